@@ -543,8 +543,9 @@ void tier_arith(int mode, int tier, int njob, Arith *ar, int refine_x1 = 0, int 
 // tab[t][p]: arithmetic of job p for the systems in tier t; tiers_present:
 // bit t set when some active system is in tier t (the per-system tiers are in
 // h->sd.tier on the device)
+// lin: an active system's c_lin is not 0
 StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
-                   const Arith (*tab)[kMaxJobs], unsigned tiers_present) {
+                   const Arith (*tab)[kMaxJobs], unsigned tiers_present, bool lin) {
     cudaStream_t st = h->stream;
     const int NB = in.NB, b = in.b, njob = jt.njob;
     const size_t bb = (size_t)b * b;
@@ -600,9 +601,10 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
     // are large (above 4 GiB the solve's time dwarfs a re-allocation)
     const size_t big = size_t(4) << 30;
     if (!tc && in.ophi.cap * sizeof(uint16_t) > big) in.ophi.release();
+    if (!(tc && lin) && h->tcw.xlin.cap * sizeof(float) > big) h->tcw.xlin.release();
     if (!f32_planes && in.opf32.cap * sizeof(float) > big) in.opf32.release();
     if (!any_c[1] && in.opf32lo.cap * sizeof(float) > big) in.opf32lo.release();
-    if (tc) prepare_operands(in, tc_ar, h->tcw, st);
+    if (tc) prepare_operands(in, tc_ar, lin, h->tcw, st);
     if (any_oz) prepare_oz_operands(in, h->ozw, st);
     else if (h->ozw.slices.cap * sizeof(uint16_t) > big) h->ozw.slices.release();
     if (f32_planes) {
@@ -988,7 +990,7 @@ void set_products(rdm_handle *h, MatSet &in, const JobTable &jt, const std::vect
     h2d(h->sd.tier.p, zero.data(), S, h->stream);
     Arith tab[kMaxTiers][kMaxJobs];
     for (int p = 0; p < kMaxJobs; ++p) tab[0][p] = ar;
-    multiply(h, in, out, jt, tab, 1u);
+    multiply(h, in, out, jt, tab, 1u, std::any_of(cl.begin(), cl.end(), [](double c) { return c != 0.0; }));
 }
 
 // the same with one coefficient pair, in FP64
@@ -1360,6 +1362,8 @@ int run_solve(rdm_handle *h, rdm_info *info_out) {
                 for (int p = 0; p < jt.njob; ++p) ar[p] = tab[t][p];
                 break;
             }
+        bool lin = false;     // an active system has a linear term
+        for (int s = 0; s < S; ++s) lin = lin || (act[s] && c_lin[s] != 0.0);
         h2d(h->sd.tier.p, tier_of.data(), S, st);
         h2d(h->sd.c_lin.p, c_lin.data(), S, st);
         h2d(h->sd.c_sq.p, c_sq.data(), S, st);
@@ -1368,7 +1372,7 @@ int run_solve(rdm_handle *h, rdm_info *info_out) {
         h2d(h->sd.active.p, act.data(), S, st);
         RDM_CUDA_TRY(cudaEventRecord(ev0, st));
         MatSet &Xn = h->X[1 - h->cur];
-        StepStats sst = multiply(h, Xc, Xn, jt, tab, tiers_present);
+        StepStats sst = multiply(h, Xc, Xn, jt, tab, tiers_present, lin);
         RDM_CUDA_TRY(cudaEventRecord(ev1, st));
         RDM_CUDA_TRY(cudaEventSynchronize(ev1));
         float ms = 0;
@@ -1838,6 +1842,7 @@ void release_work(rdm_handle *h) {
     h->tcw.tile_cnt.release();
     h->tcw.tile_off.release();
     h->tcw.zero.release();
+    h->tcw.xlin.release();
     h->pool_cap_hint = 0;
     h->solved = false;
 }
@@ -2420,7 +2425,7 @@ int rdm_block_product(rdm_handle *h, const rdm_bsr *A, const rdm_bsr *B, const r
         if (slices) tab[0][0] = AR_OZ;
         else tier_arith(mode, 0, jt.njob, tab[0]);
         MatSet res;
-        multiply(&t, in, res, jt, tab, 1u);
+        multiply(&t, in, res, jt, tab, 1u, c_lin != 0.0);
         int64_t n = res.nnzb[0];
         if (needed) *needed = n;
         if (!out || !out->row_ptr || out->nnzb < n || (n && (!out->col_idx || !out->vals))) {

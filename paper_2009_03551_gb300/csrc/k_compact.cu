@@ -4,6 +4,7 @@
 // the upper triangle and the copy writes each lower block as the transpose
 // of its upper partner.  Also builds the work list of upper-triangle output
 // blocks for the numeric phase.
+#include "fp_bits.cuh"
 #include "rdm_internal.cuh"
 
 #include <algorithm>
@@ -85,7 +86,7 @@ __global__ void k_compact_count(CompactArgs c, int *cnt) {
     int n = 0;
     for (int p = c.out_rp[r] + lane; p < c.out_rp[r + 1]; p += 32) {
         const bool up = c.out_col[p] >= c.slot_row[p];
-        n += c.keep[up ? p : c.slot_t[p]] ? 1 : 0;
+        n += c.keep[up ? p : c.slot_t[p]] & kKeepBlock;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
@@ -108,7 +109,7 @@ __global__ void k_compact_index(CompactArgs c) {
         if (p < rend) {
             up = c.out_col[p] >= c.slot_row[p];
             src = up ? p : c.slot_t[p];
-            k = c.keep[src] != 0;
+            k = (c.keep[src] & kKeepBlock) != 0;
         }
         const unsigned m = __ballot_sync(0xffffffffu, k);
         if (k) {
@@ -123,16 +124,47 @@ __global__ void k_compact_index(CompactArgs c) {
 }
 
 // one CTA per kept block (grid-stride): upper blocks are copied, lower ones
-// transposed through shared memory (b x (b+1) doubles) from their upper
-// partner, which is in this group's buffer or already compacted
+// are the transpose of their upper partner, which is in this group's buffer or
+// already compacted.  FP32 blocks of the buffer are widened: 12 bytes move per
+// element instead of 16, and either orientation reads its source in whole
+// sectors, a warp at a time, so only FP64 sources are transposed through
+// shared memory (b x (b+1) doubles).
 __global__ void __launch_bounds__(128) k_compact_vals(CompactArgs c, int d1) {
     extern __shared__ double tile[];
     const int b = c.b, bb = b * b, ld = b + 1;
     for (int d = c.d0 + blockIdx.x; d < d1; d += gridDim.x) {
         const int p = c.src[d - c.d0];
         double *out = c.new_val + (size_t)d * bb;
-        if (c.out_col[p] >= c.slot_row[p]) {
-            const double *s = c.out_val + (size_t)(c.uidx[p] - c.u0) * bb;
+        const bool up = c.out_col[p] >= c.slot_row[p];
+        const int t = up ? p : c.slot_t[p];
+        const int ut = c.uidx[t];
+        const bool here = ut >= c.u0;
+        const double *s = here ? c.out_val + (size_t)(ut - c.u0) * bb : c.new_val + (size_t)c.dest[t] * bb;
+        if (here && (c.keep[t] & kBlockF32)) {
+            const float4 *f = reinterpret_cast<const float4 *>(s);
+            const int q4 = b >> 2;
+            if (up) {
+                // a thread widens 4 columns of a row: the threads of a row are neighbours
+                for (int e = threadIdx.x; e < bb / 4; e += blockDim.x) {
+                    const int r = e / q4, c4 = e % q4;
+                    const float4 v = f[c4 * b + r];
+                    double2 *o = reinterpret_cast<double2 *>(out + r * b + 4 * c4);
+                    o[0] = make_double2(f32_to_f64(v.x), f32_to_f64(v.y));
+                    o[1] = make_double2(f32_to_f64(v.z), f32_to_f64(v.w));
+                }
+            } else {
+                // 4 source columns of source row k are column k of 4 output rows
+                for (int e = threadIdx.x; e < bb / 4; e += blockDim.x) {
+                    const int k = e % b, c4 = e / b;
+                    const float4 v = f[c4 * b + k];
+                    double *o = out + 4 * c4 * b + k;
+                    o[0] = f32_to_f64(v.x);
+                    o[b] = f32_to_f64(v.y);
+                    o[2 * b] = f32_to_f64(v.z);
+                    o[3 * b] = f32_to_f64(v.w);
+                }
+            }
+        } else if (up) {
             if ((bb & 1) == 0) {
                 const double2 *s2 = reinterpret_cast<const double2 *>(s);
                 double2 *o2 = reinterpret_cast<double2 *>(out);
@@ -141,10 +173,6 @@ __global__ void __launch_bounds__(128) k_compact_vals(CompactArgs c, int d1) {
                 for (int e = threadIdx.x; e < bb; e += blockDim.x) out[e] = s[e];
             }
         } else {
-            const int t = c.slot_t[p];
-            const int ut = c.uidx[t];
-            const double *s = ut >= c.u0 ? c.out_val + (size_t)(ut - c.u0) * bb
-                                         : c.new_val + (size_t)c.dest[t] * bb;
             for (int e = threadIdx.x; e < bb; e += blockDim.x) tile[(e / b) * ld + (e % b)] = s[e];
             __syncthreads();
             for (int e = threadIdx.x; e < bb; e += blockDim.x) out[e] = tile[(e % b) * ld + (e / b)];

@@ -13,6 +13,7 @@
 // operand blocks of each pair are staged in shared memory, each thread owns
 // ceil(b^2 / threads) outputs.  On GB300 the FP64 rate is the bound of this
 // kernel; the FP32 variant converts the FP64 master values on load.
+#include "fp_bits.cuh"
 #include "rdm_internal.cuh"
 
 #include <algorithm>
@@ -437,7 +438,7 @@ __global__ void __launch_bounds__(64, 8) k_numeric_f32_t84(NumArgs a) {
         for (int e = tid; e < 1024; e += 64) {
             const int r = e >> 5, c = e & 31, o = r * kF32Ld + c;
             float x = cq * (sA[0][o] + sA[1][o]);
-            if (gx) x = fmaf(cl, (float)gx[e], x);
+            if (gx) x = fmaf(cl, f64_to_f32(gx[e]), x);
             sC[r * 33 + c] = x;
         }
         __syncthreads();
@@ -464,11 +465,14 @@ __global__ void __launch_bounds__(64, 8) k_numeric_f32_t84(NumArgs a) {
         __syncthreads();
         const float nrm = sqrtf(red[0] + red[1]) * (1.0f + 1e-6f);
         const bool keep = ((double)nrm >= tau) && (nrm > 0.f);
-        double *o = a.out_val + (size_t)(a.uidx[s] - a.u0) * 1024;
-        for (int e = tid; e < 1024; e += 64) o[e] = (double)sC[(e >> 5) * 33 + (e & 31)];
+        float4 *o = reinterpret_cast<float4 *>(a.out_val + (size_t)(a.uidx[s] - a.u0) * 1024);
+        for (int e = tid; e < 256; e += 64) {      // layout f32_index: 4 columns of row e % 32
+            const float *x = &sC[(e & 31) * 33 + 4 * (e >> 5)];
+            o[e] = make_float4(x[0], x[1], x[2], x[3]);
+        }
         if (tid == 0) {
             a.out_nrm[s] = nrm;
-            a.keep[s] = keep;
+            a.keep[s] = (keep ? kKeepBlock : 0) | kBlockF32;
         }
     }
 }
@@ -478,9 +482,9 @@ __global__ void k_split_f32(const double *__restrict__ v, float *__restrict__ hi
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= n) return;
     const double x = v[e];
-    const float h = (float)x;
+    const float h = f64_to_f32(x);
     hi[e] = h;
-    if (lo) lo[e] = (float)(x - (double)h);
+    if (lo) lo[e] = f64_to_f32(x - f32_to_f64(h));
 }
 
 

@@ -65,6 +65,7 @@
 
 #include <algorithm>
 
+#include "fp_bits.cuh"
 #include "tc_gemm.cuh"
 #include "tc_plan.cuh"
 #include "tc_ptx.cuh"
@@ -178,10 +179,13 @@ __global__ void k_matrix_scales(const unsigned *__restrict__ mxbits, int nmat, i
 
 // one thread per 8 consecutive elements of a block row (one core-matrix row):
 // 64 bytes of FP64 in, 16 bytes of hi and 16 bytes of lo out
+// and, with xlin, the FP32 values of the upper blocks for the linear term, in
+// the layout of f32_index (32 bytes)
 template <bool BF16, int B>
 __global__ void k_split_planes(const double *__restrict__ val, int64_t nblk, uint16_t *__restrict__ hi,
                                const float *__restrict__ scale,
-                               const int *__restrict__ mat_first, int nmat, const int *__restrict__ tpos) {
+                               const int *__restrict__ mat_first, int nmat, const int *__restrict__ tpos,
+                               float *__restrict__ xlin) {
     constexpr int kPE = B * B;
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= nblk * (kPE / 8)) return;
@@ -193,13 +197,20 @@ __global__ void k_split_planes(const double *__restrict__ val, int64_t nblk, uin
     const float sc = scale[m];
     const double2 *v2 = reinterpret_cast<const double2 *>(val + p * kPE + rc0);
     uint16_t h[8], l[8];
+    double2 x2[4];
+    float xf[8];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) x2[k] = v2[k];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const double2 x2 = v2[k];
-        const float xs[2] = {(float)x2.x * sc, (float)x2.y * sc};
+        xf[2 * k] = f64_to_f32(x2[k].x);
+        xf[2 * k + 1] = f64_to_f32(x2[k].y);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-            const float x = xs[u];
+            const float x = xf[2 * k + u] * sc;
             if (BF16) {
                 const __nv_bfloat16 bh = __float2bfloat16_rn(x);
                 const __nv_bfloat16 bl = __float2bfloat16_rn(x - __bfloat162float(bh));
@@ -223,6 +234,11 @@ __global__ void k_split_planes(const double *__restrict__ val, int64_t nblk, uin
     // its own position without one
     const int64_t at = tpos ? (int64_t)tpos[p] : p;
     if (at < 0) return;
+    if (xlin && at >= p) {      // the transposed block of an upper block comes later
+        float *x = xlin + p * kPE;
+        *reinterpret_cast<float4 *>(x + f32_index(B, r, c0)) = make_float4(xf[0], xf[1], xf[2], xf[3]);
+        *reinterpret_cast<float4 *>(x + f32_index(B, r, c0 + 4)) = make_float4(xf[4], xf[5], xf[6], xf[7]);
+    }
     uint16_t *o = hi + at * (2 * kPE);
     *reinterpret_cast<uint4 *>(o + pair_offset<B>(r, c0, 0)) = hv;
     *reinterpret_cast<uint4 *>(o + pair_offset<B>(r, c0, 1)) = lv;
@@ -270,12 +286,13 @@ struct TcArgs {
     const float *scale;           // per matrix operand scale
     int job_a[kMaxJobs], job_b[kMaxJobs];
     // epilogue
-    const double *in_val;
+    const float *xlin;      // FP32 values of the input set's upper blocks, layout f32_index, or null:
+    const double *in_val;   // the FP64 values
     const int *slot_row, *slot_job, *slot_x, *slot_t;
     const int *sys_of_row;
     const double *c_lin, *c_sq, *tau0, *tau1;
     int job_tau_sel[kMaxJobs];
-    double *out_val;        // upper slot s at index uidx[s] - u0
+    double *out_val;        // upper slot s at index uidx[s] - u0, FP32 in layout f32_index
     float *out_nrm;
     uint8_t *keep;
     const int *uidx;
@@ -352,8 +369,8 @@ __device__ __forceinline__ void prefetch_old_blocks(const TcArgs &A, int tn, int
     if (s < 0) return;
     const int sx = A.slot_x[s];
     if (sx < 0 || A.c_lin[A.sys_of_row[A.slot_row[s]]] == 0.0) return;
-    const double *px = A.in_val + (size_t)sx * (B * B);
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(px), "r"(8 * B * B) : "memory");
+    const void *px = A.xlin ? (const void *)(A.xlin + (size_t)sx * (B * B)) : (const void *)(A.in_val + (size_t)sx * (B * B));
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(px), "r"((A.xlin ? 4 : 8) * B * B) : "memory");
 }
 
 // b = 64: one step of the handshake of the two epilogue warps that share a
@@ -590,30 +607,33 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
                     const bool diag = __float_as_int(q[2 * MW]) != 0;
                     const int oidx = __float_as_int(q[3 * MW]);
                     __syncwarp();
-                    // linear term: the old block is staged in S (coalesced row reads,
-                    // rounded to FP32), then each lane takes its own row
-                    if (sx >= 0 && cl != 0.f) {
-                        const double *gx = A.in_val + (size_t)sx * G::kPlaneElems;
-#pragma unroll 8
-                        for (int r = 0; r < 32; ++r) S[r * 33 + lane] = (float)gx[r * 32 + lane];
-                        __syncwarp();
+                    // linear term: four columns of the lane's row at a time, 512
+                    // contiguous bytes for the warp (f32_index)
+                    if (sx >= 0 && cl != 0.f && !A.xlin) {
+                        const double *gx = A.in_val + (size_t)sx * G::kPlaneElems + lane * 32;
 #pragma unroll
-                        for (int c = 0; c < 32; ++c) acc[c] = fmaf(cl, S[lane * 33 + c], cq * acc[c]);
-                        __syncwarp();
+                        for (int c = 0; c < 32; ++c) acc[c] = fmaf(cl, (float)gx[c], cq * acc[c]);
+                    } else if (sx >= 0 && cl != 0.f) {
+                        const float4 *gx = reinterpret_cast<const float4 *>(A.xlin + (size_t)sx * G::kPlaneElems) + lane;
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) {
+                            const float4 x = gx[c * 32];
+                            acc[4 * c] = fmaf(cl, x.x, cq * acc[4 * c]);
+                            acc[4 * c + 1] = fmaf(cl, x.y, cq * acc[4 * c + 1]);
+                            acc[4 * c + 2] = fmaf(cl, x.z, cq * acc[4 * c + 2]);
+                            acc[4 * c + 3] = fmaf(cl, x.w, cq * acc[4 * c + 3]);
+                        }
                     } else {
 #pragma unroll
                         for (int c = 0; c < 32; ++c) acc[c] = cq * acc[c];
                     }
                     // a diagonal block is symmetrised as (X + X^T) / 2
-#pragma unroll
-                    for (int c = 0; c < 32; ++c) S[lane * 33 + c] = acc[c];
-                    __syncwarp();
                     if (diag) {
 #pragma unroll
-                        for (int c = 0; c < 32; ++c) acc[c] = 0.5f * (S[lane * 33 + c] + S[c * 33 + lane]);
+                        for (int c = 0; c < 32; ++c) S[lane * 33 + c] = acc[c];
                         __syncwarp();
 #pragma unroll
-                        for (int c = 0; c < 32; ++c) S[lane * 33 + c] = acc[c];
+                        for (int c = 0; c < 32; ++c) acc[c] = 0.5f * (acc[c] + S[c * 33 + lane]);
                         __syncwarp();
                     }
                     float ss = 0.f;
@@ -623,13 +643,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
                     for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
                     const float nrm = sqrtf(ss) * (1.0f + 1e-6f);
                     const bool kp = ((double)nrm >= tau) && (nrm > 0.f);
-                    double *o = A.out_val + (size_t)oidx * G::kPlaneElems;
-                    for (int r = 0; r < 32; ++r) o[r * 32 + lane] = (double)S[r * 33 + lane];
+                    float4 *o = reinterpret_cast<float4 *>(A.out_val + (size_t)oidx * G::kPlaneElems) + lane;
+#pragma unroll
+                    for (int c = 0; c < 8; ++c)
+                        o[c * 32] = make_float4(acc[4 * c], acc[4 * c + 1], acc[4 * c + 2], acc[4 * c + 3]);
                     if (lane == 0) {
                         A.out_nrm[s] = nrm;
-                        A.keep[s] = kp;
+                        A.keep[s] = (kp ? kKeepBlock : 0) | kBlockF32;
                     }
-                    __syncwarp();
                 }
             } else if constexpr (B == 16) {
                 // half-warp h = lane / 16 holds rows of block row 2 eq + h: lane l
@@ -647,31 +668,35 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
                     const int oidx = __float_as_int(q[3 * MW]);
                     const bool lin = s >= 0 && sx >= 0 && cl != 0.f;
                     float acc[16];
-                    __syncwarp();
-                    if (lin) {
-                        const double *gx = A.in_val + (size_t)sx * G::kPlaneElems;
+                    if (lin && !A.xlin) {
+                        const double *gx = A.in_val + (size_t)sx * G::kPlaneElems + c16 * 16;
 #pragma unroll
-                        for (int r = 0; r < 16; ++r) S[(16 * h + r) * 33 + c16] = (float)gx[r * 16 + c16];
+                        for (int c = 0; c < 16; ++c) acc[c] = fmaf(cl, (float)gx[c], cq * racc[n * 16 + c]);
+                    } else if (lin) {
+                        const float4 *gx = reinterpret_cast<const float4 *>(A.xlin + (size_t)sx * G::kPlaneElems) + c16;
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            const float4 x = gx[c * 16];
+                            acc[4 * c] = fmaf(cl, x.x, cq * racc[n * 16 + 4 * c]);
+                            acc[4 * c + 1] = fmaf(cl, x.y, cq * racc[n * 16 + 4 * c + 1]);
+                            acc[4 * c + 2] = fmaf(cl, x.z, cq * racc[n * 16 + 4 * c + 2]);
+                            acc[4 * c + 3] = fmaf(cl, x.w, cq * racc[n * 16 + 4 * c + 3]);
+                        }
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < 16; ++c) acc[c] = cq * racc[n * 16 + c];
                     }
-                    __syncwarp();
-#pragma unroll
-                    for (int c = 0; c < 16; ++c)
-                        acc[c] = lin ? fmaf(cl, S[lane * 33 + c], cq * racc[n * 16 + c]) : cq * racc[n * 16 + c];
-                    __syncwarp();
-#pragma unroll
-                    for (int c = 0; c < 16; ++c) S[lane * 33 + c] = acc[c];
-                    __syncwarp();
                     // a diagonal block is symmetrised as (X + X^T) / 2
-                    if (diag) {
-#pragma unroll
-                        for (int c = 0; c < 16; ++c) acc[c] = 0.5f * (S[lane * 33 + c] + S[(16 * h + c) * 33 + c16]);
-                    }
-                    __syncwarp();
-                    if (diag) {
+                    if (__any_sync(0xffffffffu, diag)) {
 #pragma unroll
                         for (int c = 0; c < 16; ++c) S[lane * 33 + c] = acc[c];
+                        __syncwarp();
+                        if (diag) {
+#pragma unroll
+                            for (int c = 0; c < 16; ++c) acc[c] = 0.5f * (acc[c] + S[(16 * h + c) * 33 + c16]);
+                        }
+                        __syncwarp();
                     }
-                    __syncwarp();
                     float ss = 0.f;
 #pragma unroll
                     for (int c = 0; c < 16; ++c) ss = fmaf(acc[c], acc[c], ss);
@@ -680,15 +705,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
                     const float nrm = sqrtf(ss) * (1.0f + 1e-6f);
                     const bool kp = ((double)nrm >= tau) && (nrm > 0.f);
                     if (s >= 0) {
-                        double *o = A.out_val + (size_t)oidx * G::kPlaneElems;
+                        float4 *o = reinterpret_cast<float4 *>(A.out_val + (size_t)oidx * G::kPlaneElems) + c16;
 #pragma unroll
-                        for (int r = 0; r < 16; ++r) o[r * 16 + c16] = (double)S[(16 * h + r) * 33 + c16];
+                        for (int c = 0; c < 4; ++c)
+                            o[c * 16] = make_float4(acc[4 * c], acc[4 * c + 1], acc[4 * c + 2], acc[4 * c + 3]);
                         if (c16 == 0) {
                             A.out_nrm[s] = nrm;
-                            A.keep[s] = kp;
+                            A.keep[s] = (kp ? kKeepBlock : 0) | kBlockF32;
                         }
                     }
-                    __syncwarp();
                 }
             } else {
                 // b = 64: lane l holds row 32 rh + l of 2 blocks of 64 columns; the
@@ -708,22 +733,26 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
                     const int sx = __float_as_int(q[1 * MW]);
                     const bool diag = __float_as_int(q[2 * MW]) != 0;
                     const int oidx = __float_as_int(q[3 * MW]);
-                    // linear term, one 32-column half of the old rows at a time
+                    // linear term: four columns of the lane's row at a time
+                    if (sx >= 0 && cl != 0.f && !A.xlin) {
+                        const double *gx = A.in_val + (size_t)sx * G::kPlaneElems + (size_t)(32 * rh + lane) * 64;
 #pragma unroll
-                    for (int ch = 0; ch < 2; ++ch) {
-                        __syncwarp();
-                        if (sx >= 0 && cl != 0.f) {
-                            const double *gx = A.in_val + (size_t)sx * G::kPlaneElems + (size_t)(32 * rh) * 64 + 32 * ch;
-#pragma unroll 8
-                            for (int r = 0; r < 32; ++r) S[r * 33 + lane] = (float)gx[r * 64 + lane];
-                            __syncwarp();
+                        for (int c = 0; c < 64; ++c)
+                            racc[n * 64 + c] = fmaf(cl, (float)gx[c], cq * racc[n * 64 + c]);
+                    } else if (sx >= 0 && cl != 0.f) {
+                        const float4 *gx = reinterpret_cast<const float4 *>(A.xlin + (size_t)sx * G::kPlaneElems) + 32 * rh + lane;
 #pragma unroll
-                            for (int c = 0; c < 32; ++c)
-                                racc[n * 64 + 32 * ch + c] = fmaf(cl, S[lane * 33 + c], cq * racc[n * 64 + 32 * ch + c]);
-                        } else {
-#pragma unroll
-                            for (int c = 0; c < 32; ++c) racc[n * 64 + 32 * ch + c] = cq * racc[n * 64 + 32 * ch + c];
+                        for (int c = 0; c < 16; ++c) {
+                            const float4 x = gx[c * 64];
+                            float *a4 = racc + n * 64 + 4 * c;
+                            a4[0] = fmaf(cl, x.x, cq * a4[0]);
+                            a4[1] = fmaf(cl, x.y, cq * a4[1]);
+                            a4[2] = fmaf(cl, x.z, cq * a4[2]);
+                            a4[3] = fmaf(cl, x.w, cq * a4[3]);
                         }
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < 64; ++c) racc[n * 64 + c] = cq * racc[n * 64 + c];
                     }
                     if (diag) {
                         // (X + X^T) / 2: the off-diagonal quarter (rh, 1 - rh) pairs with
@@ -774,19 +803,16 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
                     const float tot = rh == 0 ? ss + other : other + ss;
                     const float nrm = sqrtf(tot) * (1.0f + 1e-6f);
                     const bool kp = ((double)nrm >= tau) && (nrm > 0.f);
-                    // store this warp's 32 rows, one 32-column half at a time
-                    double *o = A.out_val + (size_t)oidx * G::kPlaneElems + (size_t)(32 * rh) * 64;
+                    // store this warp's 32 rows
+                    float4 *o = reinterpret_cast<float4 *>(A.out_val + (size_t)oidx * G::kPlaneElems) + 32 * rh + lane;
 #pragma unroll
-                    for (int ch = 0; ch < 2; ++ch) {
-                        __syncwarp();
-#pragma unroll
-                        for (int c = 0; c < 32; ++c) S[lane * 33 + c] = racc[n * 64 + 32 * ch + c];
-                        __syncwarp();
-                        for (int r = 0; r < 32; ++r) o[r * 64 + 32 * ch + lane] = (double)S[r * 33 + lane];
+                    for (int c = 0; c < 16; ++c) {
+                        const float *a4 = racc + n * 64 + 4 * c;
+                        o[c * 64] = make_float4(a4[0], a4[1], a4[2], a4[3]);
                     }
                     if (lane == 0 && rh == 0) {
                         A.out_nrm[s] = nrm;
-                        A.keep[s] = kp;
+                        A.keep[s] = (kp ? kKeepBlock : 0) | kBlockF32;
                     }
                     // the partner reuses pair_ss and its S only after this point
                     ok = pair_sync(ctl, pr, pround, lane, abort_flag, A.wait_cycles) && ok;
@@ -822,10 +848,10 @@ void split_planes(MatSet &in, Arith ar, TcWork &w, cudaStream_t st) {
     const int *tpos = w.tpos_valid ? w.tpos.p : nullptr;
     if (ar == AR_BF16X3)
         k_split_planes<true, B><<<(unsigned)grid, 256, 0, st>>>(in.val.p, in.total, in.ophi.p, w.scale.p,
-                                                                w.mat_first.p, in.nmat, tpos);
+                                                                w.mat_first.p, in.nmat, tpos, w.lin ? w.xlin.p : nullptr);
     else
         k_split_planes<false, B><<<(unsigned)grid, 256, 0, st>>>(in.val.p, in.total, in.ophi.p, w.scale.p,
-                                                                 w.mat_first.p, in.nmat, tpos);
+                                                                 w.mat_first.p, in.nmat, tpos, w.lin ? w.xlin.p : nullptr);
     RDM_LAUNCH_CHECK();
 }
 
@@ -852,7 +878,7 @@ double launch_tc(const NumArgs &a, const MatSet &in, const JobTable &jt, Arith a
         A.job_a[p] = p < jt.njob ? jt.job[p].a[0] : 0;
         A.job_b[p] = p < jt.njob ? jt.job[p].b[0] : 0;
     }
-    A.in_val = a.in_val; A.slot_row = a.slot_row; A.slot_job = a.slot_job; A.slot_x = a.slot_x;
+    A.xlin = w.lin ? w.xlin.p : nullptr; A.in_val = a.in_val; A.slot_row = a.slot_row; A.slot_job = a.slot_job; A.slot_x = a.slot_x;
     A.slot_t = a.slot_t; A.sys_of_row = a.sys_of_row; A.c_lin = a.c_lin; A.c_sq = a.c_sq;
     A.tau0 = a.tau0; A.tau1 = a.tau1;
     for (int p = 0; p < kMaxJobs; ++p) A.job_tau_sel[p] = a.job_tau_sel[p];
@@ -875,9 +901,10 @@ bool tc_block_size_ok(int b) { return b == 16 || b == 32 || b == 64; }
 
 int tc_tile_rows(int b) { return tc_block_size_ok(b) ? 128 / b : 4; }
 
-void prepare_operands(MatSet &in, Arith ar, TcWork &w, cudaStream_t st) {
+void prepare_operands(MatSet &in, Arith ar, bool lin, TcWork &w, cudaStream_t st) {
     if (!tc_block_size_ok(in.b)) throw Error{-1, "the tensor-core path handles 16 x 16, 32 x 32 and 64 x 64 blocks"};
     if (ar != AR_BF16X3 && ar != AR_FP16X3) throw Error{-1, "tensor-core arithmetic not available"};
+    w.lin = lin;
     const int nmat = in.nmat;
     std::vector<int> first(nmat + 1, 0);
     for (int m = 0; m < nmat; ++m) first[m + 1] = first[m] + (int)in.nnzb[m];
@@ -895,6 +922,12 @@ void prepare_operands(MatSet &in, Arith ar, TcWork &w, cudaStream_t st) {
     RDM_LAUNCH_CHECK();
     const int64_t n = in.total * (int64_t)in.b * in.b;
     in.ophi.ensure(std::max<int64_t>(2 * n, 1));   // hi and lo, interleaved per block
+    if (w.lin && w.xlin.cap < (size_t)n) {
+        size_t fr = 0, tot = 0;
+        RDM_CUDA_TRY(cudaMemGetInfo(&fr, &tot));
+        if ((size_t)n * sizeof(float) > (fr + w.xlin.cap * sizeof(float)) / 4) w.lin = false;
+        else w.xlin.ensure((size_t)n);
+    }
     w.pre_err.ensure(1);
     RDM_CUDA_TRY(cudaMemsetAsync(w.pre_err.p, 0, sizeof(int), st));
     w.tpos_valid = false;

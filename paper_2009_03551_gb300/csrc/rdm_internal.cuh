@@ -257,6 +257,16 @@ void launch_pairs(const MatSet &in, const JobTable &jt, const SysDev &sd, const 
                   const int64_t *pair_off, int64_t nslot, int NB, int *pair_a, int *pair_b,
                   int *slot_x, int *slot_t, int *err, cudaStream_t st, JobMask fill);
 
+// A product kernel that computes in FP32 leaves its untruncated block in FP32
+// (kBlockF32 in the slot's keep byte) and the compaction widens it: element
+// (r, c) of the b x b block at this index of the slot.  Four columns of a row
+// are adjacent and the rows follow, so that a lane that holds a row writes 16
+// bytes beside its neighbours', and the compaction reads the block's rows and
+// its columns (for the transposed block) equally well.  The FP32 copies of
+// the old blocks for the linear terms have the same layout.
+constexpr uint8_t kKeepBlock = 1, kBlockF32 = 2;
+__host__ __device__ inline int f32_index(int b, int r, int c) { return ((c >> 2) * b + r) * 4 + (c & 3); }
+
 // k_numeric.cu: C(upper slot) = c_lin X + c_sq sum(pairs); lower slot = transpose
 struct NumArgs {
     const double *in_val;
@@ -276,7 +286,8 @@ struct NumArgs {
     // outputs: only upper-triangle slots (col >= row) are computed; the
     // values of upper slot s go to out_val at index uidx[s] - u0 (uidx: rank
     // of s among the upper slots, u0: that of the group's first one);
-    // norm bound and keep flag to out_nrm[s], keep[s]
+    // (b*b doubles apart; FP64, or FP32 as kBlockF32 says), norm bound and
+    // keep flag to out_nrm[s], keep[s]
     double *out_val;
     float *out_nrm;
     uint8_t *keep;

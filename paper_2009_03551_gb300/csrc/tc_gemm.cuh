@@ -32,6 +32,8 @@ struct TcWork {
     DevBuf<int> mat_first;      // per matrix: first global block index (nmat+1)
     DevBuf<int> tpos;           // per block (i, k) of the input set: global index of block (k, i)
     DevBuf<int> pre_err;        // error bits of the operand preparation (8: a transposed block missing)
+    DevBuf<float> xlin;         // FP32 values of the input set's upper blocks (layout f32_index)
+    bool lin = false;           // xlin is filled for this step
     bool tpos_valid = false;    // the planes sit at tpos and the K-step lists point there
 };
 
@@ -59,7 +61,7 @@ int tc_tile_rows(int b);
 // every matrix is first scaled by a power of two (from its largest block
 // norm) so that its values sit in the normal range of fp16; the product
 // kernel divides the scale back out per job.
-void prepare_operands(MatSet &in, Arith ar, TcWork &w, cudaStream_t st);
+void prepare_operands(MatSet &in, Arith ar, bool lin, TcWork &w, cudaStream_t st);
 
 // Tile lists of one multiplication step from the output mask, for the jobs
 // selected by job_mask (per system tier) and the super-row units
