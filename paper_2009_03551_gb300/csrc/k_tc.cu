@@ -25,26 +25,31 @@
 // groups of a block's hi and lo planes alternating (16 b bytes each, 32 b
 // bytes between the groups of one plane): one bulk copy of 4 b^2 bytes per
 // block lands both planes ready for the MMA, and blocks stacked in a stage
-// continue the same stride, so that a side of a K-step is one operand.  A
-// streaming probe (one CTA per SM, no MMA) moves at most ~6.5 TB/s over the
-// GPU in 4 KB bulk copies, from L2 as from DRAM, and ~7.4-8.9 TB/s in
-// 16-32 KB copies: the rate of such copies into each SM bounds this kernel.
-// So the planes of the operand block (i, k) are stored at the position of
+// continue the same stride, so that a side of a K-step is one operand.
+// Bulk copies fill an SM's shared memory at up to 70 bytes per clock from L2,
+// less ~54 clocks per copy (measured: 4 KB copies 38 bytes per clock, 12 KB
+// 57), so the planes of the operand block (i, k) are stored at the position of
 // block (k, i) (the patterns are symmetric): the A blocks (i_0..i_3, k) of a
 // K-step are then neighbours in block row k, and so are its B blocks
-// (j_0..j_7, k) wherever row k holds them all, and the copy warp moves every
+// (j_0..j_7, k) wherever row k holds them all, and a copy warp moves every
 // run of slots whose blocks are neighbours in memory with one copy.
 //
-// Warp roles (320 threads, one CTA per SM, persistent over a static tile
-// schedule, tiles round robin): warp 0 issues the bulk copies into a ring of stages, warp 1
-// owns the tensor-memory allocation and one thread issues the MMAs, warps
-// 2-9 (two per TMEM lane quarter, 128 accumulator columns each) run the
-// epilogue.  Ten warps put three on some SM sub-partitions, which caps a
-// thread at 168 registers: the epilogue keeps its 128 accumulators in
-// registers and parks the tile metadata in shared memory.  At b = 64 an
-// output block spans two lane quarters, so the two warps that share its
-// columns combine their halves (norm, transpose of diagonal blocks) through
-// shared memory, synchronised by a bounded mbarrier handshake.
+// Warp roles (384 threads, one CTA per SM, persistent over a static tile
+// schedule, tiles round robin): warps 0 and 2 issue the bulk copies into a
+// ring of stages, every second K-step each, warp 1 owns the tensor-memory
+// allocation and one thread issues the MMAs, warps 4-11 (two per TMEM lane
+// quarter, 128 accumulator columns each) run the epilogue.  Two copy warps,
+// because finding and issuing a K-step's ~3.5 copies keeps one busy for 930
+// clocks (index load, ballots, ~100 per copy), longer than the K-step's MMAs
+// (768): with one, a K-step of the 2,000-atom cluster took 1,158 clocks, with
+// two 1,026 (919 where the operands stay in L2), and the MMA thread's wait for
+// a stage fell from 495 to 313 clocks, what L2 misses leave.  Twelve warps put
+// three on every SM sub-partition, which allows a thread 168 registers: the
+// epilogue keeps its 128 accumulators in registers and the tile metadata in
+// shared memory, gathered a tile ahead.  At b = 64 an output block spans two
+// lane quarters, so the two warps that share its columns combine their halves
+// (norm, transpose of diagonal blocks) through shared memory, synchronised by
+// a bounded mbarrier handshake.
 //
 // Accumulation in segments.  The tensor cores' FP32 accumulation truncates
 // (it is not round-to-nearest), so a long accumulation chain drifts towards
@@ -56,7 +61,13 @@
 // buffer.  The drift is then that of one segment (-7e-7 relative),
 // independent of the tile's length.  After the last segment:
 // C = c_lin X + c_sq D, diagonal blocks symmetrised, block Frobenius norm,
-// truncation flag, FP64 store of the (upper-triangle) block; the old X
+// truncation flag, and the (upper-triangle) block is stored in FP32, 512
+// contiguous bytes per warp instruction straight from the registers
+// (f32_index); the linear term reads an FP32 copy of X of the same layout.
+// Neither goes through FP64 here: conversions between FP32 and FP64 run at 2
+// per clock and SM on this part, and a tile has 32,768 of each (the FP64
+// version's epilogue held up the MMAs of the next tile: 75 against 64 ms of
+// products for the 2,000-atom cluster in the bf16 ladder).  The old X
 // blocks of the next tile's linear terms are prefetched into L2 two segments
 // before this tile ends.  Every wait is bounded: on timeout the kernel raises
 // an error flag, drains what it issued and frees its tensor memory.
@@ -81,7 +92,7 @@ struct Geo : PlanGeo<128 / B, 256 / B> {
     static constexpr int kPairBytes = 4 * B * B;        // hi and lo planes of one block, interleaved
     static constexpr int kSideABytes = P::TBM * kPairBytes;     // A side of a stage: TBM blocks stacked
     static constexpr int kStageBytes = P::kSlots * kPairBytes;  // A side, then the TBN blocks of the B side
-    static constexpr int kStages = B == 16 ? 7 : B == 32 ? 4 : 2;   // fit checked below
+    static constexpr int kStages = B == 16 ? 8 : B == 32 ? 4 : 2;   // even: one producer per parity; fit checked below
     static constexpr int kSegSteps = 128 / B;           // K-steps per accumulation segment (128 K)
     static constexpr int kSub = B / 16;                 // MMAs of K = 16 per K-step and product
     static constexpr uint32_t kSBO = 32 * B;            // bytes between the 8-row groups of one plane
@@ -90,18 +101,20 @@ struct Geo : PlanGeo<128 / B, 256 / B> {
 
 constexpr int kTileN = 256;                  // MMA N = accumulator columns in tensor memory
 constexpr int kEpiWarps = 8;                 // epilogue warps: 2 per TMEM lane quarter
-constexpr int kThreads = 64 + 32 * kEpiWarps;
+constexpr int kEpiWarp0 = 4;                 // warps 0 and 2 copy, warp 1 issues the MMAs, warp 3 idles
+constexpr int kThreads = 32 * (kEpiWarp0 + kEpiWarps);
 constexpr int kSegBufs = 512 / kTileN;       // segment accumulators: the 512 TMEM columns
-// epilogue metadata per warp (8 words per output block): at b = 32 and 64
-// (4 and 2 blocks per warp) it is parked in the padding column of the warp's
-// 32 x 33 staging tile; at b = 16 (16 blocks per warp) in a region of its own
-template <int B>
-constexpr int meta_words() { return B == 16 ? 16 * 8 : 0; }
-template <int B>
-constexpr int meta_stride() { return B == 16 ? 1 : 33; }
 // output blocks whose metadata an epilogue warp holds (one lane each)
 template <int B>
 constexpr int blocks_per_warp() { return B == 16 ? 16 : B == 32 ? 4 : 2; }
+// epilogue metadata: 8 words per output block, two tiles per warp (the current
+// one and the next)
+template <int B>
+constexpr int meta_words() { return 2 * 8 * blocks_per_warp<B>(); }
+// b = 64: a 32 x 33 staging tile per epilogue warp for the diagonal blocks,
+// whose transposed quarters sit in the partner warp
+template <int B>
+constexpr int stage_words() { return B == 64 ? kEpiWarps * 32 * 33 : 0; }
 static_assert(kSegBufs >= 2 && (kSegBufs & (kSegBufs - 1)) == 0, "tile shape");
 
 // Stays 0 for the life of the program: the test setting `hold` makes the
@@ -317,9 +330,7 @@ struct __align__(8) SmemCtl {
 // Epilogue metadata of one output block, gathered by one lane while the
 // tile's MMAs run and parked in shared memory (8 words per block: slot, old
 // slot, diagonal, output index, c_lin, c_sq, tau lo, tau hi).
-template <int B>
 __device__ __forceinline__ void gather_meta(const TcArgs &A, int s, float *q) {
-    constexpr int W = meta_stride<B>();
     int m_sx = -1, m_diag = 0, m_keepidx = 0;
     float m_cl = 0.f, m_cq = 0.f;
     double m_tau = 0.0;
@@ -336,13 +347,13 @@ __device__ __forceinline__ void gather_meta(const TcArgs &A, int s, float *q) {
         m_keepidx = A.uidx[s] - (int)A.u0;
     }
     q[0] = __int_as_float(s);
-    q[W] = __int_as_float(m_sx);
-    q[2 * W] = __int_as_float(m_diag);
-    q[3 * W] = __int_as_float(m_keepidx);
-    q[4 * W] = m_cl;
-    q[5 * W] = m_cq;
-    q[6 * W] = __int_as_float(__double2loint(m_tau));
-    q[7 * W] = __int_as_float(__double2hiint(m_tau));
+    q[1] = __int_as_float(m_sx);
+    q[2] = __int_as_float(m_diag);
+    q[3] = __int_as_float(m_keepidx);
+    q[4] = m_cl;
+    q[5] = m_cq;
+    q[6] = __int_as_float(__double2loint(m_tau));
+    q[7] = __int_as_float(__double2hiint(m_tau));
 }
 
 // The output block (slot) whose metadata lane `lane` of epilogue warp
@@ -397,8 +408,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
     using G = Geo<B>;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t *stages = smem_raw;                                                    // kStages stages
-    float *stage_ep = reinterpret_cast<float *>(smem_raw + G::kStages * G::kStageBytes);   // kEpiWarps x 32 x 33
-    float *meta_all = stage_ep + kEpiWarps * 32 * 33;                              // kEpiWarps x meta_words
+    float *stage_ep = reinterpret_cast<float *>(smem_raw + G::kStages * G::kStageBytes);   // stage_words
+    float *meta_all = stage_ep + stage_words<B>();                                 // kEpiWarps x meta_words
     SmemCtl *ctl = reinterpret_cast<SmemCtl *>(meta_all + kEpiWarps * meta_words<B>());
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -426,70 +437,89 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
     fence_after();
     const uint32_t tmem = ctl->tmem_base;
 
-    if (warp == 0) {
-        // ---------------- producer: bulk copies of the operand blocks ----------------
-        // Lane m < kSlots owns slot m of every stage (slot m < TBM: A block row
-        // m, else B block row m - TBM; slot m at m * kPairBytes): it loads the
-        // block index of the next K-step while the current step's copies are
-        // issued.  A slot whose block is missing needs zeros; a stage slot that
-        // already holds zeros from its previous use is not copied again (zmask).
-        uint32_t it = 0;
+    if (warp == 0 || warp == 2) {
+        // ---------------- producers: bulk copies of the operand blocks ----------------
+        // The K-steps of the CTA's tiles are one stream; this warp (pr = 0, 1)
+        // takes every second one.  Lane m < kSlots owns slot m of every stage
+        // (slot m < TBM: A block row m, else B block row m - TBM; slot m at
+        // m * kPairBytes).  A slot whose block is missing needs zeros; a stage
+        // slot that already holds zeros from its previous use is not copied
+        // again (zmask).
+        const uint32_t pr = (uint32_t)warp >> 1;
+        uint32_t it = pr;
         bool ok = true;
-        uint32_t zmask[G::kStages];
+        uint32_t zmask[G::kStages / 2];
 #pragma unroll
-        for (int k = 0; k < G::kStages; ++k) zmask[k] = 0u;
-        for (int t = blockIdx.x; t < A.ntile && ok; t += gridDim.x) {
-            const int64_t s0 = A.step_off[t], s1 = A.step_off[t + 1];
-            int nxt = (s0 < s1 && lane < G::kSlots) ? A.steps[s0 * G::kSlots + lane] : -1;
-            for (int64_t q = s0; q < s1; ++q, ++it) {
-                const int cur = nxt;
-                if (q + 1 < s1 && lane < G::kSlots) nxt = A.steps[(q + 1) * G::kSlots + lane];
-                const int st = it % G::kStages;
-                const uint32_t ph = (it / G::kStages) & 1;
-                const uint32_t zbits = __ballot_sync(0xffffffffu, lane < G::kSlots && cur < 0);
-                uint32_t zprev = 0u;
+        for (int k = 0; k < G::kStages / 2; ++k) zmask[k] = 0u;
+        // lq < le: the next step of this warp, in tile lt; [nq, ne): the tile
+        // after it (its range is loaded a tile ahead)
+        int lt = blockIdx.x;
+        int64_t lq = 0, le = 0, nq = 0, ne = 0;
+        if (lt < A.ntile) { lq = A.step_off[lt]; le = A.step_off[lt + 1]; }
+        if (lt + (int)gridDim.x < A.ntile) { nq = A.step_off[lt + gridDim.x]; ne = A.step_off[lt + gridDim.x + 1]; }
+        lq += pr;
+        // block index of this lane's slot in the warp's next step, loaded
+        // while the current step's copies are issued
+        int nxt = -1;
+        auto fetch = [&]() {
+            while (lq >= le && lt < A.ntile) {
+                lt += gridDim.x;
+                lq = nq + (lq - le);
+                le = ne;
+                if (lt + (int)gridDim.x < A.ntile) { nq = A.step_off[lt + gridDim.x]; ne = A.step_off[lt + gridDim.x + 1]; }
+            }
+            if (lt < A.ntile && lane < G::kSlots) nxt = A.steps[lq * G::kSlots + lane];
+        };
+        for (fetch(); lt < A.ntile; it += 2) {
+            const int cur = nxt;
+            lq += 2;
+            fetch();
+            const int st = it % G::kStages;
+            const uint32_t ph = (it / G::kStages) & 1;
+            const uint32_t zbits = __ballot_sync(0xffffffffu, lane < G::kSlots && cur < 0);
+            uint32_t zprev = 0u;
 #pragma unroll
-                for (int k = 0; k < G::kStages; ++k)
-                    if (k == st) zprev = zmask[k];
-                const bool skip = lane >= G::kSlots || (cur < 0 && ((zprev >> lane) & 1u));
-                const uint32_t need = __ballot_sync(0xffffffffu, !skip);
-                int waited = 1;
-                if (lane == 0) {
-                    waited = mbar_wait(&ctl->empty[st], ph ^ 1, abort_flag, A.wait_cycles) ? 1 : 0;
-                    if (waited) mbar_expect_tx(&ctl->full[st], (uint32_t)__popc(need) * G::kPairBytes);
+            for (int k = 0; k < G::kStages / 2; ++k)
+                if (k == (st >> 1)) {
+                    zprev = zmask[k];
+                    zmask[k] = zbits;
                 }
-                waited = __shfl_sync(0xffffffffu, waited, 0);
-                if (!waited) { ok = false; break; }
-#pragma unroll
-                for (int k = 0; k < G::kStages; ++k)
-                    if (k == st) zmask[k] = zbits;
-                // zero blocks: one per CTA and slot (so that the CTAs do not all
-                // read the same few L2 sectors), adjacent like the slots
-                const uint16_t *src = cur >= 0 ? A.planes + (size_t)cur * (2 * G::kPlaneElems)
-                                               : A.zero + ((size_t)blockIdx.x * G::kSlots + lane) * (2 * G::kPlaneElems);
-                // runs: a slot whose source follows its left neighbour's in
-                // memory joins that neighbour's copy; the first slot of a run
-                // copies the whole run
-                const uint16_t *left = reinterpret_cast<const uint16_t *>(
-                    __shfl_up_sync(0xffffffffu, reinterpret_cast<unsigned long long>(src), 1));
-                const bool joins = A.runs && lane > 0 && !skip && ((need >> (lane - 1)) & 1u) &&
-                                   src == left + 2 * G::kPlaneElems;
-                const uint32_t jm = __ballot_sync(0xffffffffu, joins);
-                if (!skip && !joins) {
-                    const uint32_t above = lane < 31 ? jm >> (lane + 1) : 0u;
-                    const uint32_t len = (uint32_t)__ffs(~above);      // this slot and the slots that join it
-                    bulk_g2s(stages + st * G::kStageBytes + lane * G::kPairBytes, src, len * G::kPairBytes,
-                             &ctl->full[st]);
-                }
+            const bool skip = lane >= G::kSlots || (cur < 0 && ((zprev >> lane) & 1u));
+            const uint32_t need = __ballot_sync(0xffffffffu, !skip);
+            // zero blocks: one per CTA and slot (so that the CTAs do not all
+            // read the same few L2 sectors), adjacent like the slots
+            const uint16_t *src = cur >= 0 ? A.planes + (size_t)cur * (2 * G::kPlaneElems)
+                                           : A.zero + ((size_t)blockIdx.x * G::kSlots + lane) * (2 * G::kPlaneElems);
+            // runs: a slot whose source follows its left neighbour's in
+            // memory joins that neighbour's copy; the first slot of a run
+            // copies the whole run
+            const uint16_t *left = reinterpret_cast<const uint16_t *>(
+                __shfl_up_sync(0xffffffffu, reinterpret_cast<unsigned long long>(src), 1));
+            const bool joins = A.runs && lane > 0 && !skip && ((need >> (lane - 1)) & 1u) &&
+                               src == left + 2 * G::kPlaneElems;
+            const uint32_t jm = __ballot_sync(0xffffffffu, joins);
+            int waited = 1;
+            if (lane == 0) {
+                waited = mbar_wait(&ctl->empty[st], ph ^ 1, abort_flag, A.wait_cycles) ? 1 : 0;
+                if (waited) mbar_expect_tx(&ctl->full[st], (uint32_t)__popc(need) * G::kPairBytes);
+            }
+            waited = __shfl_sync(0xffffffffu, waited, 0);
+            if (!waited) { ok = false; break; }
+            if (!skip && !joins) {
+                const uint32_t above = lane < 31 ? jm >> (lane + 1) : 0u;
+                const uint32_t len = (uint32_t)__ffs(~above);      // this slot and the slots that join it
+                bulk_g2s(stages + st * G::kStageBytes + lane * G::kPairBytes, src, len * G::kPairBytes,
+                         &ctl->full[st]);
             }
         }
         if (!ok && lane == 0) {
-            // after an abort, wait (bounded) until the copies of the stages
-            // still in flight have landed before the CTA leaves: the last
-            // min(it, kStages) issued stages, each at the phase of its last use
-            const uint32_t n = it < (uint32_t)G::kStages ? it : (uint32_t)G::kStages;
-            for (uint32_t q = it - n; q < it; ++q)
-                mbar_wait_drain(&ctl->full[q % G::kStages], (q / G::kStages) & 1, A.wait_cycles);
+            // after an abort, wait (bounded) until this warp's copies still in
+            // flight have landed before the CTA leaves: those of its last
+            // kStages / 2 issued steps, each at the phase of its last use
+            for (int k = 1; k <= G::kStages / 2; ++k) {
+                const int64_t q = (int64_t)it - 2 * k;
+                if (q >= 0) mbar_wait_drain(&ctl->full[q % G::kStages], (uint32_t)(q / G::kStages) & 1, A.wait_cycles);
+            }
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -498,8 +528,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
             if (A.hold) hold_until_timeout(abort_flag, A.wait_cycles);
             uint32_t it = 0, seg = 0;
             bool issued = false;
+            int64_t n0 = 0, n1 = 0;          // step range of the next tile, loaded a tile ahead
+            if (blockIdx.x < A.ntile) { n0 = A.step_off[blockIdx.x]; n1 = A.step_off[blockIdx.x + 1]; }
             for (int t = blockIdx.x; t < A.ntile && !*abort_flag; t += gridDim.x) {
-                const int64_t s0 = A.step_off[t], s1 = A.step_off[t + 1];
+                const int64_t s0 = n0, s1 = n1;
+                if (t + (int)gridDim.x < A.ntile) { n0 = A.step_off[t + gridDim.x]; n1 = A.step_off[t + gridDim.x + 1]; }
                 bool ok = true;
                 for (int64_t q = s0; q < s1 && ok; ++seg) {
                     // one segment: up to kSegSteps K-steps into a fresh accumulator
@@ -541,26 +574,31 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
                 }
             }
         }
-    } else {
-        // ---------------- epilogue: warps 2..9 ----------------
+    } else if (warp >= kEpiWarp0) {
+        // ---------------- epilogue: warps 4..11 ----------------
         const int eq = warp & 3;                        // TMEM lanes 32*eq .. 32*eq+31
-        const int colhalf = (warp - 2) >> 2;            // accumulator columns 128*colhalf .. +127
-        float *S = stage_ep + (warp - 2) * 32 * 33;     // one 32 x 32 tile, transposed through shared memory
-        // metadata of block n, word w at meta[(8 n + w) * MW]
-        constexpr int MW = meta_stride<B>();
-        float *meta = B == 16 ? meta_all + (warp - 2) * meta_words<B>() : S + 32;
-        uint32_t seg = 0, pround = 0;
-        for (int t = blockIdx.x; t < A.ntile && !*abort_flag; t += gridDim.x) {
+        const int colhalf = (warp - kEpiWarp0) >> 2;            // accumulator columns 128*colhalf .. +127
+        float *S = stage_ep + (warp - kEpiWarp0) * 32 * 33;     // b = 64: a 32 x 32 tile
+        // metadata (one lane per block) and step count of a tile, gathered
+        // while the previous tile's MMAs run: the chain of dependent loads
+        // takes about as long as a segment
+        float *const meta2 = meta_all + (warp - kEpiWarp0) * meta_words<B>();
+        int nst_next = 0;
+        auto gather = [&](int t, int par) {
             const int *d = A.tiles + (size_t)t * G::kTileInts;
-            // metadata of this warp's output blocks, one lane each
-            {
-                const int s = lane_slot<B, G>(d, eq, colhalf, lane);
-                // blocks per warp: 4 at b = 32, 16 at b = 16, 2 at b = 64 (each shared
-                // with the partner warp that holds the other row half)
-                if (lane < blocks_per_warp<B>()) gather_meta<B>(A, s, meta + lane * 8 * MW);
-            }
+            nst_next = d[3];
+            const int s = lane_slot<B, G>(d, eq, colhalf, lane);
+            if (lane < blocks_per_warp<B>())
+                gather_meta(A, s, meta2 + (par * blocks_per_warp<B>() + lane) * 8);
+        };
+        uint32_t seg = 0, pround = 0;
+        int par = 0;
+        if (blockIdx.x < A.ntile) gather(blockIdx.x, 0);
+        for (int t = blockIdx.x; t < A.ntile && !*abort_flag; t += gridDim.x, par ^= 1) {
+            const float *meta = meta2 + par * blocks_per_warp<B>() * 8;
             __syncwarp();
-            const int nst = d[3];
+            const int nst = nst_next;
+            const bool more = t + (int)gridDim.x < A.ntile;
             if (nst < 0 && lane == 0) atomicOr(A.err, 4);
             // the tile's accumulator: sum of its segments, added with
             // round-to-nearest in registers (row 32*eq + lane, this warp's 128 columns)
@@ -572,8 +610,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
             for (int g = 0; g < nseg; ++g, ++seg) {
                 const int buf = seg & (kSegBufs - 1);
                 const uint32_t use = seg / kSegBufs;
-                if (g == (nseg > 2 ? nseg - 2 : 0) && t + (int)gridDim.x < A.ntile)
+                if (g == (nseg > 2 ? nseg - 2 : 0) && more) {
                     prefetch_old_blocks<B, G>(A, t + gridDim.x, eq, colhalf, lane);
+                    gather(t + gridDim.x, par ^ 1);
+                }
                 if (!mbar_wait(&ctl->seg_full[buf], use & 1, abort_flag, A.wait_cycles)) { ok = false; break; }
                 fence_after();
                 const uint32_t ta = tmem + ((uint32_t)(32 * eq) << 16) + buf * kTileN + 128 * colhalf;
@@ -589,23 +629,24 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
                 if (lane == 0) mbar_arrive(&ctl->seg_empty[buf]);
             }
             if (!ok) break;
+            if (nseg == 0 && more) gather(t + gridDim.x, par ^ 1);
 
             if constexpr (B == 32) {
                 // lane l holds row l of 4 blocks of 32 columns
 #pragma unroll
                 for (int n = 0; n < 4; ++n) {
-                    const float *q = meta + n * 8 * MW;
+                    const float *q = meta + n * 8;
                     const int s = __float_as_int(q[0]);
                     if (s < 0) continue;
                     float acc[32];
 #pragma unroll
                     for (int c = 0; c < 32; ++c) acc[c] = racc[n * 32 + c];
-                    const float cl = q[4 * MW];
-                    const float cq = q[5 * MW];
-                    const double tau = __hiloint2double(__float_as_int(q[7 * MW]), __float_as_int(q[6 * MW]));
-                    const int sx = __float_as_int(q[1 * MW]);
-                    const bool diag = __float_as_int(q[2 * MW]) != 0;
-                    const int oidx = __float_as_int(q[3 * MW]);
+                    const float cl = q[4];
+                    const float cq = q[5];
+                    const double tau = __hiloint2double(__float_as_int(q[7]), __float_as_int(q[6]));
+                    const int sx = __float_as_int(q[1]);
+                    const bool diag = __float_as_int(q[2]) != 0;
+                    const int oidx = __float_as_int(q[3]);
                     __syncwarp();
                     // linear term: four columns of the lane's row at a time, 512
                     // contiguous bytes for the warp (f32_index)
@@ -628,12 +669,18 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
                         for (int c = 0; c < 32; ++c) acc[c] = cq * acc[c];
                     }
                     // a diagonal block is symmetrised as (X + X^T) / 2
+                    // (the transpose comes back from the output slot: one block
+                    // in a row is diagonal)
+                    float4 *o = reinterpret_cast<float4 *>(A.out_val + (size_t)oidx * G::kPlaneElems) + lane;
                     if (diag) {
 #pragma unroll
-                        for (int c = 0; c < 32; ++c) S[lane * 33 + c] = acc[c];
+                        for (int c = 0; c < 8; ++c)
+                            o[c * 32] = make_float4(acc[4 * c], acc[4 * c + 1], acc[4 * c + 2], acc[4 * c + 3]);
                         __syncwarp();
+                        const volatile float *tr = reinterpret_cast<const float *>(A.out_val + (size_t)oidx * G::kPlaneElems) +
+                                                   f32_index(32, 0, lane);
 #pragma unroll
-                        for (int c = 0; c < 32; ++c) acc[c] = 0.5f * (acc[c] + S[c * 33 + lane]);
+                        for (int c = 0; c < 32; ++c) acc[c] = 0.5f * (acc[c] + tr[4 * c]);
                         __syncwarp();
                     }
                     float ss = 0.f;
@@ -643,7 +690,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
                     for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
                     const float nrm = sqrtf(ss) * (1.0f + 1e-6f);
                     const bool kp = ((double)nrm >= tau) && (nrm > 0.f);
-                    float4 *o = reinterpret_cast<float4 *>(A.out_val + (size_t)oidx * G::kPlaneElems) + lane;
 #pragma unroll
                     for (int c = 0; c < 8; ++c)
                         o[c * 32] = make_float4(acc[4 * c], acc[4 * c + 1], acc[4 * c + 2], acc[4 * c + 3]);
@@ -658,14 +704,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
                 const int h = lane >> 4, c16 = lane & 15;
 #pragma unroll
                 for (int n = 0; n < 8; ++n) {
-                    const float *q = meta + (h * 8 + n) * 8 * MW;
+                    const float *q = meta + (h * 8 + n) * 8;
                     const int s = __float_as_int(q[0]);
-                    const float cl = q[4 * MW];
-                    const float cq = q[5 * MW];
-                    const double tau = __hiloint2double(__float_as_int(q[7 * MW]), __float_as_int(q[6 * MW]));
-                    const int sx = __float_as_int(q[1 * MW]);
-                    const bool diag = s >= 0 && __float_as_int(q[2 * MW]) != 0;
-                    const int oidx = __float_as_int(q[3 * MW]);
+                    const float cl = q[4];
+                    const float cq = q[5];
+                    const double tau = __hiloint2double(__float_as_int(q[7]), __float_as_int(q[6]));
+                    const int sx = __float_as_int(q[1]);
+                    const bool diag = s >= 0 && __float_as_int(q[2]) != 0;
+                    const int oidx = __float_as_int(q[3]);
                     const bool lin = s >= 0 && sx >= 0 && cl != 0.f;
                     float acc[16];
                     if (lin && !A.xlin) {
@@ -687,13 +733,19 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
                         for (int c = 0; c < 16; ++c) acc[c] = cq * racc[n * 16 + c];
                     }
                     // a diagonal block is symmetrised as (X + X^T) / 2
+                    float4 *o = reinterpret_cast<float4 *>(A.out_val + (size_t)oidx * G::kPlaneElems) + c16;
                     if (__any_sync(0xffffffffu, diag)) {
-#pragma unroll
-                        for (int c = 0; c < 16; ++c) S[lane * 33 + c] = acc[c];
-                        __syncwarp();
                         if (diag) {
 #pragma unroll
-                            for (int c = 0; c < 16; ++c) acc[c] = 0.5f * (acc[c] + S[(16 * h + c) * 33 + c16]);
+                            for (int c = 0; c < 4; ++c)
+                                o[c * 16] = make_float4(acc[4 * c], acc[4 * c + 1], acc[4 * c + 2], acc[4 * c + 3]);
+                        }
+                        __syncwarp();
+                        if (diag) {
+                            const volatile float *tr = reinterpret_cast<const float *>(A.out_val + (size_t)oidx * G::kPlaneElems) +
+                                                       f32_index(16, 0, c16);
+#pragma unroll
+                            for (int c = 0; c < 16; ++c) acc[c] = 0.5f * (acc[c] + tr[4 * c]);
                         }
                         __syncwarp();
                     }
@@ -705,7 +757,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
                     const float nrm = sqrtf(ss) * (1.0f + 1e-6f);
                     const bool kp = ((double)nrm >= tau) && (nrm > 0.f);
                     if (s >= 0) {
-                        float4 *o = reinterpret_cast<float4 *>(A.out_val + (size_t)oidx * G::kPlaneElems) + c16;
 #pragma unroll
                         for (int c = 0; c < 4; ++c)
                             o[c * 16] = make_float4(acc[4 * c], acc[4 * c + 1], acc[4 * c + 2], acc[4 * c + 3]);
@@ -720,19 +771,19 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
                 // partner warp (warp ^ 1) holds the other 32 rows of the same blocks
                 // (both see the same slots, so both take the same branches and
                 // handshakes; after an abort both skip the rest)
-                const int rh = eq & 1, pr = (warp - 2) >> 1;
-                const float *Sp = stage_ep + ((warp ^ 1) - 2) * 32 * 33;   // the partner's staging tile
+                const int rh = eq & 1, pr = (warp - kEpiWarp0) >> 1;
+                const float *Sp = stage_ep + ((warp ^ 1) - kEpiWarp0) * 32 * 33;   // the partner's staging tile
 #pragma unroll
                 for (int n = 0; n < 2; ++n) {
-                    const float *q = meta + n * 8 * MW;
+                    const float *q = meta + n * 8;
                     const int s = __float_as_int(q[0]);
                     if (s < 0 || !ok) continue;
-                    const float cl = q[4 * MW];
-                    const float cq = q[5 * MW];
-                    const double tau = __hiloint2double(__float_as_int(q[7 * MW]), __float_as_int(q[6 * MW]));
-                    const int sx = __float_as_int(q[1 * MW]);
-                    const bool diag = __float_as_int(q[2 * MW]) != 0;
-                    const int oidx = __float_as_int(q[3 * MW]);
+                    const float cl = q[4];
+                    const float cq = q[5];
+                    const double tau = __hiloint2double(__float_as_int(q[7]), __float_as_int(q[6]));
+                    const int sx = __float_as_int(q[1]);
+                    const bool diag = __float_as_int(q[2]) != 0;
+                    const int oidx = __float_as_int(q[3]);
                     // linear term: four columns of the lane's row at a time
                     if (sx >= 0 && cl != 0.f && !A.xlin) {
                         const double *gx = A.in_val + (size_t)sx * G::kPlaneElems + (size_t)(32 * rh + lane) * 64;
@@ -797,9 +848,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
                     for (int c = 0; c < 64; ++c) ss = fmaf(racc[n * 64 + c], racc[n * 64 + c], ss);
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-                    if (lane == 0) ctl->pair_ss[warp - 2] = ss;
+                    if (lane == 0) ctl->pair_ss[warp - kEpiWarp0] = ss;
                     ok = pair_sync(ctl, pr, pround, lane, abort_flag, A.wait_cycles) && ok;
-                    const float other = *(volatile float *)&ctl->pair_ss[(warp ^ 1) - 2];
+                    const float other = *(volatile float *)&ctl->pair_ss[(warp ^ 1) - kEpiWarp0];
                     const float tot = rh == 0 ? ss + other : other + ss;
                     const float nrm = sqrtf(tot) * (1.0f + 1e-6f);
                     const bool kp = ((double)nrm >= tau) && (nrm > 0.f);
@@ -834,8 +885,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
 
 template <int B>
 constexpr size_t smem_bytes() {
-    return (size_t)Geo<B>::kStages * Geo<B>::kStageBytes + kEpiWarps * 32 * 33 * sizeof(float) +
-           kEpiWarps * meta_words<B>() * sizeof(float) + sizeof(SmemCtl) + 1024;
+    return (size_t)Geo<B>::kStages * Geo<B>::kStageBytes + stage_words<B>() * sizeof(float) +
+           kEpiWarps * meta_words<B>() * sizeof(float) + sizeof(SmemCtl);
 }
 static_assert(smem_bytes<16>() <= 227 * 1024 && smem_bytes<32>() <= 227 * 1024 && smem_bytes<64>() <= 227 * 1024,
               "shared memory of the tensor-core kernel exceeds 227 KB");
