@@ -59,7 +59,10 @@ extern "C" {
 #define RDM_ESTATE          -7   /* call made in the wrong state (e.g. getter before solve) */
 
 /* ---- precision modes (rdm_params.mode) ------------------------------- */
-#define RDM_MODE_FP64        0   /* every product in FP64 (CUDA cores) */
+#define RDM_MODE_FP64        0   /* every product to FP64 accuracy: FP64 FMAs on the CUDA cores, or
+                                    (32 x 32 blocks, truncation threshold >= 1e-10) exact sums of
+                                    products of 8 bf16 slices per element on the tensor cores,
+                                    rounded to FP64 once */
 #define RDM_MODE_FP32        1   /* every product in FP32 (CUDA cores), FP64 scalars */
 #define RDM_MODE_MIXED_BF16  2   /* bf16 hi+lo split products on the tensor cores
                                     (tcgen05, FP32 accumulate) until the idempotency
@@ -192,10 +195,11 @@ typedef struct {
     double  issued_flops;   /* flops the kernels executed (split products count 3x, padding counted) */
     double  kernel_ms[8];   /* device time per kernel class (CUDA events on the handle's stream):
                                0 symbolic mask + pair / tile lists, 1 tensor-core split products,
-                               2 FP64 CUDA-core products, 3 FP32 CUDA-core products (and copies
+                               2 FP64 products, 3 FP32 CUDA-core products (and copies
                                of converged systems), 4 truncation compaction, 5 reductions,
                                set-up and host decisions (the remainder of the solve),
-                               6 double-FP32 CUDA-core products, 7 tensor-core slice products */
+                               6 double-FP32 CUDA-core products, 7 tensor-core slice products
+                               (REFINE_SLICES) */
     double  kernel_flops[5];   /* useful flops (2 b^3 per block triple) of the tensor-core split (0),
                                   FP64 (1), FP32 (2), double-FP32 (3) and slice-product (4) launches */
     int64_t kernel_launches;   /* kernels launched by the solve */

@@ -485,6 +485,7 @@ struct StepStats {
     int64_t npairs = 0;
     int64_t nslot = 0;
     int64_t pairs_tc = 0, pairs_64 = 0, pairs_32 = 0, pairs_ff = 0, pairs_oz = 0;   // block triples per class
+    int64_t pairs_simt = 0;                 // block triples computed on the CUDA cores
     double issued_tc = 0, issued_oz = 0;
     double bytes = 0;
     double ms[7] = {0, 0, 0, 0, 0, 0, 0};   // symbolic, tc, fp64, fp32, compaction, double-fp32, slice products
@@ -540,6 +541,21 @@ void tier_arith(int mode, int tier, int njob, Arith *ar, int refine_x1 = 0, int 
     }
 }
 
+// FP64 products of an FP64-mode step with threshold tau: 8-slice products on
+// the tensor cores for 32 x 32 blocks (12 times the FP64 pipe's rate on the
+// 300-atom cluster, and closer to the exact product, k_oz.cu).  Their error is
+// absolute, ~2^-60 of the largest elements of a row and a column; an element
+// far below that, which an FP64 FMA chain might still resolve, lies in a block
+// that the filter drops.  So they need a threshold well above that error:
+// below kSliceTau (an exact solve, tau = 0, foremost) the products stay on the
+// FP64 pipe.  So do the FP64 products of the mixed modes: their results go
+// through the rounding of the split operands, where a last-bit difference
+// comes out as one of 2^-22.
+constexpr double kSliceTau = 1e-10;
+Arith fp64_arith(int mode, int b, double tau) {
+    return mode == RDM_MODE_FP64 && b == 32 && tau >= kSliceTau ? AR_OZ8 : AR_FP64;
+}
+
 // tab[t][p]: arithmetic of job p for the systems in tier t; tiers_present:
 // bit t set when some active system is in tier t (the per-system tiers are in
 // h->sd.tier on the device)
@@ -555,16 +571,21 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
     // CUDA-core classes, launched in this order: FP64, double-FP32, FP32
     constexpr int kSimt = 3;
     const Arith simt_ar[kSimt] = {AR_FP64, AR_FF, AR_FP32};
-    JobMask tcm{}, cm[kSimt]{}, simt{}, ozm{};
+    JobMask tcm{}, cm[kSimt]{}, simt{}, ozm{}, m64{}, moz{};   // m64, moz: accounting (FP64, slices)
     Arith tc_ar = AR_FP16X3;
-    bool any_tc = false, any_oz = false, any_c[kSimt] = {false, false, false};
+    bool any_tc = false, any_oz = false, any_oz8 = false, any_c[kSimt] = {false, false, false};
+    int oz_nmat = 0;
     for (int t = 0; t < kMaxTiers; ++t) {
         if (!((tiers_present >> t) & 1u)) continue;
         for (int p = 0; p < njob; ++p) {
             const Arith a = tab[t][p];
-            if (a == AR_OZ) {
+            if (a == AR_OZ || a == AR_OZ8) {
                 ozm.m[t] |= 1u << p;
+                (a == AR_OZ ? moz : m64).m[t] |= 1u << p;
                 any_oz = true;
+                any_oz8 = any_oz8 || a == AR_OZ8;
+                for (int k = 0; k < jt.job[p].nterm; ++k)
+                    oz_nmat = std::max(oz_nmat, 1 + std::max(jt.job[p].a[k], jt.job[p].b[k]));
                 continue;
             }
             if (is_tc(a)) {
@@ -577,8 +598,20 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
             cm[c].m[t] |= 1u << p;
             any_c[c] = true;
         }
-        simt.m[t] = cm[0].m[t] | cm[1].m[t] | cm[2].m[t];
+        m64.m[t] |= cm[0].m[t];
     }
+    h->ensure_events();
+    RDM_CUDA_TRY(cudaEventRecord(h->ev[0], st));
+    if (any_oz && !prepare_oz_operands(in, oz_nmat, any_oz8 ? 8 : 7, h->ozw, st)) {
+        // no room for the slices: the FP64 pipe
+        for (int t = 0; t < kMaxTiers; ++t) {
+            cm[0].m[t] |= ozm.m[t];
+            ozm.m[t] = 0;
+        }
+        any_oz = any_oz8 = false;
+        any_c[0] = true;
+    }
+    for (int t = 0; t < kMaxTiers; ++t) simt.m[t] = cm[0].m[t] | cm[1].m[t] | cm[2].m[t];
     // the first class present also copies the blocks of converged systems (the
     // FP32 class when no CUDA-core product is left)
     int first_c = kSimt - 1;
@@ -586,8 +619,6 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
         if (any_c[c]) first_c = c;
     const bool tc = any_tc;
     const bool f32_planes = any_c[1] || any_c[2];
-    h->ensure_events();
-    RDM_CUDA_TRY(cudaEventRecord(h->ev[0], st));
     // operand copies are made afresh from the input set at every step: one
     // set of buffers, moved to whichever set is the input, serves both
     auto take = [](auto &mine, auto &other) {
@@ -605,8 +636,10 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
     if (!f32_planes && in.opf32.cap * sizeof(float) > big) in.opf32.release();
     if (!any_c[1] && in.opf32lo.cap * sizeof(float) > big) in.opf32lo.release();
     if (tc) prepare_operands(in, tc_ar, lin, h->tcw, st);
-    if (any_oz) prepare_oz_operands(in, h->ozw, st);
-    else if (h->ozw.slices.cap * sizeof(uint16_t) > big) h->ozw.slices.release();
+    if (!any_oz && h->ozw.slices_a.cap * sizeof(uint16_t) > big) {
+        h->ozw.slices_a.release();
+        h->ozw.slices_b.release();
+    }
     if (f32_planes) {
         in.opf32.ensure(std::max<int64_t>(in.total, 1) * bb);
         if (any_c[1]) in.opf32lo.ensure(std::max<int64_t>(in.total, 1) * bb);
@@ -664,7 +697,7 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
     h->class_pairs.ensure(5);
     RDM_CUDA_TRY(cudaMemsetAsync(h->class_pairs.p, 0, 5 * sizeof(unsigned long long), st));
     launch_class_pairs(h->slot_row.p, mcol, h->slot_npair.p, h->slot_job.p, nslot, h->sd.sys_of_row.p,
-                       h->sd.active.p, h->sd.tier.p, tcm, cm[0], cm[2], cm[1], ozm, h->class_pairs.p, st);
+                       h->sd.active.p, h->sd.tier.p, tcm, m64, cm[2], cm[1], moz, h->class_pairs.p, st);
     unsigned long long cls[5] = {0, 0, 0, 0, 0};
     d2h(cls, h->class_pairs.p, 5, st);
     sync(h);
@@ -674,6 +707,7 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
     ss.pairs_32 = (int64_t)cls[2];
     ss.pairs_ff = (int64_t)cls[3];
     ss.pairs_oz = (int64_t)cls[4];
+    ss.pairs_simt = (any_oz8 ? 0 : ss.pairs_64) + ss.pairs_32 + ss.pairs_ff;
     if (any_c[0] || any_c[1] || any_c[2]) {
         h->pair_a.ensure(std::max<int64_t>(npairs, 1));
         h->pair_b.ensure(std::max<int64_t>(npairs, 1));
@@ -822,7 +856,7 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
         RDM_CUDA_TRY(cudaEventRecord(h->ev[2], st));
         if (oz_g) {
             const long long lt = g_kernel_launches;
-            ss.issued_oz += launch_numeric_oz(a, in, mcol, h->ozw, h->tcw_oz, oplan, st);
+            ss.issued_oz += launch_numeric_oz(a, in, jt, mcol, h->ozw, h->tcw_oz, oplan, st);
             ss.oz_launches += (int)(g_kernel_launches - lt);
         }
         RDM_CUDA_TRY(cudaEventRecord(h->ev[7], st));
@@ -873,7 +907,7 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
         for (int c = 0; c < kSimt; ++c) t_simt[c] += mc[c];
         t_tc += m42; t_cmp += m23; t_oz += moz;
     }
-    ss.bytes = ((double)in.total * (tc ? 4.0 : 8.0) + (any_oz ? (double)in.nnzb[0] * 14.0 : 0.0) +
+    ss.bytes = ((double)in.total * (tc ? 4.0 : 8.0) + (any_oz ? (double)in.nnzb[0] * 2.0 * h->ozw.nslice : 0.0) +
                 (double)nupper * 8.0) * (double)bb;
     out.total = kept;
     std::vector<int> rp(nrows + 1);
@@ -882,7 +916,11 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
     float mall = 0;
     cudaEventElapsedTime(&mall, h->ev[0], h->ev[3]);
     ss.ms[1] = t_tc;          // tensor-core products
-    ss.ms[2] = t_simt[0];     // FP64 products
+    // FP64 products: on the CUDA cores, or the slice launch when it held no others
+    bool oz_other = false;
+    for (int t = 0; t < kMaxTiers; ++t) oz_other = oz_other || moz.m[t];
+    if (any_oz8 && !oz_other) std::swap(t_simt[0], t_oz);
+    ss.ms[2] = t_simt[0];
     ss.ms[3] = t_simt[2];     // FP32 products (and copies of converged systems)
     ss.ms[4] = t_cmp;
     ss.ms[5] = t_simt[1];     // double-FP32 products
@@ -988,6 +1026,7 @@ void set_products(rdm_handle *h, MatSet &in, const JobTable &jt, const std::vect
     h2d(h->sd.tau1.p, t.data(), S, h->stream);
     h2d(h->sd.active.p, one.data(), S, h->stream);
     h2d(h->sd.tier.p, zero.data(), S, h->stream);
+    if (ar == AR_FP64) ar = fp64_arith(h->prm.mode, h->bs, tau);
     Arith tab[kMaxTiers][kMaxJobs];
     for (int p = 0; p < kMaxJobs; ++p) tab[0][p] = ar;
     multiply(h, in, out, jt, tab, 1u, std::any_of(cl.begin(), cl.end(), [](double c) { return c != 0.0; }));
@@ -999,10 +1038,11 @@ void fp64_products(rdm_handle *h, MatSet &in, const JobTable &jt, double c_lin, 
     set_products(h, in, jt, std::vector<double>(h->S, c_lin), std::vector<double>(h->S, c_sq), tau, AR_FP64, out);
 }
 
-// FP64-class products: double-FP32 at b = 32 (about 46 bits), FP64 otherwise
+// FP64-class products: double-FP32 at b = 32 (about 46 bits) where FP64 ones
+// would run on the FP64 pipe, FP64 ones otherwise
 void fp64_class_products(rdm_handle *h, MatSet &in, const JobTable &jt, const std::vector<double> &cl,
                          const std::vector<double> &cq, double tau, MatSet &out) {
-    set_products(h, in, jt, cl, cq, tau, h->bs == 32 ? AR_FF : AR_FP64, out);
+    set_products(h, in, jt, cl, cq, tau, h->bs == 32 && fp64_arith(h->prm.mode, 32, tau) == AR_FP64 ? AR_FF : AR_FP64, out);
 }
 
 // Job: out p = c_lin X_x + c_sq (A B + B A), or A A (a == b, one term)
@@ -1350,7 +1390,13 @@ int run_solve(rdm_handle *h, rdm_info *info_out) {
         Arith tab[kMaxTiers][kMaxJobs];
         unsigned tiers_present = 0;
         std::vector<int> tier_of(S, 0);
-        for (int t = 0; t <= final_tier; ++t) tier_arith(P.mode, t, jt.njob, tab[t], P.refine_x1, P.refine_x0, b);
+        for (int t = 0; t <= final_tier; ++t) {
+            tier_arith(P.mode, t, jt.njob, tab[t], P.refine_x1, P.refine_x0, b);
+            const bool ref = mixed && t == final_tier;
+            for (int p = 0; p < jt.njob; ++p)
+                if (tab[t][p] == AR_FP64)
+                    tab[t][p] = fp64_arith(P.mode, b, jt.job[p].tau_sel ? (ref ? tau1_ref : tau1) : (ref ? tau_ref : tau0));
+        }
         for (int s = 0; s < S; ++s) {
             tier_of[s] = ss[s].tier;
             if (act[s]) tiers_present |= 1u << ss[s].tier;
@@ -1384,7 +1430,7 @@ int run_solve(rdm_handle *h, rdm_info *info_out) {
         flops_32 += (double)sst.pairs_32 * fpb;
         flops_ff += (double)sst.pairs_ff * fpb;
         flops_oz += (double)sst.pairs_oz * fpb;
-        issued += sst.issued_tc + sst.issued_oz + (double)(sst.pairs_64 + sst.pairs_32 + sst.pairs_ff) * fpb;
+        issued += sst.issued_tc + sst.issued_oz + (double)sst.pairs_simt * fpb;
         nbytes += sst.bytes;
         tc_launches += sst.tc_launches;
         oz_launches += sst.oz_launches;

@@ -183,8 +183,9 @@ struct JobTable {
 
 // Operand arithmetic of a numeric launch
 // (AR_FF: double-FP32 products on the FP32 pipe, about 46 bits; AR_OZ:
-// exact bf16 slice products on the tensor cores, FP64-class)
-enum Arith { AR_FP64 = 0, AR_FP32 = 1, AR_BF16X3 = 2, AR_FP16X3 = 3, AR_FF = 5, AR_OZ = 6 };
+// exact bf16 slice products on the tensor cores, 7 slices, FP64-class; AR_OZ8:
+// FP64 products as 8-slice products)
+enum Arith { AR_FP64 = 0, AR_FP32 = 1, AR_BF16X3 = 2, AR_FP16X3 = 3, AR_FF = 5, AR_OZ = 6, AR_OZ8 = 7 };
 
 // Jobs selected per precision tier: bit p of m[t] selects job p for the rows
 // of systems currently in tier t (systems of a batch move through the tiers

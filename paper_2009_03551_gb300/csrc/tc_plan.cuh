@@ -16,7 +16,7 @@ struct PlanGeo {
     static constexpr int TBM = TBM_;                    // block rows per tile
     static constexpr int TBN = TBN_;                    // block columns per tile
     static constexpr int kSlots = TBM + TBN;            // operand blocks per K-step: A rows, then B rows
-    static constexpr int kColOff = 4 + TBM * TBN;       // tile record: job, super-row, -, nsteps,
+    static constexpr int kColOff = 4 + TBM * TBN;       // tile record: job, super-row, steps of term 0, nsteps,
     static constexpr int kTileInts = kColOff + TBN;     //   mask slot[TBM x TBN], column j of each tile column
     static_assert(kSlots <= 32, "one producer lane per slot");
 };
@@ -250,6 +250,7 @@ __device__ void tile_steps_serial(const TileBuild &T, int t, int fill) {
                 ++n;
             }
         }
+        if (!fill && term == 0) T.tiles[(size_t)t * G::kTileInts + 2] = n;
     }
     if (!fill) T.step_cnt[t] = n;
     else if (n != (int)(T.step_off[t + 1] - T.step_off[t])) T.tiles[(size_t)t * G::kTileInts + 3] = -1;
@@ -311,7 +312,7 @@ __global__ void __launch_bounds__(32 * kStepWarps) k_tile_steps(TileBuild T, int
         return;
     }
     int64_t w = fill ? T.step_off[t] : 0;
-    int n = 0;
+    int n = 0, n_first = 0;
     for (int term = 0; term < job.nterm; ++term) {
         const int lo = lo_t[term], hi = hi_t[term];
         if (hi < lo) continue;
@@ -366,8 +367,10 @@ __global__ void __launch_bounds__(32 * kStepWarps) k_tile_steps(TileBuild T, int
             __syncwarp();
         }
         n += carry;
+        if (!fill && term == 0) n_first = n;
     }
     if (lane == 0) {
+        if (!fill) T.tiles[(size_t)t * G::kTileInts + 2] = n_first;
         if (!fill) T.step_cnt[t] = n;
         else if (n != (int)(T.step_off[t + 1] - T.step_off[t])) T.tiles[(size_t)t * G::kTileInts + 3] = -1;
     }
