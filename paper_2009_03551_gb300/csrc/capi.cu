@@ -941,12 +941,12 @@ JobTable solve_jobs(int nd) {
 
 // per-system stats of the current X: [S][3+nd]
 std::vector<double> stats(rdm_handle *h, MatSet &X) {
-    const int nq = 3 + h->nd;
-    h->row_part.ensure((size_t)nq * h->NB);
+    const int nq = 3 + h->nd, parts = row_stats_parts(h->NB);
+    h->row_part.ensure((size_t)nq * h->NB * parts);
     h->sys_q.ensure((size_t)nq * h->S);
     launch_row_stats(X.row_ptr.p, X.col.p, X.val.p, X.nmat, h->NB, h->bs, h->H0.row_ptr.p,
-                     h->H0.col.p, h->H0.val.p, h->row_part.p, h->stream);
-    launch_sys_sum(h->row_part.p, nq, h->NB, h->sd.row0.p, h->sd.nbs.p, h->S, h->sys_q.p, h->stream);
+                     h->H0.col.p, h->H0.val.p, parts, h->row_part.p, h->stream);
+    launch_sys_sum(h->row_part.p, nq, h->NB, h->sd.row0.p, h->sd.nbs.p, h->S, h->sys_q.p, h->stream, parts);
     std::vector<double> q((size_t)nq * h->S);
     d2h(q.data(), h->sys_q.p, q.size(), h->stream);
     sync(h);
@@ -1121,7 +1121,7 @@ void lowdin_forward(rdm_handle *h) {
     JobTable jt{};
     double prev = 1e300;
     int it = 0;
-    const int nq = 3;     // Tr T, ||T||^2, Tr(T T) from the stats of a one-matrix set
+    const int nq = 2;     // Tr T, ||T||^2
     for (it = 0; it < 100; ++it) {
         concat(h, {{&Z, 0, 1}, {&Y, 0, 1}, {&I, 0, 1}}, in);
         jt.njob = 1;
@@ -1130,7 +1130,7 @@ void lowdin_forward(rdm_handle *h) {
         // ||T - I||_F^2 = ||T||^2 - 2 Tr T + n per system (padding rows included)
         h->row_part.ensure((size_t)nq * NB);
         h->sys_q.ensure((size_t)nq * S);
-        launch_row_stats(T.row_ptr.p, T.col.p, T.val.p, 1, NB, b, T.row_ptr.p, T.col.p, T.val.p, h->row_part.p, st);
+        launch_row_trace_norm(T.row_ptr.p, T.col.p, T.val.p, NB, b, h->row_part.p, st);
         launch_sys_sum(h->row_part.p, nq, NB, h->sd.row0.p, h->sd.nbs.p, S, h->sys_q.p, st);
         std::vector<double> q((size_t)nq * S);
         d2h(q.data(), h->sys_q.p, q.size(), st);

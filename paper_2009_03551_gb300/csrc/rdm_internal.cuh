@@ -224,11 +224,17 @@ void launch_check_values(const int *row_ptr, const int *col, const double *val, 
 // k_stats.cu: per-row partial sums then a deterministic per-system reduction.
 // q-layout of the per-system output (double, [S][nq]):
 //   0: Tr X0, 1: ||X0||_F^2, 2: Tr(X0 H0), 3+g: Tr(X1_g H0)
+// A block row's sums come in `parts` partial sums (row_stats_parts), so that
+// row_part has [q][NB * parts] entries.
+int row_stats_parts(int NB);
 void launch_row_stats(const int *row_ptr, const int *col, const double *val, int nmat, int NB,
-                      int b, const int *h_row_ptr, const int *h_col, const double *h_val,
+                      int b, const int *h_row_ptr, const int *h_col, const double *h_val, int parts,
                       double *row_part, cudaStream_t st);
+// Tr X and ||X||_F^2 of one matrix, row_part [2][NB]
+void launch_row_trace_norm(const int *row_ptr, const int *col, const double *val, int NB, int b, double *row_part,
+                           cudaStream_t st);
 void launch_sys_sum(const double *row_part, int nq, int NB, const int *row0, const int *nbs,
-                    int S, double *out, cudaStream_t st);
+                    int S, double *out, cudaStream_t st, int parts = 1);
 
 // alpha: per-row partials of <P1_d, H1_g> over intersecting blocks
 void launch_row_dots(const int *p_row_ptr, const int *p_col, const double *p_val, int np,
