@@ -85,6 +85,46 @@ struct SysState {
 
 }  // namespace
 
+// pinned host memory, grow-only
+template <class T>
+struct PinBuf {
+    T *p = nullptr;
+    size_t cap = 0;
+    PinBuf() = default;
+    PinBuf(const PinBuf &) = delete;
+    PinBuf &operator=(const PinBuf &) = delete;
+    ~PinBuf() { release(); }
+    T *ensure(size_t n) {
+        if (n <= cap && p) return p;
+        release();
+        RDM_CUDA_TRY(cudaHostAlloc((void **)&p, n * sizeof(T), cudaHostAllocDefault));
+        cap = n;
+        return p;
+    }
+    void release() {
+        if (p) cudaFreeHost(p);
+        p = nullptr;
+        cap = 0;
+    }
+};
+
+// device counters of a multiplication step (rdm_handle::counters, ints)
+enum {
+    kCtrTop = 0,         // pool_top, overflow of the symbolic phase
+    kCtrErr = 2,         // error bits of the pair lists
+    kCtrPairs = 4,       // 64 bits: pairs of all upper slots
+    kCtrClass = 6,       // 5 x 64 bits: pairs per kernel class
+    kCtrWork = 16,       // work items of the three CUDA-core classes (zeroed for every group, with the next)
+    kCtrNext = 20,       // next item to hand out, per class
+    kCtrInts = 24
+};
+struct HostStep {
+    int ctr[kCtrInts];
+    int nupper, kept;
+    int tc[8], oz[8];                 // TcWork::counters of the two plans
+    int rp[kMaxJobs + 1];             // first block of every output matrix
+};
+
 struct rdm_handle {
     int device = 0;
     cudaStream_t stream = nullptr;
@@ -120,16 +160,17 @@ struct rdm_handle {
     int cur = 0;
 
     // work buffers
-    DevBuf<int> row_cnt, row_off, pool_col, pool_npair, counters, mask_col;
+    DevBuf<int> row_off, pool_col, pool_npair, counters, mask_col;
+    DevBuf<int64_t> row_cnt;
     DevBuf<int> out_rp, slot_row, slot_job, slot_npair, slot_x, slot_t, work, work2, work3;
     DevBuf<int64_t> pair_off, scan_tmp64;
     DevBuf<int> scan_tmp32, pair_a, pair_b, cnt_rows;
-    DevBuf<int> uidx, scan_tmp_s, urp, dest, cpsrc;   // upper-slot ranks, compaction maps
-    DevBuf<int> work_ctr;                             // work-item counters of the CUDA-core launches
+    DevBuf<int> uidx, urp, dest, cpsrc;               // upper-slot ranks, compaction maps
     DevBuf<double> out_val, row_part, sys_q;
     DevBuf<float> out_nrm;
     DevBuf<uint8_t> keep;
-    DevBuf<unsigned long long> class_pairs;
+    PinBuf<HostStep> step_host;   // what the host reads back during a step
+    PinBuf<double> scalars_host;  // the step's scalars on their way to SysDev::step, and statistics back
     DevBuf<double> row_lo, row_hi;
     TcWork tcw, tcw_oz;      // plans of the split and of the slice-product tensor-core launches
     OzWork ozw;
@@ -465,8 +506,8 @@ void init_sys_scalars(rdm_handle *h) {
     const int S = h->S, NB = h->NB;
     SysDev &sd = h->sd;
     sd.row0.ensure(S); sd.nbs.ensure(S); sd.n_orb.ensure(S);
-    sd.emin.ensure(S); sd.emax.ensure(S); sd.c_lin.ensure(S); sd.c_sq.ensure(S);
-    sd.tau0.ensure(S); sd.tau1.ensure(S); sd.active.ensure(S); sd.tier.ensure(S);
+    sd.emin.ensure(S); sd.emax.ensure(S);
+    sd.ensure_step(S);
     sd.sys_of_row.ensure(NB);
     std::vector<int> sor(NB);
     for (int s = 0; s < S; ++s)
@@ -491,7 +532,60 @@ struct StepStats {
     double ms[7] = {0, 0, 0, 0, 0, 0, 0};   // symbolic, tc, fp64, fp32, compaction, double-fp32, slice products
     int tc_launches = 0, oz_launches = 0, simt_launches = 0;
     int groups = 1;                         // job groups of the numeric phase
+    // times of the launches; the last group's are added by finish_step
+    float t_simt[3] = {0, 0, 0}, t_tc = 0, t_cmp = 0, t_oz = 0;
+    bool oz_is_fp64 = false;                // the slice launch held FP64 products only
 };
+
+// Uploads the scalars of a step (per system) in one copy.  Every step waits
+// for the device at least once before the next upload, so the staging memory
+// is free again.
+void upload_step(rdm_handle *h, const std::vector<double> &c_lin, const std::vector<double> &c_sq,
+                 const std::vector<double> &t0, const std::vector<double> &t1, const std::vector<int> &active,
+                 const std::vector<int> &tier) {
+    const size_t S = c_lin.size(), n = SysDev::step_doubles((int)S);
+    double *q = h->scalars_host.ensure(n);
+    std::copy(c_lin.begin(), c_lin.end(), q);
+    std::copy(c_sq.begin(), c_sq.end(), q + S);
+    std::copy(t0.begin(), t0.end(), q + 2 * S);
+    std::copy(t1.begin(), t1.end(), q + 3 * S);
+    int *a = reinterpret_cast<int *>(q + 4 * S);
+    std::copy(active.begin(), active.end(), a);
+    std::copy(tier.begin(), tier.end(), a + S);
+    h2d(h->sd.step.p, q, n, h->stream);
+}
+
+// adds the times of the events of the last group, which must have completed
+void add_times(rdm_handle *h, StepStats &ss) {
+    const int ev_simt[3] = {5, 6, 4};   // events after each CUDA-core class
+    float m[6] = {0, 0, 0, 0, 0, 0};
+    cudaEventElapsedTime(&m[0], h->ev[1], h->ev[ev_simt[0]]);             // FP64 class
+    cudaEventElapsedTime(&m[1], h->ev[ev_simt[0]], h->ev[ev_simt[1]]);    // double-FP32 class
+    cudaEventElapsedTime(&m[2], h->ev[ev_simt[1]], h->ev[ev_simt[2]]);    // FP32 class (and copies)
+    cudaEventElapsedTime(&m[3], h->ev[ev_simt[2]], h->ev[2]);             // tensor-core launch
+    cudaEventElapsedTime(&m[4], h->ev[2], h->ev[7]);                      // slice-product launch
+    cudaEventElapsedTime(&m[5], h->ev[7], h->ev[3]);                      // compaction
+    for (int c = 0; c < 3; ++c) ss.t_simt[c] += m[c];
+    ss.t_tc += m[3];
+    ss.t_oz += m[4];
+    ss.t_cmp += m[5];
+}
+
+// the step's times per kernel class, once the device has finished it
+void finish_step(rdm_handle *h, StepStats &ss) {
+    add_times(h, ss);
+    float mall = 0;
+    cudaEventElapsedTime(&mall, h->ev[0], h->ev[3]);
+    const float rest = ss.t_simt[0] + ss.t_simt[1] + ss.t_simt[2] + ss.t_tc + ss.t_cmp + ss.t_oz;
+    if (ss.oz_is_fp64) std::swap(ss.t_simt[0], ss.t_oz);
+    ss.ms[1] = ss.t_tc;          // tensor-core products
+    ss.ms[2] = ss.t_simt[0];     // FP64 products: on the CUDA cores, or slices
+    ss.ms[3] = ss.t_simt[2];     // FP32 products (and copies of converged systems)
+    ss.ms[4] = ss.t_cmp;
+    ss.ms[5] = ss.t_simt[1];     // double-FP32 products
+    ss.ms[6] = ss.t_oz;          // tensor-core slice products
+    ss.ms[0] = std::max(0.f, mall - rest);   // mask, lists, plans
+}
 
 bool is_tc(Arith a) { return a == AR_BF16X3 || a == AR_FP16X3; }
 
@@ -559,9 +653,12 @@ Arith fp64_arith(int mode, int b, double tau) {
 // tab[t][p]: arithmetic of job p for the systems in tier t; tiers_present:
 // bit t set when some active system is in tier t (the per-system tiers are in
 // h->sd.tier on the device)
-// lin: an active system's c_lin is not 0
+// lin: an active system's c_lin is not 0; copies: some system is not active
+// (its blocks are copied).  The host waits twice, for the size of the mask and
+// for that of the result (and once more per further group); the device may
+// still be working on the compaction when the call returns (finish_step).
 StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
-                   const Arith (*tab)[kMaxJobs], unsigned tiers_present, bool lin) {
+                   const Arith (*tab)[kMaxJobs], unsigned tiers_present, bool lin, bool copies) {
     cudaStream_t st = h->stream;
     const int NB = in.NB, b = in.b, njob = jt.njob;
     const size_t bb = (size_t)b * b;
@@ -632,7 +729,7 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
     // are large (above 4 GiB the solve's time dwarfs a re-allocation)
     const size_t big = size_t(4) << 30;
     if (!tc && in.ophi.cap * sizeof(uint16_t) > big) in.ophi.release();
-    if (!(tc && lin) && h->tcw.xlin.cap * sizeof(float) > big) h->tcw.xlin.release();
+    if (!tc && h->tcw.xlin.cap * sizeof(float) > big) h->tcw.xlin.release();
     if (!f32_planes && in.opf32.cap * sizeof(float) > big) in.opf32.release();
     if (!any_c[1] && in.opf32lo.cap * sizeof(float) > big) in.opf32lo.release();
     if (tc) prepare_operands(in, tc_ar, lin, h->tcw, st);
@@ -646,94 +743,76 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
         launch_to_f32(in.val.p, in.opf32.p, in.total * (int64_t)bb, st, any_c[1] ? in.opf32lo.p : nullptr);
     }
 
+    // symbolic phase: the mask, its row pointers and the ranks of its upper slots
     h->row_cnt.ensure(nrows);
     h->row_off.ensure(nrows);
-    h->counters.ensure(8);
+    h->out_rp.ensure(nrows + 1);
+    h->urp.ensure(nrows + 1);
+    h->scan_tmp32.ensure(scan_tmp_elems(nrows + 1));
+    h->scan_tmp64.ensure(scan_tmp_elems(nrows + 1));
+    h->counters.ensure(kCtrInts);
+    HostStep *hs = h->step_host.ensure(1);
     int64_t cap = std::max<int64_t>(h->pool_cap_hint, 4 * in.total + 1024);
-    int top = 0;
-    for (int attempt = 0; attempt < 4; ++attempt) {
+    SymOut so{};
+    for (int attempt = 0;; ++attempt) {
         if (cap > INT32_MAX / 2) throw Error{RDM_ECAPACITY, "symbolic pool exceeds 2^30 blocks"};
         h->pool_col.ensure(cap);
         h->pool_npair.ensure(cap);
-        RDM_CUDA_TRY(cudaMemsetAsync(h->counters.p, 0, 8 * sizeof(int), st));
-        SymOut so{h->row_cnt.p, h->row_off.p, h->pool_col.p, h->pool_npair.p, h->counters.p,
-                  (int)h->pool_col.cap, h->counters.p + 1};
+        RDM_CUDA_TRY(cudaMemsetAsync(h->counters.p, 0, kCtrInts * sizeof(int), st));
+        so = SymOut{h->row_cnt.p, h->row_off.p, h->pool_col.p, h->pool_npair.p, h->counters.p + kCtrTop,
+                    (int)h->pool_col.cap, h->counters.p + kCtrTop + 1,
+                    reinterpret_cast<unsigned long long *>(h->counters.p + kCtrPairs)};
         launch_symbolic(in, jt, h->sd, h->S, so, st, h->prm.symbolic_hash ? kSymMaxNs + 1 : max_ns);
-        int hc[2];
-        d2h(hc, h->counters.p, 2, st);
+        scan_exclusive_pair(h->row_cnt.p, h->out_rp.p, h->urp.p, nrows, h->scan_tmp64.p, st);
+        d2h(hs->ctr, h->counters.p, kCtrInts, st);
+        d2h(&hs->nupper, h->urp.p + nrows, 1, st);
         sync(h);
-        top = hc[0];
-        if (!hc[1]) break;
-        if (hc[1] == 2)
+        const int top = hs->ctr[kCtrTop], over = hs->ctr[kCtrTop + 1];
+        if (!over) break;
+        if (over == 2)
             throw Error{RDM_ECAPACITY, "a block row of a product reaches more than 6144 distinct block columns"};
-        cap = (int64_t)top + top / 4 + 1024;
         if (attempt == 3) throw Error{RDM_ECAPACITY, "symbolic pool overflow after retries"};
+        cap = (int64_t)top + top / 4 + 1024;
     }
-    h->pool_cap_hint = std::max<int64_t>(h->pool_cap_hint, top);
-
-    // output pattern
-    h->out_rp.ensure(nrows + 1);
-    h->scan_tmp32.ensure(scan_tmp_elems(nrows + 1));
-    scan_exclusive_i32(h->row_cnt.p, h->out_rp.p, nrows, h->scan_tmp32.p, st);
-    const int64_t nslot = top;
+    const int64_t nslot = hs->ctr[kCtrTop], nupper = hs->nupper;
+    const int64_t npairs = *reinterpret_cast<int64_t *>(hs->ctr + kCtrPairs);
+    h->pool_cap_hint = std::max<int64_t>(h->pool_cap_hint, nslot);
     ss.nslot = nslot;
+    ss.npairs = npairs;
+
+    // output pattern, pair lists (only for the jobs on the CUDA cores; the
+    // tensor-core kernels build their own K-steps), slot_x / slot_t for every job
     out.nmat = njob;
     out.NB = NB;
     out.b = b;
-    int *mcol = h->mask_col.ensure(std::max<int64_t>(nslot, 1));
-    h->slot_row.ensure(std::max<int64_t>(nslot, 1));
-    h->slot_job.ensure(std::max<int64_t>(nslot, 1));
-    h->slot_npair.ensure(std::max<int64_t>(nslot, 1));
-    SymOut so{h->row_cnt.p, h->row_off.p, h->pool_col.p, h->pool_npair.p, h->counters.p,
-              (int)h->pool_col.cap, h->counters.p + 1};
-    launch_gather(so, njob, NB, h->out_rp.p, mcol, h->slot_row.p, h->slot_job.p,
-                  h->slot_npair.p, st);
-    h->pair_off.ensure(nslot + 1);
-    h->scan_tmp64.ensure(scan_tmp_elems((int)nslot + 1));
-    scan_exclusive_i64(h->slot_npair.p, h->pair_off.p, (int)nslot, h->scan_tmp64.p, st);
-    int64_t npairs = 0;
-    d2h(&npairs, h->pair_off.p + nslot, 1, st);
-    // block triples per kernel class (tensor cores, FP64, FP32, double-FP32) for the accounting
-    h->class_pairs.ensure(5);
-    RDM_CUDA_TRY(cudaMemsetAsync(h->class_pairs.p, 0, 5 * sizeof(unsigned long long), st));
-    launch_class_pairs(h->slot_row.p, mcol, h->slot_npair.p, h->slot_job.p, nslot, h->sd.sys_of_row.p,
-                       h->sd.active.p, h->sd.tier.p, tcm, m64, cm[2], cm[1], moz, h->class_pairs.p, st);
-    unsigned long long cls[5] = {0, 0, 0, 0, 0};
-    d2h(cls, h->class_pairs.p, 5, st);
-    sync(h);
-    ss.npairs = npairs;
-    ss.pairs_tc = (int64_t)cls[0];
-    ss.pairs_64 = (int64_t)cls[1];
-    ss.pairs_32 = (int64_t)cls[2];
-    ss.pairs_ff = (int64_t)cls[3];
-    ss.pairs_oz = (int64_t)cls[4];
-    ss.pairs_simt = (any_oz8 ? 0 : ss.pairs_64) + ss.pairs_32 + ss.pairs_ff;
-    if (any_c[0] || any_c[1] || any_c[2]) {
+    const int64_t ns1 = std::max<int64_t>(nslot, 1);
+    int *mcol = h->mask_col.ensure(ns1);
+    h->slot_row.ensure(ns1);
+    h->slot_job.ensure(ns1);
+    h->uidx.ensure(ns1);
+    h->slot_x.ensure(ns1);
+    h->slot_t.ensure(ns1);
+    const bool lists = any_c[0] || any_c[1] || any_c[2];
+    if (lists) {
+        h->slot_npair.ensure(ns1);
+        h->pair_off.ensure(nslot + 1);
+        h->scan_tmp64.ensure(scan_tmp_elems((int)nslot + 1));
         h->pair_a.ensure(std::max<int64_t>(npairs, 1));
         h->pair_b.ensure(std::max<int64_t>(npairs, 1));
     }
-    h->slot_x.ensure(std::max<int64_t>(nslot, 1));
-    h->slot_t.ensure(std::max<int64_t>(nslot, 1));
-    // pair lists only for the jobs on the CUDA cores (the tensor-core kernel
-    // builds its own K-steps); slot_x / slot_t for every job
-    launch_pairs(in, jt, h->sd, h->out_rp.p, mcol, h->slot_row.p, h->slot_job.p, h->pair_off.p,
-                 nslot, NB, h->pair_a.p, h->pair_b.p, h->slot_x.p, h->slot_t.p, h->counters.p + 2, st,
-                 simt);
+    const ClassMasks masks{{tcm, m64, cm[2], cm[1], moz}};
+    launch_gather(so, njob, NB, h->out_rp.p, h->urp.p, mcol, h->slot_row.p, h->slot_job.p,
+                  lists ? h->slot_npair.p : nullptr, h->uidx.p, h->sd, masks,
+                  reinterpret_cast<unsigned long long *>(h->counters.p + kCtrClass), st);
+    if (lists) scan_exclusive_i64(h->slot_npair.p, h->pair_off.p, (int)nslot, h->scan_tmp64.p, st);
+    launch_pairs(in, jt, h->sd, h->out_rp.p, mcol, h->slot_row.p, h->slot_job.p, lists ? h->pair_off.p : nullptr,
+                 nslot, NB, h->pair_a.p, h->pair_b.p, h->slot_x.p, h->slot_t.p, h->counters.p + kCtrErr, st, simt);
     DevBuf<int> *worklist[kSimt] = {&h->work, &h->work2, &h->work3};
-    for (int c = 0; c < kSimt; ++c)
-        if (any_c[c] || c == first_c) worklist[c]->ensure(std::max<int64_t>(nslot, 1));
-    // rank of every upper slot among the upper slots (the products store
-    // only those; compaction writes the lower blocks as transposes)
-    h->uidx.ensure(nslot + 1);
-    h->scan_tmp_s.ensure(scan_tmp_elems((int)nslot + 1));
-    launch_upper_flags(h->slot_row.p, mcol, nslot, h->uidx.p, st);
-    scan_exclusive_i32(h->uidx.p, h->uidx.p, (int)nslot, h->scan_tmp_s.p, st);
-    int hq[2] = {0, 0};
-    d2h(&hq[0], h->counters.p + 2, 1, st);
-    d2h(&hq[1], h->uidx.p + nslot, 1, st);
-    sync(h);
-    if (hq[0]) throw Error{RDM_ECUDA, "internal error: pair lists inconsistent with the mask (code " + std::to_string(hq[0]) + ")"};
-    const int64_t nupper = hq[1];
+    bool run_c[kSimt];
+    for (int c = 0; c < kSimt; ++c) {
+        run_c[c] = any_c[c] || (c == first_c && copies);
+        if (run_c[c]) worklist[c]->ensure(ns1);
+    }
 
     // Numeric phase, fused truncation and compaction, one group of
     // consecutive super-rows (the block rows of a tensor-core tile, 128 / b of
@@ -770,8 +849,6 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
     if (nupper <= budget) {
         gunit.push_back(nunit);
     } else {
-        h->urp.ensure(nrows + 1);
-        launch_gather_i32(h->out_rp.p, h->uidx.p, nrows, h->urp.p, st);
         hrp.resize(nrows + 1);
         hurp.resize(nrows + 1);
         d2h(hrp.data(), h->out_rp.p, nrows + 1, st);
@@ -798,83 +875,98 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
     h->cnt_rows.ensure(nrows + 1);
     out.row_ptr.ensure(nrows + 1);
     int kept = 0;
-    float t_simt[kSimt] = {0, 0, 0}, t_tc = 0, t_cmp = 0, t_oz = 0;
     const int ev_simt[kSimt] = {5, 6, 4};   // events after each CUDA-core class
     for (int g = 0; g < ngroup; ++g) {
         const int ua = gunit[g], ub = gunit[g + 1];
-        const int64_t s0 = gslot(ua), s1 = gslot(ub), u0 = gupper(ua);
+        const int64_t s0 = gslot(ua), s1 = gslot(ub), u0 = gupper(ua), nup = gupper(ub) - u0;
         const int r0 = unit_row(ua), nr = unit_row(ub) - r0;
-        RDM_CUDA_TRY(cudaMemsetAsync(h->counters.p + 3, 0, kSimt * sizeof(int), st));
-        // CUDA-core work per class: the selected jobs, and in the first class
-        // the copies of converged systems
-        for (int c = 0; c < kSimt; ++c)
-            if (any_c[c] || c == first_c)
-                launch_build_work(h->slot_row.p, mcol, s0, s1, worklist[c]->p, h->counters.p + 3 + c, st,
-                                  h->sd.sys_of_row.p, h->sd.active.p, h->slot_job.p, h->sd.tier.p, cm[c],
-                                  c == first_c ? 1 : 0);
-        TcPlan plan{}, oplan{};
-        if (tc) plan = build_tc_plan(in, jt, h->sd, h->out_rp.p, mcol, h->tcw, tcm, ua, ub, st);
-        if (any_oz) oplan = build_oz_plan(in, jt, h->sd, h->out_rp.p, mcol, h->tcw_oz, ozm, ua, ub, st);
-        const bool tc_g = tc && plan.ntile > 0;
-        const bool oz_g = any_oz && oplan.ntile > 0;
-        int nwork[kSimt];
-        d2h(nwork, h->counters.p + 3, kSimt, st);
-        sync(h);
-
-        NumArgs a{};
-        a.in_val = in.val.p; a.in_nrm = in.nrm.p;
-        a.in_f32 = f32_planes ? in.opf32.p : nullptr;
-        a.in_f32lo = any_c[1] ? in.opf32lo.p : nullptr;
-        a.pair_a = h->pair_a.p; a.pair_b = h->pair_b.p; a.pair_off = h->pair_off.p;
-        a.slot_row = h->slot_row.p; a.slot_job = h->slot_job.p; a.slot_x = h->slot_x.p; a.slot_t = h->slot_t.p;
-        a.sys_of_row = h->sd.sys_of_row.p;
-        a.c_lin = h->sd.c_lin.p; a.c_sq = h->sd.c_sq.p; a.tau0 = h->sd.tau0.p; a.tau1 = h->sd.tau1.p;
-        a.active = h->sd.active.p;
-        for (int p = 0; p < njob; ++p) a.job_tau_sel[p] = jt.job[p].tau_sel;
-        a.out_val = h->out_val.p; a.out_nrm = h->out_nrm.p; a.keep = h->keep.p;
-        a.uidx = h->uidx.p; a.u0 = u0; a.b = b;
-        h->work_ctr.ensure(kSimt);
-        RDM_CUDA_TRY(cudaMemsetAsync(h->work_ctr.p, 0, kSimt * sizeof(int), st));
-        RDM_CUDA_TRY(cudaEventRecord(h->ev[1], st));
-        const long long lg = g_kernel_launches;
-        for (int c = 0; c < kSimt; ++c) {
-            if (nwork[c]) {
-                NumArgs ac = a;
-                ac.work = worklist[c]->p;
-                ac.nwork = nwork[c];
-                ac.work_next = h->work_ctr.p + c;
-                launch_numeric_simt(ac, simt_ar[c], st);
-            }
-            RDM_CUDA_TRY(cudaEventRecord(h->ev[ev_simt[c]], st));
-        }
-        ss.simt_launches += (int)(g_kernel_launches - lg);
-        if (tc_g) {
-            const long long lt = g_kernel_launches;
-            ss.issued_tc += launch_numeric_tc(a, in, jt, tc_ar, h->tcw, NB, plan, st);
-            ss.tc_launches += (int)(g_kernel_launches - lt);
-        }
-        RDM_CUDA_TRY(cudaEventRecord(h->ev[2], st));
-        if (oz_g) {
-            const long long lt = g_kernel_launches;
-            ss.issued_oz += launch_numeric_oz(a, in, jt, mcol, h->ozw, h->tcw_oz, oplan, st);
-            ss.oz_launches += (int)(g_kernel_launches - lt);
-        }
-        RDM_CUDA_TRY(cudaEventRecord(h->ev[7], st));
-
-        // compaction of the group's rows, appended after the previous groups
+        // room for the K-steps (a tile of 4 x 8 blocks has 5 to 12 pairs to a
+        // step, one of 4 x 2 about 3); a plan that needs more is built again
+        const int64_t gpairs = (int64_t)((double)npairs * (double)nup / (double)std::max<int64_t>(nupper, 1)) + 1;
+        int64_t steps_tc = std::min(gpairs, gpairs / 4 + 65536) + 1024, steps_oz = gpairs / 2 + 1024;
         CompactArgs ca{};
-        ca.out_rp = h->out_rp.p; ca.out_col = mcol; ca.slot_row = h->slot_row.p; ca.slot_t = h->slot_t.p;
-        ca.uidx = h->uidx.p; ca.out_val = h->out_val.p; ca.out_nrm = h->out_nrm.p; ca.keep = h->keep.p;
-        ca.u0 = u0; ca.dest = h->dest.p; ca.new_rp = out.row_ptr.p; ca.r0 = r0; ca.nrows = nr; ca.b = b;
-        launch_compact_count(ca, h->cnt_rows.p, st);
-        scan_exclusive_i32(h->cnt_rows.p, out.row_ptr.p + r0, nr, h->scan_tmp32.p, st, kept);
         int kept_end = 0;
-        d2h(&kept_end, out.row_ptr.p + r0 + nr, 1, st);
-        int tc_err = 0, oz_err = 0;
-        if (tc_g) d2h(&tc_err, h->tcw.counters.p, 1, st);
-        if (oz_g) d2h(&oz_err, h->tcw_oz.counters.p, 1, st);
-        sync(h);
-        tc_err |= oz_err;
+        for (int attempt = 0;; ++attempt) {
+            RDM_CUDA_TRY(cudaMemsetAsync(h->counters.p + kCtrWork, 0, (kCtrInts - kCtrWork) * sizeof(int), st));
+            // CUDA-core work per class: the selected jobs, and in the first class
+            // the copies of converged systems
+            for (int c = 0; c < kSimt; ++c)
+                if (run_c[c])
+                    launch_build_work(h->slot_row.p, mcol, s0, s1, worklist[c]->p, h->counters.p + kCtrWork + c, st,
+                                      h->sd.sys_of_row.p, h->sd.active.p, h->slot_job.p, h->sd.tier.p, cm[c],
+                                      c == first_c ? 1 : 0);
+            TcPlan plan{}, oplan{};
+            if (tc) plan = build_tc_plan(in, jt, h->sd, h->out_rp.p, mcol, h->tcw, tcm, ua, ub, nup, steps_tc, st);
+            if (any_oz) oplan = build_oz_plan(in, jt, h->sd, h->out_rp.p, mcol, h->tcw_oz, ozm, ua, ub, nup, steps_oz, st);
+
+            NumArgs a{};
+            a.in_val = in.val.p; a.in_nrm = in.nrm.p;
+            a.in_f32 = f32_planes ? in.opf32.p : nullptr;
+            a.in_f32lo = any_c[1] ? in.opf32lo.p : nullptr;
+            a.pair_a = h->pair_a.p; a.pair_b = h->pair_b.p; a.pair_off = lists ? h->pair_off.p : nullptr;
+            a.slot_row = h->slot_row.p; a.slot_job = h->slot_job.p; a.slot_x = h->slot_x.p; a.slot_t = h->slot_t.p;
+            a.sys_of_row = h->sd.sys_of_row.p;
+            a.c_lin = h->sd.c_lin.p; a.c_sq = h->sd.c_sq.p; a.tau0 = h->sd.tau0.p; a.tau1 = h->sd.tau1.p;
+            a.active = h->sd.active.p;
+            for (int p = 0; p < njob; ++p) a.job_tau_sel[p] = jt.job[p].tau_sel;
+            a.out_val = h->out_val.p; a.out_nrm = h->out_nrm.p; a.keep = h->keep.p;
+            a.uidx = h->uidx.p; a.u0 = u0; a.b = b;
+            RDM_CUDA_TRY(cudaEventRecord(h->ev[1], st));
+            const long long lg = g_kernel_launches;
+            for (int c = 0; c < kSimt; ++c) {
+                if (run_c[c]) {
+                    NumArgs ac = a;
+                    ac.work = worklist[c]->p;
+                    ac.nwork = h->counters.p + kCtrWork + c;
+                    ac.max_work = (int)nup;
+                    ac.work_next = h->counters.p + kCtrNext + c;
+                    launch_numeric_simt(ac, simt_ar[c], st);
+                }
+                RDM_CUDA_TRY(cudaEventRecord(h->ev[ev_simt[c]], st));
+            }
+            ss.simt_launches += (int)(g_kernel_launches - lg);
+            const long long lt = g_kernel_launches;
+            if (tc) launch_numeric_tc(a, in, jt, tc_ar, h->tcw, NB, plan, st);
+            ss.tc_launches += (int)(g_kernel_launches - lt);
+            RDM_CUDA_TRY(cudaEventRecord(h->ev[2], st));
+            const long long lo = g_kernel_launches;
+            if (any_oz) launch_numeric_oz(a, in, jt, mcol, h->ozw, h->tcw_oz, oplan, st);
+            ss.oz_launches += (int)(g_kernel_launches - lo);
+            if (any_oz8) launch_diag_fp64(a, in, jt, m64, h->out_rp.p, mcol, h->sd.tier.p, r0, nr, st);
+            RDM_CUDA_TRY(cudaEventRecord(h->ev[7], st));
+
+            // compaction of the group's rows, appended after the previous groups
+            ca = CompactArgs{};
+            ca.out_rp = h->out_rp.p; ca.out_col = mcol; ca.slot_row = h->slot_row.p; ca.slot_t = h->slot_t.p;
+            ca.uidx = h->uidx.p; ca.out_val = h->out_val.p; ca.out_nrm = h->out_nrm.p; ca.keep = h->keep.p;
+            ca.u0 = u0; ca.dest = h->dest.p; ca.new_rp = out.row_ptr.p; ca.r0 = r0; ca.nrows = nr; ca.b = b;
+            launch_compact_count(ca, h->cnt_rows.p, st);
+            scan_exclusive_i32(h->cnt_rows.p, out.row_ptr.p + r0, nr, h->scan_tmp32.p, st, kept);
+            d2h(&hs->kept, out.row_ptr.p + r0 + nr, 1, st);
+            d2h(hs->ctr, h->counters.p, kCtrInts, st);
+            if (tc) d2h(hs->tc, h->tcw.counters.p, 8, st);
+            if (any_oz) d2h(hs->oz, h->tcw_oz.counters.p, 8, st);
+            if (g == ngroup - 1 && NB)
+                RDM_CUDA_TRY(cudaMemcpy2DAsync(hs->rp, sizeof(int), out.row_ptr.p, (size_t)NB * sizeof(int), sizeof(int),
+                                               njob + 1, cudaMemcpyDeviceToHost, st));
+            sync(h);
+            if (hs->ctr[kCtrErr])
+                throw Error{RDM_ECUDA, "internal error: pair lists inconsistent with the mask (code " +
+                                           std::to_string(hs->ctr[kCtrErr]) + ")"};
+            const int64_t nst_tc = tc ? *reinterpret_cast<int64_t *>(hs->tc + 4) : 0;
+            const int64_t nst_oz = any_oz ? *reinterpret_cast<int64_t *>(hs->oz + 4) : 0;
+            const bool again = (tc && hs->tc[1]) || (any_oz && hs->oz[1]);
+            if (!again) {
+                ss.issued_tc += (double)nst_tc * tc_step_flops(b);
+                if (any_oz) ss.issued_oz += (double)nst_oz * oz_step_flops(h->ozw);
+                break;
+            }
+            if (attempt == 3) throw Error{RDM_ECAPACITY, "K-step lists outgrew their buffers repeatedly"};
+            steps_tc = std::max(steps_tc, nst_tc);
+            steps_oz = std::max(steps_oz, nst_oz);
+        }
+        kept_end = hs->kept;
+        const int tc_err = (tc ? hs->tc[0] : 0) | (any_oz ? hs->oz[0] : 0);
         if (tc_err & 8) throw Error{RDM_EBADBSR, "an operand's block pattern is not symmetric"};
         if (tc_err)
             throw Error{tc_err & 1 ? RDM_ETIMEOUT : RDM_ECUDA,
@@ -896,38 +988,25 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
         launch_compact_copy(ca, kept_end, st);
         kept = kept_end;
         RDM_CUDA_TRY(cudaEventRecord(h->ev[3], st));
-        RDM_CUDA_TRY(cudaEventSynchronize(h->ev[3]));
-        float mc[kSimt] = {0, 0, 0}, m42 = 0, m23 = 0, moz = 0;
-        cudaEventElapsedTime(&mc[0], h->ev[1], h->ev[ev_simt[0]]);             // FP64 class
-        cudaEventElapsedTime(&mc[1], h->ev[ev_simt[0]], h->ev[ev_simt[1]]);    // double-FP32 class
-        cudaEventElapsedTime(&mc[2], h->ev[ev_simt[1]], h->ev[ev_simt[2]]);    // FP32 class (and copies)
-        cudaEventElapsedTime(&m42, h->ev[ev_simt[2]], h->ev[2]);               // tensor-core launch
-        cudaEventElapsedTime(&moz, h->ev[2], h->ev[7]);                        // slice-product launch
-        cudaEventElapsedTime(&m23, h->ev[7], h->ev[3]);                        // compaction
-        for (int c = 0; c < kSimt; ++c) t_simt[c] += mc[c];
-        t_tc += m42; t_cmp += m23; t_oz += moz;
+        if (g + 1 < ngroup) {
+            RDM_CUDA_TRY(cudaEventSynchronize(h->ev[3]));
+            add_times(h, ss);
+        }
     }
+    const unsigned long long *cls = reinterpret_cast<unsigned long long *>(hs->ctr + kCtrClass);
+    ss.pairs_tc = (int64_t)cls[0];
+    ss.pairs_64 = (int64_t)cls[1];
+    ss.pairs_32 = (int64_t)cls[2];
+    ss.pairs_ff = (int64_t)cls[3];
+    ss.pairs_oz = (int64_t)cls[4];
+    ss.pairs_simt = (any_oz8 ? 0 : ss.pairs_64) + ss.pairs_32 + ss.pairs_ff;
+    ss.oz_is_fp64 = any_oz8;
+    for (int t = 0; t < kMaxTiers; ++t) ss.oz_is_fp64 = ss.oz_is_fp64 && !moz.m[t];
     ss.bytes = ((double)in.total * (tc ? 4.0 : 8.0) + (any_oz ? (double)in.nnzb[0] * 2.0 * h->ozw.nslice : 0.0) +
                 (double)nupper * 8.0) * (double)bb;
     out.total = kept;
-    std::vector<int> rp(nrows + 1);
-    d2h(rp.data(), out.row_ptr.p, nrows + 1, st);
-    sync(h);
-    float mall = 0;
-    cudaEventElapsedTime(&mall, h->ev[0], h->ev[3]);
-    ss.ms[1] = t_tc;          // tensor-core products
-    // FP64 products: on the CUDA cores, or the slice launch when it held no others
-    bool oz_other = false;
-    for (int t = 0; t < kMaxTiers; ++t) oz_other = oz_other || moz.m[t];
-    if (any_oz8 && !oz_other) std::swap(t_simt[0], t_oz);
-    ss.ms[2] = t_simt[0];
-    ss.ms[3] = t_simt[2];     // FP32 products (and copies of converged systems)
-    ss.ms[4] = t_cmp;
-    ss.ms[5] = t_simt[1];     // double-FP32 products
-    ss.ms[6] = t_oz;          // tensor-core slice products
-    ss.ms[0] = std::max(0.f, mall - (t_simt[0] + t_simt[1] + t_simt[2] + t_tc + t_cmp + t_oz));  // mask, lists, plans
     out.nnzb.assign(njob, 0);
-    for (int p = 0; p < njob; ++p) out.nnzb[p] = rp[(size_t)(p + 1) * NB] - rp[(size_t)p * NB];
+    for (int p = 0; p < njob; ++p) out.nnzb[p] = hs->rp[p + 1] - hs->rp[p];
     return ss;
 }
 
@@ -941,16 +1020,17 @@ JobTable solve_jobs(int nd) {
 
 // per-system stats of the current X: [S][3+nd]
 std::vector<double> stats(rdm_handle *h, MatSet &X) {
-    const int nq = 3 + h->nd, parts = row_stats_parts(h->NB);
+    const int nq = 3 + h->nd, parts = row_stats_parts();
     h->row_part.ensure((size_t)nq * h->NB * parts);
     h->sys_q.ensure((size_t)nq * h->S);
     launch_row_stats(X.row_ptr.p, X.col.p, X.val.p, X.nmat, h->NB, h->bs, h->H0.row_ptr.p,
-                     h->H0.col.p, h->H0.val.p, parts, h->row_part.p, h->stream);
+                     h->H0.col.p, h->H0.val.p, h->row_part.p, h->stream);
     launch_sys_sum(h->row_part.p, nq, h->NB, h->sd.row0.p, h->sd.nbs.p, h->S, h->sys_q.p, h->stream, parts);
-    std::vector<double> q((size_t)nq * h->S);
-    d2h(q.data(), h->sys_q.p, q.size(), h->stream);
+    const size_t n = (size_t)nq * h->S;
+    double *q = h->scalars_host.ensure(std::max(n, SysDev::step_doubles(h->S)));
+    d2h(q, h->sys_q.p, n, h->stream);
     sync(h);
-    return q;
+    return std::vector<double>(q, q + n);
 }
 
 // ---------------------------------------------------------------------------
@@ -1018,18 +1098,12 @@ void concat(rdm_handle *h, std::initializer_list<SetRange> parts, MatSet &out) {
 void set_products(rdm_handle *h, MatSet &in, const JobTable &jt, const std::vector<double> &cl,
                   const std::vector<double> &cq, double tau, Arith ar, MatSet &out) {
     const int S = h->S;
-    std::vector<double> t(S, tau);
-    std::vector<int> one(S, 1), zero(S, 0);
-    h2d(h->sd.c_lin.p, cl.data(), S, h->stream);
-    h2d(h->sd.c_sq.p, cq.data(), S, h->stream);
-    h2d(h->sd.tau0.p, t.data(), S, h->stream);
-    h2d(h->sd.tau1.p, t.data(), S, h->stream);
-    h2d(h->sd.active.p, one.data(), S, h->stream);
-    h2d(h->sd.tier.p, zero.data(), S, h->stream);
+    const std::vector<double> t(S, tau);
+    upload_step(h, cl, cq, t, t, std::vector<int>(S, 1), std::vector<int>(S, 0));
     if (ar == AR_FP64) ar = fp64_arith(h->prm.mode, h->bs, tau);
     Arith tab[kMaxTiers][kMaxJobs];
     for (int p = 0; p < kMaxJobs; ++p) tab[0][p] = ar;
-    multiply(h, in, out, jt, tab, 1u, std::any_of(cl.begin(), cl.end(), [](double c) { return c != 0.0; }));
+    multiply(h, in, out, jt, tab, 1u, std::any_of(cl.begin(), cl.end(), [](double c) { return c != 0.0; }), false);
 }
 
 // the same with one coefficient pair, in FP64
@@ -1270,10 +1344,9 @@ int run_solve(rdm_handle *h, rdm_info *info_out) {
     RDM_CUDA_TRY(cudaEventCreate(&ev1));
     int it = 0;
     bool any_active = true;
-    std::vector<double> q;
+    std::vector<double> q = stats(h, X);      // of the current X, from here on
     for (it = 0; it <= P.max_iter; ++it) {
         MatSet &Xc = h->X[h->cur];
-        q = stats(h, Xc);
         const int nq = 3 + nd;
         any_active = false;
         for (int s = 0; s < S; ++s) {
@@ -1408,19 +1481,18 @@ int run_solve(rdm_handle *h, rdm_info *info_out) {
                 for (int p = 0; p < jt.njob; ++p) ar[p] = tab[t][p];
                 break;
             }
-        bool lin = false;     // an active system has a linear term
-        for (int s = 0; s < S; ++s) lin = lin || (act[s] && c_lin[s] != 0.0);
-        h2d(h->sd.tier.p, tier_of.data(), S, st);
-        h2d(h->sd.c_lin.p, c_lin.data(), S, st);
-        h2d(h->sd.c_sq.p, c_sq.data(), S, st);
-        h2d(h->sd.tau0.p, t0.data(), S, st);
-        h2d(h->sd.tau1.p, t1.data(), S, st);
-        h2d(h->sd.active.p, act.data(), S, st);
+        bool lin = false, copies = false;     // an active system has a linear term; a system is not active
+        for (int s = 0; s < S; ++s) {
+            lin = lin || (act[s] && c_lin[s] != 0.0);
+            copies = copies || !act[s];
+        }
+        upload_step(h, c_lin, c_sq, t0, t1, act, tier_of);
         RDM_CUDA_TRY(cudaEventRecord(ev0, st));
         MatSet &Xn = h->X[1 - h->cur];
-        StepStats sst = multiply(h, Xc, Xn, jt, tab, tiers_present, lin);
+        StepStats sst = multiply(h, Xc, Xn, jt, tab, tiers_present, lin, copies);
         RDM_CUDA_TRY(cudaEventRecord(ev1, st));
-        RDM_CUDA_TRY(cudaEventSynchronize(ev1));
+        q = stats(h, Xn);                     // waits for the step
+        finish_step(h, sst);
         float ms = 0;
         cudaEventElapsedTime(&ms, ev0, ev1);
         const double fpb = 2.0 * b * b * b;
@@ -1463,10 +1535,10 @@ int run_solve(rdm_handle *h, rdm_info *info_out) {
 
     // polarizability: alpha[g][d] = -spin * <P1_d, H1_g>
     MatSet &Xf = h->X[h->cur];
-    compute_alpha(h);
     // final pattern on the host for the getters, summary per system
     h->final_rp.resize((size_t)Xf.nmat * NB + 1);
     d2h(h->final_rp.data(), Xf.row_ptr.p, h->final_rp.size(), st);
+    compute_alpha(h);
     sync(h);
     auto t_end = std::chrono::steady_clock::now();
     double wall_ms = std::chrono::duration<double, std::milli>(t_end - t_start).count();
@@ -1508,8 +1580,6 @@ int run_solve(rdm_handle *h, rdm_info *info_out) {
         I.device_bytes_peak = (int64_t)g_dev_bytes_peak.load();
         I.product_groups = max_groups;
     }
-    // band energy of the result: recompute the stats of the final X
-    q = stats(h, Xf);
     for (int s = 0; s < S; ++s) {
         h->info[s].band_energy0 = q[(size_t)s * nq + 2];
         h->info[s].trace_error = q[(size_t)s * nq] - nocc[s];
@@ -1867,11 +1937,12 @@ int run_solve_dirs(rdm_handle *h, rdm_info *info_out) {
 // between autotuning probes at different block sizes, whose grow-only buffers
 // would otherwise add up.
 void release_work(rdm_handle *h) {
-    for (auto *b : {&h->row_cnt, &h->row_off, &h->pool_col, &h->pool_npair, &h->mask_col, &h->out_rp, &h->slot_row,
+    for (auto *b : {&h->row_off, &h->pool_col, &h->pool_npair, &h->mask_col, &h->out_rp, &h->slot_row,
                     &h->slot_job, &h->slot_npair, &h->slot_x, &h->slot_t, &h->work, &h->work2, &h->work3,
-                    &h->scan_tmp32, &h->pair_a, &h->pair_b, &h->cnt_rows, &h->uidx, &h->scan_tmp_s, &h->urp,
+                    &h->scan_tmp32, &h->pair_a, &h->pair_b, &h->cnt_rows, &h->uidx, &h->urp,
                     &h->dest, &h->cpsrc})
         b->release();
+    h->row_cnt.release();
     h->pair_off.release();
     h->scan_tmp64.release();
     h->out_val.release();
@@ -2448,19 +2519,12 @@ int rdm_block_product(rdm_handle *h, const rdm_bsr *A, const rdm_bsr *B, const r
         t.norb = {A->n};
         SysDev &sd = t.sd;
         sd.row0.ensure(1); sd.nbs.ensure(1); sd.n_orb.ensure(1); sd.sys_of_row.ensure(NB);
-        sd.c_lin.ensure(1); sd.c_sq.ensure(1); sd.tau0.ensure(1); sd.tau1.ensure(1); sd.active.ensure(1);
-        sd.tier.ensure(1);
-        RDM_CUDA_TRY(cudaMemsetAsync(sd.tier.p, 0, sizeof(int), t.stream));
+        sd.ensure_step(1);
         RDM_CUDA_TRY(cudaMemsetAsync(sd.row0.p, 0, sizeof(int), t.stream));
         RDM_CUDA_TRY(cudaMemsetAsync(sd.sys_of_row.p, 0, NB * sizeof(int), t.stream));
-        int one = 1;
         h2d(sd.nbs.p, &NB, 1, t.stream);
         h2d(sd.n_orb.p, &A->n, 1, t.stream);
-        h2d(sd.active.p, &one, 1, t.stream);
-        h2d(sd.c_lin.p, &c_lin, 1, t.stream);
-        h2d(sd.c_sq.p, &c_sq, 1, t.stream);
-        h2d(sd.tau0.p, &tau, 1, t.stream);
-        h2d(sd.tau1.p, &tau, 1, t.stream);
+        upload_step(&t, {c_lin}, {c_sq}, {tau}, {tau}, {1}, {0});
         JobTable jt{};
         jt.njob = 1;
         int ia = idx[0], ib = terms == 2 ? idx[1] : idx[0];
@@ -2471,7 +2535,7 @@ int rdm_block_product(rdm_handle *h, const rdm_bsr *A, const rdm_bsr *B, const r
         if (slices) tab[0][0] = AR_OZ;
         else tier_arith(mode, 0, jt.njob, tab[0]);
         MatSet res;
-        multiply(&t, in, res, jt, tab, 1u, c_lin != 0.0);
+        multiply(&t, in, res, jt, tab, 1u, c_lin != 0.0, false);
         int64_t n = res.nnzb[0];
         if (needed) *needed = n;
         if (!out || !out->row_ptr || out->nnzb < n || (n && (!out->col_idx || !out->vals))) {

@@ -36,46 +36,6 @@ __global__ void k_build_work(const int *__restrict__ slot_row, const int *__rest
     if (up) work[base + __popc(m & ((1u << lane) - 1u))] = (int)s;
 }
 
-__global__ void k_class_pairs(const int *__restrict__ slot_row, const int *__restrict__ out_col,
-                              const int *__restrict__ slot_npair, const int *__restrict__ slot_job, int64_t nslot,
-                              const int *__restrict__ sys_of_row, const int *__restrict__ active,
-                              const int *__restrict__ sys_tier, JobMask tc, JobMask m64, JobMask m32,
-                              JobMask mff, JobMask moz, unsigned long long *out) {
-    int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    unsigned long long c[5] = {0, 0, 0, 0, 0};
-    if (s < nslot && out_col[s] >= slot_row[s]) {
-        const int sys = sys_of_row[slot_row[s]];
-        if (active[sys]) {
-            const int t = sys_tier[sys] & (kMaxTiers - 1);
-            const unsigned bit = 1u << slot_job[s];
-            const unsigned long long np = (unsigned long long)slot_npair[s];
-            if (tc.m[t] & bit) c[0] = np;
-            else if (m64.m[t] & bit) c[1] = np;
-            else if (m32.m[t] & bit) c[2] = np;
-            else if (mff.m[t] & bit) c[3] = np;
-            else if (moz.m[t] & bit) c[4] = np;
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-        unsigned long long v = c[k];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if ((threadIdx.x & 31) == 0 && v) atomicAdd(&out[k], v);
-    }
-}
-
-__global__ void k_upper_flags(const int *__restrict__ slot_row, const int *__restrict__ out_col,
-                              int64_t nslot, int *__restrict__ uidx) {
-    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s < nslot) uidx[s] = out_col[s] >= slot_row[s] ? 1 : 0;
-}
-
-__global__ void k_gather_i32(const int *__restrict__ idx, const int *__restrict__ src, int n,
-                             int *__restrict__ dst) {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r <= n) dst[r] = src[idx[r]];
-}
-
 // one warp per row of the group: kept blocks (an upper slot on its own flag,
 // a lower one on its upper partner's)
 __global__ void k_compact_count(CompactArgs c, int *cnt) {
@@ -190,29 +150,6 @@ void launch_build_work(const int *slot_row, const int *out_col, int64_t s0, int6
     int64_t grid = (s1 - s0 + 255) / 256;
     k_build_work<<<(unsigned)grid, 256, 0, st>>>(slot_row, out_col, s0, s1, work, nwork, sys_of_row,
                                                  active, slot_job, sys_tier, job_mask, with_inactive);
-    RDM_LAUNCH_CHECK();
-}
-
-void launch_class_pairs(const int *slot_row, const int *out_col, const int *slot_npair, const int *slot_job,
-                        int64_t nslot, const int *sys_of_row, const int *active, const int *sys_tier,
-                        JobMask tc, JobMask m64, JobMask m32, JobMask mff, JobMask moz, unsigned long long *out,
-                        cudaStream_t st) {
-    if (nslot == 0) return;
-    const int64_t grid = (nslot + 255) / 256;
-    k_class_pairs<<<(unsigned)grid, 256, 0, st>>>(slot_row, out_col, slot_npair, slot_job, nslot, sys_of_row,
-                                                  active, sys_tier, tc, m64, m32, mff, moz, out);
-    RDM_LAUNCH_CHECK();
-}
-
-void launch_upper_flags(const int *slot_row, const int *out_col, int64_t nslot, int *uidx,
-                        cudaStream_t st) {
-    if (nslot == 0) return;
-    k_upper_flags<<<(unsigned)((nslot + 255) / 256), 256, 0, st>>>(slot_row, out_col, nslot, uidx);
-    RDM_LAUNCH_CHECK();
-}
-
-void launch_gather_i32(const int *idx, const int *src, int n, int *dst, cudaStream_t st) {
-    k_gather_i32<<<(n + 256) / 256, 256, 0, st>>>(idx, src, n, dst);
     RDM_LAUNCH_CHECK();
 }
 

@@ -53,6 +53,7 @@ __global__ void __launch_bounds__(Cfg<B>::NT) k_numeric_simt(NumArgs a) {
     const int tid = threadIdx.x;
 
     __shared__ int s_w;
+    const int nwork = *a.nwork;
     for (;;) {
         // work items are handed out in list order by an atomic counter, so the
         // blocks in flight stay close in the list and share operands in L2
@@ -60,14 +61,14 @@ __global__ void __launch_bounds__(Cfg<B>::NT) k_numeric_simt(NumArgs a) {
         __syncthreads();
         const int w = s_w;
         __syncthreads();
-        if (w >= a.nwork) break;
+        if (w >= nwork) break;
         const int s = a.work[w];
         const int i = a.slot_row[s];
         const int sys = a.sys_of_row[i];
         const int job = a.slot_job[s];
         const double cl = a.c_lin[sys], cq = a.c_sq[sys];
         const double tau = a.job_tau_sel[job] ? a.tau1[sys] : a.tau0[sys];
-        const int64_t p0 = a.pair_off[s], p1 = a.pair_off[s + 1];
+        const int64_t p0 = a.pair_off ? a.pair_off[s] : 0, p1 = a.pair_off ? a.pair_off[s + 1] : 0;
         const int st = a.slot_t[s], sx = a.slot_x[s];
 
         T acc[PER];
@@ -180,6 +181,7 @@ __global__ void __launch_bounds__(64) k_numeric_ff_b32(NumArgs a) {
     const float *planes[2] = {a.in_f32, a.in_f32lo};
 
     __shared__ int s_w;
+    const int nwork = *a.nwork;
     for (;;) {
         // work items are handed out in list order by an atomic counter, so the
         // blocks in flight stay close in the list and share operands in L2
@@ -187,13 +189,13 @@ __global__ void __launch_bounds__(64) k_numeric_ff_b32(NumArgs a) {
         __syncthreads();
         const int w = s_w;
         __syncthreads();
-        if (w >= a.nwork) break;
+        if (w >= nwork) break;
         const int s = a.work[w];
         const int i = a.slot_row[s];
         const int sys = a.sys_of_row[i];
         const int job = a.slot_job[s];
         const double tau = a.job_tau_sel[job] ? a.tau1[sys] : a.tau0[sys];
-        const int64_t p0 = a.pair_off[s], p1 = a.pair_off[s + 1];
+        const int64_t p0 = a.pair_off ? a.pair_off[s] : 0, p1 = a.pair_off ? a.pair_off[s + 1] : 0;
         const int st = a.slot_t[s], sx = a.slot_x[s];
 
         float acc[4][4], accl[4][4];
@@ -356,18 +358,19 @@ __global__ void __launch_bounds__(64, 8) k_numeric_f32_t84(NumArgs a) {
     const int kh = hw & 1, ch = hw >> 1;
     const int r0 = l >> 2, c0 = 16 * ch + (l & 3);
     const int k0 = 16 * kh;
+    const int nwork = *a.nwork;
     for (;;) {
         if (threadIdx.x == 0) s_w = atomicAdd(a.work_next, 1);
         __syncthreads();
         const int w = s_w;
         __syncthreads();
-        if (w >= a.nwork) break;
+        if (w >= nwork) break;
         const int s = a.work[w];
         const int i = a.slot_row[s];
         const int sys = a.sys_of_row[i];
         const int job = a.slot_job[s];
         const double tau = a.job_tau_sel[job] ? a.tau1[sys] : a.tau0[sys];
-        const int64_t p0 = a.pair_off[s], p1 = a.pair_off[s + 1];
+        const int64_t p0 = a.pair_off ? a.pair_off[s] : 0, p1 = a.pair_off ? a.pair_off[s + 1] : 0;
         const int st = a.slot_t[s], sx = a.slot_x[s];
 
         float acc[8][4];
@@ -477,6 +480,47 @@ __global__ void __launch_bounds__(64, 8) k_numeric_f32_t84(NumArgs a) {
     }
 }
 
+// Diagonal elements of A A (32 x 32 blocks) as FP64 FMA chains, written over
+// those of the slice product in out_val.  The trace of X0^2 decides the branch
+// of Eq. TC2, at convergence by its last bits (Tr X0 is then N_occ up to
+// rounding), so it keeps the rounding of the chains that the CUDA-core kernel
+// computes: block by block along the row, k ascending, the linear term last.
+// One warp per block row, a lane per element; it waits for its chain (1,600
+// dependent FMAs in a row of 50 blocks, ~40 us beside ~2 ms of products).
+__global__ void __launch_bounds__(32) k_diag_fp64(const int *__restrict__ rp, const int *__restrict__ out_rp,
+                                                  const int *__restrict__ out_col, NumArgs a, JobTable jt, JobMask jobs,
+                                                  const int *__restrict__ sys_tier, int NB, int r0, int nrows) {
+    const int r = r0 + blockIdx.x, p = r / NB, i = r - p * NB;
+    const int lane = threadIdx.x;
+    const int sys = a.sys_of_row[i];
+    const Job &job = jt.job[p];
+    if (!a.active[sys] || job.nterm != 1 || !((jobs.m[sys_tier[sys] & (kMaxTiers - 1)] >> p) & 1u)) return;
+    int lo = out_rp[r], hi = out_rp[r + 1];
+    const int end = hi;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (out_col[mid] < i) lo = mid + 1; else hi = mid;
+    }
+    if (lo >= end || out_col[lo] != i) return;             // no diagonal block in the mask
+    double acc = 0.0;
+    const int q1 = rp[job.a[0] * NB + i + 1];
+    for (int q = rp[job.a[0] * NB + i]; q < q1; ++q) {
+        const double2 *x = reinterpret_cast<const double2 *>(a.in_val + (size_t)q * 1024 + lane * 32);
+        double2 v[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) v[k] = x[k];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            acc = fma(v[k].x, v[k].x, acc);
+            acc = fma(v[k].y, v[k].y, acc);
+        }
+    }
+    double c = a.c_sq[sys] * acc;
+    const int sx = a.slot_x[lo];
+    if (sx >= 0) c = fma(a.c_lin[sys], a.in_val[(size_t)sx * 1024 + lane * 33], c);
+    a.out_val[(size_t)(a.uidx[lo] - a.u0) * 1024 + lane * 33] = c;
+}
+
 // FP64 masters -> FP32 hi plane and (optionally) FP32 lo plane, x = hi + lo
 __global__ void k_split_f32(const double *__restrict__ v, float *__restrict__ hi, float *__restrict__ lo, int64_t n) {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -503,7 +547,7 @@ void launch_b(const NumArgs &a, cudaStream_t st) {
         RDM_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
         resident = std::max(1, per_sm) * nsm;
     }
-    const int grid = a.nwork < resident ? a.nwork : resident;
+    const int grid = a.max_work < resident ? a.max_work : resident;
     if (grid <= 0) return;
     k_numeric_simt<B, T><<<grid, NT, smem, st>>>(a);
     RDM_LAUNCH_CHECK();
@@ -536,21 +580,28 @@ int resident_blocks(K k, int nt) {
 }  // namespace
 
 void launch_numeric_simt(const NumArgs &a, Arith ar, cudaStream_t st) {
-    if (a.nwork == 0) return;
+    if (a.max_work == 0) return;
     if (ar == AR_FF) {
         if (a.b != 32 || !a.in_f32 || !a.in_f32lo) throw Error{-1, "double-FP32 products need 32 x 32 blocks"};
         static const int res = resident_blocks(k_numeric_ff_b32, 64);
-        k_numeric_ff_b32<<<std::min(a.nwork, res), 64, 0, st>>>(a);
+        k_numeric_ff_b32<<<std::min(a.max_work, res), 64, 0, st>>>(a);
         RDM_LAUNCH_CHECK();
     } else if (ar == AR_FP64) {
         dispatch<double>(a, st);
     } else if (a.b == 32 && a.in_f32) {
         static const int res = resident_blocks(k_numeric_f32_t84, 64);
-        k_numeric_f32_t84<<<std::min(a.nwork, res), 64, 0, st>>>(a);
+        k_numeric_f32_t84<<<std::min(a.max_work, res), 64, 0, st>>>(a);
         RDM_LAUNCH_CHECK();
     } else {
         dispatch<float>(a, st);
     }
+}
+
+void launch_diag_fp64(const NumArgs &a, const MatSet &in, const JobTable &jt, JobMask jobs, const int *out_rp,
+                      const int *out_col, const int *sys_tier, int r0, int nrows, cudaStream_t st) {
+    if (nrows == 0) return;
+    k_diag_fp64<<<nrows, 32, 0, st>>>(in.row_ptr.p, out_rp, out_col, a, jt, jobs, sys_tier, in.NB, r0, nrows);
+    RDM_LAUNCH_CHECK();
 }
 
 void launch_to_f32(const double *val, float *f32, int64_t n, cudaStream_t st, float *f32lo) {

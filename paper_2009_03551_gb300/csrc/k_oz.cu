@@ -67,7 +67,8 @@
 // groups equally spaced over the 4 stacked blocks (groups outermost, slices
 // inside) and B its slices (slices outermost), so both layouts are stored.
 // FP64 solve of a 300-atom cluster: products 652 ms on the FP64 pipe, 37 ms here
-// (21 TFLOP/s useful).  Bounded waits and the abort drain are those of the
+// (21 TFLOP/s useful, the 2 ms of k_diag_fp64 included: the diagonal elements
+// of X0^2 keep the FMA chains' rounding, because the trace decides branches).  Bounded waits and the abort drain are those of the
 // split kernel (k_tc.cu).
 #include <cuda_bf16.h>
 
@@ -306,7 +307,8 @@ struct OzArgs {
     const int *tiles;
     const int64_t *step_off;
     const int *steps;
-    int ntile, NB;
+    const int *flags;             // TcWork::counters
+    int NB;
     // epilogue
     const double *in_val;
     const int *slot_row, *slot_job, *slot_x;
@@ -344,6 +346,8 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_tc_oz(OzArgs A) {
     OzCtl *ctl = reinterpret_cast<OzCtl *>(smem_raw + G::kStages * G::kStageBytes);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     volatile int *abort_flag = &ctl->abort_flag;
+    if (A.flags[1]) return;               // the K-step list outgrew its buffer: the host builds it again
+    const int ntile = A.flags[2];
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < G::kStages; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
@@ -373,7 +377,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_tc_oz(OzArgs A) {
 #pragma unroll
         for (int k = 0; k < G::kStages; ++k) zmask[k] = 0u;
         const uint16_t *base = lane < G::TBM ? A.slices_a : A.slices_b;
-        for (int t = blockIdx.x; t < A.ntile && ok; t += gridDim.x) {
+        for (int t = blockIdx.x; t < ntile && ok; t += gridDim.x) {
             const int64_t s0 = A.step_off[t], s1 = A.step_off[t + 1];
             int nxt = (s0 < s1 && lane < G::kSlots) ? A.steps[s0 * G::kSlots + lane] : -1;
             for (int64_t q = s0; q < s1; ++q, ++it) {
@@ -419,7 +423,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_tc_oz(OzArgs A) {
             const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 4) << 24);
             uint32_t it = 0, seg = 0;
             bool issued = false;
-            for (int t = blockIdx.x; t < A.ntile && !*abort_flag; t += gridDim.x) {
+            for (int t = blockIdx.x; t < ntile && !*abort_flag; t += gridDim.x) {
                 const int *d = A.tiles + (size_t)t * G::kTileInts;
                 const int nst = d[3], n1 = d[2];
                 bool ok = true;
@@ -470,7 +474,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_tc_oz(OzArgs A) {
         const int bc = (warp - kOzEpiWarp0) >> 2;       // block column of the tile
         const uint32_t ta = tmem + ((uint32_t)(32 * eq) << 16) + bc * G::kAccCols;
         uint32_t seg = 0;
-        for (int t = blockIdx.x; t < A.ntile && !*abort_flag; t += gridDim.x) {
+        for (int t = blockIdx.x; t < ntile && !*abort_flag; t += gridDim.x) {
             const int *d = A.tiles + (size_t)t * G::kTileInts;
             const int s = d[4 + eq * G::TBN + bc];
             const int nst = d[3], n1 = d[2];
@@ -633,7 +637,7 @@ constexpr size_t oz_smem() { return (size_t)GeoOz<S>::kStages * GeoOz<S>::kStage
 static_assert(oz_smem<8>() <= 227 * 1024, "shared memory of the slice-product kernel exceeds 227 KB");
 
 template <int S>
-double launch_oz(OzArgs &A, const TcPlan &plan, OzWork &ow, cudaStream_t st) {
+void launch_oz(OzArgs &A, const TcPlan &plan, OzWork &ow, cudaStream_t st) {
     using G = GeoOz<S>;
     int dev = 0, nsm = 0;
     RDM_CUDA_TRY(cudaGetDevice(&dev));
@@ -645,10 +649,9 @@ double launch_oz(OzArgs &A, const TcPlan &plan, OzWork &ow, cudaStream_t st) {
     }
     A.zero = ow.zero.p;
     func_smem_once((const void *)k_tc_oz<S>, (int)oz_smem<S>());
-    const int grid = plan.ntile < nsm ? plan.ntile : nsm;
+    const int grid = plan.max_tile < nsm ? plan.max_tile : nsm;
     k_tc_oz<S><<<grid, kOzThreads, oz_smem<S>(), st>>>(A);
     RDM_LAUNCH_CHECK();
-    return (double)plan.nsteps * G::kPairs * 2.0 * 2.0 * 128.0 * 64.0 * 16.0;
 }
 
 }  // namespace
@@ -685,20 +688,23 @@ bool prepare_oz_operands(const MatSet &in, int nmat, int slices, OzWork &w, cuda
 }
 
 TcPlan build_oz_plan(const MatSet &in, const JobTable &jt, const SysDev &sd, const int *out_rp, const int *mcol,
-                     TcWork &w, JobMask job_mask, int unit0, int unit1, cudaStream_t st) {
+                     TcWork &w, JobMask job_mask, int unit0, int unit1, int64_t nupper, int64_t min_steps,
+                     cudaStream_t st) {
     if (in.b != 32) throw Error{-1, "the slice-product (FP64-class tensor-core) path handles 32 x 32 blocks"};
-    return build_plan<GeoOz<8>>(in, jt, sd, out_rp, mcol, w, job_mask, unit0, unit1, st);
+    return build_plan<GeoOz<8>>(in, jt, sd, out_rp, mcol, w, job_mask, unit0, unit1, nupper, min_steps, st);
 }
 
-double launch_numeric_oz(const NumArgs &a, const MatSet &in, const JobTable &jt, const int *mcol, OzWork &ow,
+double oz_step_flops(const OzWork &ow) { return ow.nslice * (ow.nslice + 1) / 2 * 2.0 * 2.0 * 128.0 * 64.0 * 16.0; }
+
+void launch_numeric_oz(const NumArgs &a, const MatSet &in, const JobTable &jt, const int *mcol, OzWork &ow,
                          TcWork &w, const TcPlan &plan, cudaStream_t st) {
-    if (plan.ntile == 0) return 0.0;
+    if (plan.max_tile == 0) return;
     OzArgs A{};
     A.slices_a = ow.slices_a.p;
     A.slices_b = ow.slices_b.p;
     A.e = ow.e.p;
     A.NB = in.NB;
-    A.tiles = w.tiles.p; A.step_off = w.step_off.p; A.steps = w.steps.p; A.ntile = plan.ntile;
+    A.tiles = w.tiles.p; A.step_off = w.step_off.p; A.steps = w.steps.p; A.flags = w.counters.p;
     A.in_val = a.in_val; A.slot_row = a.slot_row; A.slot_job = a.slot_job; A.slot_x = a.slot_x; A.mcol = mcol;
     A.sys_of_row = a.sys_of_row; A.c_lin = a.c_lin; A.c_sq = a.c_sq; A.tau0 = a.tau0; A.tau1 = a.tau1;
     for (int p = 0; p < kMaxJobs; ++p) A.job_tau_sel[p] = a.job_tau_sel[p];
@@ -712,7 +718,8 @@ double launch_numeric_oz(const NumArgs &a, const MatSet &in, const JobTable &jt,
     A.out_val = a.out_val; A.out_nrm = a.out_nrm; A.keep = a.keep; A.uidx = a.uidx; A.u0 = a.u0;
     A.err = w.counters.p;
     A.wait_cycles = w.knobs.wait_cycles > 0 ? w.knobs.wait_cycles : kWaitCycles;
-    return ow.nslice == 8 ? launch_oz<8>(A, plan, ow, st) : launch_oz<7>(A, plan, ow, st);
+    if (ow.nslice == 8) launch_oz<8>(A, plan, ow, st);
+    else launch_oz<7>(A, plan, ow, st);
 }
 
 }  // namespace rdm

@@ -1,8 +1,10 @@
-// Exclusive prefix sums used to turn per-row / per-slot counts into offsets.
-// Three launches: per-tile sums, a single-CTA scan of the tile sums, and the
-// per-tile scan with the tile offset added.  out[n] receives the total; an
-// initial value `init` is added to every output.
-// The scan is deterministic (integer addition).
+// Exclusive prefix sums used to turn per-row / per-tile counts into offsets.
+// One launch of one CTA up to kOneCta elements (a solve's scans mostly are
+// that short, and a launch costs 2.5 to 4 us on either side); above that two:
+// per-tile sums, then the per-tile scan, whose CTAs add up the sums of the
+// tiles before theirs themselves.  out[n] receives the total; an initial value
+// `init` is added to every output.  The element count may be in device memory.
+// Deterministic (integer addition).
 #include "rdm_internal.cuh"
 
 namespace rdm {
@@ -11,6 +13,7 @@ namespace {
 constexpr int kThreads = 512;
 constexpr int kItems = 8;
 constexpr int kTile = kThreads * kItems;
+constexpr int kOneCta = 4 * kTile;
 
 template <class T>
 __device__ T block_exclusive_scan(T v, T *sh, T *total) {
@@ -40,66 +43,89 @@ __device__ T block_exclusive_scan(T v, T *sh, T *total) {
     return excl;
 }
 
-template <class In, class Out>
-__global__ void tile_sums(const In *__restrict__ in, int n, Out *__restrict__ tile_sum) {
-    __shared__ Out sh[32];
-    int64_t base = (int64_t)blockIdx.x * kTile + (int64_t)threadIdx.x * kItems;
-    Out s = 0;
+// where the prefix sums go: one array, or the two halves of packed counts
+template <class T>
+struct Plain {
+    T *out;
+    __device__ void put(int64_t i, T v) const { out[i] = v; }
+};
+struct Halves {
+    int *lo, *hi;
+    __device__ void put(int64_t i, int64_t v) const {
+        lo[i] = (int)(v & 0xffffffffll);
+        hi[i] = (int)(v >> 32);
+    }
+};
+
+// the tile of kTile elements at `base`, with `carry` added; returns its total
+template <class In, class T, class Dst>
+__device__ T scan_tile(const In *in, int64_t base0, int n, T carry, const Dst &dst, T *sh) {
+    const int64_t base = base0 + (int64_t)threadIdx.x * kItems;
+    T v[kItems], s = 0;
+#pragma unroll
+    for (int k = 0; k < kItems; ++k) {
+        v[k] = base + k < n ? (T)in[base + k] : T(0);
+        s += v[k];
+    }
+    T tot;
+    T e = block_exclusive_scan<T>(s, sh, &tot) + carry;
+#pragma unroll
+    for (int k = 0; k < kItems; ++k) {
+        if (base + k < n) dst.put(base + k, e);
+        e += v[k];
+    }
+    return tot;
+}
+
+template <class In, class T, class Dst>
+__global__ void __launch_bounds__(kThreads) k_scan_one(const In *in, int n, const int *n_dev, Dst dst, T init) {
+    __shared__ T sh[32];
+    if (n_dev) n = *n_dev;
+    T carry = init;
+    for (int64_t base = 0; base < n; base += kTile) carry += scan_tile<In, T, Dst>(in, base, n, carry, dst, sh);
+    if (threadIdx.x == 0) dst.put(n, carry);
+}
+
+template <class In, class T>
+__global__ void __launch_bounds__(kThreads) k_tile_sums(const In *__restrict__ in, int n, const int *n_dev,
+                                                        T *__restrict__ tile_sum) {
+    __shared__ T sh[32];
+    if (n_dev) n = *n_dev;
+    const int64_t base = (int64_t)blockIdx.x * kTile + (int64_t)threadIdx.x * kItems;
+    T s = 0;
 #pragma unroll
     for (int k = 0; k < kItems; ++k)
-        if (base + k < n) s += (Out)in[base + k];
-    Out tot;
-    block_exclusive_scan<Out>(s, sh, &tot);
+        if (base + k < n) s += (T)in[base + k];
+    T tot;
+    block_exclusive_scan<T>(s, sh, &tot);
     if (threadIdx.x == 0) tile_sum[blockIdx.x] = tot;
 }
 
-template <class Out>
-__global__ void scan_tiles(Out *tile_sum, int ntiles, Out *total_out, Out init) {
-    __shared__ Out sh[32];
-    Out carry = init;
-    for (int base = 0; base < ntiles; base += kThreads) {
-        int i = base + threadIdx.x;
-        Out v = i < ntiles ? tile_sum[i] : Out(0);
-        Out tot;
-        Out e = block_exclusive_scan<Out>(v, sh, &tot);
-        if (i < ntiles) tile_sum[i] = e + carry;
-        carry += tot;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *total_out = carry;
+template <class In, class T, class Dst>
+__global__ void __launch_bounds__(kThreads) k_scan_apply(const In *in, int n, const int *n_dev,
+                                                         const T *__restrict__ tile_sum, Dst dst, T init) {
+    __shared__ T sh[32];
+    if (n_dev) n = *n_dev;
+    // sum of the tiles before this one
+    T s = 0, before;
+    for (int k = threadIdx.x; k < (int)blockIdx.x; k += kThreads) s += tile_sum[k];
+    block_exclusive_scan<T>(s, sh, &before);
+    const T tot = scan_tile<In, T, Dst>(in, (int64_t)blockIdx.x * kTile, n, init + before, dst, sh);
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) dst.put(n, init + before + tot);
 }
 
-template <class In, class Out>
-__global__ void scan_apply(const In *in, int n, const Out *__restrict__ tile_sum, Out *out) {
-    __shared__ Out sh[32];
-    int64_t base = (int64_t)blockIdx.x * kTile + (int64_t)threadIdx.x * kItems;
-    Out v[kItems];
-    Out s = 0;
-#pragma unroll
-    for (int k = 0; k < kItems; ++k) {
-        v[k] = (base + k < n) ? (Out)in[base + k] : Out(0);
-        s += v[k];
-    }
-    Out e = block_exclusive_scan<Out>(s, sh, nullptr) + tile_sum[blockIdx.x];
-#pragma unroll
-    for (int k = 0; k < kItems; ++k) {
-        if (base + k < n) out[base + k] = e;
-        e += v[k];
-    }
-}
-
-template <class In, class Out>
-void scan_impl(const In *in, Out *out, int n, Out *tmp, cudaStream_t st, Out init) {
-    int ntiles = (n + kTile - 1) / kTile;
-    if (ntiles < 1) ntiles = 1;
-    tile_sums<In, Out><<<ntiles, kThreads, 0, st>>>(in, n, tmp);
-    RDM_LAUNCH_CHECK();
-    scan_tiles<Out><<<1, kThreads, 0, st>>>(tmp, ntiles, out + n, init);
-    RDM_LAUNCH_CHECK();
-    if (n > 0) {
-        scan_apply<In, Out><<<ntiles, kThreads, 0, st>>>(in, n, tmp, out);
+template <class In, class T, class Dst>
+void scan_impl(const In *in, Dst dst, int n, const int *n_dev, T *tmp, cudaStream_t st, T init) {
+    if (n <= kOneCta) {
+        k_scan_one<In, T, Dst><<<1, kThreads, 0, st>>>(in, n, n_dev, dst, init);
         RDM_LAUNCH_CHECK();
+        return;
     }
+    const int ntiles = (n + kTile - 1) / kTile;
+    k_tile_sums<In, T><<<ntiles, kThreads, 0, st>>>(in, n, n_dev, tmp);
+    RDM_LAUNCH_CHECK();
+    k_scan_apply<In, T, Dst><<<ntiles, kThreads, 0, st>>>(in, n, n_dev, tmp, dst, init);
+    RDM_LAUNCH_CHECK();
 }
 
 }  // namespace
@@ -107,10 +133,13 @@ void scan_impl(const In *in, Out *out, int n, Out *tmp, cudaStream_t st, Out ini
 size_t scan_tmp_elems(int n) { return (size_t)((n + kTile - 1) / kTile + 1); }
 
 void scan_exclusive_i32(const int *in, int *out, int n, int *tmp, cudaStream_t st, int init) {
-    scan_impl<int, int>(in, out, n, tmp, st, init);
+    scan_impl<int, int>(in, Plain<int>{out}, n, nullptr, tmp, st, init);
 }
-void scan_exclusive_i64(const int *in, int64_t *out, int n, int64_t *tmp, cudaStream_t st) {
-    scan_impl<int, int64_t>(in, out, n, tmp, st, int64_t(0));
+void scan_exclusive_i64(const int *in, int64_t *out, int n, int64_t *tmp, cudaStream_t st, const int *n_dev) {
+    scan_impl<int, int64_t>(in, Plain<int64_t>{out}, n, n_dev, tmp, st, int64_t(0));
+}
+void scan_exclusive_pair(const int64_t *in, int *out_lo, int *out_hi, int n, int64_t *tmp, cudaStream_t st) {
+    scan_impl<int64_t, int64_t>(in, Halves{out_lo, out_hi}, n, nullptr, tmp, st, int64_t(0));
 }
 
 }  // namespace rdm

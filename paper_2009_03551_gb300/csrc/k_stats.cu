@@ -2,12 +2,10 @@
 // band energies of the stopping rule (Sec. 2.2: E0 = Tr(P0 H0),
 // E1 = Tr(P1 H0)), and the polarizability trace (Eq. polar).
 //
-// Every reduction is two-stage and deterministic: one CTA (or `parts` of them)
-// per block row writes partial sums (warp-shuffle reductions, added in a fixed
-// order), then one CTA per (system, quantity) adds the rows in a fixed order.
+// Every reduction is two-stage and deterministic: warps write partial sums of
+// their block row (warp-shuffle reductions), then one CTA per (system,
+// quantity) adds them, row by row, in a fixed order.
 // The branch decision therefore never depends on atomic ordering.
-#include <algorithm>
-
 #include "rdm_internal.cuh"
 
 namespace rdm {
@@ -33,91 +31,84 @@ __device__ __forceinline__ int warp_find_col(const int *__restrict__ col, int lo
     return -1;
 }
 
-// row_part layout: [q][NB * parts], q = 0 trace, 1 sumsq, 2 E0, 3+m-1 E1 of
-// matrix m.  A block row is shared by `parts` CTAs (consecutive entries), warps
-// over blocks, lanes over elements; the warp partials are added in a fixed
-// order.  Tr X0 and ||X0||_F^2 run over the blocks of X0, the band energies
-// Tr(X H0) only over the blocks of H0 (where H0 is zero they get no
-// contribution), each looking up the matching block of X.  The matrices are
-// symmetric: only blocks on and above the diagonal are read, those above
-// count twice.  Bound by the FP64 pipe (2 FMAs per clock and SM), hence the
-// upper triangle only and `parts` for systems with fewer block rows than would
-// fill the chip (38 block rows, 1,300 blocks of X0: 155 -> 43 us; 1,250 block
-// rows, 110,000 blocks: 0.9 -> 0.5 ms).
-constexpr int kStatWarps = 8;
-constexpr int kStatQ = 3 + 7;    // up to 7 first-order matrices
+// row_part layout: [q][NB][kStatWarps], q = 0 trace, 1 sumsq, 2 E0, 3+m-1 E1 of
+// matrix m.  Warp w of block row i adds the blocks w, w + 8, ... of the row,
+// lanes over elements; Tr X0 and ||X0||_F^2 run over the blocks of X0, the band
+// energies Tr(X H0) only over the blocks of H0 (where H0 is zero they get no
+// contribution), each looking up the matching block of X.  k_sys_sum adds the
+// warps' sums of a row in order.  A sum that ends within its rounding of an
+// integer decides a branch (Tr X0 against N_occ at convergence), so the order
+// of the additions is fixed: per warp and lane one chain over the blocks and
+// elements of its share.  Bound by the FP64 pipe (2 FMAs per clock and SM); the
+// chains of a row (8 warps, 2 + nmat sums) are spread over 2 (1 + nmat) CTAs, so
+// that a system of few block rows fills the chip (38 block rows, 1,300 blocks of
+// X0: 155 us in one CTA per row, 27 us spread).
+constexpr int kStatWarps = 8;    // warps per block row
+constexpr int kStatCta = 4;      // of them in one CTA
 
-__global__ void __launch_bounds__(kStatWarps * 32) k_row_stats(
-    const int *__restrict__ rp, const int *__restrict__ col, const double *__restrict__ val, int nmat, int NB, int b,
-    const int *__restrict__ hrp, const int *__restrict__ hcol, const double *__restrict__ hval, int parts,
+__global__ void __launch_bounds__(kStatCta * 32) k_row_stats(
+    const int *__restrict__ rp, const int *__restrict__ col, const double *__restrict__ val, int NB, int b,
+    const int *__restrict__ hrp, const int *__restrict__ hcol, const double *__restrict__ hval,
     double *__restrict__ row_part) {
-    __shared__ double sh[kStatWarps][kStatQ];
-    const int i = blockIdx.x / parts, part = blockIdx.x % parts;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int first = part * kStatWarps + wid, stride = parts * kStatWarps;
+    const int lane = threadIdx.x & 31;
+    const int slot = blockIdx.x * kStatCta + (threadIdx.x >> 5);     // row, warp of the row
+    const int i = slot / kStatWarps, w = slot % kStatWarps;
     const int bb = b * b;
-    double q[kStatQ];
-#pragma unroll
-    for (int k = 0; k < kStatQ; ++k) q[k] = 0.0;
-    // trace and squared norm of X0 (first: the warp's first block of the row)
-    for (int p = rp[i] + first; p < rp[i + 1]; p += stride) {
-        const int j = col[p];
-        if (j < i) continue;
-        const double *x = val + (size_t)p * bb;
-        double s0 = 0.0, s1 = 0.0;
-        int e = lane;
-        for (; e + 96 < bb; e += 128) {
-            const double v0 = x[e], v1 = x[e + 32], v2 = x[e + 64], v3 = x[e + 96];
-            s0 = fma(v0, v0, s0);
-            s1 = fma(v1, v1, s1);
-            s0 = fma(v2, v2, s0);
-            s1 = fma(v3, v3, s1);
-        }
-        for (; e < bb; e += 32) s0 = fma(x[e], x[e], s0);
-        q[1] += j == i ? s0 + s1 : 2.0 * (s0 + s1);
-        if (j == i)
-            for (int r = lane; r < b; r += 32) q[0] += x[(size_t)r * (b + 1)];
-    }
-    // band energies over the pattern of H0
-    for (int ph = hrp[i] + first; ph < hrp[i + 1]; ph += stride) {
-        const int j = hcol[ph];
-        if (j < i) continue;
-        const double *h = hval + (size_t)ph * bb;
-        for (int m = 0; m < nmat; ++m) {
-            const int *rpm = rp + (size_t)m * NB;
-            const int p = warp_find_col(col, rpm[i], rpm[i + 1], j, lane);
-            if (p < 0) continue;
+    const size_t nslot = (size_t)NB * kStatWarps;
+    if (blockIdx.y == 0) {
+        // trace and squared norm of X0
+        double tr = 0.0, ss = 0.0;
+        for (int p = rp[i] + w; p < rp[i + 1]; p += kStatWarps) {
             const double *x = val + (size_t)p * bb;
-            double e0 = 0.0, e1 = 0.0;
             int e = lane;
-            for (; e + 96 < bb; e += 128) {
-                const double v0 = x[e], v1 = x[e + 32], v2 = x[e + 64], v3 = x[e + 96];
-                const double h0 = h[e], h1 = h[e + 32], h2 = h[e + 64], h3 = h[e + 96];
-                e0 = fma(v0, h0, e0);
-                e1 = fma(v1, h1, e1);
-                e0 = fma(v2, h2, e0);
-                e1 = fma(v3, h3, e1);
+            for (; e + 224 < bb; e += 256) {
+                double v[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) v[k] = x[e + 32 * k];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) ss = fma(v[k], v[k], ss);
             }
-            for (; e < bb; e += 32) e0 = fma(x[e], h[e], e0);
-            const double eb = j == i ? e0 + e1 : 2.0 * (e0 + e1);
-#pragma unroll
-            for (int k = 0; k < kStatQ - 2; ++k)
-                if (k == m) q[2 + k] += eb;
+            for (; e < bb; e += 32) ss = fma(x[e], x[e], ss);
+            if (col[p] == i)
+                // the lane's elements in order, those on the diagonal
+                for (e = lane; e < bb; e += 32)
+                    if (e / b == e % b) tr += x[e];
         }
+        tr = warp_sum(tr);
+        ss = warp_sum(ss);
+        if (lane == 0) {
+            row_part[slot] = tr;
+            row_part[nslot + slot] = ss;
+        }
+        return;
     }
+    // band energy of matrix m over the pattern of H0
+    const int m = blockIdx.y - 1;
+    const int *rpm = rp + (size_t)m * NB;
+    const int lo = rpm[i], hi = rpm[i + 1];
+    double q = 0.0;
+    for (int ph = hrp[i] + w; ph < hrp[i + 1]; ph += kStatWarps) {
+        const int p = warp_find_col(col, lo, hi, hcol[ph], lane);
+        if (p < 0) continue;
+        const double *h = hval + (size_t)ph * bb;
+        const double *x = val + (size_t)p * bb;
+        double eb = 0.0;
+        int e = lane;
+        for (; e + 224 < bb; e += 256) {
+            double v[8], u[8];
 #pragma unroll
-    for (int k = 0; k < kStatQ; ++k) {
-        if (k >= 2 + nmat) break;
-        const double v = warp_sum(q[k]);
-        if (lane == 0) sh[wid][k] = v;
+            for (int k = 0; k < 8; ++k) {
+                v[k] = x[e + 32 * k];
+                u[k] = h[e + 32 * k];
+            }
+#pragma unroll
+            for (int k = 0; k < 8; ++k) eb = fma(v[k], u[k], eb);
+        }
+        for (; e < bb; e += 32) eb = fma(x[e], h[e], eb);
+        q += eb;
     }
-    __syncthreads();
-    if (threadIdx.x < 2 + nmat) {
-        const int k = threadIdx.x;
-        double t = 0.0;
-        for (int w = 0; w < kStatWarps; ++w) t += sh[w][k];
-        row_part[(size_t)k * NB * parts + blockIdx.x] = t;
-    }
+    q = warp_sum(q);
+    if (lane == 0) row_part[(2 + m) * nslot + slot] = q;
 }
 
 // Tr X and ||X||_F^2 of one matrix over all its blocks, row_part layout [2][NB]
@@ -190,7 +181,12 @@ __global__ void k_sys_sum(const double *__restrict__ row_part, int nq, int NB,
     int s = blockIdx.x, q = blockIdx.y;
     const double *r = row_part + ((size_t)q * NB + row0[s]) * parts;
     double acc = 0.0;
-    for (int i = threadIdx.x; i < nbs[s] * parts; i += blockDim.x) acc += r[i];
+    for (int i = threadIdx.x; i < nbs[s]; i += blockDim.x) {
+        double t = parts > 1 ? 0.0 : r[i];
+        if (parts > 1)
+            for (int w = 0; w < parts; ++w) t += r[(size_t)i * parts + w];
+        acc += t;
+    }
     acc = warp_sum(acc);
     int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (lane == 0) sh[w] = acc;
@@ -204,18 +200,14 @@ __global__ void k_sys_sum(const double *__restrict__ row_part, int nq, int NB,
 
 }  // namespace
 
-int row_stats_parts(int NB) {
-    // enough CTAs for four per SM, at most one per warp's worth of a row of 64 blocks
-    return std::max(1, std::min(8, 608 / std::max(NB, 1)));
-}
+int row_stats_parts() { return kStatWarps; }
 
 void launch_row_stats(const int *row_ptr, const int *col, const double *val, int nmat, int NB,
-                      int b, const int *h_row_ptr, const int *h_col, const double *h_val, int parts,
+                      int b, const int *h_row_ptr, const int *h_col, const double *h_val,
                       double *row_part, cudaStream_t st) {
     if (NB == 0) return;
-    if (nmat > kStatQ - 2) throw Error{-1, "at most 7 first-order matrices"};
-    k_row_stats<<<(unsigned)NB * parts, kStatWarps * 32, 0, st>>>(row_ptr, col, val, nmat, NB, b, h_row_ptr, h_col,
-                                                                  h_val, parts, row_part);
+    k_row_stats<<<dim3((unsigned)NB * (kStatWarps / kStatCta), 1 + nmat), kStatCta * 32, 0, st>>>(
+        row_ptr, col, val, NB, b, h_row_ptr, h_col, h_val, row_part);
     RDM_LAUNCH_CHECK();
 }
 

@@ -82,6 +82,9 @@ __device__ T block_excl_scan(T v, T *sh, T *total) {
     return ex;
 }
 
+// kept blocks of a row (low 32 bits) and those with col >= row (high)
+__device__ __forceinline__ int64_t pack_counts(int n, int upper) { return (int64_t)n | ((int64_t)upper << 32); }
+
 struct SymParams {
     const int *rp;       // flat row_ptr of the input set (nmat*NB+1)
     const int *col;
@@ -93,6 +96,13 @@ struct SymParams {
     const int *active;
     SymOut so;
 };
+
+// adds the warp's pair counts to *total
+__device__ __forceinline__ void add_pairs(unsigned long long np, unsigned long long *total) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) np += __shfl_xor_sync(0xffffffffu, np, o);
+    if ((threadIdx.x & 31) == 0 && np) atomicAdd(total, np);
+}
 
 // grid (NB, njob); dynamic shared memory: acc[ns] (u64) + cnt[ns] (u32)
 __global__ void __launch_bounds__(kSymThreads) k_symbolic(SymParams P) {
@@ -117,7 +127,7 @@ __global__ void __launch_bounds__(kSymThreads) k_symbolic(SymParams P) {
             int off = atomicAdd(P.so.pool_top, n);
             if (off + n > P.so.pool_cap) { atomicExch(P.so.overflow, 1); off = -1; }
             sh_off = off;
-            P.so.row_cnt[out_r] = n;
+            P.so.row_cnt[out_r] = pack_counts(n, hi - lower_bound(P.col, lo, hi, i));
             P.so.row_off[out_r] = off;
         }
         __syncthreads();
@@ -166,19 +176,26 @@ __global__ void __launch_bounds__(kSymThreads) k_symbolic(SymParams P) {
     __syncthreads();
 
     const unsigned long long thr = (unsigned long long)kFixOne;
-    // pass 1: count kept columns
-    int my = 0;
+    // pass 1: count the kept columns, those on or above the diagonal and their pairs
+    int my = 0, up = 0;
+    unsigned long long np = 0;
     for (int t = tid; t < ns; t += blockDim.x) {
         bool keep = exact ? (cnt[t] != 0u) : (sm_acc[t] >= thr);
         my += keep ? 1 : 0;
+        if (keep && c0 + t >= i) {
+            ++up;
+            np += cnt[t] & 0x7fffffffu;
+        }
     }
-    int total;
+    int total, upper;
     block_excl_scan<int>(my, sh_scan, &total);
+    block_excl_scan<int>(up, sh_scan, &upper);
+    add_pairs(np, P.so.npairs);
     if (tid == 0) {
         int off = atomicAdd(P.so.pool_top, total);
         if (off + total > P.so.pool_cap) { atomicExch(P.so.overflow, 1); off = -1; }
         sh_off = off;
-        P.so.row_cnt[out_r] = total;
+        P.so.row_cnt[out_r] = pack_counts(total, upper);
         P.so.row_off[out_r] = off;
     }
     __syncthreads();
@@ -252,7 +269,7 @@ __global__ void __launch_bounds__(kSymThreads) k_symbolic_hash(SymParams P) {
             int off = atomicAdd(P.so.pool_top, n);
             if (off + n > P.so.pool_cap) { atomicExch(P.so.overflow, 1); off = -1; }
             sh_off = off;
-            P.so.row_cnt[out_r] = n;
+            P.so.row_cnt[out_r] = pack_counts(n, hi - lower_bound(P.col, lo, hi, i));
             P.so.row_off[out_r] = off;
         }
         __syncthreads();
@@ -309,7 +326,8 @@ __global__ void __launch_bounds__(kSymThreads) k_symbolic_hash(SymParams P) {
     }
     // keep decision, packed as (column << 32 | pair count); dropped slots sort last
     const unsigned long long thr = (unsigned long long)kFixOne;
-    int my = 0;
+    int my = 0, up = 0;
+    unsigned long long npt = 0;
     for (int t = tid; t < kHashSlots; t += blockDim.x) {
         unsigned long long packed = ~0ull;
         if (keys[t] >= 0) {
@@ -319,12 +337,16 @@ __global__ void __launch_bounds__(kSymThreads) k_symbolic_hash(SymParams P) {
                 const unsigned np = (j >= i) ? (cnt[t] & 0x7fffffffu) : 0u;
                 packed = ((unsigned long long)(unsigned)j << 32) | np;
                 ++my;
+                up += j >= i ? 1 : 0;
+                npt += np;
             }
         }
         sm_acc[t] = packed;
     }
-    int total;
+    int total, upper;
     block_excl_scan<int>(my, sh_scan, &total);
+    block_excl_scan<int>(up, sh_scan, &upper);
+    add_pairs(npt, P.so.npairs);
     // bitonic sort of the packed keys (ascending)
     for (int k = 2; k <= kHashSlots; k <<= 1) {
         for (int jj = k >> 1; jj > 0; jj >>= 1) {
@@ -343,7 +365,7 @@ __global__ void __launch_bounds__(kSymThreads) k_symbolic_hash(SymParams P) {
         int off = atomicAdd(P.so.pool_top, total);
         if (off + total > P.so.pool_cap) { atomicExch(P.so.overflow, 1); off = -1; }
         sh_off = off;
-        P.so.row_cnt[out_r] = total;
+        P.so.row_cnt[out_r] = pack_counts(total, upper);
         P.so.row_off[out_r] = off;
     }
     __syncthreads();
@@ -355,20 +377,46 @@ __global__ void __launch_bounds__(kSymThreads) k_symbolic_hash(SymParams P) {
     }
 }
 
-// one warp per (job,row): copy the pool lists into the output pattern
-__global__ void k_gather(SymOut so, int nrows, const int *__restrict__ out_rp, int *out_col,
-                         int *slot_row, int *slot_job, int *slot_npair, int NB) {
-    int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    int lane = threadIdx.x & 31;
-    if (r >= nrows) return;
-    int n = so.row_cnt[r], off = so.row_off[r], dst = out_rp[r];
-    int i = r % NB, p = r / NB;
+struct GatherParams {
+    SymOut so;
+    int nrows, NB;
+    const int *out_rp, *out_urp;
+    int *out_col, *slot_row, *slot_job, *slot_npair, *uidx;
+    const int *sys_of_row, *active, *sys_tier;
+    ClassMasks cm;
+    unsigned long long *cls;
+};
+
+// one warp per (job,row): copy the pool lists into the output pattern.  The
+// columns of a row are sorted, so its upper slots are the last ones and their
+// ranks follow from the counts per row.
+__global__ void k_gather(GatherParams P) {
+    const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    if (r >= P.nrows) return;
+    const int dst = P.out_rp[r], n = P.out_rp[r + 1] - dst;
+    const int u0 = P.out_urp[r], nlow = n - (P.out_urp[r + 1] - u0);
+    const int off = P.so.row_off[r];
+    const int i = r % P.NB, p = r / P.NB;
+    unsigned long long np = 0;
     for (int t = lane; t < n; t += 32) {
-        out_col[dst + t] = so.pool_col[off + t];
-        slot_npair[dst + t] = so.pool_npair[off + t];
-        slot_row[dst + t] = i;
-        slot_job[dst + t] = p;
+        const int c = P.so.pool_npair[off + t];
+        P.out_col[dst + t] = P.so.pool_col[off + t];
+        if (P.slot_npair) P.slot_npair[dst + t] = c;
+        P.slot_row[dst + t] = i;
+        P.slot_job[dst + t] = p;
+        if (t >= nlow) P.uidx[dst + t] = u0 + (t - nlow);
+        np += (unsigned long long)c;       // 0 for lower slots
     }
+    const int sys = P.sys_of_row[i];
+    if (!P.active[sys]) return;
+    const int tier = P.sys_tier[sys] & (kMaxTiers - 1);
+#pragma unroll
+    for (int k = 0; k < 5; ++k)
+        if ((P.cm.m[k].m[tier] >> p) & 1u) {
+            add_pairs(np, &P.cls[k]);
+            return;
+        }
 }
 
 struct PairParams {
@@ -408,7 +456,7 @@ __global__ void k_pairs(PairParams P) {
     }
     // a converged system's blocks are copied: the symbolic phase gave them no pairs
     const int sys = P.sys_of_row[i];
-    if (!P.active[sys] || !((P.fill.m[P.sys_tier[sys] & (kMaxTiers - 1)] >> p) & 1u)) return;
+    if (!P.pair_off || !P.active[sys] || !((P.fill.m[P.sys_tier[sys] & (kMaxTiers - 1)] >> p) & 1u)) return;
     int64_t w = P.pair_off[s];
     const int64_t wend = P.pair_off[s + 1];
     for (int t = 0; t < job.nterm; ++t) {
@@ -460,13 +508,15 @@ void launch_symbolic(const MatSet &in, const JobTable &jt, const SysDev &sd, int
     RDM_LAUNCH_CHECK();
 }
 
-void launch_gather(const SymOut &so, int njob, int NB, const int *out_row_ptr, int *out_col,
-                   int *slot_row, int *slot_job, int *slot_npair, cudaStream_t st) {
-    int nrows = njob * NB;
+void launch_gather(const SymOut &so, int njob, int NB, const int *out_row_ptr, const int *out_urp, int *out_col,
+                   int *slot_row, int *slot_job, int *slot_npair, int *uidx, const SysDev &sd,
+                   const ClassMasks &cm, unsigned long long *cls, cudaStream_t st) {
+    const int nrows = njob * NB;
     if (nrows == 0) return;
-    int wpb = 8;
-    k_gather<<<(nrows + wpb - 1) / wpb, wpb * 32, 0, st>>>(so, nrows, out_row_ptr, out_col,
-                                                           slot_row, slot_job, slot_npair, NB);
+    GatherParams P{so, nrows, NB, out_row_ptr, out_urp, out_col, slot_row, slot_job, slot_npair, uidx,
+                   sd.sys_of_row.p, sd.active.p, sd.tier.p, cm, cls};
+    const int wpb = 8;
+    k_gather<<<(nrows + wpb - 1) / wpb, wpb * 32, 0, st>>>(P);
     RDM_LAUNCH_CHECK();
 }
 

@@ -148,18 +148,20 @@ __device__ __forceinline__ int pair_offset(int r, int c, int plane) {
     return (r >> 3) * (16 * B) + plane * (8 * B) + ((c >> 3) << 6) + ((r & 7) << 3) + (c & 7);
 }
 
-// Largest block norm of every matrix of the set: each CTA takes a contiguous
-// chunk of blocks and folds the part of every matrix it overlaps into mx[m]
-// (norms are non-negative, so their bit patterns order like the values).
-__global__ void k_matrix_max(const float *__restrict__ nrm, const int *__restrict__ mat_first, int nmat,
+// Largest block norm of every matrix of the set (matrix m: blocks
+// [rp[m NB], rp[(m + 1) NB])): each CTA takes a contiguous chunk of blocks and
+// folds the part of every matrix it overlaps into mx[m] (norms are
+// non-negative, so their bit patterns order like the values).
+__global__ void k_matrix_max(const float *__restrict__ nrm, const int *__restrict__ rp, int NB, int nmat,
                              unsigned *__restrict__ mx) {
-    const int64_t total = mat_first[nmat];
+    const int64_t total = rp[(size_t)nmat * NB];
     const int64_t per = (total + gridDim.x - 1) / gridDim.x;
     const int64_t c0 = (int64_t)blockIdx.x * per, c1 = c0 + per < total ? c0 + per : total;
     __shared__ float sh[32];
     for (int m = 0; m < nmat; ++m) {
-        const int64_t a = c0 > mat_first[m] ? c0 : mat_first[m];
-        const int64_t b = c1 < mat_first[m + 1] ? c1 : mat_first[m + 1];
+        const int64_t m0 = rp[(size_t)m * NB], m1 = rp[(size_t)(m + 1) * NB];
+        const int64_t a = c0 > m0 ? c0 : m0;
+        const int64_t b = c1 < m1 ? c1 : m1;
         if (a >= b) continue;                               // the same for the whole CTA
         float v = 0.f;
         for (int64_t p = a + threadIdx.x; p < b; p += blockDim.x) v = fmaxf(v, nrm[p]);
@@ -174,20 +176,19 @@ __global__ void k_matrix_max(const float *__restrict__ nrm, const int *__restric
     }
 }
 
-// per matrix m: scale[m] = 2^floor(log2(2^14 / max block norm)) for fp16 (the
-// largest element then sits below 2^14, far from fp16 overflow, and values
-// down to ~1e-9 of it stay normal); 1 for bf16, whose exponent range is FP32's
-__global__ void k_matrix_scales(const unsigned *__restrict__ mxbits, int nmat, int fp16, float *__restrict__ scale) {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= nmat) return;
-    const float mx = __uint_as_float(mxbits[m]);
+// operand scale of a matrix with largest block norm mx: 2^floor(log2(2^14 / mx))
+// for fp16 (the largest element then sits below 2^14, far from fp16 overflow,
+// and values down to ~1e-9 of it stay normal); 1 for bf16, whose exponent
+// range is FP32's
+__device__ __forceinline__ float matrix_scale(unsigned mxbits, bool fp16) {
+    const float mx = __uint_as_float(mxbits);
     float s = 1.f;
     if (fp16 && mx > 0.f) {
         int e = (int)floorf(log2f(16384.f / mx));
         e = max(-60, min(60, e));
         s = ldexpf(1.f, e);
     }
-    scale[m] = s;
+    return s;
 }
 
 // one thread per 8 consecutive elements of a block row (one core-matrix row):
@@ -196,9 +197,11 @@ __global__ void k_matrix_scales(const unsigned *__restrict__ mxbits, int nmat, i
 // the layout of f32_index (32 bytes)
 template <bool BF16, int B>
 __global__ void k_split_planes(const double *__restrict__ val, int64_t nblk, uint16_t *__restrict__ hi,
-                               const float *__restrict__ scale,
-                               const int *__restrict__ mat_first, int nmat, const int *__restrict__ tpos,
+                               const unsigned *__restrict__ mx, float *__restrict__ scale,
+                               const int *__restrict__ rp, int NB, int nmat, const int *__restrict__ tpos,
                                float *__restrict__ xlin) {
+    // the scales, for the product kernel too
+    if (blockIdx.x == 0 && (int)threadIdx.x < nmat) scale[threadIdx.x] = matrix_scale(mx[threadIdx.x], !BF16);
     constexpr int kPE = B * B;
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= nblk * (kPE / 8)) return;
@@ -206,8 +209,8 @@ __global__ void k_split_planes(const double *__restrict__ val, int64_t nblk, uin
     const int rc0 = (int)(g % (kPE / 8)) * 8;     // first element (row r, columns c0..c0+7)
     const int r = rc0 / B, c0 = rc0 % B;
     int m = 0;
-    while (m + 1 < nmat && p >= mat_first[m + 1]) ++m;
-    const float sc = scale[m];
+    while (m + 1 < nmat && p >= rp[(size_t)(m + 1) * NB]) ++m;
+    const float sc = matrix_scale(mx[m], !BF16);
     const double2 *v2 = reinterpret_cast<const double2 *>(val + p * kPE + rc0);
     uint16_t h[8], l[8];
     double2 x2[4];
@@ -294,7 +297,7 @@ struct TcArgs {
     const int *tiles;
     const int64_t *step_off;
     const int *steps;
-    int ntile;
+    const int *flags;             // TcWork::counters
     uint32_t idesc;
     const float *scale;           // per matrix operand scale
     int job_a[kMaxJobs], job_b[kMaxJobs];
@@ -414,6 +417,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     volatile int *abort_flag = &ctl->abort_flag;
+    if (A.flags[1]) return;               // the K-step list outgrew its buffer: the host builds it again
+    const int ntile = A.flags[2];
 
     if (threadIdx.x == 0) {
         if (blockIdx.x == 0 && *A.pre_err) atomicOr(A.err, *A.pre_err);
@@ -455,22 +460,22 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
         // after it (its range is loaded a tile ahead)
         int lt = blockIdx.x;
         int64_t lq = 0, le = 0, nq = 0, ne = 0;
-        if (lt < A.ntile) { lq = A.step_off[lt]; le = A.step_off[lt + 1]; }
-        if (lt + (int)gridDim.x < A.ntile) { nq = A.step_off[lt + gridDim.x]; ne = A.step_off[lt + gridDim.x + 1]; }
+        if (lt < ntile) { lq = A.step_off[lt]; le = A.step_off[lt + 1]; }
+        if (lt + (int)gridDim.x < ntile) { nq = A.step_off[lt + gridDim.x]; ne = A.step_off[lt + gridDim.x + 1]; }
         lq += pr;
         // block index of this lane's slot in the warp's next step, loaded
         // while the current step's copies are issued
         int nxt = -1;
         auto fetch = [&]() {
-            while (lq >= le && lt < A.ntile) {
+            while (lq >= le && lt < ntile) {
                 lt += gridDim.x;
                 lq = nq + (lq - le);
                 le = ne;
-                if (lt + (int)gridDim.x < A.ntile) { nq = A.step_off[lt + gridDim.x]; ne = A.step_off[lt + gridDim.x + 1]; }
+                if (lt + (int)gridDim.x < ntile) { nq = A.step_off[lt + gridDim.x]; ne = A.step_off[lt + gridDim.x + 1]; }
             }
-            if (lt < A.ntile && lane < G::kSlots) nxt = A.steps[lq * G::kSlots + lane];
+            if (lt < ntile && lane < G::kSlots) nxt = A.steps[lq * G::kSlots + lane];
         };
-        for (fetch(); lt < A.ntile; it += 2) {
+        for (fetch(); lt < ntile; it += 2) {
             const int cur = nxt;
             lq += 2;
             fetch();
@@ -529,10 +534,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
             uint32_t it = 0, seg = 0;
             bool issued = false;
             int64_t n0 = 0, n1 = 0;          // step range of the next tile, loaded a tile ahead
-            if (blockIdx.x < A.ntile) { n0 = A.step_off[blockIdx.x]; n1 = A.step_off[blockIdx.x + 1]; }
-            for (int t = blockIdx.x; t < A.ntile && !*abort_flag; t += gridDim.x) {
+            if (blockIdx.x < ntile) { n0 = A.step_off[blockIdx.x]; n1 = A.step_off[blockIdx.x + 1]; }
+            for (int t = blockIdx.x; t < ntile && !*abort_flag; t += gridDim.x) {
                 const int64_t s0 = n0, s1 = n1;
-                if (t + (int)gridDim.x < A.ntile) { n0 = A.step_off[t + gridDim.x]; n1 = A.step_off[t + gridDim.x + 1]; }
+                if (t + (int)gridDim.x < ntile) { n0 = A.step_off[t + gridDim.x]; n1 = A.step_off[t + gridDim.x + 1]; }
                 bool ok = true;
                 for (int64_t q = s0; q < s1 && ok; ++seg) {
                     // one segment: up to kSegSteps K-steps into a fresh accumulator
@@ -593,12 +598,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
         };
         uint32_t seg = 0, pround = 0;
         int par = 0;
-        if (blockIdx.x < A.ntile) gather(blockIdx.x, 0);
-        for (int t = blockIdx.x; t < A.ntile && !*abort_flag; t += gridDim.x, par ^= 1) {
+        if (blockIdx.x < ntile) gather(blockIdx.x, 0);
+        for (int t = blockIdx.x; t < ntile && !*abort_flag; t += gridDim.x, par ^= 1) {
             const float *meta = meta2 + par * blocks_per_warp<B>() * 8;
             __syncwarp();
             const int nst = nst_next;
-            const bool more = t + (int)gridDim.x < A.ntile;
+            const bool more = t + (int)gridDim.x < ntile;
             if (nst < 0 && lane == 0) atomicOr(A.err, 4);
             // the tile's accumulator: sum of its segments, added with
             // round-to-nearest in registers (row 32*eq + lane, this warp's 128 columns)
@@ -898,16 +903,18 @@ void split_planes(MatSet &in, Arith ar, TcWork &w, cudaStream_t st) {
     const int64_t grid = (n / 8 + 255) / 256;
     const int *tpos = w.tpos_valid ? w.tpos.p : nullptr;
     if (ar == AR_BF16X3)
-        k_split_planes<true, B><<<(unsigned)grid, 256, 0, st>>>(in.val.p, in.total, in.ophi.p, w.scale.p,
-                                                                w.mat_first.p, in.nmat, tpos, w.lin ? w.xlin.p : nullptr);
+        k_split_planes<true, B><<<(unsigned)grid, 256, 0, st>>>(
+            in.val.p, in.total, in.ophi.p, (unsigned *)w.pre_err.p + 1, w.scale.p, in.row_ptr.p, in.NB, in.nmat, tpos,
+            w.lin ? w.xlin.p : nullptr);
     else
-        k_split_planes<false, B><<<(unsigned)grid, 256, 0, st>>>(in.val.p, in.total, in.ophi.p, w.scale.p,
-                                                                 w.mat_first.p, in.nmat, tpos, w.lin ? w.xlin.p : nullptr);
+        k_split_planes<false, B><<<(unsigned)grid, 256, 0, st>>>(
+            in.val.p, in.total, in.ophi.p, (unsigned *)w.pre_err.p + 1, w.scale.p, in.row_ptr.p, in.NB, in.nmat, tpos,
+            w.lin ? w.xlin.p : nullptr);
     RDM_LAUNCH_CHECK();
 }
 
 template <int B>
-double launch_tc(const NumArgs &a, const MatSet &in, const JobTable &jt, Arith ar, TcWork &w,
+void launch_tc(const NumArgs &a, const MatSet &in, const JobTable &jt, Arith ar, TcWork &w,
                  const TcPlan &plan, cudaStream_t st) {
     using G = Geo<B>;
     int dev = 0, nsm = 0;
@@ -920,7 +927,7 @@ double launch_tc(const NumArgs &a, const MatSet &in, const JobTable &jt, Arith a
     }
     TcArgs A{};
     A.planes = in.ophi.p; A.zero = w.zero.p;
-    A.tiles = w.tiles.p; A.step_off = w.step_off.p; A.steps = w.steps.p; A.ntile = plan.ntile;
+    A.tiles = w.tiles.p; A.step_off = w.step_off.p; A.steps = w.steps.p; A.flags = w.counters.p;
     // kind::f16: D = F32 (bit 4), A/B = BF16 (1) or F16 (0), K-major, N = kTileN, M = 128
     const uint32_t ab = ar == AR_BF16X3 ? 1u : 0u;
     A.idesc = (1u << 4) | (ab << 7) | (ab << 10) | (((uint32_t)kTileN >> 3) << 17) | ((128u >> 4) << 24);
@@ -940,10 +947,9 @@ double launch_tc(const NumArgs &a, const MatSet &in, const JobTable &jt, Arith a
     A.runs = w.tpos_valid ? 1 : 0;
     A.pre_err = w.pre_err.p;
     func_smem_once((const void *)k_tc_bf16x3<B>, (int)smem_bytes<B>());
-    const int grid = plan.ntile < nsm ? plan.ntile : nsm;
+    const int grid = plan.max_tile < nsm ? plan.max_tile : nsm;
     k_tc_bf16x3<B><<<grid, kThreads, smem_bytes<B>(), st>>>(A);
     RDM_LAUNCH_CHECK();
-    return (double)plan.nsteps * 3.0 * 2.0 * 128.0 * kTileN * B;
 }
 
 }  // namespace
@@ -957,20 +963,9 @@ void prepare_operands(MatSet &in, Arith ar, bool lin, TcWork &w, cudaStream_t st
     if (ar != AR_BF16X3 && ar != AR_FP16X3) throw Error{-1, "tensor-core arithmetic not available"};
     w.lin = lin;
     const int nmat = in.nmat;
-    std::vector<int> first(nmat + 1, 0);
-    for (int m = 0; m < nmat; ++m) first[m + 1] = first[m] + (int)in.nnzb[m];
-    w.mat_first.ensure(nmat + 1);
     w.scale.ensure(std::max(nmat, 1));
-    RDM_CUDA_TRY(cudaMemcpyAsync(w.mat_first.p, first.data(), (nmat + 1) * sizeof(int), cudaMemcpyHostToDevice, st));
-    w.mx.ensure(std::max(nmat, 1));
-    RDM_CUDA_TRY(cudaMemsetAsync(w.mx.p, 0, std::max(nmat, 1) * sizeof(unsigned), st));
-    if (in.total > 0) {
-        const int grid = (int)std::min<int64_t>(4 * 152, (in.total + 255) / 256);
-        k_matrix_max<<<grid, 256, 0, st>>>(in.nrm.p, w.mat_first.p, nmat, w.mx.p);
-        RDM_LAUNCH_CHECK();
-    }
-    k_matrix_scales<<<(nmat + 31) / 32, 32, 0, st>>>(w.mx.p, nmat, ar == AR_FP16X3 ? 1 : 0, w.scale.p);
-    RDM_LAUNCH_CHECK();
+    w.pre_err.ensure(1 + std::max(nmat, 1));
+    RDM_CUDA_TRY(cudaMemsetAsync(w.pre_err.p, 0, (1 + nmat) * sizeof(int), st));
     const int64_t n = in.total * (int64_t)in.b * in.b;
     in.ophi.ensure(std::max<int64_t>(2 * n, 1));   // hi and lo, interleaved per block
     if (w.lin && w.xlin.cap < (size_t)n) {
@@ -979,10 +974,11 @@ void prepare_operands(MatSet &in, Arith ar, bool lin, TcWork &w, cudaStream_t st
         if ((size_t)n * sizeof(float) > (fr + w.xlin.cap * sizeof(float)) / 4) w.lin = false;
         else w.xlin.ensure((size_t)n);
     }
-    w.pre_err.ensure(1);
-    RDM_CUDA_TRY(cudaMemsetAsync(w.pre_err.p, 0, sizeof(int), st));
     w.tpos_valid = false;
     if (n == 0) return;
+    const int mgrid = (int)std::min<int64_t>(4 * 152, (in.total + 255) / 256);
+    k_matrix_max<<<mgrid, 256, 0, st>>>(in.nrm.p, in.row_ptr.p, in.NB, nmat, (unsigned *)w.pre_err.p + 1);
+    RDM_LAUNCH_CHECK();
     // planes at the positions of the transposed blocks (the plan builder
     // points the K-step lists there), unless the test setting asks for one
     // copy per block
@@ -1000,11 +996,13 @@ void prepare_operands(MatSet &in, Arith ar, bool lin, TcWork &w, cudaStream_t st
     }
 }
 
-double launch_numeric_tc(const NumArgs &a, const MatSet &in, const JobTable &jt, Arith ar, TcWork &w,
-                         int NB, const TcPlan &plan, cudaStream_t st) {
+double tc_step_flops(int b) { return 3.0 * 2.0 * 128.0 * kTileN * b; }
+
+void launch_numeric_tc(const NumArgs &a, const MatSet &in, const JobTable &jt, Arith ar, TcWork &w,
+                       int NB, const TcPlan &plan, cudaStream_t st) {
     (void)NB;
     if (!tc_block_size_ok(in.b)) throw Error{-1, "the tensor-core path handles 16 x 16, 32 x 32 and 64 x 64 blocks"};
-    if (plan.ntile == 0) return 0.0;
+    if (plan.max_tile == 0) return;
     switch (in.b) {
         case 16: return launch_tc<16>(a, in, jt, ar, w, plan, st);
         case 32: return launch_tc<32>(a, in, jt, ar, w, plan, st);
@@ -1013,11 +1011,12 @@ double launch_numeric_tc(const NumArgs &a, const MatSet &in, const JobTable &jt,
 }
 
 TcPlan build_tc_plan(const MatSet &in, const JobTable &jt, const SysDev &sd, const int *out_rp,
-                     const int *mcol, TcWork &w, JobMask job_mask, int unit0, int unit1, cudaStream_t st) {
+                     const int *mcol, TcWork &w, JobMask job_mask, int unit0, int unit1, int64_t nupper,
+                     int64_t min_steps, cudaStream_t st) {
     switch (in.b) {
-        case 16: return build_plan<Geo<16>>(in, jt, sd, out_rp, mcol, w, job_mask, unit0, unit1, st);
-        case 32: return build_plan<Geo<32>>(in, jt, sd, out_rp, mcol, w, job_mask, unit0, unit1, st);
-        case 64: return build_plan<Geo<64>>(in, jt, sd, out_rp, mcol, w, job_mask, unit0, unit1, st);
+        case 16: return build_plan<Geo<16>>(in, jt, sd, out_rp, mcol, w, job_mask, unit0, unit1, nupper, min_steps, st);
+        case 32: return build_plan<Geo<32>>(in, jt, sd, out_rp, mcol, w, job_mask, unit0, unit1, nupper, min_steps, st);
+        case 64: return build_plan<Geo<64>>(in, jt, sd, out_rp, mcol, w, job_mask, unit0, unit1, nupper, min_steps, st);
         default: throw Error{-1, "the tensor-core path handles 16 x 16, 32 x 32 and 64 x 64 blocks"};
     }
 }

@@ -139,10 +139,20 @@ struct SysDev {
     DevBuf<int> row0, nbs, n_orb;      // [S]
     DevBuf<int> sys_of_row;            // [NB]
     DevBuf<double> emin, emax;         // [S]
-    DevBuf<double> c_lin, c_sq;        // [S]   branch coefficients of the current step
-    DevBuf<double> tau0, tau1;         // [S]   truncation thresholds of the current step
-    DevBuf<int> active;                // [S]   1 = still iterating
-    DevBuf<int> tier;                  // [S]
+    // scalars of the current step, one buffer that a step uploads in one copy
+    template <class T>
+    struct View { T *p = nullptr; };
+    DevBuf<double> step;               // c_lin, c_sq, tau0, tau1 [S], then active, tier [S] (int)
+    View<double> c_lin, c_sq;          // branch coefficients
+    View<double> tau0, tau1;           // truncation thresholds
+    View<int> active;                  // 1 = still iterating
+    View<int> tier;
+    static size_t step_doubles(int S) { return (size_t)5 * S; }
+    void ensure_step(int S) {
+        double *q = step.ensure(step_doubles(S));
+        c_lin.p = q; c_sq.p = q + S; tau0.p = q + 2 * (size_t)S; tau1.p = q + 3 * (size_t)S;
+        active.p = reinterpret_cast<int *>(q + 4 * (size_t)S); tier.p = active.p + S;
+    }
 };
 
 struct MatSet {
@@ -199,9 +209,13 @@ struct JobMask {
 // kernel launchers (implemented in the k_*.cu files)
 // ---------------------------------------------------------------------------
 
-// k_scan.cu: exclusive scan (out may alias in); returns nothing, total at out[n]
+// k_scan.cu: exclusive scan (out may alias in); returns nothing, total at out[n].
+// With n_dev the element count is *n_dev <= n (device memory).
 void scan_exclusive_i32(const int *in, int *out, int n, int *tmp, cudaStream_t st, int init = 0);
-void scan_exclusive_i64(const int *in, int64_t *out, int n, int64_t *tmp, cudaStream_t st);
+void scan_exclusive_i64(const int *in, int64_t *out, int n, int64_t *tmp, cudaStream_t st,
+                        const int *n_dev = nullptr);
+// two counts per element (low and high 32 bits), totals below 2^31 each
+void scan_exclusive_pair(const int64_t *in, int *out_lo, int *out_hi, int n, int64_t *tmp, cudaStream_t st);
 size_t scan_tmp_elems(int n);
 
 // k_setup.cu
@@ -224,11 +238,11 @@ void launch_check_values(const int *row_ptr, const int *col, const double *val, 
 // k_stats.cu: per-row partial sums then a deterministic per-system reduction.
 // q-layout of the per-system output (double, [S][nq]):
 //   0: Tr X0, 1: ||X0||_F^2, 2: Tr(X0 H0), 3+g: Tr(X1_g H0)
-// A block row's sums come in `parts` partial sums (row_stats_parts), so that
-// row_part has [q][NB * parts] entries.
-int row_stats_parts(int NB);
+// A block row's sums come in row_stats_parts() partial sums: row_part has
+// [q][NB][parts] entries.
+int row_stats_parts();
 void launch_row_stats(const int *row_ptr, const int *col, const double *val, int nmat, int NB,
-                      int b, const int *h_row_ptr, const int *h_col, const double *h_val, int parts,
+                      int b, const int *h_row_ptr, const int *h_col, const double *h_val,
                       double *row_part, cudaStream_t st);
 // Tr X and ||X||_F^2 of one matrix, row_part [2][NB]
 void launch_row_trace_norm(const int *row_ptr, const int *col, const double *val, int NB, int b, double *row_part,
@@ -243,22 +257,31 @@ void launch_row_dots(const int *p_row_ptr, const int *p_col, const double *p_val
 
 // k_symbolic.cu
 struct SymOut {
-    int *row_cnt;        // [njob*NB] kept blocks per (job,row)
+    int64_t *row_cnt;    // [njob*NB] kept blocks per (job,row); high 32 bits: those with col >= row
     int *row_off;        // [njob*NB] offset of the row's list in the pool
     int *pool_col;       // pool of kept columns
     int *pool_npair;     // pool of pair counts (per kept column)
     int *pool_top;       // [1] pool allocation counter
     int pool_cap;
     int *overflow;       // [1] set when the pool is too small
+    unsigned long long *npairs;   // [1] pairs of the kept upper-triangle blocks
 };
 // largest system (in block rows) the shared-memory row accumulator handles
 constexpr int kSymMaxNs = 8192;
 void launch_symbolic(const MatSet &in, const JobTable &jt, const SysDev &sd, int S,
                      SymOut so, cudaStream_t st, int max_ns);
-// gathers the pool into the output pattern; writes slot_row/slot_job and the
-// per-slot pair counts (0 for lower-triangle slots)
-void launch_gather(const SymOut &so, int njob, int NB, const int *out_row_ptr, int *out_col,
-                   int *slot_row, int *slot_job, int *slot_npair, cudaStream_t st);
+// Gathers the pool into the output pattern: columns, row and job of every
+// slot, its pair count (slot_npair may be null), and uidx, the rank of an
+// upper slot (col >= row) among the upper slots (out_urp: their count before
+// each row).  cls accumulates the pairs of active systems per kernel class.
+struct ClassMasks {
+    JobMask m[5];        // tensor cores, FP64, FP32, double-FP32, tensor-core slices
+};
+void launch_gather(const SymOut &so, int njob, int NB, const int *out_row_ptr, const int *out_urp, int *out_col,
+                   int *slot_row, int *slot_job, int *slot_npair, int *uidx, const SysDev &sd,
+                   const ClassMasks &cm, unsigned long long *cls, cudaStream_t st);
+// pair lists of the jobs in `fill` (pair_off: offsets of every slot's list;
+// null when no job is) and slot_x / slot_t of every slot
 void launch_pairs(const MatSet &in, const JobTable &jt, const SysDev &sd, const int *out_row_ptr,
                   const int *out_col, const int *slot_row, const int *slot_job,
                   const int64_t *pair_off, int64_t nslot, int NB, int *pair_a, int *pair_b,
@@ -281,11 +304,12 @@ struct NumArgs {
     const float *in_f32lo;     // in_val - in_f32 rounded to FP32 (double-FP32 products), may be null
     const float *in_nrm;
     const int *pair_a, *pair_b;
-    const int64_t *pair_off;
+    const int64_t *pair_off;   // null: no slot has pairs (copies of converged systems only)
     const int *slot_row, *slot_job, *slot_x, *slot_t;
     const int *work;        // upper slots to process
+    const int *nwork;       // their number
     int *work_next;         // zeroed counter: next work item to hand out
-    int nwork;
+    int max_work;           // bound of *nwork
     const int *sys_of_row;
     const double *c_lin, *c_sq, *tau0, *tau1;
     const int *active;
@@ -303,18 +327,15 @@ struct NumArgs {
     int b;
 };
 void launch_numeric_simt(const NumArgs &a, Arith ar, cudaStream_t st);
+// diagonal elements of the one-term products A A of the jobs in `jobs` as FP64
+// FMA chains, over those in out_val; flat rows [r0, r0 + nrows) of the mask
+void launch_diag_fp64(const NumArgs &a, const MatSet &in, const JobTable &jt, JobMask jobs, const int *out_rp,
+                      const int *out_col, const int *sys_tier, int r0, int nrows, cudaStream_t st);
 // FP32 copy of the FP64 master values (for the FP32 products)
 // FP32 copy (and, with f32lo, the FP32 remainder) of FP64 values
 void launch_to_f32(const double *val, float *f32, int64_t n, cudaStream_t st, float *f32lo = nullptr);
 
 // k_compact.cu
-// block triples of the upper slots of active systems per kernel class:
-// out[0] tensor cores (tc), out[1] FP64 (m64), out[2] FP32 (m32), out[3] double-FP32 (mff),
-// out[4] tensor-core slice products (moz)
-void launch_class_pairs(const int *slot_row, const int *out_col, const int *slot_npair, const int *slot_job,
-                        int64_t nslot, const int *sys_of_row, const int *active, const int *sys_tier,
-                        JobMask tc, JobMask m64, JobMask m32, JobMask mff, JobMask moz, unsigned long long *out,
-                        cudaStream_t st);
 // upper slots of the active systems' jobs selected by job_mask (per system
 // tier), plus (with_inactive) all upper slots of converged systems
 // (slots [s0, s1) only)
@@ -322,12 +343,6 @@ void launch_build_work(const int *slot_row, const int *out_col, int64_t s0, int6
                        int *work, int *nwork, cudaStream_t st, const int *sys_of_row,
                        const int *active, const int *slot_job, const int *sys_tier, JobMask job_mask,
                        int with_inactive);
-// uidx[s] = 1 for upper slots (col >= row), else 0 (scanned afterwards)
-void launch_upper_flags(const int *slot_row, const int *out_col, int64_t nslot, int *uidx,
-                        cudaStream_t st);
-// urp[r] = uidx[out_row_ptr[r]] for r in [0, n]
-void launch_gather_i32(const int *idx, const int *src, int n, int *dst, cudaStream_t st);
-
 // Compaction of the rows [r0, r0 + nrows) of the mask.  An upper slot is kept
 // on its own flag; a lower slot t on that of its upper partner slot_t[t],
 // and receives that block's transpose, read from out_val when the partner

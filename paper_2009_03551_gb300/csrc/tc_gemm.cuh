@@ -24,14 +24,16 @@ struct TcWork {
     DevBuf<int> step_cnt;
     DevBuf<int64_t> step_off;
     DevBuf<int> steps;          // per K-step: TBM A block indices, TBN B block indices (-1 = zero)
-    DevBuf<int> counters;       // [0]: error bits of the product kernel
+    // [0]: error bits of the product kernel, [1]: a list outgrew its buffer
+    // (the product kernel then does nothing), [2]: tiles, [4..5]: K-steps (64 bits)
+    DevBuf<int> counters;
     DevBuf<int> scan32;
     DevBuf<int64_t> scan64;
     DevBuf<float> scale;        // per matrix: power-of-two scale of its operand planes
-    DevBuf<unsigned> mx;        // per matrix: largest block norm (bit pattern)
-    DevBuf<int> mat_first;      // per matrix: first global block index (nmat+1)
     DevBuf<int> tpos;           // per block (i, k) of the input set: global index of block (k, i)
-    DevBuf<int> pre_err;        // error bits of the operand preparation (8: a transposed block missing)
+    // [0]: error bits of the operand preparation (8: a transposed block missing);
+    // [1 + m]: largest block norm of matrix m (bit pattern)
+    DevBuf<int> pre_err;
     DevBuf<float> xlin;         // FP32 values of the input set's upper blocks (layout f32_index)
     bool lin = false;           // xlin is filled for this step
     bool tpos_valid = false;    // the planes sit at tpos and the K-step lists point there
@@ -46,9 +48,11 @@ struct OzWork {
     DevBuf<uint16_t> zero;      // zero blocks: one per CTA and K-step slot
 };
 
+// Lists of one launch.  Their lengths stay on the device (TcWork::counters);
+// the host has bounds.
 struct TcPlan {
-    int ntile;
-    int64_t nsteps;
+    int max_tile = 0;           // bound of the number of tiles (0: no tile)
+    int64_t cap_steps = 0;      // K-steps that the list has room for
 };
 
 // Block sizes the tensor-core kernel handles (16, 32, 64), and the block rows
@@ -64,29 +68,35 @@ int tc_tile_rows(int b);
 // kernel divides the scale back out per job.
 void prepare_operands(MatSet &in, Arith ar, bool lin, TcWork &w, cudaStream_t st);
 
-// Tile lists of one multiplication step from the output mask, for the jobs
-// selected by job_mask (per system tier) and the super-row units
+// Tile and K-step lists of one multiplication step from the output mask, for
+// the jobs selected by job_mask (per system tier) and the super-row units
 // [unit0, unit1) (unit = job * ceil(NB/TR) + I covers block rows
-// TR I .. TR I + TR - 1 of the job, TR = tc_tile_rows(b)).
+// TR I .. TR I + TR - 1 of the job, TR = tc_tile_rows(b)), which have nupper
+// upper slots.  Nothing is waited for: min_steps is the least room made for
+// K-steps, and a list that needs more (counters[1], with the number in
+// counters[4..5]) has to be built again.
 TcPlan build_tc_plan(const MatSet &in, const JobTable &jt, const SysDev &sd, const int *out_rp,
-                     const int *mcol, TcWork &w, JobMask job_mask, int unit0, int unit1, cudaStream_t st);
+                     const int *mcol, TcWork &w, JobMask job_mask, int unit0, int unit1, int64_t nupper,
+                     int64_t min_steps, cudaStream_t st);
 
 // Numeric phase on the tensor cores; same output contract as
-// launch_numeric_simt for the slots of active systems.  Returns the flops
-// issued to the tensor cores.
-double launch_numeric_tc(const NumArgs &a, const MatSet &in, const JobTable &jt, Arith ar, TcWork &w,
+// launch_numeric_simt for the slots of active systems.
+void launch_numeric_tc(const NumArgs &a, const MatSet &in, const JobTable &jt, Arith ar, TcWork &w,
                          int NB, const TcPlan &plan, cudaStream_t st);
 
 // FP64-class products on the tensor cores from exact bf16 slices (32 x 32
 // blocks; k_oz.cu): the slices (7 or 8 per element) and row scales of the
 // first nmat matrices of `in` (false, with nothing done, when the device has
 // no room for them), the tile lists (128 x 64 tiles) of the jobs in job_mask,
-// and the launch (same output contract as the other numeric launches; returns
-// the MMA flops issued).
+// and the launch (same output contract as the other numeric launches).
+// tc_step_flops / oz_step_flops: the MMA flops issued per K-step.
 bool prepare_oz_operands(const MatSet &in, int nmat, int slices, OzWork &w, cudaStream_t st);
 TcPlan build_oz_plan(const MatSet &in, const JobTable &jt, const SysDev &sd, const int *out_rp, const int *mcol,
-                     TcWork &w, JobMask job_mask, int unit0, int unit1, cudaStream_t st);
-double launch_numeric_oz(const NumArgs &a, const MatSet &in, const JobTable &jt, const int *mcol, OzWork &ow,
+                     TcWork &w, JobMask job_mask, int unit0, int unit1, int64_t nupper, int64_t min_steps,
+                     cudaStream_t st);
+double tc_step_flops(int b);
+double oz_step_flops(const OzWork &ow);
+void launch_numeric_oz(const NumArgs &a, const MatSet &in, const JobTable &jt, const int *mcol, OzWork &ow,
                          TcWork &w, const TcPlan &plan, cudaStream_t st);
 
 }  // namespace rdm

@@ -40,7 +40,9 @@ struct TileBuild {
     int *step_cnt;       // [ntile]
     const int64_t *step_off;
     int *steps;          // [nsteps * kSlots]
-    int ntile;
+    const int *ntile;    // number of tiles
+    int64_t cap_steps;   // room in steps
+    int *flags;          // TcWork::counters
     int max_words;       // bitmap window in 32-column words (<= 512); wider windows: serial merge
     const int *tpos;     // K-step entries point at tpos[e] (the planes' position), or at e if null
 };
@@ -243,7 +245,7 @@ __device__ void tile_steps_serial(const TileBuild &T, int t, int fill) {
                 }
             }
             if (anyA && anyB) {
-                if (fill && w + n < T.step_off[t + 1]) {
+                if (fill && w + n < T.step_off[t + 1] && w + n < T.cap_steps) {
                     int *s = T.steps + (size_t)(w + n) * G::kSlots;
                     for (int q = 0; q < G::kSlots; ++q) s[q] = idx[q] >= 0 && T.tpos ? T.tpos[idx[q]] : idx[q];
                 }
@@ -253,148 +255,183 @@ __device__ void tile_steps_serial(const TileBuild &T, int t, int fill) {
         if (!fill && term == 0) T.tiles[(size_t)t * G::kTileInts + 2] = n;
     }
     if (!fill) T.step_cnt[t] = n;
-    else if (n != (int)(T.step_off[t + 1] - T.step_off[t])) T.tiles[(size_t)t * G::kTileInts + 3] = -1;
+    else T.tiles[(size_t)t * G::kTileInts + 3] = n == (int)(T.step_off[t + 1] - T.step_off[t]) ? n : -1;
 }
 
-// K-steps of one tile, warp-parallel: per term, the columns k of the tile's
+// K-steps of one tile, one CTA per tile: per term, the columns k of the tile's
 // TBM A rows and of its TBN B rows are marked in two shared-memory bitmaps
 // over the window where both can have columns; a K-step is a k marked in
 // both, its index the rank of k among those (prefix popcounts).  Each list
 // entry at such a k writes its block index into its slot of the step; the
 // other slots stay -1 (zero block).  Same steps, same order as the serial
-// merge, which lane 0 runs for windows wider than the bitmaps.
+// merge, which thread 0 runs for windows wider than the bitmaps.  The kernel
+// waits for loads, so a tile's slots are spread over four warps (one warp per
+// tile took 25 us for the ~180 tiles of a 150-atom cluster).
 constexpr int kStepWarps = 4, kStepWords = 512;    // 16,384 columns per window
 template <class G>
 __global__ void __launch_bounds__(32 * kStepWarps) k_tile_steps(TileBuild T, int fill) {
-    __shared__ unsigned ba_s[kStepWarps][kStepWords], bb_s[kStepWarps][kStepWords];
-    __shared__ int rank_s[kStepWarps][kStepWords];
-    const int wq = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int t = blockIdx.x * kStepWarps + wq;
-    if (t >= T.ntile) return;
-    unsigned *ba = ba_s[wq], *bb = bb_s[wq];
-    int *wr = rank_s[wq];
-    const int *d = T.tiles + (size_t)t * G::kTileInts;
-    const int p = d[0], I = d[1];
-    const Job &job = T.jt.job[p];
-    // the window of every term must fit the bitmaps, else the serial merge
-    int lo_t[2], hi_t[2], cur[2][G::kSlots], end[2][G::kSlots];
-    bool fits = true;
-    for (int term = 0; term < job.nterm; ++term) {
-        const int am = job.a[term], bm = job.b[term];
-        int loA = 0x7fffffff, hiA = -1, loB = 0x7fffffff, hiB = -1;
-        for (int q = 0; q < G::TBM; ++q) {
-            const int i = G::TBM * I + q;
-            cur[term][q] = end[term][q] = 0;
-            if (i < T.NB) { cur[term][q] = T.rp[am * T.NB + i]; end[term][q] = T.rp[am * T.NB + i + 1]; }
-            if (cur[term][q] < end[term][q]) {
-                loA = min(loA, T.col[cur[term][q]]);
-                hiA = max(hiA, T.col[end[term][q] - 1]);
-            }
-        }
-        for (int q = 0; q < G::TBN; ++q) {
-            const int j = d[G::kColOff + q];
-            cur[term][G::TBM + q] = end[term][G::TBM + q] = 0;
-            if (j >= 0) {
-                cur[term][G::TBM + q] = T.rp[bm * T.NB + j];
-                end[term][G::TBM + q] = T.rp[bm * T.NB + j + 1];
-            }
-            if (cur[term][G::TBM + q] < end[term][G::TBM + q]) {
-                loB = min(loB, T.col[cur[term][G::TBM + q]]);
-                hiB = max(hiB, T.col[end[term][G::TBM + q] - 1]);
-            }
-        }
-        lo_t[term] = max(loA, loB);
-        hi_t[term] = min(hiA, hiB);
-        if (hi_t[term] >= lo_t[term] && ((hi_t[term] - lo_t[term]) >> 5) + 1 > T.max_words) fits = false;
+    __shared__ unsigned ba[kStepWords], bb[kStepWords];
+    __shared__ int wr[kStepWords];
+    __shared__ int cur[2][G::kSlots], end[2][G::kSlots], lo_c[2][G::kSlots], hi_c[2][G::kSlots];
+    __shared__ int sh_carry;
+    static_assert(2 * G::kSlots <= 32 * kStepWarps, "one thread per slot and term");
+    const int tid = threadIdx.x, wq = tid >> 5, lane = tid & 31;
+    const int ntile = *T.ntile;
+    if (fill && blockIdx.x == 0 && tid == 0) {
+        const int64_t n = T.step_off[ntile];
+        if (n > T.cap_steps) T.flags[1] = 1;
+        T.flags[2] = ntile;
+        *reinterpret_cast<int64_t *>(T.flags + 4) = n;
     }
-    if (!fits) {
-        if (lane == 0) tile_steps_serial<G>(T, t, fill);
-        return;
-    }
-    int64_t w = fill ? T.step_off[t] : 0;
-    int n = 0, n_first = 0;
-    for (int term = 0; term < job.nterm; ++term) {
-        const int lo = lo_t[term], hi = hi_t[term];
-        if (hi < lo) continue;
-        const int nw = ((hi - lo) >> 5) + 1;
-        for (int x = lane; x < nw; x += 32) { ba[x] = 0u; bb[x] = 0u; }
-        __syncwarp();
-        for (int q = 0; q < G::kSlots; ++q) {
-            unsigned *bmap = q < G::TBM ? ba : bb;
-            for (int e = cur[term][q] + lane; e < end[term][q]; e += 32) {
-                const int k = T.col[e];
-                if (k < lo || k > hi) continue;
-                atomicOr(&bmap[(k - lo) >> 5], 1u << ((k - lo) & 31));
-            }
-        }
-        __syncwarp();
-        int carry = 0;
-        for (int x0 = 0; x0 < nw; x0 += 32) {
-            const int x = x0 + lane;
-            unsigned both = 0u;
-            if (x < nw) {
-                both = ba[x] & bb[x];
-                ba[x] = both;
-            }
-            const int c = __popc(both);
-            int y = c;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int z = __shfl_up_sync(0xffffffffu, y, o);
-                if (lane >= o) y += z;
-            }
-            if (x < nw) wr[x] = carry + y - c;
-            carry += __shfl_sync(0xffffffffu, y, 31);
-        }
-        __syncwarp();
-        if (fill) {
-            const int64_t wend = T.step_off[t + 1];
-            for (int64_t q = w + n + lane; q < min(w + n + carry, wend); q += 32) {
-                int *st = T.steps + (size_t)q * G::kSlots;
-                for (int k = 0; k < G::kSlots; ++k) st[k] = -1;
-            }
-            __syncwarp();
-            for (int q = 0; q < G::kSlots; ++q)
-                for (int e = cur[term][q] + lane; e < end[term][q]; e += 32) {
-                    const int k = T.col[e];
-                    if (k < lo || k > hi) continue;
-                    const int kk = k - lo;
-                    const unsigned word = ba[kk >> 5];
-                    if (!((word >> (kk & 31)) & 1u)) continue;
-                    const int r = wr[kk >> 5] + __popc(word & ((1u << (kk & 31)) - 1u));
-                    if (w + n + r < wend) T.steps[(size_t)(w + n + r) * G::kSlots + q] = T.tpos ? T.tpos[e] : e;
+    for (int t = blockIdx.x; t < ntile; t += gridDim.x) {
+        const int *d = T.tiles + (size_t)t * G::kTileInts;
+        const int p = d[0], I = d[1];
+        const Job &job = T.jt.job[p];
+        if (tid < job.nterm * G::kSlots) {
+            const int term = tid / G::kSlots, q = tid % G::kSlots;
+            const int mat = q < G::TBM ? job.a[term] : job.b[term];
+            const int row = q < G::TBM ? G::TBM * I + q : d[G::kColOff + q - G::TBM];
+            int c = 0, e = 0, l = 0x7fffffff, h = -1;
+            if (row >= 0 && row < T.NB) {
+                c = T.rp[mat * T.NB + row];
+                e = T.rp[mat * T.NB + row + 1];
+                if (c < e) {
+                    l = T.col[c];
+                    h = T.col[e - 1];
                 }
-            __syncwarp();
+            }
+            cur[term][q] = c;
+            end[term][q] = e;
+            lo_c[term][q] = l;
+            hi_c[term][q] = h;
         }
-        n += carry;
-        if (!fill && term == 0) n_first = n;
-    }
-    if (lane == 0) {
-        if (!fill) T.tiles[(size_t)t * G::kTileInts + 2] = n_first;
-        if (!fill) T.step_cnt[t] = n;
-        else if (n != (int)(T.step_off[t + 1] - T.step_off[t])) T.tiles[(size_t)t * G::kTileInts + 3] = -1;
+        __syncthreads();
+        // the window of every term must fit the bitmaps, else the serial merge
+        int lo_t[2], hi_t[2];
+        bool fits = true;
+#pragma unroll
+        for (int term = 0; term < 2; ++term) {
+            lo_t[term] = 0;
+            hi_t[term] = -1;
+            if (term >= job.nterm) continue;
+            int loA = 0x7fffffff, hiA = -1, loB = 0x7fffffff, hiB = -1;
+            for (int q = 0; q < G::TBM; ++q) {
+                loA = min(loA, lo_c[term][q]);
+                hiA = max(hiA, hi_c[term][q]);
+            }
+            for (int q = G::TBM; q < G::kSlots; ++q) {
+                loB = min(loB, lo_c[term][q]);
+                hiB = max(hiB, hi_c[term][q]);
+            }
+            lo_t[term] = max(loA, loB);
+            hi_t[term] = min(hiA, hiB);
+            if (hi_t[term] >= lo_t[term] && ((hi_t[term] - lo_t[term]) >> 5) + 1 > T.max_words) fits = false;
+        }
+        if (!fits) {
+            if (tid == 0) tile_steps_serial<G>(T, t, fill);
+            __syncthreads();
+            continue;
+        }
+        int64_t w = fill ? T.step_off[t] : 0;
+        const int64_t wcap = fill ? min(T.step_off[t + 1], T.cap_steps) : 0;
+        int n = 0, n_first = 0;
+#pragma unroll
+        for (int term = 0; term < 2; ++term) {
+            const int lo = lo_t[term], hi = hi_t[term];
+            if (hi >= lo) {
+                const int nw = ((hi - lo) >> 5) + 1;
+                for (int x = tid; x < nw; x += 32 * kStepWarps) { ba[x] = 0u; bb[x] = 0u; }
+                __syncthreads();
+                for (int q = wq; q < G::kSlots; q += kStepWarps) {
+                    unsigned *bmap = q < G::TBM ? ba : bb;
+                    const int qe = end[term][q];
+                    for (int e = cur[term][q] + lane; e < qe; e += 32) {
+                        const int k = T.col[e];
+                        if (k < lo || k > hi) continue;
+                        atomicOr(&bmap[(k - lo) >> 5], 1u << ((k - lo) & 31));
+                    }
+                }
+                __syncthreads();
+                if (wq == 0) {
+                    int carry = 0;
+                    for (int x0 = 0; x0 < nw; x0 += 32) {
+                        const int x = x0 + lane;
+                        unsigned both = 0u;
+                        if (x < nw) {
+                            both = ba[x] & bb[x];
+                            ba[x] = both;
+                        }
+                        const int c = __popc(both);
+                        int y = c;
+#pragma unroll
+                        for (int o = 1; o < 32; o <<= 1) {
+                            const int z = __shfl_up_sync(0xffffffffu, y, o);
+                            if (lane >= o) y += z;
+                        }
+                        if (x < nw) wr[x] = carry + y - c;
+                        carry += __shfl_sync(0xffffffffu, y, 31);
+                    }
+                    if (lane == 0) sh_carry = carry;
+                }
+                __syncthreads();
+                const int carry = sh_carry;
+                if (fill) {
+                    // -1 everywhere, then the stored blocks
+                    const int64_t f0 = (w + n) * G::kSlots, f1 = min(w + n + carry, wcap) * G::kSlots;
+                    for (int64_t q = f0 + tid; q < f1; q += 32 * kStepWarps) T.steps[q] = -1;
+                    __syncthreads();
+                    for (int q = wq; q < G::kSlots; q += kStepWarps) {
+                        const int qe = end[term][q];
+                        for (int e = cur[term][q] + lane; e < qe; e += 32) {
+                            const int k = T.col[e];
+                            if (k < lo || k > hi) continue;
+                            const int kk = k - lo;
+                            const unsigned word = ba[kk >> 5];
+                            if (!((word >> (kk & 31)) & 1u)) continue;
+                            const int r = wr[kk >> 5] + __popc(word & ((1u << (kk & 31)) - 1u));
+                            if (w + n + r < wcap) T.steps[(size_t)(w + n + r) * G::kSlots + q] = T.tpos ? T.tpos[e] : e;
+                        }
+                    }
+                }
+                n += carry;
+                __syncthreads();
+            }
+            if (term == 0) n_first = n;
+        }
+        if (tid == 0) {
+            if (!fill) {
+                T.tiles[(size_t)t * G::kTileInts + 2] = n_first;
+                T.step_cnt[t] = n;
+            } else {
+                T.tiles[(size_t)t * G::kTileInts + 3] = n == (int)(T.step_off[t + 1] - T.step_off[t]) ? n : -1;
+            }
+        }
     }
 }
-
-template <class G>
-__global__ void k_set_nsteps(int *tiles, const int *step_cnt, int ntile) {
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < ntile) tiles[(size_t)t * G::kTileInts + 3] = step_cnt[t];
-}
-
 
 template <class G>
 TcPlan build_plan(const MatSet &in, const JobTable &jt, const SysDev &sd, const int *out_rp, const int *mcol,
-                  TcWork &w, JobMask job_mask, int unit0, int unit1, cudaStream_t st) {
+                  TcWork &w, JobMask job_mask, int unit0, int unit1, int64_t nupper, int64_t min_steps,
+                  cudaStream_t st) {
     TcPlan plan{};
     const int NB = in.NB, NBT = (NB + G::TBM - 1) / G::TBM;
     const int nrowt = unit1 - unit0;
-    if (nrowt <= 0) return plan;
     w.counters.ensure(8);
     RDM_CUDA_TRY(cudaMemsetAsync(w.counters.p, 0, 8 * sizeof(int), st));
+    if (nrowt <= 0 || nupper <= 0) return plan;
+    // every tile of a super-row but its last one has TBN columns, each with at
+    // least one upper slot
+    const int64_t max_tile = nupper / G::TBN + nrowt;
+    plan.max_tile = (int)max_tile;
     w.tile_cnt.ensure(nrowt + 1);
     w.tile_off.ensure(nrowt + 1);
     w.scan32.ensure(scan_tmp_elems(nrowt + 1));
+    w.tiles.ensure((size_t)max_tile * G::kTileInts);
+    w.step_cnt.ensure(max_tile + 1);
+    w.step_off.ensure(max_tile + 1);
+    w.scan64.ensure(scan_tmp_elems((int)max_tile + 1));
+    w.steps.ensure((size_t)std::max<int64_t>(min_steps, 1) * G::kSlots);
+    plan.cap_steps = (int64_t)(w.steps.cap / G::kSlots);
     TileBuild T{};
     T.rp = in.row_ptr.p; T.col = in.col.p; T.NB = NB; T.NBT = NBT; T.jt = jt;
     T.out_rp = out_rp; T.mcol = mcol; T.sys_of_row = sd.sys_of_row.p; T.active = sd.active.p;
@@ -403,39 +440,22 @@ TcPlan build_plan(const MatSet &in, const JobTable &jt, const SysDev &sd, const 
     T.sys_tier = sd.tier.p;
     T.tile_cnt = w.tile_cnt.p; T.tile_off = w.tile_off.p;
     T.tpos = w.tpos_valid ? w.tpos.p : nullptr;
+    T.tiles = w.tiles.p; T.step_cnt = w.step_cnt.p; T.step_off = w.step_off.p; T.steps = w.steps.p;
+    T.ntile = w.tile_off.p + nrowt; T.cap_steps = plan.cap_steps; T.flags = w.counters.p;
     static_assert(kTileRowWords == kStepWords, "one window bound for both plan builders");
     T.max_words = w.knobs.window_words > 0 && w.knobs.window_words < kTileRowWords ? w.knobs.window_words
                                                                                     : kTileRowWords;
-    k_tile_rows<G><<<(nrowt + kTileRowWarps - 1) / kTileRowWarps, 32 * kTileRowWarps, 0, st>>>(T, 0);
+    const int rgrid = (nrowt + kTileRowWarps - 1) / kTileRowWarps;
+    const int sgrid = (int)std::min<int64_t>(max_tile, 152 * 16);
+    k_tile_rows<G><<<rgrid, 32 * kTileRowWarps, 0, st>>>(T, 0);
     RDM_LAUNCH_CHECK();
     scan_exclusive_i32(w.tile_cnt.p, w.tile_off.p, nrowt, w.scan32.p, st);
-    int ntile = 0;
-    RDM_CUDA_TRY(cudaMemcpyAsync(&ntile, w.tile_off.p + nrowt, sizeof(int), cudaMemcpyDeviceToHost, st));
-    RDM_CUDA_TRY(cudaStreamSynchronize(st));
-    plan.ntile = ntile;
-    if (ntile == 0) return plan;
-    w.tiles.ensure((size_t)ntile * G::kTileInts);
-    T.tiles = w.tiles.p;
-    k_tile_rows<G><<<(nrowt + kTileRowWarps - 1) / kTileRowWarps, 32 * kTileRowWarps, 0, st>>>(T, 1);
+    k_tile_rows<G><<<rgrid, 32 * kTileRowWarps, 0, st>>>(T, 1);
     RDM_LAUNCH_CHECK();
-    w.step_cnt.ensure(ntile + 1);
-    w.step_off.ensure(ntile + 1);
-    w.scan64.ensure(scan_tmp_elems(ntile + 1));
-    T.ntile = ntile;
-    T.step_cnt = w.step_cnt.p;
-    k_tile_steps<G><<<(ntile + kStepWarps - 1) / kStepWarps, 32 * kStepWarps, 0, st>>>(T, 0);
+    k_tile_steps<G><<<sgrid, 32 * kStepWarps, 0, st>>>(T, 0);
     RDM_LAUNCH_CHECK();
-    scan_exclusive_i64(w.step_cnt.p, w.step_off.p, ntile, w.scan64.p, st);
-    int64_t nsteps = 0;
-    RDM_CUDA_TRY(cudaMemcpyAsync(&nsteps, w.step_off.p + ntile, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
-    RDM_CUDA_TRY(cudaStreamSynchronize(st));
-    plan.nsteps = nsteps;
-    w.steps.ensure(std::max<int64_t>(nsteps, 1) * G::kSlots);
-    T.step_off = w.step_off.p;
-    T.steps = w.steps.p;
-    k_set_nsteps<G><<<(ntile + 127) / 128, 128, 0, st>>>(w.tiles.p, w.step_cnt.p, ntile);
-    RDM_LAUNCH_CHECK();
-    k_tile_steps<G><<<(ntile + kStepWarps - 1) / kStepWarps, 32 * kStepWarps, 0, st>>>(T, 1);
+    scan_exclusive_i64(w.step_cnt.p, w.step_off.p, (int)max_tile, w.scan64.p, st, T.ntile);
+    k_tile_steps<G><<<sgrid, 32 * kStepWarps, 0, st>>>(T, 1);
     RDM_LAUNCH_CHECK();
     return plan;
 }
