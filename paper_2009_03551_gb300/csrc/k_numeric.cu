@@ -9,8 +9,8 @@
 // C_mn and C_nm differs.  The block Frobenius norm is reduced in FP64 and the
 // block is kept iff norm >= tau (the block-wise "filter" of Sec. 2.3).
 //
-// One CTA per output block (grid-stride over the work list); the two
-// operand blocks of each pair are staged in shared memory, each thread owns
+// One CTA per output block (work items from an atomic counter) for b >= 8; the
+// two operand blocks of each pair are staged in shared memory, each thread owns
 // ceil(b^2 / threads) outputs.  On GB300 the FP64 rate is the bound of this
 // kernel; the FP32 variant converts the FP64 master values on load.
 #include "fp_bits.cuh"
@@ -40,6 +40,28 @@ __device__ __forceinline__ double block_sum(double v, double *sh) {
     for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += sh[k];
     __syncthreads();
     return t;
+}
+
+template <class T>
+__device__ __forceinline__ T operand(double x) {
+    if constexpr (std::is_same<T, float>::value) return f64_to_f32(x);
+    else return x;
+}
+
+// B consecutive doubles (a row of a block, aligned to its size)
+template <int B>
+__device__ __forceinline__ void load_row(const double *p, double (&v)[B]) {
+    if constexpr (B == 4) {
+        asm volatile("ld.global.v4.f64 {%0,%1,%2,%3}, [%4];"
+                     : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3])
+                     : "l"(p));
+    } else if constexpr (B == 2) {
+        const double2 x = *reinterpret_cast<const double2 *>(p);
+        v[0] = x.x;
+        v[1] = x.y;
+    } else {
+        v[0] = p[0];
+    }
 }
 
 template <int B, class T>
@@ -80,8 +102,8 @@ __global__ void __launch_bounds__(Cfg<B>::NT) k_numeric_simt(NumArgs a) {
             const double *gb = a.in_val + (size_t)a.pair_b[q] * BB;
             __syncthreads();
             for (int e = tid; e < BB; e += NT) {
-                As[(e / B) * LD + (e % B)] = (T)ga[e];
-                Bs[(e / B) * LD + (e % B)] = (T)gb[e];
+                As[(e / B) * LD + (e % B)] = operand<T>(ga[e]);
+                Bs[(e / B) * LD + (e % B)] = operand<T>(gb[e]);
             }
             __syncthreads();
 #pragma unroll
@@ -139,6 +161,77 @@ __global__ void __launch_bounds__(Cfg<B>::NT) k_numeric_simt(NumArgs a) {
         if (tid == 0) {
             a.out_nrm[s] = __double2float_ru(nrm);
             a.keep[s] = keep;
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Blocks of 1, 2 and 4: b*b lanes per output block, a lane its element, rows of
+// the operand blocks read straight into registers, four pairs ahead of the
+// FMAs.  With so few operations per pair the kernel waits for loads; staging
+// each pair in shared memory between barriers, with half of a CTA's 32 threads
+// idle at b = 4, took 87 us for the 4,160 blocks of up to 128 pairs of a
+// 64-atom chain, 59 us here, 5 more than its FMAs take on the FP64 pipe.  Same chains of FMAs and the same sums as
+// k_numeric_simt.
+// ---------------------------------------------------------------------------
+template <int B, class T>
+__global__ void __launch_bounds__(128) k_numeric_small(NumArgs a) {
+    constexpr int L = B * B, PB = 128 / L, BB = B * B, U = 4;
+    __shared__ int s_w;
+    const int nwork = *a.nwork;
+    const int g = threadIdx.x / L, e = threadIdx.x % L, m = e / B, n = e % B;
+    for (;;) {
+        if (threadIdx.x == 0) s_w = atomicAdd(a.work_next, PB);
+        __syncthreads();
+        const int w0 = s_w, w = w0 + g;
+        __syncthreads();
+        if (w0 >= nwork) break;
+        const bool on = w < nwork;
+        const int s = on ? a.work[w] : 0;
+        const int64_t p0 = on && a.pair_off ? a.pair_off[s] : 0, p1 = on && a.pair_off ? a.pair_off[s + 1] : 0;
+        T acc = T(0);
+        int64_t q = p0;
+        for (; q + U <= p1; q += U) {
+            double x[U][B], y[U][B];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                load_row<B>(a.in_val + (size_t)a.pair_a[q + u] * BB + m * B, x[u]);
+                load_row<B>(a.in_val + (size_t)a.pair_b[q + u] * BB + n * B, y[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int k = 0; k < B; ++k) acc = fma(operand<T>(x[u][k]), operand<T>(y[u][k]), acc);
+        }
+        for (; q < p1; ++q) {
+            double x[B], y[B];
+            load_row<B>(a.in_val + (size_t)a.pair_a[q] * BB + m * B, x);
+            load_row<B>(a.in_val + (size_t)a.pair_b[q] * BB + n * B, y);
+#pragma unroll
+            for (int k = 0; k < B; ++k) acc = fma(operand<T>(x[k]), operand<T>(y[k]), acc);
+        }
+        double out = 0.0, tau = 0.0;
+        bool diag = false;
+        if (on) {
+            const int sys = a.sys_of_row[a.slot_row[s]];
+            const int job = a.slot_job[s], sx = a.slot_x[s];
+            tau = a.job_tau_sel[job] ? a.tau1[sys] : a.tau0[sys];
+            out = a.c_sq[sys] * (double)acc;
+            if (sx >= 0) out = fma(a.c_lin[sys], a.in_val[(size_t)sx * BB + e], out);
+            diag = a.slot_t[s] == s;
+        }
+        const double tr = __shfl_sync(0xffffffffu, out, (threadIdx.x & 31) - e + n * B + m);
+        if (diag) out = 0.5 * (out + tr);
+        double ss = out * out;
+#pragma unroll
+        for (int o = L / 2; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+        if (on) {
+            const double nrm = sqrt(ss);
+            a.out_val[(size_t)(a.uidx[s] - a.u0) * BB + e] = out;
+            if (e == 0) {
+                a.out_nrm[s] = __double2float_ru(nrm);
+                a.keep[s] = (nrm >= tau) && (nrm > 0.0);
+            }
         }
     }
 }
@@ -553,20 +646,6 @@ void launch_b(const NumArgs &a, cudaStream_t st) {
     RDM_LAUNCH_CHECK();
 }
 
-template <class T>
-void dispatch(const NumArgs &a, cudaStream_t st) {
-    switch (a.b) {
-        case 1: launch_b<1, T>(a, st); break;
-        case 2: launch_b<2, T>(a, st); break;
-        case 4: launch_b<4, T>(a, st); break;
-        case 8: launch_b<8, T>(a, st); break;
-        case 16: launch_b<16, T>(a, st); break;
-        case 32: launch_b<32, T>(a, st); break;
-        case 64: launch_b<64, T>(a, st); break;
-        default: throw Error{-1, "block size must be 1, 2, 4, 8, 16, 32 or 64"};
-    }
-}
-
 // blocks of kernel k (threads per block nt, static shared memory) resident on the whole GPU
 template <class K>
 int resident_blocks(K k, int nt) {
@@ -575,6 +654,28 @@ int resident_blocks(K k, int nt) {
     RDM_CUDA_TRY(cudaGetDevice(&dev));
     RDM_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     return std::max(1, per_sm) * nsm;
+}
+
+template <int B, class T>
+void launch_small(const NumArgs &a, cudaStream_t st) {
+    static const int res = resident_blocks(k_numeric_small<B, T>, 128);
+    const int per = 128 / (B * B);
+    k_numeric_small<B, T><<<std::min((a.max_work + per - 1) / per, res), 128, 0, st>>>(a);
+    RDM_LAUNCH_CHECK();
+}
+
+template <class T>
+void dispatch(const NumArgs &a, cudaStream_t st) {
+    switch (a.b) {
+        case 1: launch_small<1, T>(a, st); break;
+        case 2: launch_small<2, T>(a, st); break;
+        case 4: launch_small<4, T>(a, st); break;
+        case 8: launch_b<8, T>(a, st); break;
+        case 16: launch_b<16, T>(a, st); break;
+        case 32: launch_b<32, T>(a, st); break;
+        case 64: launch_b<64, T>(a, st); break;
+        default: throw Error{-1, "block size must be 1, 2, 4, 8, 16, 32 or 64"};
+    }
 }
 
 }  // namespace
