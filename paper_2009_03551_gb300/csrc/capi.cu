@@ -159,6 +159,9 @@ struct rdm_handle {
     MatSet X[2];
     int cur = 0;
 
+    // scratch of the uploads (pattern, system tables, error word), kept between them
+    DevBuf<int> up_rp, up_col, up_sys, up_z, up_err, up_orow, up_ocol;
+
     // work buffers
     DevBuf<int> row_off, pool_col, pool_npair, counters, mask_col;
     DevBuf<int64_t> row_cnt;
@@ -246,6 +249,7 @@ void d2h(T *dst, const T *src, size_t n, cudaStream_t st) {
 // upload and validation
 // ---------------------------------------------------------------------------
 
+// (that every (i, j) has its (j, i) is checked with the values, in a kernel)
 void check_pattern(const rdm_bsr *A, const std::vector<int> &rp, const std::vector<int> &col,
                    bool need_diag) {
     const int nb = A->nb;
@@ -264,13 +268,6 @@ void check_pattern(const rdm_bsr *A, const std::vector<int> &rp, const std::vect
         if (need_diag && !diag)
             throw Error{RDM_EBADBSR, "diagonal block missing in block row " + std::to_string(i)};
     }
-    // symmetric pattern: every (i,j) has (j,i)
-    for (int i = 0; i < nb; ++i)
-        for (int p = rp[i]; p < rp[i + 1]; ++p) {
-            int j = col[p];
-            if (!std::binary_search(col.begin() + rp[j], col.begin() + rp[j + 1], i))
-                throw Error{RDM_EBADBSR, "block pattern is not symmetric"};
-        }
 }
 
 void upload_matrix(rdm_handle *h, const rdm_bsr *A, std::vector<int> &rp, std::vector<int> &col,
@@ -298,7 +295,7 @@ void upload_matrix(rdm_handle *h, const rdm_bsr *A, std::vector<int> &rp, std::v
                                      A->on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
                                      h->stream));
     // value checks on the device: finite, symmetric (1e-12 max|H|), zero padding
-    DevBuf<int> drp, dcol, derr, dsys, dz;
+    DevBuf<int> &drp = h->up_rp, &dcol = h->up_col, &derr = h->up_err, &dsys = h->up_sys, &dz = h->up_z;
     drp.ensure(nb + 1);
     dcol.ensure(std::max<int64_t>(1, A->nnzb));
     derr.ensure(4);
@@ -315,7 +312,6 @@ void upload_matrix(rdm_handle *h, const rdm_bsr *A, std::vector<int> &rp, std::v
     int herr[4];
     d2h(herr, derr.p, 4, h->stream);
     sync(h);
-    drp.release(); dcol.release(); derr.release(); dsys.release(); dz.release();
     if (herr[0] & 1) throw Error{RDM_EBADBSR, "matrix has non-finite values"};
     if (herr[0] & 8) throw Error{RDM_EBADBSR, "block pattern is not symmetric"};
     if (herr[0] & 2) throw Error{RDM_EBADBSR, "matrix values are not symmetric (tolerance 1e-12 max|H|)"};
@@ -341,7 +337,7 @@ void ensure_reblocked(rdm_handle *h, int s, int bs) {
         std::vector<int> orow(nout);
         for (int i = 0; i + 1 < (int)orp.size(); ++i)
             for (int p = orp[i]; p < orp[i + 1]; ++p) orow[p] = i;
-        DevBuf<int> drp, dcol, dorow, docol;
+        DevBuf<int> &drp = h->up_rp, &dcol = h->up_col, &dorow = h->up_orow, &docol = h->up_ocol;
         drp.ensure(rp.size());
         dcol.ensure(std::max<size_t>(col.size(), 1));
         dorow.ensure(std::max<int64_t>(nout, 1));
@@ -2238,8 +2234,16 @@ int rdm_batch_create(rdm_handle *h, int n_systems) {
     if (n_systems < 1 || n_systems > 65536) return fail(h, RDM_EINVAL, "n_systems out of range");
     return guarded(h, [&] {
         DeviceGuard dg(h->device);
-        h->hs.clear();
+        // the systems' device buffers stay for the next uploads (those of
+        // systems beyond n_systems are freed)
         h->hs.resize(n_systems);
+        for (HostSys &y : h->hs) {
+            y.has_h0 = y.has_s = false;
+            for (bool &f : y.has_h1) f = false;
+            y.rb.b = 0;
+            y.nb = y.n = 0;
+            y.n_elec = 0;
+        }
         h->S = n_systems;
         h->b = 0;
         h->solved = false;
@@ -2269,7 +2273,7 @@ int rdm_upload_h0(rdm_handle *h, int sys, const rdm_bsr *H0, int64_t n_electrons
             throw;
         }
         y.has_h0 = true;
-        y.rb = SysMats{};
+        y.rb.b = 0;       // made again at the next solve that needs it
         y.nb = H0->nb;
         y.n = H0->n;
         y.n_elec = n_electrons;
@@ -2297,7 +2301,7 @@ int rdm_upload_h1(rdm_handle *h, int sys, int dir, const rdm_bsr *H1) {
             return fail(h, RDM_EINVAL, "H1 must have the same nb, b and n as H0");
         upload_matrix(h, H1, y.rp1[dir], y.col1[dir], y.val1[dir], false);
         y.has_h1[dir] = true;
-        y.rb = SysMats{};
+        y.rb.b = 0;       // made again at the next solve that needs it
         h->solved = false;
         return RDM_OK;
     });
@@ -2316,7 +2320,7 @@ int rdm_upload_s(rdm_handle *h, int sys, const rdm_bsr *S) {
             return fail(h, RDM_EINVAL, "S must have the same nb, b and n as H0");
         upload_matrix(h, S, y.rps, y.cols, y.vals, true);
         y.has_s = true;
-        y.rb = SysMats{};
+        y.rb.b = 0;       // made again at the next solve that needs it
         h->solved = false;
         return RDM_OK;
     });
