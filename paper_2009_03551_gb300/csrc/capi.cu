@@ -122,6 +122,7 @@ struct HostStep {
     int ctr[kCtrInts];
     int nupper, kept;
     int tc[8], oz[8];                 // TcWork::counters of the two plans
+    int pre_err;                      // error bits of the transposed positions (FP32 products)
     int rp[kMaxJobs + 1];             // first block of every output matrix
 };
 
@@ -738,6 +739,15 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
         if (any_c[1]) in.opf32lo.ensure(std::max<int64_t>(in.total, 1) * bb);
         launch_to_f32(in.val.p, in.opf32.p, in.total * (int64_t)bb, st, any_c[1] ? in.opf32lo.p : nullptr);
     }
+    // the FP32 products stage the transposed blocks (patterns are symmetric)
+    const bool f32_t = any_c[2] && b == 32;
+    if (f32_t && !(tc && h->tcw.tpos_valid)) {
+        if (!tc) {
+            h->tcw.pre_err.ensure(1);
+            RDM_CUDA_TRY(cudaMemsetAsync(h->tcw.pre_err.p, 0, sizeof(int), st));
+        }
+        find_transposes(in, h->tcw, st);
+    }
 
     // symbolic phase: the mask, its row pointers and the ranks of its upper slots
     h->row_cnt.ensure(nrows);
@@ -898,6 +908,7 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
             NumArgs a{};
             a.in_val = in.val.p; a.in_nrm = in.nrm.p;
             a.in_f32 = f32_planes ? in.opf32.p : nullptr;
+            a.tpos = f32_t ? h->tcw.tpos.p : nullptr;
             a.in_f32lo = any_c[1] ? in.opf32lo.p : nullptr;
             a.pair_a = h->pair_a.p; a.pair_b = h->pair_b.p; a.pair_off = lists ? h->pair_off.p : nullptr;
             a.slot_row = h->slot_row.p; a.slot_job = h->slot_job.p; a.slot_x = h->slot_x.p; a.slot_t = h->slot_t.p;
@@ -942,6 +953,7 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
             d2h(hs->ctr, h->counters.p, kCtrInts, st);
             if (tc) d2h(hs->tc, h->tcw.counters.p, 8, st);
             if (any_oz) d2h(hs->oz, h->tcw_oz.counters.p, 8, st);
+            if (f32_t) d2h(&hs->pre_err, h->tcw.pre_err.p, 1, st);
             if (g == ngroup - 1 && NB)
                 RDM_CUDA_TRY(cudaMemcpy2DAsync(hs->rp, sizeof(int), out.row_ptr.p, (size_t)NB * sizeof(int), sizeof(int),
                                                njob + 1, cudaMemcpyDeviceToHost, st));
@@ -962,7 +974,7 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
             steps_oz = std::max(steps_oz, nst_oz);
         }
         kept_end = hs->kept;
-        const int tc_err = (tc ? hs->tc[0] : 0) | (any_oz ? hs->oz[0] : 0);
+        const int tc_err = (f32_t ? hs->pre_err & 8 : 0) | (tc ? hs->tc[0] : 0) | (any_oz ? hs->oz[0] : 0);
         if (tc_err & 8) throw Error{RDM_EBADBSR, "an operand's block pattern is not symmetric"};
         if (tc_err)
             throw Error{tc_err & 1 ? RDM_ETIMEOUT : RDM_ECUDA,

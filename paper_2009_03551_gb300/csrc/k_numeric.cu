@@ -427,36 +427,41 @@ __global__ void __launch_bounds__(64) k_numeric_ff_b32(NumArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-// FP32 products of 32 x 32 blocks with 8 x 4 register tiles.  A 4 x 4 tile
-// (the layout of k_numeric_ff_b32) reads 2 bytes of shared memory per FMA, and a warp's 16-byte read takes four
-// shared-memory cycles whatever it broadcasts, so the operand reads allow
-// about half of the SM's FMA rate (ncu on the 4 x 4 version: FMA pipe 54%,
-// short-scoreboard stalls first).  Here half-warp h of the CTA's four covers
-// the k-half kh = h % 2 (k = 16 kh .. 16 kh + 15 of every pair) and the
-// column half ch = h / 2, lane l of it rows r0 + 4u (u = 0..7) and columns
-// 16 ch + c0 + 4v (v = 0..3), r0 = l / 4, c0 = l % 4: 12 reads of 16 bytes per
-// 128 FMAs (1.5 bytes per FMA) within 128 registers, so that eight CTAs
-// share an SM (44.5 against 41.6 TFLOP/s for the 4 x 4 version; an 8 x 8
-// tile at 222 registers, four CTAs per SM, gained nothing).  A quarter warp reads two A rows (broadcast) and four B rows,
-// in distinct banks.  The two k-halves are added in a fixed order at the end.
+// FP32 products of 32 x 32 blocks, one warp per output block, two FMAs per
+// instruction (fma.rn.f32x2: both halves are IEEE FMAs).  Half-warp kh covers
+// k = 16 kh .. 16 kh + 15 of every pair, lane l of it the 8 x 8 tile of rows
+// 8 (l / 4) .. and columns 8 (l % 4) ..; per k it reads 8 elements of each
+// operand (4 shared-memory reads of 16 bytes for 64 FMAs, 1 byte per FMA).
+// The operands are staged as [k][row] and [k][column], which for a symmetric
+// matrix is the block at the transposed position as it is stored, so that
+// adjacent rows are register pairs as loaded and only the 8 column elements
+// are doubled by moves: 52 issue slots per 64 FMAs, whose pipe takes 64 clocks.
+// A version with 64 threads per block, 8 x 4 tiles and 16-byte reads along k
+// (1.5 bytes per FMA, where a 16-byte warp read takes 4 shared-memory cycles)
+// was bound by those reads: 44.5 TFLOP/s with the FMA pipe at 58%; this one 58.6 TFLOP/s (1,000-atom
+// cluster, 125 -> 94.5 ms of products).  The
+// k-halves' sums and the norm keep the order of that version.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(64, 8) k_numeric_f32_t84(NumArgs a) {
-    __shared__ __align__(16) float sA[2][32 * kF32Ld];
-    __shared__ __align__(16) float sB[2][32 * kF32Ld];
-    __shared__ float sC[32 * 33];
-    __shared__ float red[2];
-    __shared__ int s_w;
-    const int tid = threadIdx.x;
-    const int hw = tid >> 4, l = tid & 15;
-    const int kh = hw & 1, ch = hw >> 1;
-    const int r0 = l >> 2, c0 = 16 * ch + (l & 3);
-    const int k0 = 16 * kh;
+__device__ __forceinline__ void fma2(unsigned long long &d, unsigned long long a, unsigned long long b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ unsigned long long dup2(float x) {
+    unsigned long long d;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(d) : "f"(x));
+    return d;
+}
+
+__global__ void __launch_bounds__(32, 13) k_numeric_f32_x2(NumArgs a) {
+    __shared__ __align__(16) float sm[2][2][1024];         // [buffer][operand][k][row or column]
+    float *sC = &sm[0][0][0];                              // 32 x 33, after the products
+    const int lane = threadIdx.x;
+    const int kh = lane >> 4, l = lane & 15;
+    const int r0 = 8 * (l >> 2), c0 = 8 * (l & 3), k0 = 16 * kh;
     const int nwork = *a.nwork;
     for (;;) {
-        if (threadIdx.x == 0) s_w = atomicAdd(a.work_next, 1);
-        __syncthreads();
-        const int w = s_w;
-        __syncthreads();
+        int w = 0;
+        if (lane == 0) w = atomicAdd(a.work_next, 1);
+        w = __shfl_sync(0xffffffffu, w, 0);
         if (w >= nwork) break;
         const int s = a.work[w];
         const int i = a.slot_row[s];
@@ -466,110 +471,126 @@ __global__ void __launch_bounds__(64, 8) k_numeric_f32_t84(NumArgs a) {
         const int64_t p0 = a.pair_off ? a.pair_off[s] : 0, p1 = a.pair_off ? a.pair_off[s + 1] : 0;
         const int st = a.slot_t[s], sx = a.slot_x[s];
 
-        float acc[8][4];
+        unsigned long long acc[4][8];                      // rows 2u, 2u + 1 of the tile, column v
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
+        for (int u = 0; u < 4; ++u)
 #pragma unroll
-            for (int v = 0; v < 4; ++v) acc[u][v] = 0.f;
-
-        auto issue = [&](int64_t q, int buf) {
-            const float *ga = a.in_f32 + (size_t)a.pair_a[q] * 1024;
-            const float *gb = a.in_f32 + (size_t)a.pair_b[q] * 1024;
+            for (int v = 0; v < 8; ++v) acc[u][v] = 0ull;
+        int na = 0, nb = 0;                                // positions of the next pair to stage
+        auto look = [&](int64_t q) {
+            if (q < p1) {
+                na = max(a.tpos[a.pair_a[q]], 0);     // (-1, a missing transpose, is reported by the host)
+                nb = max(a.tpos[a.pair_b[q]], 0);
+            }
+        };
+        auto issue = [&](int buf) {
+            const float *ga = a.in_f32 + (size_t)na * 1024 + 4 * lane;
+            const float *gb = a.in_f32 + (size_t)nb * 1024 + 4 * lane;
 #pragma unroll
-            for (int c = tid; c < 256; c += 64) {
-                const int row = c >> 3, col4 = (c & 7) * 4;
-                cp_async16(&sA[buf][row * kF32Ld + col4], ga + row * 32 + col4);
-                cp_async16(&sB[buf][row * kF32Ld + col4], gb + row * 32 + col4);
+            for (int c = 0; c < 8; ++c) {
+                cp_async16(&sm[buf][0][128 * c + 4 * lane], ga + 128 * c);
+                cp_async16(&sm[buf][1][128 * c + 4 * lane], gb + 128 * c);
             }
             cp_async_commit();
         };
-        __syncthreads();
-        if (p0 < p1) issue(p0, 0);
+        __syncwarp();
+        look(p0);
+        if (p0 < p1) issue(0);
+        look(p0 + 1);
         for (int64_t q = p0; q < p1; ++q) {
             const int buf = (int)((q - p0) & 1);
             if (q + 1 < p1) {
-                issue(q + 1, buf ^ 1);
+                issue(buf ^ 1);
+                look(q + 2);
                 cp_async_wait1();
             } else {
                 cp_async_wait0();
             }
-            __syncthreads();
-            const float *A_ = sA[buf];
-            const float *B_ = sB[buf];
+            __syncwarp();
+            const float *A_ = &sm[buf][0][k0 * 32 + r0], *B_ = &sm[buf][1][k0 * 32 + c0];
+#pragma unroll 4
+            for (int k = 0; k < 16; ++k) {
+                const ulonglong2 x0 = *reinterpret_cast<const ulonglong2 *>(A_ + 32 * k);
+                const ulonglong2 x1 = *reinterpret_cast<const ulonglong2 *>(A_ + 32 * k + 4);
+                const float4 y0 = *reinterpret_cast<const float4 *>(B_ + 32 * k);
+                const float4 y1 = *reinterpret_cast<const float4 *>(B_ + 32 * k + 4);
+                const unsigned long long x[4] = {x0.x, x0.y, x1.x, x1.y};
+                const float y[8] = {y0.x, y0.y, y0.z, y0.w, y1.x, y1.y, y1.z, y1.w};
 #pragma unroll
-            for (int kk = 0; kk < 16; kk += 4) {
-                float4 av[8], bv[4];
+                for (int v = 0; v < 8; ++v) {
+                    const unsigned long long yy = dup2(y[v]);
 #pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    av[u] = *reinterpret_cast<const float4 *>(&A_[(r0 + 4 * u) * kF32Ld + k0 + kk]);
-#pragma unroll
-                for (int v = 0; v < 4; ++v)
-                    bv[v] = *reinterpret_cast<const float4 *>(&B_[(c0 + 4 * v) * kF32Ld + k0 + kk]);
-#pragma unroll
-                for (int u = 0; u < 8; ++u)
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) {
-                        float t = acc[u][v];
-                        t = fmaf(av[u].x, bv[v].x, t);
-                        t = fmaf(av[u].y, bv[v].y, t);
-                        t = fmaf(av[u].z, bv[v].z, t);
-                        t = fmaf(av[u].w, bv[v].w, t);
-                        acc[u][v] = t;
-                    }
+                    for (int u = 0; u < 4; ++u) fma2(acc[u][v], x[u], yy);
+                }
             }
-            __syncthreads();
+            __syncwarp();
         }
 
-        // the two k-halves' partial blocks into the free operand buffers, then
-        // C = c_lin X + c_sq (P_0 + P_1)
-        float *part = sA[kh];
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) part[(r0 + 4 * u) * kF32Ld + c0 + 4 * v] = acc[u][v];
-        __syncthreads();
-        const double *gx = sx >= 0 ? a.in_val + (size_t)sx * 1024 : nullptr;
+        // P_0 + P_1 (the half-warps hold the same tiles), then C = c_lin X + c_sq P;
+        // half-warp kh finishes columns 4 kh .. 4 kh + 3 of each tile
+        const float *gx = sx >= 0 ? a.in_f32 + (size_t)sx * 1024 : nullptr;
         const bool diag = (st == s);
         const float cl = (float)a.c_lin[sys], cq = (float)a.c_sq[sys];
-        for (int e = tid; e < 1024; e += 64) {
-            const int r = e >> 5, c = e & 31, o = r * kF32Ld + c;
-            float x = cq * (sA[0][o] + sA[1][o]);
-            if (gx) x = fmaf(cl, f64_to_f32(gx[e]), x);
-            sC[r * 33 + c] = x;
-        }
-        __syncthreads();
-        float sym[16];
-        if (diag) {
+        float t[8][4];
 #pragma unroll
-            for (int t = 0; t < 16; ++t) {
-                const int e = tid + 64 * t, r = e >> 5, c = e & 31;
-                sym[t] = 0.5f * (sC[r * 33 + c] + sC[c * 33 + r]);
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int v = 0; v < 8; ++v) {
+                const unsigned long long o = __shfl_xor_sync(0xffffffffu, acc[u][v], 16);
+                const float lo = __uint_as_float((unsigned)acc[u][v]) + __uint_as_float((unsigned)o);
+                const float hi = __uint_as_float((unsigned)(acc[u][v] >> 32)) + __uint_as_float((unsigned)(o >> 32));
+                if ((v >> 2) == kh) {
+                    t[2 * u][v & 3] = lo;
+                    t[2 * u + 1][v & 3] = hi;
+                }
+            }
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            const int c = c0 + 4 * kh;
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (gx) x = *reinterpret_cast<const float4 *>(gx + (r0 + r) * 32 + c);
+            float *o = sC + (r0 + r) * 33 + c;
+            o[0] = gx ? fmaf(cl, x.x, cq * t[r][0]) : cq * t[r][0];
+            o[1] = gx ? fmaf(cl, x.y, cq * t[r][1]) : cq * t[r][1];
+            o[2] = gx ? fmaf(cl, x.z, cq * t[r][2]) : cq * t[r][2];
+            o[3] = gx ? fmaf(cl, x.w, cq * t[r][3]) : cq * t[r][3];
+        }
+        __syncwarp();
+        if (diag) {
+            // (X + X^T) / 2 of the elements on and above the diagonal, mirrored
+            for (int r = 0; r < 32; ++r) {
+                float y = 0.f;
+                if (lane >= r) y = 0.5f * (sC[r * 33 + lane] + sC[lane * 33 + r]);
+                __syncwarp();
+                if (lane >= r) sC[r * 33 + lane] = sC[lane * 33 + r] = y;
+                __syncwarp();
             }
         }
-        __syncthreads();
-        float ss = 0.f;
+        float s0 = 0.f, s1 = 0.f;                          // even and odd rows
 #pragma unroll
-        for (int t = 0; t < 16; ++t) {
-            const int e = tid + 64 * t, r = e >> 5, c = e & 31;
-            if (diag) sC[r * 33 + c] = sym[t];
-            const float x = diag ? sym[t] : sC[r * 33 + c];
-            ss = fmaf(x, x, ss);
+        for (int r = 0; r < 32; r += 2) {
+            const float x = sC[r * 33 + lane], y = sC[(r + 1) * 33 + lane];
+            s0 = fmaf(x, x, s0);
+            s1 = fmaf(y, y, s1);
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-        if ((tid & 31) == 0) red[tid >> 5] = ss;
-        __syncthreads();
-        const float nrm = sqrtf(red[0] + red[1]) * (1.0f + 1e-6f);
+        for (int o = 16; o > 0; o >>= 1) {
+            s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+            s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+        }
+        const float nrm = sqrtf(s0 + s1) * (1.0f + 1e-6f);
         const bool keep = ((double)nrm >= tau) && (nrm > 0.f);
         float4 *o = reinterpret_cast<float4 *>(a.out_val + (size_t)(a.uidx[s] - a.u0) * 1024);
-        for (int e = tid; e < 256; e += 64) {      // layout f32_index: 4 columns of row e % 32
-            const float *x = &sC[(e & 31) * 33 + 4 * (e >> 5)];
-            o[e] = make_float4(x[0], x[1], x[2], x[3]);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {                      // layout f32_index: 4 columns of row `lane`
+            const float *x = &sC[lane * 33 + 4 * c];
+            o[c * 32 + lane] = make_float4(x[0], x[1], x[2], x[3]);
         }
-        if (tid == 0) {
+        if (lane == 0) {
             a.out_nrm[s] = nrm;
             a.keep[s] = (keep ? kKeepBlock : 0) | kBlockF32;
         }
+        __syncwarp();
     }
 }
 
@@ -690,8 +711,9 @@ void launch_numeric_simt(const NumArgs &a, Arith ar, cudaStream_t st) {
     } else if (ar == AR_FP64) {
         dispatch<double>(a, st);
     } else if (a.b == 32 && a.in_f32) {
-        static const int res = resident_blocks(k_numeric_f32_t84, 64);
-        k_numeric_f32_t84<<<std::min(a.max_work, res), 64, 0, st>>>(a);
+        if (!a.tpos) throw Error{-1, "FP32 products of 32 x 32 blocks need the transposed positions"};
+        static const int res = resident_blocks(k_numeric_f32_x2, 32);
+        k_numeric_f32_x2<<<std::min(a.max_work, res), 32, 0, st>>>(a);
         RDM_LAUNCH_CHECK();
     } else {
         dispatch<float>(a, st);

@@ -431,9 +431,35 @@ struct PairParams {
     JobMask fill;    // jobs whose pair lists are filled, per tier (others: only slot_x / slot_t)
 };
 
-// one warp per output slot; only upper-triangle slots (j >= i) do work.
-// slot_t pairs every off-diagonal upper slot with its lower mirror (both
-// ways); a diagonal slot maps to itself
+// slot_x and slot_t of slot s = (i, j), j >= i.  slot_t pairs every
+// off-diagonal upper slot with its lower mirror (both ways); a diagonal slot
+// maps to itself
+__device__ __forceinline__ void slot_maps(const PairParams &P, int64_t s, int i, int j, int p) {
+    const int NB = P.NB;
+    const Job &job = P.jt.job[p];
+    int t = (int)s;
+    if (j > i) {
+        t = find_col(P.out_col, P.out_rp[p * NB + j], P.out_rp[p * NB + j + 1], i);
+        if (t < 0) atomicOr(P.err, 1);
+    }
+    P.slot_t[s] = t;
+    if (t >= 0 && t != s) P.slot_t[t] = (int)s;   // the lower partner points back
+    int x = -1;
+    if (job.xmat >= 0) x = find_col(P.col, P.rp[job.xmat * NB + i], P.rp[job.xmat * NB + i + 1], j);
+    P.slot_x[s] = x;
+}
+
+// without pair lists: one thread per output slot (with a warp each the
+// searches took 75 us for the 300,000 slots of a 2,000-atom cluster, 12 us so)
+__global__ void __launch_bounds__(256) k_slot_maps(PairParams P) {
+    const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (s >= P.nslot) return;
+    const int i = P.slot_row[s], j = P.out_col[s];
+    if (j >= i) slot_maps(P, s, i, j, P.slot_job[s]);
+}
+
+// with pair lists: one warp per output slot; only upper-triangle slots
+// (j >= i) do work
 __global__ void k_pairs(PairParams P) {
     int64_t s = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     int lane = threadIdx.x & 31;
@@ -442,21 +468,10 @@ __global__ void k_pairs(PairParams P) {
     if (j < i) return;
     const int NB = P.NB;
     const Job &job = P.jt.job[p];
-    if (lane == 0) {
-        int t = s;
-        if (j > i) {
-            t = find_col(P.out_col, P.out_rp[p * NB + j], P.out_rp[p * NB + j + 1], i);
-            if (t < 0) atomicOr(P.err, 1);
-        }
-        P.slot_t[s] = t;
-        if (t >= 0 && t != s) P.slot_t[t] = (int)s;   // the lower partner points back
-        int x = -1;
-        if (job.xmat >= 0) x = find_col(P.col, P.rp[job.xmat * NB + i], P.rp[job.xmat * NB + i + 1], j);
-        P.slot_x[s] = x;
-    }
+    if (lane == 0) slot_maps(P, s, i, j, p);
     // a converged system's blocks are copied: the symbolic phase gave them no pairs
     const int sys = P.sys_of_row[i];
-    if (!P.pair_off || !P.active[sys] || !((P.fill.m[P.sys_tier[sys] & (kMaxTiers - 1)] >> p) & 1u)) return;
+    if (!P.active[sys] || !((P.fill.m[P.sys_tier[sys] & (kMaxTiers - 1)] >> p) & 1u)) return;
     int64_t w = P.pair_off[s];
     const int64_t wend = P.pair_off[s + 1];
     for (int t = 0; t < job.nterm; ++t) {
@@ -533,6 +548,11 @@ void launch_pairs(const MatSet &in, const JobTable &jt, const SysDev &sd, const 
     P.pair_off = pair_off; P.nslot = nslot; P.pair_a = pair_a; P.pair_b = pair_b;
     P.slot_x = slot_x; P.slot_t = slot_t; P.err = err;
     P.sys_of_row = sd.sys_of_row.p; P.active = sd.active.p;
+    if (!pair_off) {
+        k_slot_maps<<<(unsigned)((nslot + 255) / 256), 256, 0, st>>>(P);
+        RDM_LAUNCH_CHECK();
+        return;
+    }
     int wpb = 8;
     int64_t grid = (nslot + wpb - 1) / wpb;
     k_pairs<<<(unsigned)grid, wpb * 32, 0, st>>>(P);

@@ -958,6 +958,14 @@ bool tc_block_size_ok(int b) { return b == 16 || b == 32 || b == 64; }
 
 int tc_tile_rows(int b) { return tc_block_size_ok(b) ? 128 / b : 4; }
 
+void find_transposes(const MatSet &in, TcWork &w, cudaStream_t st) {
+    if (in.total == 0) return;
+    w.tpos.ensure(in.total);
+    k_transpose_pos<<<(unsigned)((in.total + 255) / 256), 256, 0, st>>>(in.row_ptr.p, in.col.p, in.nmat * in.NB, in.NB,
+                                                                         in.total, w.tpos.p, w.pre_err.p);
+    RDM_LAUNCH_CHECK();
+}
+
 void prepare_operands(MatSet &in, Arith ar, bool lin, TcWork &w, cudaStream_t st) {
     if (!tc_block_size_ok(in.b)) throw Error{-1, "the tensor-core path handles 16 x 16, 32 x 32 and 64 x 64 blocks"};
     if (ar != AR_BF16X3 && ar != AR_FP16X3) throw Error{-1, "tensor-core arithmetic not available"};
@@ -983,10 +991,7 @@ void prepare_operands(MatSet &in, Arith ar, bool lin, TcWork &w, cudaStream_t st
     // points the K-step lists there), unless the test setting asks for one
     // copy per block
     if (!w.knobs.block_copies) {
-        w.tpos.ensure(in.total);
-        k_transpose_pos<<<(unsigned)((in.total + 255) / 256), 256, 0, st>>>(
-            in.row_ptr.p, in.col.p, nmat * in.NB, in.NB, in.total, w.tpos.p, w.pre_err.p);
-        RDM_LAUNCH_CHECK();
+        find_transposes(in, w, st);
         w.tpos_valid = true;
     }
     switch (in.b) {

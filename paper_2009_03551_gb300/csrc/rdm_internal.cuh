@@ -301,6 +301,7 @@ __host__ __device__ inline int f32_index(int b, int r, int c) { return ((c >> 2)
 struct NumArgs {
     const double *in_val;
     const float *in_f32;       // FP32 copy of in_val (FP32 products), may be null
+    const int *tpos;           // position of every block's transpose (with in_f32 and b = 32)
     const float *in_f32lo;     // in_val - in_f32 rounded to FP32 (double-FP32 products), may be null
     const float *in_nrm;
     const int *pair_a, *pair_b;

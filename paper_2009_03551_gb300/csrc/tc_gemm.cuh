@@ -68,6 +68,10 @@ int tc_tile_rows(int b);
 // kernel divides the scale back out per job.
 void prepare_operands(MatSet &in, Arith ar, bool lin, TcWork &w, cudaStream_t st);
 
+// Positions of the transposed blocks of the set (w.tpos); a pattern that is not
+// symmetric sets error bit 8 of pre_err[0].
+void find_transposes(const MatSet &in, TcWork &w, cudaStream_t st);
+
 // Tile and K-step lists of one multiplication step from the output mask, for
 // the jobs selected by job_mask (per system tier) and the super-row units
 // [unit0, unit1) (unit = job * ceil(NB/TR) + I covers block rows
