@@ -464,6 +464,7 @@ void init_x(rdm_handle *h) {
     const size_t bb = (size_t)b * b;
     MatSet &X = h->X[0];
     h->cur = 0;
+    X.planes_ar = -1;
     X.nmat = 1 + nd;
     X.NB = NB;
     X.b = b;
@@ -651,11 +652,13 @@ Arith fp64_arith(int mode, int b, double tau) {
 // bit t set when some active system is in tier t (the per-system tiers are in
 // h->sd.tier on the device)
 // lin: an active system's c_lin is not 0; copies: some system is not active
-// (its blocks are copied).  The host waits twice, for the size of the mask and
+// (its blocks are copied); next_ar: split arithmetic (Arith) of a step that takes
+// `out` as its input, whose operands the compaction then writes (-1: none).
+// The host waits twice, for the size of the mask and
 // for that of the result (and once more per further group); the device may
 // still be working on the compaction when the call returns (finish_step).
 StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
-                   const Arith (*tab)[kMaxJobs], unsigned tiers_present, bool lin, bool copies) {
+                   const Arith (*tab)[kMaxJobs], unsigned tiers_present, bool lin, bool copies, int next_ar = -1) {
     cudaStream_t st = h->stream;
     const int NB = in.NB, b = in.b, njob = jt.njob;
     const size_t bb = (size_t)b * b;
@@ -719,7 +722,9 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
         if (other.cap > mine.cap) mine.swap(other);
         other.release();
     };
-    take(in.ophi, out.ophi);
+    const bool have_planes = tc && reuse_operands(in, tc_ar, lin, h->tcw);
+    out.planes_ar = -1;
+    if (!have_planes) take(in.ophi, out.ophi);
     take(in.opf32, out.opf32);
     take(in.opf32lo, out.opf32lo);
     // copies the step does not use are kept for the next solve, unless they
@@ -729,7 +734,7 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
     if (!tc && h->tcw.xlin.cap * sizeof(float) > big) h->tcw.xlin.release();
     if (!f32_planes && in.opf32.cap * sizeof(float) > big) in.opf32.release();
     if (!any_c[1] && in.opf32lo.cap * sizeof(float) > big) in.opf32lo.release();
-    if (tc) prepare_operands(in, tc_ar, lin, h->tcw, st);
+    if (tc && !have_planes) prepare_operands(in, tc_ar, lin, h->tcw, st);
     if (!any_oz && h->ozw.slices_a.cap * sizeof(uint16_t) > big) {
         h->ozw.slices_a.release();
         h->ozw.slices_b.release();
@@ -993,6 +998,10 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
         ca.new_col = out.col.p; ca.new_val = out.val.p; ca.new_nrm = out.nrm.p;
         ca.src = h->cpsrc.ensure(std::max(kept_end - kept, 1));
         ca.d0 = kept;
+        ca.NB = NB;
+        ca.slot_job = h->slot_job.p;
+        if (next_ar >= 0 && ngroup == 1 && tc_block_size_ok(b) && !h->tcw.knobs.block_copies)
+            operands_from_compaction(ca, out, in.ophi, kept_end, njob, (Arith)next_ar, h->tcw, st);
         launch_compact_copy(ca, kept_end, st);
         kept = kept_end;
         RDM_CUDA_TRY(cudaEventRecord(h->ev[3], st));
@@ -1068,6 +1077,7 @@ void concat(rdm_handle *h, std::initializer_list<SetRange> parts, MatSet &out) {
     out.nmat = nmat;
     out.NB = NB;
     out.b = b;
+    out.planes_ar = -1;
     out.nnzb.assign(nmat, 0);
     int m = 0;
     for (size_t k = 0; k < parts.size(); ++k) {
@@ -1497,7 +1507,8 @@ int run_solve(rdm_handle *h, rdm_info *info_out) {
         upload_step(h, c_lin, c_sq, t0, t1, act, tier_of);
         RDM_CUDA_TRY(cudaEventRecord(ev0, st));
         MatSet &Xn = h->X[1 - h->cur];
-        StepStats sst = multiply(h, Xc, Xn, jt, tab, tiers_present, lin, copies);
+        StepStats sst = multiply(h, Xc, Xn, jt, tab, tiers_present, lin, copies,
+                                 P.mode == RDM_MODE_MIXED_BF16 ? AR_BF16X3 : mixed ? AR_FP16X3 : -1);
         RDM_CUDA_TRY(cudaEventRecord(ev1, st));
         q = stats(h, Xn);                     // waits for the step
         finish_step(h, sst);

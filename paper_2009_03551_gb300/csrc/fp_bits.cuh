@@ -45,5 +45,16 @@ __device__ __forceinline__ float f64_to_f32(double x) {
     return __uint_as_float(t | (hi & 0x80000000u));
 }
 
+// 32 bytes of global memory (32-byte aligned)
+__device__ __forceinline__ void ld_f64x4(const double *p, double (&v)[4]) {
+    asm volatile("ld.global.v4.f64 {%0,%1,%2,%3}, [%4];"
+                 : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3])
+                 : "l"(p)
+                 : "memory");
+}
+__device__ __forceinline__ void st_f64x4(double *p, const double (&v)[4]) {
+    asm volatile("st.global.v4.f64 [%0], {%1,%2,%3,%4};" ::"l"(p), "d"(v[0]), "d"(v[1]), "d"(v[2]), "d"(v[3]) : "memory");
+}
+
 }  // namespace
 }  // namespace rdm

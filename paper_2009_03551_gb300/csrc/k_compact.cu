@@ -6,6 +6,7 @@
 // blocks for the numeric phase.
 #include "fp_bits.cuh"
 #include "rdm_internal.cuh"
+#include "tc_split.cuh"
 
 #include <algorithm>
 
@@ -62,6 +63,7 @@ __global__ void k_compact_index(CompactArgs c) {
     const int r = c.r0 + rr;
     const int rend = c.out_rp[r + 1];
     int dst = c.new_rp[r];
+    float mx = 0.f;
     for (int base = c.out_rp[r]; base < rend; base += 32) {
         const int p = base + lane;
         bool k = false, up = false;
@@ -75,70 +77,160 @@ __global__ void k_compact_index(CompactArgs c) {
         if (k) {
             const int d = dst + __popc(m & ((1u << lane) - 1u));
             c.new_col[d] = c.out_col[p];
-            c.new_nrm[d] = c.out_nrm[src];
+            const float nrm = c.out_nrm[src];
+            c.new_nrm[d] = nrm;
+            mx = fmaxf(mx, nrm);
             c.src[d - c.d0] = p;
-            if (up) c.dest[p] = d;
+            c.dest[p] = d;
         }
         dst += __popc(m);
     }
+    if (c.mx) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        if (lane == 0 && mx > 0.f) atomicMax(&c.mx[r / c.NB], __float_as_uint(mx));
+    }
 }
 
-// one CTA per kept block (grid-stride): upper blocks are copied, lower ones
-// are the transpose of their upper partner, which is in this group's buffer or
-// already compacted.  FP32 blocks of the buffer are widened: 12 bytes move per
-// element instead of 16, and either orientation reads its source in whole
-// sectors, a warp at a time, so only FP64 sources are transposed through
-// shared memory (b x (b+1) doubles).
+// Values of the kept blocks, block sizes that the tensor cores do not take: one
+// CTA per block (grid-stride), upper blocks are copied, lower ones transposed
+// through shared memory (b x (b+1) doubles) from their upper partner, which is
+// in this group's buffer or already compacted.
 __global__ void __launch_bounds__(128) k_compact_vals(CompactArgs c, int d1) {
     extern __shared__ double tile[];
     const int b = c.b, bb = b * b, ld = b + 1;
     for (int d = c.d0 + blockIdx.x; d < d1; d += gridDim.x) {
         const int p = c.src[d - c.d0];
         double *out = c.new_val + (size_t)d * bb;
-        const bool up = c.out_col[p] >= c.slot_row[p];
-        const int t = up ? p : c.slot_t[p];
-        const int ut = c.uidx[t];
-        const bool here = ut >= c.u0;
-        const double *s = here ? c.out_val + (size_t)(ut - c.u0) * bb : c.new_val + (size_t)c.dest[t] * bb;
-        if (here && (c.keep[t] & kBlockF32)) {
-            const float4 *f = reinterpret_cast<const float4 *>(s);
-            const int q4 = b >> 2;
-            if (up) {
-                // a thread widens 4 columns of a row: the threads of a row are neighbours
-                for (int e = threadIdx.x; e < bb / 4; e += blockDim.x) {
-                    const int r = e / q4, c4 = e % q4;
-                    const float4 v = f[c4 * b + r];
-                    double2 *o = reinterpret_cast<double2 *>(out + r * b + 4 * c4);
-                    o[0] = make_double2(f32_to_f64(v.x), f32_to_f64(v.y));
-                    o[1] = make_double2(f32_to_f64(v.z), f32_to_f64(v.w));
-                }
-            } else {
-                // 4 source columns of source row k are column k of 4 output rows
-                for (int e = threadIdx.x; e < bb / 4; e += blockDim.x) {
-                    const int k = e % b, c4 = e / b;
-                    const float4 v = f[c4 * b + k];
-                    double *o = out + 4 * c4 * b + k;
-                    o[0] = f32_to_f64(v.x);
-                    o[b] = f32_to_f64(v.y);
-                    o[2 * b] = f32_to_f64(v.z);
-                    o[3 * b] = f32_to_f64(v.w);
-                }
-            }
-        } else if (up) {
-            if ((bb & 1) == 0) {
-                const double2 *s2 = reinterpret_cast<const double2 *>(s);
-                double2 *o2 = reinterpret_cast<double2 *>(out);
-                for (int e = threadIdx.x; e < bb / 2; e += blockDim.x) o2[e] = s2[e];
-            } else {
-                for (int e = threadIdx.x; e < bb; e += blockDim.x) out[e] = s[e];
-            }
+        if (c.out_col[p] >= c.slot_row[p]) {
+            const double *s = c.out_val + (size_t)(c.uidx[p] - c.u0) * bb;
+            for (int e = threadIdx.x; e < bb; e += blockDim.x) out[e] = s[e];
         } else {
+            const int t = c.slot_t[p];
+            const int ut = c.uidx[t];
+            const double *s = ut >= c.u0 ? c.out_val + (size_t)(ut - c.u0) * bb
+                                         : c.new_val + (size_t)c.dest[t] * bb;
             for (int e = threadIdx.x; e < bb; e += blockDim.x) tile[(e / b) * ld + (e % b)] = s[e];
             __syncthreads();
             for (int e = threadIdx.x; e < bb; e += blockDim.x) out[e] = tile[(e % b) * ld + (e / b)];
             __syncthreads();
         }
     }
+}
+
+// The same for B = 16, 32, 64, a warp per block, without shared memory: a lane
+// takes 8 neighbouring columns of a row of an upper block, and for a lower
+// block 8 rows x 4 columns of its partner, which are 8 neighbouring columns of
+// 4 rows of the transpose.  FP32 sources (kBlockF32) are widened.  PL = 1 (fp16)
+// or 2 (bf16): the same pass writes the next step's operand planes, at the
+// transposed block's position, and the FP32 copy for its linear terms, instead
+// of a second one that reads the FP64 values back.  Bound by memory: 18 bytes
+// per element of the result where the two passes moved 26 (2,000-atom cluster,
+// 300,000 blocks of 32: 292 + 271 us per step in two passes, 537 in one;
+// 150 atoms, 5,500 blocks: 16.5 + 13.5 us, 21 in one, and four launches less).
+template <int B, int PL>
+__global__ void __launch_bounds__(128) k_compact_blocks(CompactArgs c, int d1) {
+    constexpr int BB = B * B, C8 = B / 8;
+    const int lane = threadIdx.x & 31;
+    if (PL && blockIdx.x == 0 && (int)threadIdx.x < c.njob) c.scale[threadIdx.x] = matrix_scale(c.mx[threadIdx.x], PL == 1);
+    for (int d = c.d0 + blockIdx.x * 4 + (threadIdx.x >> 5); d < d1; d += gridDim.x * 4) {
+        const int p = c.src[d - c.d0];
+        double *out = c.new_val + (size_t)d * BB;
+        const bool up = c.out_col[p] >= c.slot_row[p];
+        const int partner = c.slot_t[p], t = up ? p : partner;
+        const int ut = c.uidx[t];
+        const bool here = ut >= c.u0;
+        const double *s = here ? c.out_val + (size_t)(ut - c.u0) * BB : c.new_val + (size_t)c.dest[t] * BB;
+        const float4 *f = here && (c.keep[t] & kBlockF32) ? reinterpret_cast<const float4 *>(s) : nullptr;
+        uint16_t *planes = nullptr;
+        float sc = 1.f;
+        if constexpr (PL != 0) {
+            const int at = c.dest[partner];
+            if (lane == 0) c.tpos[d] = at;
+            planes = c.planes + (size_t)at * (2 * BB);
+            sc = matrix_scale(c.mx[c.slot_job[p]], PL == 1);
+        }
+        if (up) {
+            for (int k = lane; k < B * C8; k += 32) {
+                const int r = k / C8, c0 = 8 * (k % C8);
+                double v[2][4];
+                float x[8];
+                if (f) {
+                    const float4 a0 = f[(c0 >> 2) * B + r], a1 = f[((c0 >> 2) + 1) * B + r];
+                    x[0] = a0.x; x[1] = a0.y; x[2] = a0.z; x[3] = a0.w;
+                    x[4] = a1.x; x[5] = a1.y; x[6] = a1.z; x[7] = a1.w;
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) v[u >> 2][u & 3] = f32_to_f64(x[u]);
+                } else {
+                    ld_f64x4(s + r * B + c0, v[0]);
+                    ld_f64x4(s + r * B + c0 + 4, v[1]);
+                    if constexpr (PL != 0) {
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) x[u] = f64_to_f32(v[u >> 2][u & 3]);
+                    }
+                }
+                st_f64x4(out + r * B + c0, v[0]);
+                st_f64x4(out + r * B + c0 + 4, v[1]);
+                if constexpr (PL != 0) {
+                    store_planes<PL == 2, B>(planes, r, c0, x, sc);
+                    if (c.xlin) {
+                        float *xl = c.xlin + (size_t)d * BB;
+                        *reinterpret_cast<float4 *>(xl + f32_index(B, r, c0)) = make_float4(x[0], x[1], x[2], x[3]);
+                        *reinterpret_cast<float4 *>(xl + f32_index(B, r, c0 + 4)) = make_float4(x[4], x[5], x[6], x[7]);
+                    }
+                }
+            }
+        } else {
+            for (int k = lane; k < (B / 4) * C8; k += 32) {
+                const int c4 = k / C8, r0 = 8 * (k % C8);       // source columns 4 c4 .., rows r0 ..
+                if (f) {
+                    float4 a[8];
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) a[q] = f[c4 * B + r0 + q];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        float x[8];
+                        double v[2][4];
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) {
+                            x[q] = u == 0 ? a[q].x : u == 1 ? a[q].y : u == 2 ? a[q].z : a[q].w;
+                            v[q >> 2][q & 3] = f32_to_f64(x[q]);
+                        }
+                        st_f64x4(out + (4 * c4 + u) * B + r0, v[0]);
+                        st_f64x4(out + (4 * c4 + u) * B + r0 + 4, v[1]);
+                        if constexpr (PL != 0) store_planes<PL == 2, B>(planes, 4 * c4 + u, r0, x, sc);
+                    }
+                } else {
+                    double a[8][4];
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) ld_f64x4(s + (r0 + q) * B + 4 * c4, a[q]);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        double v[2][4];
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) v[q >> 2][q & 3] = a[q][u];
+                        st_f64x4(out + (4 * c4 + u) * B + r0, v[0]);
+                        st_f64x4(out + (4 * c4 + u) * B + r0 + 4, v[1]);
+                        if constexpr (PL != 0) {
+                            float x[8];
+#pragma unroll
+                            for (int q = 0; q < 8; ++q) x[q] = f64_to_f32(a[q][u]);
+                            store_planes<PL == 2, B>(planes, 4 * c4 + u, r0, x, sc);
+                        }
+                    }
+                }
+            }
+        }
+    }
+}
+
+template <int B>
+void launch_blocks(const CompactArgs &c, int d1, cudaStream_t st) {
+    const int grid = (int)std::min<int64_t>(((int64_t)d1 - c.d0 + 3) / 4, 152 * 16);
+    if (!c.planes) k_compact_blocks<B, 0><<<grid, 128, 0, st>>>(c, d1);
+    else if (c.bf16) k_compact_blocks<B, 2><<<grid, 128, 0, st>>>(c, d1);
+    else k_compact_blocks<B, 1><<<grid, 128, 0, st>>>(c, d1);
+    RDM_LAUNCH_CHECK();
 }
 
 }  // namespace
@@ -166,8 +258,13 @@ void launch_compact_copy(const CompactArgs &c, int d1, cudaStream_t st) {
     k_compact_index<<<(c.nrows + wpb - 1) / wpb, wpb * 32, 0, st>>>(c);
     RDM_LAUNCH_CHECK();
     if (d1 <= c.d0) return;
+    switch (c.b) {
+        case 16: return launch_blocks<16>(c, d1, st);
+        case 32: return launch_blocks<32>(c, d1, st);
+        case 64: return launch_blocks<64>(c, d1, st);
+        default: break;
+    }
     const size_t smem = (size_t)c.b * (c.b + 1) * sizeof(double);
-    func_smem_once((const void *)k_compact_vals, 64 * 65 * (int)sizeof(double));
     const int grid = (int)std::min<int64_t>((int64_t)d1 - c.d0, 152 * 16);
     k_compact_vals<<<grid, 128, smem, st>>>(c, d1);
     RDM_LAUNCH_CHECK();

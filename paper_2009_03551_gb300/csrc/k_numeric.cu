@@ -52,9 +52,7 @@ __device__ __forceinline__ T operand(double x) {
 template <int B>
 __device__ __forceinline__ void load_row(const double *p, double (&v)[B]) {
     if constexpr (B == 4) {
-        asm volatile("ld.global.v4.f64 {%0,%1,%2,%3}, [%4];"
-                     : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3])
-                     : "l"(p));
+        ld_f64x4(p, v);
     } else if constexpr (B == 2) {
         const double2 x = *reinterpret_cast<const double2 *>(p);
         v[0] = x.x;

@@ -71,15 +71,13 @@
 // blocks of the next tile's linear terms are prefetched into L2 two segments
 // before this tile ends.  Every wait is bounded: on timeout the kernel raises
 // an error flag, drains what it issued and frees its tensor memory.
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
-
 #include <algorithm>
 
 #include "fp_bits.cuh"
 #include "tc_gemm.cuh"
 #include "tc_plan.cuh"
 #include "tc_ptx.cuh"
+#include "tc_split.cuh"
 
 namespace rdm {
 namespace {
@@ -136,18 +134,9 @@ __device__ __noinline__ void hold_until_timeout(volatile int *abort_flag, long l
 }
 
 // ---------------------------------------------------------------------------
-// operand planes: hi/lo split in the K-major core-matrix layout
+// operand planes: hi/lo split in the K-major core-matrix layout, from the FP64
+// values (a solve's first step; afterwards the compaction makes them)
 // ---------------------------------------------------------------------------
-template <int B>
-__device__ __forceinline__ int pair_offset(int r, int c, int plane) {
-    // element (r, c) of plane `plane` (0 hi, 1 lo) of a B x B block: the two
-    // planes' 8-row groups alternate (8 B elements each), so that one copy
-    // brings both and both are K-major core-matrix operands with a 32 B-byte
-    // stride between 8-row groups; inside a group, core matrix (c/8) at 64
-    // elements
-    return (r >> 3) * (16 * B) + plane * (8 * B) + ((c >> 3) << 6) + ((r & 7) << 3) + (c & 7);
-}
-
 // Largest block norm of every matrix of the set (matrix m: blocks
 // [rp[m NB], rp[(m + 1) NB])): each CTA takes a contiguous chunk of blocks and
 // folds the part of every matrix it overlaps into mx[m] (norms are
@@ -176,21 +165,6 @@ __global__ void k_matrix_max(const float *__restrict__ nrm, const int *__restric
     }
 }
 
-// operand scale of a matrix with largest block norm mx: 2^floor(log2(2^14 / mx))
-// for fp16 (the largest element then sits below 2^14, far from fp16 overflow,
-// and values down to ~1e-9 of it stay normal); 1 for bf16, whose exponent
-// range is FP32's
-__device__ __forceinline__ float matrix_scale(unsigned mxbits, bool fp16) {
-    const float mx = __uint_as_float(mxbits);
-    float s = 1.f;
-    if (fp16 && mx > 0.f) {
-        int e = (int)floorf(log2f(16384.f / mx));
-        e = max(-60, min(60, e));
-        s = ldexpf(1.f, e);
-    }
-    return s;
-}
-
 // one thread per 8 consecutive elements of a block row (one core-matrix row):
 // 64 bytes of FP64 in, 16 bytes of hi and 16 bytes of lo out
 // and, with xlin, the FP32 values of the upper blocks for the linear term, in
@@ -212,7 +186,6 @@ __global__ void k_split_planes(const double *__restrict__ val, int64_t nblk, uin
     while (m + 1 < nmat && p >= rp[(size_t)(m + 1) * NB]) ++m;
     const float sc = matrix_scale(mx[m], !BF16);
     const double2 *v2 = reinterpret_cast<const double2 *>(val + p * kPE + rc0);
-    uint16_t h[8], l[8];
     double2 x2[4];
     float xf[8];
 #pragma unroll
@@ -222,29 +195,6 @@ __global__ void k_split_planes(const double *__restrict__ val, int64_t nblk, uin
         xf[2 * k] = f64_to_f32(x2[k].x);
         xf[2 * k + 1] = f64_to_f32(x2[k].y);
     }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const float x = xf[2 * k + u] * sc;
-            if (BF16) {
-                const __nv_bfloat16 bh = __float2bfloat16_rn(x);
-                const __nv_bfloat16 bl = __float2bfloat16_rn(x - __bfloat162float(bh));
-                h[2 * k + u] = __bfloat16_as_ushort(bh);
-                l[2 * k + u] = __bfloat16_as_ushort(bl);
-            } else {
-                const __half hh = __float2half_rn(x);
-                const __half hl = __float2half_rn(x - __half2float(hh));
-                h[2 * k + u] = __half_as_ushort(hh);
-                l[2 * k + u] = __half_as_ushort(hl);
-            }
-        }
-    }
-    uint4 hv, lv;
-    hv.x = h[0] | ((uint32_t)h[1] << 16); hv.y = h[2] | ((uint32_t)h[3] << 16);
-    hv.z = h[4] | ((uint32_t)h[5] << 16); hv.w = h[6] | ((uint32_t)h[7] << 16);
-    lv.x = l[0] | ((uint32_t)l[1] << 16); lv.y = l[2] | ((uint32_t)l[3] << 16);
-    lv.z = l[4] | ((uint32_t)l[5] << 16); lv.w = l[6] | ((uint32_t)l[7] << 16);
     // columns c0..c0+7 of row r are 8 consecutive elements of one core matrix;
     // the block's planes go to the position of its transpose (tpos), or to
     // its own position without one
@@ -255,9 +205,7 @@ __global__ void k_split_planes(const double *__restrict__ val, int64_t nblk, uin
         *reinterpret_cast<float4 *>(x + f32_index(B, r, c0)) = make_float4(xf[0], xf[1], xf[2], xf[3]);
         *reinterpret_cast<float4 *>(x + f32_index(B, r, c0 + 4)) = make_float4(xf[4], xf[5], xf[6], xf[7]);
     }
-    uint16_t *o = hi + at * (2 * kPE);
-    *reinterpret_cast<uint4 *>(o + pair_offset<B>(r, c0, 0)) = hv;
-    *reinterpret_cast<uint4 *>(o + pair_offset<B>(r, c0, 1)) = lv;
+    store_planes<BF16, B>(hi + at * (2 * kPE), r, c0, xf, sc);
 }
 
 // Position of the transposed block: for block e = (i, k) of matrix m of the
@@ -958,7 +906,55 @@ bool tc_block_size_ok(int b) { return b == 16 || b == 32 || b == 64; }
 
 int tc_tile_rows(int b) { return tc_block_size_ok(b) ? 128 / b : 4; }
 
+namespace {
+// room for an FP32 copy of n elements, if that is at most a quarter of the free memory
+bool xlin_room(size_t n, TcWork &w) {
+    if (w.xlin.cap >= n) return true;
+    size_t fr = 0, tot = 0;
+    RDM_CUDA_TRY(cudaMemGetInfo(&fr, &tot));
+    if (n * sizeof(float) > (fr + w.xlin.cap * sizeof(float)) / 4) return false;
+    w.xlin.ensure(n);
+    return true;
+}
+}  // namespace
+
+bool reuse_operands(const MatSet &in, Arith ar, bool lin, TcWork &w) {
+    if (in.planes_ar != ar || in.planes_gen != w.gen || w.knobs.block_copies) return false;
+    w.lin = lin && w.xlin_valid;
+    w.tpos_valid = true;
+    return true;
+}
+
+void operands_from_compaction(CompactArgs &c, MatSet &out, DevBuf<uint16_t> &planes, int64_t kept, int njob, Arith ar,
+                              TcWork &w, cudaStream_t st) {
+    const size_t n = (size_t)std::max<int64_t>(kept, 1) * out.b * out.b;
+    if (planes.cap < 2 * n) {
+        // the step may be the last one: no larger buffer for operands that may not be used when memory is short
+        size_t fr = 0, tot = 0;
+        RDM_CUDA_TRY(cudaMemGetInfo(&fr, &tot));
+        if (2 * n * sizeof(uint16_t) > (fr + planes.cap * sizeof(uint16_t)) / 4) return;
+    }
+    out.ophi.release();
+    out.ophi.swap(planes);
+    out.ophi.ensure(2 * n);
+    w.tpos.ensure(std::max<int64_t>(kept, 1));
+    w.scale.ensure(njob);
+    w.pre_err.ensure(1 + njob);
+    RDM_CUDA_TRY(cudaMemsetAsync(w.pre_err.p, 0, (1 + njob) * sizeof(int), st));
+    w.xlin_valid = xlin_room(n, w);
+    c.planes = out.ophi.p;
+    c.tpos = w.tpos.p;
+    c.mx = (unsigned *)w.pre_err.p + 1;
+    c.scale = w.scale.p;
+    c.xlin = w.xlin_valid ? w.xlin.p : nullptr;
+    c.bf16 = ar == AR_BF16X3;
+    c.njob = njob;
+    out.planes_ar = ar;
+    out.planes_gen = ++w.gen;
+}
+
 void find_transposes(const MatSet &in, TcWork &w, cudaStream_t st) {
+    ++w.gen;
     if (in.total == 0) return;
     w.tpos.ensure(in.total);
     k_transpose_pos<<<(unsigned)((in.total + 255) / 256), 256, 0, st>>>(in.row_ptr.p, in.col.p, in.nmat * in.NB, in.NB,
@@ -970,18 +966,15 @@ void prepare_operands(MatSet &in, Arith ar, bool lin, TcWork &w, cudaStream_t st
     if (!tc_block_size_ok(in.b)) throw Error{-1, "the tensor-core path handles 16 x 16, 32 x 32 and 64 x 64 blocks"};
     if (ar != AR_BF16X3 && ar != AR_FP16X3) throw Error{-1, "tensor-core arithmetic not available"};
     w.lin = lin;
+    ++w.gen;
+    in.planes_ar = -1;
     const int nmat = in.nmat;
     w.scale.ensure(std::max(nmat, 1));
     w.pre_err.ensure(1 + std::max(nmat, 1));
     RDM_CUDA_TRY(cudaMemsetAsync(w.pre_err.p, 0, (1 + nmat) * sizeof(int), st));
     const int64_t n = in.total * (int64_t)in.b * in.b;
     in.ophi.ensure(std::max<int64_t>(2 * n, 1));   // hi and lo, interleaved per block
-    if (w.lin && w.xlin.cap < (size_t)n) {
-        size_t fr = 0, tot = 0;
-        RDM_CUDA_TRY(cudaMemGetInfo(&fr, &tot));
-        if ((size_t)n * sizeof(float) > (fr + w.xlin.cap * sizeof(float)) / 4) w.lin = false;
-        else w.xlin.ensure((size_t)n);
-    }
+    w.lin = w.lin && xlin_room((size_t)n, w);
     w.tpos_valid = false;
     if (n == 0) return;
     const int mgrid = (int)std::min<int64_t>(4 * 152, (in.total + 255) / 256);

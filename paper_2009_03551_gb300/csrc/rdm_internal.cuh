@@ -168,7 +168,13 @@ struct MatSet {
     DevBuf<float> opf32lo;    // lo word (x - hi) for the double-FP32 products
     std::vector<int64_t> nnzb;   // host copy, per matrix
     int64_t total = 0;
+    // arithmetic (Arith) whose operand planes ophi holds for these values, with
+    // the transposed positions, scales and FP32 copy in TcWork as of
+    // TcWork::gen == planes_gen; -1: none
+    int planes_ar = -1;
+    uint64_t planes_gen = 0;
     void release() {
+        planes_ar = -1;
         row_ptr.release(); col.release(); val.release(); nrm.release();
         ophi.release(); opf32.release(); opf32lo.release();
         nnzb.clear(); total = 0;
@@ -364,6 +370,15 @@ struct CompactArgs {
     float *new_nrm;
     int r0, nrows, b;
     int d0;                 // first output block of the group
+    // the next step's operands (null: not made): planes at the transposed
+    // positions, those positions, operand scales from the largest block norms
+    // (bit patterns, zeroed), FP32 copy for the linear terms (may be null)
+    uint16_t *planes;
+    int *tpos;
+    unsigned *mx;
+    float *scale, *xlin;
+    int bf16, njob, NB;
+    const int *slot_job;
 };
 void launch_compact_count(const CompactArgs &c, int *cnt, cudaStream_t st);
 // output blocks [d0, d1) of the group

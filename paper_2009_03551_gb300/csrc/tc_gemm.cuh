@@ -36,6 +36,8 @@ struct TcWork {
     DevBuf<int> pre_err;
     DevBuf<float> xlin;         // FP32 values of the input set's upper blocks (layout f32_index)
     bool lin = false;           // xlin is filled for this step
+    uint64_t gen = 0;           // counts the rewrites of tpos, scale and xlin
+    bool xlin_valid = false;    // xlin was written with the planes
     bool tpos_valid = false;    // the planes sit at tpos and the K-step lists point there
 };
 
@@ -67,6 +69,15 @@ int tc_tile_rows(int b);
 // norm) so that its values sit in the normal range of fp16; the product
 // kernel divides the scale back out per job.
 void prepare_operands(MatSet &in, Arith ar, bool lin, TcWork &w, cudaStream_t st);
+
+// The operands of `in` as the compaction left them (MatSet::planes_ar), if they
+// are those of arithmetic `ar`; false: prepare_operands has to make them.
+bool reuse_operands(const MatSet &in, Arith ar, bool lin, TcWork &w);
+// Room for the operands of `out` (kept blocks, njob matrices) and their
+// pointers in `c`, for the compaction to write; `planes`: the buffer of the input
+// set's operands, which the step no longer reads.
+void operands_from_compaction(CompactArgs &c, MatSet &out, DevBuf<uint16_t> &planes, int64_t kept, int njob, Arith ar,
+                              TcWork &w, cudaStream_t st);
 
 // Positions of the transposed blocks of the set (w.tpos); a pattern that is not
 // symmetric sets error bit 8 of pre_err[0].

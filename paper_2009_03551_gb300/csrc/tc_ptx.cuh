@@ -112,16 +112,6 @@ __device__ __forceinline__ void tmem_wait_ld(float (&v)[4][8]) {
                    "+f"(v[2][0]), "+f"(v[2][1]), "+f"(v[2][2]), "+f"(v[2][3]), "+f"(v[2][4]), "+f"(v[2][5]), "+f"(v[2][6]), "+f"(v[2][7]),
                    "+f"(v[3][0]), "+f"(v[3][1]), "+f"(v[3][2]), "+f"(v[3][3]), "+f"(v[3][4]), "+f"(v[3][5]), "+f"(v[3][6]), "+f"(v[3][7]));
 }
-// 32 bytes of global memory (32-byte aligned)
-__device__ __forceinline__ void ld_f64x4(const double *p, double (&v)[4]) {
-    asm volatile("ld.global.v4.f64 {%0,%1,%2,%3}, [%4];"
-                 : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3])
-                 : "l"(p)
-                 : "memory");
-}
-__device__ __forceinline__ void st_f64x4(double *p, const double (&v)[4]) {
-    asm volatile("st.global.v4.f64 [%0], {%1,%2,%3,%4};" ::"l"(p), "d"(v[0]), "d"(v[1]), "d"(v[2]), "d"(v[3]) : "memory");
-}
 
 }  // namespace
 }  // namespace rdm
