@@ -116,6 +116,7 @@ enum {
     kCtrClass = 6,       // 5 x 64 bits: pairs per kernel class
     kCtrWork = 16,       // work items of the three CUDA-core classes (zeroed for every group, with the next)
     kCtrNext = 20,       // next item to hand out, per class
+    kCtrLook = 23,       // a wait of the compaction ran out
     kCtrInts = 24
 };
 struct HostStep {
@@ -168,7 +169,8 @@ struct rdm_handle {
     DevBuf<int64_t> row_cnt;
     DevBuf<int> out_rp, slot_row, slot_job, slot_npair, slot_x, slot_t, work, work2, work3;
     DevBuf<int64_t> pair_off, scan_tmp64;
-    DevBuf<int> scan_tmp32, pair_a, pair_b, cnt_rows;
+    DevBuf<int> pair_a, pair_b;
+    DevBuf<unsigned long long> look;                  // prefix sums of the compaction
     DevBuf<int> uidx, urp, dest, cpsrc;               // upper-slot ranks, compaction maps
     DevBuf<double> out_val, row_part, sys_q;
     DevBuf<float> out_nrm;
@@ -759,7 +761,6 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
     h->row_off.ensure(nrows);
     h->out_rp.ensure(nrows + 1);
     h->urp.ensure(nrows + 1);
-    h->scan_tmp32.ensure(scan_tmp_elems(nrows + 1));
     h->scan_tmp64.ensure(scan_tmp_elems(nrows + 1));
     h->counters.ensure(kCtrInts);
     HostStep *hs = h->step_host.ensure(1);
@@ -883,8 +884,15 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
     h->out_nrm.ensure(std::max<int64_t>(nslot, 1));
     h->keep.ensure(std::max<int64_t>(nslot, 1));
     h->dest.ensure(std::max<int64_t>(nslot, 1));
-    h->cnt_rows.ensure(nrows + 1);
+    h->look.ensure(compact_look_words(nrows));
+    // the pattern of the output is written before its size is known, into room
+    // for the whole mask (12 bytes per block, against b x b values for a kept one)
     out.row_ptr.ensure(nrows + 1);
+    out.col.ensure(ns1);
+    out.nrm.ensure(ns1);
+    int64_t gslots = 1;
+    for (int g = 0; g < ngroup; ++g) gslots = std::max(gslots, gslot(gunit[g + 1]) - gslot(gunit[g]));
+    h->cpsrc.ensure(gslots);
     int kept = 0;
     const int ev_simt[kSimt] = {5, 6, 4};   // events after each CUDA-core class
     for (int g = 0; g < ngroup; ++g) {
@@ -952,8 +960,9 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
             ca.out_rp = h->out_rp.p; ca.out_col = mcol; ca.slot_row = h->slot_row.p; ca.slot_t = h->slot_t.p;
             ca.uidx = h->uidx.p; ca.out_val = h->out_val.p; ca.out_nrm = h->out_nrm.p; ca.keep = h->keep.p;
             ca.u0 = u0; ca.dest = h->dest.p; ca.new_rp = out.row_ptr.p; ca.r0 = r0; ca.nrows = nr; ca.b = b;
-            launch_compact_count(ca, h->cnt_rows.p, st);
-            scan_exclusive_i32(h->cnt_rows.p, out.row_ptr.p + r0, nr, h->scan_tmp32.p, st, kept);
+            ca.new_col = out.col.p; ca.new_nrm = out.nrm.p; ca.src = h->cpsrc.p; ca.d0 = kept; ca.NB = NB;
+            ca.look_err = h->counters.p + kCtrLook;
+            launch_compact_rows(ca, h->look.p, st);
             d2h(&hs->kept, out.row_ptr.p + r0 + nr, 1, st);
             d2h(hs->ctr, h->counters.p, kCtrInts, st);
             if (tc) d2h(hs->tc, h->tcw.counters.p, 8, st);
@@ -963,6 +972,7 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
                 RDM_CUDA_TRY(cudaMemcpy2DAsync(hs->rp, sizeof(int), out.row_ptr.p, (size_t)NB * sizeof(int), sizeof(int),
                                                njob + 1, cudaMemcpyDeviceToHost, st));
             sync(h);
+            if (hs->ctr[kCtrLook]) throw Error{RDM_ETIMEOUT, "compaction: a wait for other blocks of the kernel ran out"};
             if (hs->ctr[kCtrErr])
                 throw Error{RDM_ECUDA, "internal error: pair lists inconsistent with the mask (code " +
                                            std::to_string(hs->ctr[kCtrErr]) + ")"};
@@ -987,21 +997,14 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
         if (g == 0) {
             // the output set's old contents are dead; reserve about the input's size
             const int64_t want = ngroup > 1 ? std::max<int64_t>(kept_end, in.total) : kept_end;
-            out.col.ensure(std::max<int64_t>(want, 1));
             out.val.ensure((size_t)std::max<int64_t>(want, 1) * bb);
-            out.nrm.ensure(std::max<int64_t>(want, 1));
         } else {
-            out.col.grow_keep(std::max(kept_end, 1), kept, st);
             out.val.grow_keep((size_t)std::max(kept_end, 1) * bb, (size_t)kept * bb, st);
-            out.nrm.grow_keep(std::max(kept_end, 1), kept, st);
         }
-        ca.new_col = out.col.p; ca.new_val = out.val.p; ca.new_nrm = out.nrm.p;
-        ca.src = h->cpsrc.ensure(std::max(kept_end - kept, 1));
-        ca.d0 = kept;
-        ca.NB = NB;
+        ca.new_val = out.val.p;
         ca.slot_job = h->slot_job.p;
         if (next_ar >= 0 && ngroup == 1 && tc_block_size_ok(b) && !h->tcw.knobs.block_copies)
-            operands_from_compaction(ca, out, in.ophi, kept_end, njob, (Arith)next_ar, h->tcw, st);
+            operands_from_compaction(ca, out, in.ophi, kept_end, njob, (Arith)next_ar, h->tcw);
         launch_compact_copy(ca, kept_end, st);
         kept = kept_end;
         RDM_CUDA_TRY(cudaEventRecord(h->ev[3], st));
@@ -1958,7 +1961,7 @@ int run_solve_dirs(rdm_handle *h, rdm_info *info_out) {
 void release_work(rdm_handle *h) {
     for (auto *b : {&h->row_off, &h->pool_col, &h->pool_npair, &h->mask_col, &h->out_rp, &h->slot_row,
                     &h->slot_job, &h->slot_npair, &h->slot_x, &h->slot_t, &h->work, &h->work2, &h->work3,
-                    &h->scan_tmp32, &h->pair_a, &h->pair_b, &h->cnt_rows, &h->uidx, &h->urp,
+                    &h->pair_a, &h->pair_b, &h->uidx, &h->urp,
                     &h->dest, &h->cpsrc})
         b->release();
     h->row_cnt.release();
@@ -1973,10 +1976,7 @@ void release_work(rdm_handle *h) {
     h->H1.release();
     h->tcw.tiles.release();
     h->tcw.steps.release();
-    h->tcw.step_cnt.release();
-    h->tcw.step_off.release();
-    h->tcw.tile_cnt.release();
-    h->tcw.tile_off.release();
+    h->tcw.step_rng.release();
     h->tcw.zero.release();
     h->tcw.xlin.release();
     h->pool_cap_hint = 0;

@@ -1,10 +1,11 @@
-// Stream compaction after truncation: per-row counts of the kept blocks, a
-// scan (k_scan.cu) into the new row pointers, and an order-preserving copy of
-// the kept blocks (columns, values, norm bounds); the products compute only
+// Stream compaction after truncation: the pattern and norm bounds of the kept
+// blocks, with the new row pointers, and an order-preserving copy of their
+// values; the products compute only
 // the upper triangle and the copy writes each lower block as the transpose
 // of its upper partner.  Also builds the work list of upper-triangle output
 // blocks for the numeric phase.
 #include "fp_bits.cuh"
+#include "lookback.cuh"
 #include "rdm_internal.cuh"
 #include "tc_split.cuh"
 
@@ -37,40 +38,54 @@ __global__ void k_build_work(const int *__restrict__ slot_row, const int *__rest
     if (up) work[base + __popc(m & ((1u << lane) - 1u))] = (int)s;
 }
 
-// one warp per row of the group: kept blocks (an upper slot on its own flag,
-// a lower one on its upper partner's)
-__global__ void k_compact_count(CompactArgs c, int *cnt) {
-    const int rr = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (rr >= c.nrows) return;
-    const int r = c.r0 + rr;
+// One warp per row of the group: the kept blocks (an upper slot on its own flag,
+// a lower one on its upper partner's) are counted, the row gets its place from
+// the running sums of the CTAs before it, and their columns, norm bounds and
+// destinations are written in order; src[d - d0] receives the slot of output
+// block d, mx[m] the largest norm of matrix m.  Bound by launches and waits for
+// loads: one launch where count, scan and copy were three (150-atom cluster:
+// 16 us, 9 us so).
+constexpr int kRowWarps = 8;
+__global__ void __launch_bounds__(32 * kRowWarps) k_compact_rows(CompactArgs c) {
+    __shared__ int cnt_s[kRowWarps];
+    __shared__ int sh_bid, sh_base;
+    const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
+    const int bid = lookback_id(c.look, &sh_bid);
+    const int r = c.r0 + bid * kRowWarps + wq;
+    const bool row = r < c.r0 + c.nrows;
+    const int rbeg = row ? c.out_rp[r] : 0, rend = row ? c.out_rp[r + 1] : 0;
     int n = 0;
-    for (int p = c.out_rp[r] + lane; p < c.out_rp[r + 1]; p += 32) {
+    for (int p = rbeg + lane; p < rend; p += 32) {
         const bool up = c.out_col[p] >= c.slot_row[p];
         n += c.keep[up ? p : c.slot_t[p]] & kKeepBlock;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
-    if (lane == 0) cnt[rr] = n;
-}
-
-// one warp per row: columns, norm bounds and destinations of the kept blocks
-// (order-preserving); src[d - d0] receives the slot of output block d
-__global__ void k_compact_index(CompactArgs c) {
-    const int rr = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (rr >= c.nrows) return;
-    const int r = c.r0 + rr;
-    const int rend = c.out_rp[r + 1];
-    int dst = c.new_rp[r];
+    if (lane == 0) cnt_s[wq] = n;
+    __syncthreads();
+    int total = 0, before = 0;
+#pragma unroll
+    for (int k = 0; k < kRowWarps; ++k) {
+        if (k < wq) before += cnt_s[k];
+        total += cnt_s[k];
+    }
+    if (wq == 0) {
+        const int first = lookback_sum(c.look, bid, total, c.look_err) + c.d0;
+        if (lane == 0) {
+            sh_base = first;
+            if (bid == (int)gridDim.x - 1) c.new_rp[c.r0 + c.nrows] = first + total;
+        }
+    }
+    __syncthreads();
+    int dst = sh_base + before;
+    if (row && lane == 0) c.new_rp[r] = dst;
     float mx = 0.f;
-    for (int base = c.out_rp[r]; base < rend; base += 32) {
+    for (int base = rbeg; base < rend; base += 32) {
         const int p = base + lane;
-        bool k = false, up = false;
+        bool k = false;
         int src = p;
         if (p < rend) {
-            up = c.out_col[p] >= c.slot_row[p];
-            src = up ? p : c.slot_t[p];
+            src = c.out_col[p] >= c.slot_row[p] ? p : c.slot_t[p];
             k = (c.keep[src] & kKeepBlock) != 0;
         }
         const unsigned m = __ballot_sync(0xffffffffu, k);
@@ -85,11 +100,9 @@ __global__ void k_compact_index(CompactArgs c) {
         }
         dst += __popc(m);
     }
-    if (c.mx) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        if (lane == 0 && mx > 0.f) atomicMax(&c.mx[r / c.NB], __float_as_uint(mx));
-    }
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (row && lane == 0 && mx > 0.f) atomicMax(&c.mx[r / c.NB], __float_as_uint(mx));
 }
 
 // Values of the kept blocks, block sizes that the tensor cores do not take: one
@@ -245,18 +258,21 @@ void launch_build_work(const int *slot_row, const int *out_col, int64_t s0, int6
     RDM_LAUNCH_CHECK();
 }
 
-void launch_compact_count(const CompactArgs &c, int *cnt, cudaStream_t st) {
-    if (c.nrows == 0) return;
-    const int wpb = 8;
-    k_compact_count<<<(c.nrows + wpb - 1) / wpb, wpb * 32, 0, st>>>(c, cnt);
+int64_t compact_look_words(int nrows) { return kMaxJobs + lookback_words((nrows + kRowWarps - 1) / kRowWarps); }
+
+void launch_compact_rows(CompactArgs &c, unsigned long long *look, cudaStream_t st) {
+    RDM_CUDA_TRY(cudaMemsetAsync(look, 0, compact_look_words(c.nrows) * sizeof(unsigned long long), st));
+    c.mx = reinterpret_cast<unsigned *>(look);
+    c.look = look + kMaxJobs;
+    if (c.nrows == 0) {
+        RDM_CUDA_TRY(cudaMemsetAsync(const_cast<int *>(c.new_rp) + c.r0, 0, sizeof(int), st));
+        return;
+    }
+    k_compact_rows<<<(c.nrows + kRowWarps - 1) / kRowWarps, kRowWarps * 32, 0, st>>>(c);
     RDM_LAUNCH_CHECK();
 }
 
 void launch_compact_copy(const CompactArgs &c, int d1, cudaStream_t st) {
-    if (c.nrows == 0) return;
-    const int wpb = 8;
-    k_compact_index<<<(c.nrows + wpb - 1) / wpb, wpb * 32, 0, st>>>(c);
-    RDM_LAUNCH_CHECK();
     if (d1 <= c.d0) return;
     switch (c.b) {
         case 16: return launch_blocks<16>(c, d1, st);

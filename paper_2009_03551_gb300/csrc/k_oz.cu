@@ -305,7 +305,7 @@ struct OzArgs {
     const uint16_t *zero;         // zero blocks (kSlots per CTA)
     const int *e;                 // row exponents (flat rows of the set)
     const int *tiles;
-    const int64_t *step_off;
+    const int64_t *step_rng;
     const int *steps;
     const int *flags;             // TcWork::counters
     int NB;
@@ -378,7 +378,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_tc_oz(OzArgs A) {
         for (int k = 0; k < G::kStages; ++k) zmask[k] = 0u;
         const uint16_t *base = lane < G::TBM ? A.slices_a : A.slices_b;
         for (int t = blockIdx.x; t < ntile && ok; t += gridDim.x) {
-            const int64_t s0 = A.step_off[t], s1 = A.step_off[t + 1];
+            const int64_t s0 = A.step_rng[2 * t], s1 = A.step_rng[2 * t + 1];
             int nxt = (s0 < s1 && lane < G::kSlots) ? A.steps[s0 * G::kSlots + lane] : -1;
             for (int64_t q = s0; q < s1; ++q, ++it) {
                 const int cur = nxt;
@@ -704,7 +704,7 @@ void launch_numeric_oz(const NumArgs &a, const MatSet &in, const JobTable &jt, c
     A.slices_b = ow.slices_b.p;
     A.e = ow.e.p;
     A.NB = in.NB;
-    A.tiles = w.tiles.p; A.step_off = w.step_off.p; A.steps = w.steps.p; A.flags = w.counters.p;
+    A.tiles = w.tiles.p; A.step_rng = w.step_rng.p; A.steps = w.steps.p; A.flags = w.counters.p;
     A.in_val = a.in_val; A.slot_row = a.slot_row; A.slot_job = a.slot_job; A.slot_x = a.slot_x; A.mcol = mcol;
     A.sys_of_row = a.sys_of_row; A.c_lin = a.c_lin; A.c_sq = a.c_sq; A.tau0 = a.tau0; A.tau1 = a.tau1;
     for (int p = 0; p < kMaxJobs; ++p) A.job_tau_sel[p] = a.job_tau_sel[p];

@@ -1,10 +1,9 @@
-// Exclusive prefix sums used to turn per-row / per-tile counts into offsets.
+// Exclusive prefix sums that turn per-row and per-slot counts into offsets.
 // One launch of one CTA up to kOneCta elements (a solve's scans mostly are
 // that short, and a launch costs 2.5 to 4 us on either side); above that two:
 // per-tile sums, then the per-tile scan, whose CTAs add up the sums of the
-// tiles before theirs themselves.  out[n] receives the total; an initial value
-// `init` is added to every output.  The element count may be in device memory.
-// Deterministic (integer addition).
+// tiles before theirs themselves.  out[n] receives the total.  Deterministic
+// (integer addition).
 #include "rdm_internal.cuh"
 
 namespace rdm {
@@ -78,19 +77,16 @@ __device__ T scan_tile(const In *in, int64_t base0, int n, T carry, const Dst &d
 }
 
 template <class In, class T, class Dst>
-__global__ void __launch_bounds__(kThreads) k_scan_one(const In *in, int n, const int *n_dev, Dst dst, T init) {
+__global__ void __launch_bounds__(kThreads) k_scan_one(const In *in, int n, Dst dst) {
     __shared__ T sh[32];
-    if (n_dev) n = *n_dev;
-    T carry = init;
+    T carry = 0;
     for (int64_t base = 0; base < n; base += kTile) carry += scan_tile<In, T, Dst>(in, base, n, carry, dst, sh);
     if (threadIdx.x == 0) dst.put(n, carry);
 }
 
 template <class In, class T>
-__global__ void __launch_bounds__(kThreads) k_tile_sums(const In *__restrict__ in, int n, const int *n_dev,
-                                                        T *__restrict__ tile_sum) {
+__global__ void __launch_bounds__(kThreads) k_tile_sums(const In *__restrict__ in, int n, T *__restrict__ tile_sum) {
     __shared__ T sh[32];
-    if (n_dev) n = *n_dev;
     const int64_t base = (int64_t)blockIdx.x * kTile + (int64_t)threadIdx.x * kItems;
     T s = 0;
 #pragma unroll
@@ -102,29 +98,28 @@ __global__ void __launch_bounds__(kThreads) k_tile_sums(const In *__restrict__ i
 }
 
 template <class In, class T, class Dst>
-__global__ void __launch_bounds__(kThreads) k_scan_apply(const In *in, int n, const int *n_dev,
-                                                         const T *__restrict__ tile_sum, Dst dst, T init) {
+__global__ void __launch_bounds__(kThreads) k_scan_apply(const In *in, int n,
+                                                         const T *__restrict__ tile_sum, Dst dst) {
     __shared__ T sh[32];
-    if (n_dev) n = *n_dev;
     // sum of the tiles before this one
     T s = 0, before;
     for (int k = threadIdx.x; k < (int)blockIdx.x; k += kThreads) s += tile_sum[k];
     block_exclusive_scan<T>(s, sh, &before);
-    const T tot = scan_tile<In, T, Dst>(in, (int64_t)blockIdx.x * kTile, n, init + before, dst, sh);
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) dst.put(n, init + before + tot);
+    const T tot = scan_tile<In, T, Dst>(in, (int64_t)blockIdx.x * kTile, n, before, dst, sh);
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) dst.put(n, before + tot);
 }
 
 template <class In, class T, class Dst>
-void scan_impl(const In *in, Dst dst, int n, const int *n_dev, T *tmp, cudaStream_t st, T init) {
+void scan_impl(const In *in, Dst dst, int n, T *tmp, cudaStream_t st) {
     if (n <= kOneCta) {
-        k_scan_one<In, T, Dst><<<1, kThreads, 0, st>>>(in, n, n_dev, dst, init);
+        k_scan_one<In, T, Dst><<<1, kThreads, 0, st>>>(in, n, dst);
         RDM_LAUNCH_CHECK();
         return;
     }
     const int ntiles = (n + kTile - 1) / kTile;
-    k_tile_sums<In, T><<<ntiles, kThreads, 0, st>>>(in, n, n_dev, tmp);
+    k_tile_sums<In, T><<<ntiles, kThreads, 0, st>>>(in, n, tmp);
     RDM_LAUNCH_CHECK();
-    k_scan_apply<In, T, Dst><<<ntiles, kThreads, 0, st>>>(in, n, n_dev, tmp, dst, init);
+    k_scan_apply<In, T, Dst><<<ntiles, kThreads, 0, st>>>(in, n, tmp, dst);
     RDM_LAUNCH_CHECK();
 }
 
@@ -132,14 +127,11 @@ void scan_impl(const In *in, Dst dst, int n, const int *n_dev, T *tmp, cudaStrea
 
 size_t scan_tmp_elems(int n) { return (size_t)((n + kTile - 1) / kTile + 1); }
 
-void scan_exclusive_i32(const int *in, int *out, int n, int *tmp, cudaStream_t st, int init) {
-    scan_impl<int, int>(in, Plain<int>{out}, n, nullptr, tmp, st, init);
-}
-void scan_exclusive_i64(const int *in, int64_t *out, int n, int64_t *tmp, cudaStream_t st, const int *n_dev) {
-    scan_impl<int, int64_t>(in, Plain<int64_t>{out}, n, n_dev, tmp, st, int64_t(0));
+void scan_exclusive_i64(const int *in, int64_t *out, int n, int64_t *tmp, cudaStream_t st) {
+    scan_impl<int, int64_t>(in, Plain<int64_t>{out}, n, tmp, st);
 }
 void scan_exclusive_pair(const int64_t *in, int *out_lo, int *out_hi, int n, int64_t *tmp, cudaStream_t st) {
-    scan_impl<int64_t, int64_t>(in, Halves{out_lo, out_hi}, n, nullptr, tmp, st, int64_t(0));
+    scan_impl<int64_t, int64_t>(in, Halves{out_lo, out_hi}, n, tmp, st);
 }
 
 }  // namespace rdm

@@ -243,7 +243,7 @@ struct TcArgs {
     const uint16_t *planes;       // operand planes of the input set (hi and lo interleaved per block)
     const uint16_t *zero;         // zero blocks (kSlots per CTA)
     const int *tiles;
-    const int64_t *step_off;
+    const int64_t *step_rng;
     const int *steps;
     const int *flags;             // TcWork::counters
     uint32_t idesc;
@@ -408,8 +408,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
         // after it (its range is loaded a tile ahead)
         int lt = blockIdx.x;
         int64_t lq = 0, le = 0, nq = 0, ne = 0;
-        if (lt < ntile) { lq = A.step_off[lt]; le = A.step_off[lt + 1]; }
-        if (lt + (int)gridDim.x < ntile) { nq = A.step_off[lt + gridDim.x]; ne = A.step_off[lt + gridDim.x + 1]; }
+        if (lt < ntile) { lq = A.step_rng[2 * lt]; le = A.step_rng[2 * lt + 1]; }
+        if (lt + (int)gridDim.x < ntile) { nq = A.step_rng[2 * (lt + gridDim.x)]; ne = A.step_rng[2 * (lt + gridDim.x) + 1]; }
         lq += pr;
         // block index of this lane's slot in the warp's next step, loaded
         // while the current step's copies are issued
@@ -419,7 +419,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
                 lt += gridDim.x;
                 lq = nq + (lq - le);
                 le = ne;
-                if (lt + (int)gridDim.x < ntile) { nq = A.step_off[lt + gridDim.x]; ne = A.step_off[lt + gridDim.x + 1]; }
+                if (lt + (int)gridDim.x < ntile) { nq = A.step_rng[2 * (lt + gridDim.x)]; ne = A.step_rng[2 * (lt + gridDim.x) + 1]; }
             }
             if (lt < ntile && lane < G::kSlots) nxt = A.steps[lq * G::kSlots + lane];
         };
@@ -482,10 +482,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
             uint32_t it = 0, seg = 0;
             bool issued = false;
             int64_t n0 = 0, n1 = 0;          // step range of the next tile, loaded a tile ahead
-            if (blockIdx.x < ntile) { n0 = A.step_off[blockIdx.x]; n1 = A.step_off[blockIdx.x + 1]; }
+            if (blockIdx.x < ntile) { n0 = A.step_rng[2 * blockIdx.x]; n1 = A.step_rng[2 * blockIdx.x + 1]; }
             for (int t = blockIdx.x; t < ntile && !*abort_flag; t += gridDim.x) {
                 const int64_t s0 = n0, s1 = n1;
-                if (t + (int)gridDim.x < ntile) { n0 = A.step_off[t + gridDim.x]; n1 = A.step_off[t + gridDim.x + 1]; }
+                if (t + (int)gridDim.x < ntile) { n0 = A.step_rng[2 * (t + gridDim.x)]; n1 = A.step_rng[2 * (t + gridDim.x) + 1]; }
                 bool ok = true;
                 for (int64_t q = s0; q < s1 && ok; ++seg) {
                     // one segment: up to kSegSteps K-steps into a fresh accumulator
@@ -875,7 +875,7 @@ void launch_tc(const NumArgs &a, const MatSet &in, const JobTable &jt, Arith ar,
     }
     TcArgs A{};
     A.planes = in.ophi.p; A.zero = w.zero.p;
-    A.tiles = w.tiles.p; A.step_off = w.step_off.p; A.steps = w.steps.p; A.flags = w.counters.p;
+    A.tiles = w.tiles.p; A.step_rng = w.step_rng.p; A.steps = w.steps.p; A.flags = w.counters.p;
     // kind::f16: D = F32 (bit 4), A/B = BF16 (1) or F16 (0), K-major, N = kTileN, M = 128
     const uint32_t ab = ar == AR_BF16X3 ? 1u : 0u;
     A.idesc = (1u << 4) | (ab << 7) | (ab << 10) | (((uint32_t)kTileN >> 3) << 17) | ((128u >> 4) << 24);
@@ -926,7 +926,7 @@ bool reuse_operands(const MatSet &in, Arith ar, bool lin, TcWork &w) {
 }
 
 void operands_from_compaction(CompactArgs &c, MatSet &out, DevBuf<uint16_t> &planes, int64_t kept, int njob, Arith ar,
-                              TcWork &w, cudaStream_t st) {
+                              TcWork &w) {
     const size_t n = (size_t)std::max<int64_t>(kept, 1) * out.b * out.b;
     if (planes.cap < 2 * n) {
         // the step may be the last one: no larger buffer for operands that may not be used when memory is short
@@ -939,12 +939,9 @@ void operands_from_compaction(CompactArgs &c, MatSet &out, DevBuf<uint16_t> &pla
     out.ophi.ensure(2 * n);
     w.tpos.ensure(std::max<int64_t>(kept, 1));
     w.scale.ensure(njob);
-    w.pre_err.ensure(1 + njob);
-    RDM_CUDA_TRY(cudaMemsetAsync(w.pre_err.p, 0, (1 + njob) * sizeof(int), st));
     w.xlin_valid = xlin_room(n, w);
     c.planes = out.ophi.p;
     c.tpos = w.tpos.p;
-    c.mx = (unsigned *)w.pre_err.p + 1;
     c.scale = w.scale.p;
     c.xlin = w.xlin_valid ? w.xlin.p : nullptr;
     c.bf16 = ar == AR_BF16X3;

@@ -216,10 +216,7 @@ struct JobMask {
 // ---------------------------------------------------------------------------
 
 // k_scan.cu: exclusive scan (out may alias in); returns nothing, total at out[n].
-// With n_dev the element count is *n_dev <= n (device memory).
-void scan_exclusive_i32(const int *in, int *out, int n, int *tmp, cudaStream_t st, int init = 0);
-void scan_exclusive_i64(const int *in, int64_t *out, int n, int64_t *tmp, cudaStream_t st,
-                        const int *n_dev = nullptr);
+void scan_exclusive_i64(const int *in, int64_t *out, int n, int64_t *tmp, cudaStream_t st);
 // two counts per element (low and high 32 bits), totals below 2^31 each
 void scan_exclusive_pair(const int64_t *in, int *out_lo, int *out_hi, int n, int64_t *tmp, cudaStream_t st);
 size_t scan_tmp_elems(int n);
@@ -364,24 +361,29 @@ struct CompactArgs {
     int64_t u0;
     int *dest;
     int *src;               // [kept blocks of the group]: slot of output block d0 + k
-    const int *new_rp;
-    int *new_col;
+    int *new_rp, *new_col;
     double *new_val;
     float *new_nrm;
     int r0, nrows, b;
     int d0;                 // first output block of the group
+    int NB;
+    unsigned *mx;           // per matrix: largest block norm of the group (bit pattern)
+    unsigned long long *look;
+    int *look_err;          // set when a wait for other CTAs ran out
     // the next step's operands (null: not made): planes at the transposed
-    // positions, those positions, operand scales from the largest block norms
-    // (bit patterns, zeroed), FP32 copy for the linear terms (may be null)
+    // positions, those positions, operand scales, FP32 copy for the linear
+    // terms (may be null)
     uint16_t *planes;
     int *tpos;
-    unsigned *mx;
     float *scale, *xlin;
-    int bf16, njob, NB;
+    int bf16, njob;
     const int *slot_job;
 };
-void launch_compact_count(const CompactArgs &c, int *cnt, cudaStream_t st);
-// output blocks [d0, d1) of the group
+// pattern of the kept blocks of rows [r0, r0 + nrows) (fills mx and look from
+// `look`, compact_look_words(nrows) words of scratch), then the values of the
+// output blocks [d0, d1)
+int64_t compact_look_words(int nrows);
+void launch_compact_rows(CompactArgs &c, unsigned long long *look, cudaStream_t st);
 void launch_compact_copy(const CompactArgs &c, int d1, cudaStream_t st);
 
 // k_lowdin.cu: out = fac[sys] * val for every block of the first NB block rows

@@ -20,15 +20,13 @@ struct TcWork {
     TcKnobs knobs;
     DevBuf<uint16_t> zero;      // zero operand blocks: one per CTA and K-step slot
     DevBuf<int> tiles;          // per tile: job, I, -, nsteps, mask slot[TBM x TBN], column j[TBN]
-    DevBuf<int> tile_cnt, tile_off;
-    DevBuf<int> step_cnt;
-    DevBuf<int64_t> step_off;
+    DevBuf<int64_t> step_rng;   // per tile: its K-steps are [step_rng[2 t], step_rng[2 t + 1])
     DevBuf<int> steps;          // per K-step: TBM A block indices, TBN B block indices (-1 = zero)
     // [0]: error bits of the product kernel, [1]: a list outgrew its buffer
-    // (the product kernel then does nothing), [2]: tiles, [4..5]: K-steps (64 bits)
+    // (the product kernel then does nothing), [2]: tiles, [3]: the tile list is not
+    // complete (a wait ran out; the lists are built again), [4..5]: K-steps (64
+    // bits), [8..]: state of the tile list's prefix sums
     DevBuf<int> counters;
-    DevBuf<int> scan32;
-    DevBuf<int64_t> scan64;
     DevBuf<float> scale;        // per matrix: power-of-two scale of its operand planes
     DevBuf<int> tpos;           // per block (i, k) of the input set: global index of block (k, i)
     // [0]: error bits of the operand preparation (8: a transposed block missing);
@@ -77,7 +75,7 @@ bool reuse_operands(const MatSet &in, Arith ar, bool lin, TcWork &w);
 // pointers in `c`, for the compaction to write; `planes`: the buffer of the input
 // set's operands, which the step no longer reads.
 void operands_from_compaction(CompactArgs &c, MatSet &out, DevBuf<uint16_t> &planes, int64_t kept, int njob, Arith ar,
-                              TcWork &w, cudaStream_t st);
+                              TcWork &w);
 
 // Positions of the transposed blocks of the set (w.tpos); a pattern that is not
 // symmetric sets error bit 8 of pre_err[0].

@@ -6,6 +6,7 @@
 
 #include <algorithm>
 
+#include "lookback.cuh"
 #include "tc_gemm.cuh"
 
 namespace rdm {
@@ -34,13 +35,10 @@ struct TileBuild {
     const int *sys_of_row, *active, *sys_tier;
     JobMask job_mask;    // jobs computed on the tensor cores, per tier
     int u0, u1;          // super-row units (job * NBT + I) of this plan
-    int *tile_cnt;       // [u1 - u0]
-    const int *tile_off; // scanned
+    unsigned long long *look;   // running sums of k_tile_rows' CTAs (lookback.cuh), zeroed
     int *tiles;          // [ntile * kTileInts]
-    int *step_cnt;       // [ntile]
-    const int64_t *step_off;
+    int64_t *step_rng;   // [2 ntile]: a tile's K-steps are [step_rng[2 t], step_rng[2 t + 1])
     int *steps;          // [nsteps * kSlots]
-    const int *ntile;    // number of tiles
     int64_t cap_steps;   // room in steps
     int *flags;          // TcWork::counters
     int max_words;       // bitmap window in 32-column words (<= 512); wider windows: serial merge
@@ -73,23 +71,28 @@ __device__ __forceinline__ void tile_row_range(const TileBuild &T, int p, int I,
 // the TBM block rows are marked in a shared-memory bitmap over their column
 // window; the rank of a column among the distinct ones (prefix popcounts)
 // gives its tile (rank / TBN) and tile column (rank % TBN).  Windows wider
-// than the bitmap fall back to a serial merge by lane 0 (count or fill).
+// than the bitmap fall back to a serial merge by lane 0.  The tiles keep the
+// order of the super-rows; a CTA gets the number of tiles before its own from
+// the running sums of the CTAs before it, so that one launch counts and writes
+// (40 super-rows of a 150-atom cluster: 19 us for count, scan and fill in three
+// launches, 10 us in one).
 constexpr int kTileRowWarps = 8, kTileRowWords = 512;   // 16,384 columns per window
 template <class G>
-__device__ void tile_rows_serial(const TileBuild &T, int t, int p, int I, const int *cur0, const int *end0,
-                                 int fill);
+__device__ int tile_rows_serial(const TileBuild &T, int p, int I, const int *cur0, const int *end0, int base, bool fill);
 template <class G>
-__global__ void __launch_bounds__(32 * kTileRowWarps) k_tile_rows(TileBuild T, int fill) {
+__global__ void __launch_bounds__(32 * kTileRowWarps) k_tile_rows(TileBuild T) {
     __shared__ unsigned bits_s[kTileRowWarps][kTileRowWords];
     __shared__ int rank_s[kTileRowWarps][kTileRowWords];
+    __shared__ int cnt_s[kTileRowWarps];
+    __shared__ int sh_bid, sh_base;
     const int wq = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int t = T.u0 + blockIdx.x * kTileRowWarps + wq;
-    if (t >= T.u1) return;
+    const int bid = lookback_id(T.look, &sh_bid);
+    const int t = T.u0 + bid * kTileRowWarps + wq;
     const int p = t / T.NBT, I = t % T.NBT;
     unsigned *bm = bits_s[wq];
     int *wr = rank_s[wq];
     int c0 = 0, e0 = 0;
-    if (lane < G::TBM) tile_row_range<G>(T, p, I, lane, c0, e0);
+    if (t < T.u1 && lane < G::TBM) tile_row_range<G>(T, p, I, lane, c0, e0);
     int cur[G::TBM], end[G::TBM];
     int lo = 0x7fffffff, hi = -1;
 #pragma unroll
@@ -101,43 +104,57 @@ __global__ void __launch_bounds__(32 * kTileRowWarps) k_tile_rows(TileBuild T, i
             hi = max(hi, T.mcol[end[m] - 1]);
         }
     }
-    const int base = fill ? T.tile_off[t - T.u0] : 0;
-    if (hi < lo) {                         // no tile
-        if (!fill && lane == 0) T.tile_cnt[t - T.u0] = 0;
-        return;
-    }
-    const int nw = ((hi - lo) >> 5) + 1;
-    if (nw > T.max_words) {
-        if (lane == 0) tile_rows_serial<G>(T, t, p, I, cur, end, fill);
-        return;
-    }
-    for (int w = lane; w < nw; w += 32) bm[w] = 0u;
-    __syncwarp();
+    const int nw = hi < lo ? 0 : ((hi - lo) >> 5) + 1;
+    const bool serial = nw > T.max_words;
+    int ntile = 0;
+    if (serial) {
+        if (lane == 0) ntile = tile_rows_serial<G>(T, p, I, cur, end, 0, false);
+    } else if (nw) {
+        for (int w = lane; w < nw; w += 32) bm[w] = 0u;
+        __syncwarp();
 #pragma unroll
-    for (int m = 0; m < G::TBM; ++m)
-        for (int e = cur[m] + lane; e < end[m]; e += 32) {
-            const int j = T.mcol[e] - lo;
-            atomicOr(&bm[j >> 5], 1u << (j & 31));
-        }
-    __syncwarp();
-    // exclusive prefix of the words' popcounts
-    int carry = 0;
-    for (int w0 = 0; w0 < nw; w0 += 32) {
-        const int w = w0 + lane;
-        const int c = w < nw ? __popc(bm[w]) : 0;
-        int x = c;
+        for (int m = 0; m < G::TBM; ++m)
+            for (int e = cur[m] + lane; e < end[m]; e += 32) {
+                const int j = T.mcol[e] - lo;
+                atomicOr(&bm[j >> 5], 1u << (j & 31));
+            }
+        __syncwarp();
+        // exclusive prefix of the words' popcounts
+        int carry = 0;
+        for (int w0 = 0; w0 < nw; w0 += 32) {
+            const int w = w0 + lane;
+            const int c = w < nw ? __popc(bm[w]) : 0;
+            int x = c;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
+            if (w < nw) wr[w] = carry + x - c;
+            carry += __shfl_sync(0xffffffffu, x, 31);
         }
-        if (w < nw) wr[w] = carry + x - c;
-        carry += __shfl_sync(0xffffffffu, x, 31);
+        __syncwarp();
+        ntile = (carry + G::TBN - 1) / G::TBN;
     }
-    __syncwarp();
-    const int ndist = carry, ntile = (ndist + G::TBN - 1) / G::TBN;
-    if (!fill) {
-        if (lane == 0) T.tile_cnt[t - T.u0] = ntile;
+    if (lane == 0) cnt_s[wq] = ntile;
+    __syncthreads();
+    int total = 0, before = 0;
+#pragma unroll
+    for (int k = 0; k < kTileRowWarps; ++k) {
+        if (k < wq) before += cnt_s[k];
+        total += cnt_s[k];
+    }
+    if (wq == 0) {
+        const int first = lookback_sum(T.look, bid, total, T.flags + 3);
+        if (lane == 0) {
+            sh_base = first;
+            if (bid == (int)gridDim.x - 1) T.flags[2] = first + total;
+        }
+    }
+    __syncthreads();
+    const int base = sh_base + before;
+    if (serial) {
+        if (lane == 0) tile_rows_serial<G>(T, p, I, cur, end, base, true);
         return;
     }
     for (int q = lane; q < ntile; q += 32) {
@@ -146,6 +163,7 @@ __global__ void __launch_bounds__(32 * kTileRowWarps) k_tile_rows(TileBuild T, i
         for (int k = 4; k < G::kTileInts; ++k) d[k] = -1;
     }
     __syncwarp();
+    if (nw == 0) return;
 #pragma unroll
     for (int m = 0; m < G::TBM; ++m)
         for (int e = cur[m] + lane; e < end[m]; e += 32) {
@@ -160,15 +178,13 @@ __global__ void __launch_bounds__(32 * kTileRowWarps) k_tile_rows(TileBuild T, i
 
 // the serial TBM-way merge (same tile order as the bitmap path)
 template <class G>
-__device__ void tile_rows_serial(const TileBuild &T, int t, int p, int I, const int *cur0, const int *end0,
-                                 int fill) {
+__device__ int tile_rows_serial(const TileBuild &T, int p, int I, const int *cur0, const int *end0, int base, bool fill) {
     int cur[G::TBM], end[G::TBM];
     for (int m = 0; m < G::TBM; ++m) { cur[m] = cur0[m]; end[m] = end0[m]; }
     // the distinct columns needed by the TBM rows, in increasing order, are
     // packed TBN at a time into tiles: every tile column is needed by at least
     // one row
     int ncol = 0, n = 0;
-    const int base = fill ? T.tile_off[t - T.u0] : 0;
     int *d = nullptr;
     // list heads kept in registers: one load per advance
     int head[G::TBM];
@@ -198,17 +214,16 @@ __device__ void tile_rows_serial(const TileBuild &T, int t, int p, int I, const 
             }
         ++ncol;
     }
-    if (!fill) T.tile_cnt[t - T.u0] = n;
+    return n;
 }
 
 // one thread per tile: K-steps = union over the tile's A rows intersected with
-// the union over its B rows, for each term (count or fill)
+// the union over its B rows, for each term (count, or fill at w)
 template <class G>
-__device__ void tile_steps_serial(const TileBuild &T, int t, int fill) {
+__device__ int tile_steps_serial(const TileBuild &T, int t, int64_t w, bool fill) {
     const int *d = T.tiles + (size_t)t * G::kTileInts;
     const int p = d[0], I = d[1];
     const Job &job = T.jt.job[p];
-    int64_t w = fill ? T.step_off[t] : 0;
     int n = 0;
     for (int term = 0; term < job.nterm; ++term) {
         const int am = job.a[term], bm = job.b[term];
@@ -245,7 +260,7 @@ __device__ void tile_steps_serial(const TileBuild &T, int t, int fill) {
                 }
             }
             if (anyA && anyB) {
-                if (fill && w + n < T.step_off[t + 1] && w + n < T.cap_steps) {
+                if (fill && w + n < T.cap_steps) {
                     int *s = T.steps + (size_t)(w + n) * G::kSlots;
                     for (int q = 0; q < G::kSlots; ++q) s[q] = idx[q] >= 0 && T.tpos ? T.tpos[idx[q]] : idx[q];
                 }
@@ -254,8 +269,19 @@ __device__ void tile_steps_serial(const TileBuild &T, int t, int fill) {
         }
         if (!fill && term == 0) T.tiles[(size_t)t * G::kTileInts + 2] = n;
     }
-    if (!fill) T.step_cnt[t] = n;
-    else T.tiles[(size_t)t * G::kTileInts + 3] = n == (int)(T.step_off[t + 1] - T.step_off[t]) ? n : -1;
+    return n;
+}
+
+// room for the n K-steps of tile t: their place, and the tile's record
+template <class G>
+__device__ __forceinline__ int64_t take_steps(const TileBuild &T, int t, int n) {
+    const int64_t w = (int64_t)atomicAdd(reinterpret_cast<unsigned long long *>(T.flags + 4), (unsigned long long)n);
+    const bool room = w + n <= T.cap_steps;
+    if (!room) T.flags[1] = 1;
+    T.step_rng[2 * (size_t)t] = w;
+    T.step_rng[2 * (size_t)t + 1] = w + n;
+    T.tiles[(size_t)t * G::kTileInts + 3] = room ? n : -1;
+    return w;
 }
 
 // K-steps of one tile, one CTA per tile: per term, the columns k of the tile's
@@ -264,25 +290,28 @@ __device__ void tile_steps_serial(const TileBuild &T, int t, int fill) {
 // both, its index the rank of k among those (prefix popcounts).  Each list
 // entry at such a k writes its block index into its slot of the step; the
 // other slots stay -1 (zero block).  Same steps, same order as the serial
-// merge, which thread 0 runs for windows wider than the bitmaps.  The kernel
+// merge, which thread 0 runs for windows wider than the bitmaps.  A tile takes
+// the room for its steps from a counter as it has counted them: where its
+// list lies among the others' is left open, what is in it is not.  The kernel
 // waits for loads, so a tile's slots are spread over four warps (one warp per
-// tile took 25 us for the ~180 tiles of a 150-atom cluster).
+// tile took 25 us for the ~180 tiles of a 150-atom cluster), and counts and
+// fills in one launch (count, scan and fill in three: 26 us there and 145 us for
+// the 30,000 tiles of a 2,000-atom cluster, 12 and 112 us in one).
 constexpr int kStepWarps = 4, kStepWords = 512;    // 16,384 columns per window
 template <class G>
-__global__ void __launch_bounds__(32 * kStepWarps) k_tile_steps(TileBuild T, int fill) {
-    __shared__ unsigned ba[kStepWords], bb[kStepWords];
-    __shared__ int wr[kStepWords];
+__global__ void __launch_bounds__(32 * kStepWarps) k_tile_steps(TileBuild T) {
+    __shared__ unsigned ba[2][kStepWords], bb[kStepWords];
+    __shared__ int wr[2][kStepWords];
     __shared__ int cur[2][G::kSlots], end[2][G::kSlots], lo_c[2][G::kSlots], hi_c[2][G::kSlots];
-    __shared__ int sh_carry;
+    __shared__ int sh_n[2];
+    __shared__ int64_t sh_w;
     static_assert(2 * G::kSlots <= 32 * kStepWarps, "one thread per slot and term");
     const int tid = threadIdx.x, wq = tid >> 5, lane = tid & 31;
-    const int ntile = *T.ntile;
-    if (fill && blockIdx.x == 0 && tid == 0) {
-        const int64_t n = T.step_off[ntile];
-        if (n > T.cap_steps) T.flags[1] = 1;
-        T.flags[2] = ntile;
-        *reinterpret_cast<int64_t *>(T.flags + 4) = n;
+    if (T.flags[3]) {
+        if (blockIdx.x == 0 && tid == 0) T.flags[1] = 1;
+        return;
     }
+    const int ntile = T.flags[2];
     for (int t = blockIdx.x; t < ntile; t += gridDim.x) {
         const int *d = T.tiles + (size_t)t * G::kTileInts;
         const int p = d[0], I = d[1];
@@ -328,22 +357,24 @@ __global__ void __launch_bounds__(32 * kStepWarps) k_tile_steps(TileBuild T, int
             if (hi_t[term] >= lo_t[term] && ((hi_t[term] - lo_t[term]) >> 5) + 1 > T.max_words) fits = false;
         }
         if (!fits) {
-            if (tid == 0) tile_steps_serial<G>(T, t, fill);
+            if (tid == 0) {
+                const int n = tile_steps_serial<G>(T, t, 0, false);
+                tile_steps_serial<G>(T, t, take_steps<G>(T, t, n), true);
+            }
             __syncthreads();
             continue;
         }
-        int64_t w = fill ? T.step_off[t] : 0;
-        const int64_t wcap = fill ? min(T.step_off[t + 1], T.cap_steps) : 0;
-        int n = 0, n_first = 0;
+        // the steps of each term
 #pragma unroll
         for (int term = 0; term < 2; ++term) {
             const int lo = lo_t[term], hi = hi_t[term];
-            if (hi >= lo) {
-                const int nw = ((hi - lo) >> 5) + 1;
-                for (int x = tid; x < nw; x += 32 * kStepWarps) { ba[x] = 0u; bb[x] = 0u; }
-                __syncthreads();
+            const int nw = hi >= lo ? ((hi - lo) >> 5) + 1 : 0;
+            unsigned *both_w = ba[term];
+            for (int x = tid; x < nw; x += 32 * kStepWarps) { both_w[x] = 0u; bb[x] = 0u; }
+            __syncthreads();
+            if (nw)
                 for (int q = wq; q < G::kSlots; q += kStepWarps) {
-                    unsigned *bmap = q < G::TBM ? ba : bb;
+                    unsigned *bmap = q < G::TBM ? both_w : bb;
                     const int qe = end[term][q];
                     for (int e = cur[term][q] + lane; e < qe; e += 32) {
                         const int k = T.col[e];
@@ -351,61 +382,60 @@ __global__ void __launch_bounds__(32 * kStepWarps) k_tile_steps(TileBuild T, int
                         atomicOr(&bmap[(k - lo) >> 5], 1u << ((k - lo) & 31));
                     }
                 }
-                __syncthreads();
-                if (wq == 0) {
-                    int carry = 0;
-                    for (int x0 = 0; x0 < nw; x0 += 32) {
-                        const int x = x0 + lane;
-                        unsigned both = 0u;
-                        if (x < nw) {
-                            both = ba[x] & bb[x];
-                            ba[x] = both;
-                        }
-                        const int c = __popc(both);
-                        int y = c;
+            __syncthreads();
+            if (wq == 0) {
+                int carry = 0;
+                for (int x0 = 0; x0 < nw; x0 += 32) {
+                    const int x = x0 + lane;
+                    unsigned both = 0u;
+                    if (x < nw) {
+                        both = both_w[x] & bb[x];
+                        both_w[x] = both;
+                    }
+                    const int c = __popc(both);
+                    int y = c;
 #pragma unroll
-                        for (int o = 1; o < 32; o <<= 1) {
-                            const int z = __shfl_up_sync(0xffffffffu, y, o);
-                            if (lane >= o) y += z;
-                        }
-                        if (x < nw) wr[x] = carry + y - c;
-                        carry += __shfl_sync(0xffffffffu, y, 31);
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int z = __shfl_up_sync(0xffffffffu, y, o);
+                        if (lane >= o) y += z;
                     }
-                    if (lane == 0) sh_carry = carry;
+                    if (x < nw) wr[term][x] = carry + y - c;
+                    carry += __shfl_sync(0xffffffffu, y, 31);
                 }
-                __syncthreads();
-                const int carry = sh_carry;
-                if (fill) {
-                    // -1 everywhere, then the stored blocks
-                    const int64_t f0 = (w + n) * G::kSlots, f1 = min(w + n + carry, wcap) * G::kSlots;
-                    for (int64_t q = f0 + tid; q < f1; q += 32 * kStepWarps) T.steps[q] = -1;
-                    __syncthreads();
-                    for (int q = wq; q < G::kSlots; q += kStepWarps) {
-                        const int qe = end[term][q];
-                        for (int e = cur[term][q] + lane; e < qe; e += 32) {
-                            const int k = T.col[e];
-                            if (k < lo || k > hi) continue;
-                            const int kk = k - lo;
-                            const unsigned word = ba[kk >> 5];
-                            if (!((word >> (kk & 31)) & 1u)) continue;
-                            const int r = wr[kk >> 5] + __popc(word & ((1u << (kk & 31)) - 1u));
-                            if (w + n + r < wcap) T.steps[(size_t)(w + n + r) * G::kSlots + q] = T.tpos ? T.tpos[e] : e;
-                        }
-                    }
+                if (lane == 0) {
+                    sh_n[term] = carry;
+                    if (term == 0) T.tiles[(size_t)t * G::kTileInts + 2] = carry;
+                    else sh_w = take_steps<G>(T, t, sh_n[0] + carry);
                 }
-                n += carry;
-                __syncthreads();
             }
-            if (term == 0) n_first = n;
+            __syncthreads();
         }
-        if (tid == 0) {
-            if (!fill) {
-                T.tiles[(size_t)t * G::kTileInts + 2] = n_first;
-                T.step_cnt[t] = n;
-            } else {
-                T.tiles[(size_t)t * G::kTileInts + 3] = n == (int)(T.step_off[t + 1] - T.step_off[t]) ? n : -1;
+        // -1 everywhere, then the stored blocks (nothing without room for all)
+        const int n0 = sh_n[0], n = n0 + sh_n[1];
+        const int64_t w = sh_w;
+        if (w + n <= T.cap_steps) {
+            for (int q = tid; q < n * G::kSlots; q += 32 * kStepWarps) T.steps[(size_t)w * G::kSlots + q] = -1;
+            __syncthreads();
+#pragma unroll
+            for (int term = 0; term < 2; ++term) {
+                const int lo = lo_t[term], hi = hi_t[term];
+                if (hi < lo) continue;
+                const int64_t at = w + (term ? n0 : 0);
+                for (int q = wq; q < G::kSlots; q += kStepWarps) {
+                    const int qe = end[term][q];
+                    for (int e = cur[term][q] + lane; e < qe; e += 32) {
+                        const int k = T.col[e];
+                        if (k < lo || k > hi) continue;
+                        const int kk = k - lo;
+                        const unsigned word = ba[term][kk >> 5];
+                        if (!((word >> (kk & 31)) & 1u)) continue;
+                        const int r = wr[term][kk >> 5] + __popc(word & ((1u << (kk & 31)) - 1u));
+                        T.steps[(size_t)(at + r) * G::kSlots + q] = T.tpos ? T.tpos[e] : e;
+                    }
+                }
             }
         }
+        __syncthreads();
     }
 }
 
@@ -416,20 +446,18 @@ TcPlan build_plan(const MatSet &in, const JobTable &jt, const SysDev &sd, const 
     TcPlan plan{};
     const int NB = in.NB, NBT = (NB + G::TBM - 1) / G::TBM;
     const int nrowt = unit1 - unit0;
-    w.counters.ensure(8);
-    RDM_CUDA_TRY(cudaMemsetAsync(w.counters.p, 0, 8 * sizeof(int), st));
+    // the counters, and behind them the running sums of k_tile_rows' CTAs
+    const int rgrid = std::max(0, (nrowt + kTileRowWarps - 1) / kTileRowWarps);
+    const size_t nctr = 8 + 2 * (size_t)lookback_words(rgrid);
+    w.counters.ensure(nctr);
+    RDM_CUDA_TRY(cudaMemsetAsync(w.counters.p, 0, nctr * sizeof(int), st));
     if (nrowt <= 0 || nupper <= 0) return plan;
     // every tile of a super-row but its last one has TBN columns, each with at
     // least one upper slot
     const int64_t max_tile = nupper / G::TBN + nrowt;
     plan.max_tile = (int)max_tile;
-    w.tile_cnt.ensure(nrowt + 1);
-    w.tile_off.ensure(nrowt + 1);
-    w.scan32.ensure(scan_tmp_elems(nrowt + 1));
     w.tiles.ensure((size_t)max_tile * G::kTileInts);
-    w.step_cnt.ensure(max_tile + 1);
-    w.step_off.ensure(max_tile + 1);
-    w.scan64.ensure(scan_tmp_elems((int)max_tile + 1));
+    w.step_rng.ensure(2 * (size_t)max_tile);
     w.steps.ensure((size_t)std::max<int64_t>(min_steps, 1) * G::kSlots);
     plan.cap_steps = (int64_t)(w.steps.cap / G::kSlots);
     TileBuild T{};
@@ -438,28 +466,20 @@ TcPlan build_plan(const MatSet &in, const JobTable &jt, const SysDev &sd, const 
     T.job_mask = job_mask;
     T.u0 = unit0; T.u1 = unit1;
     T.sys_tier = sd.tier.p;
-    T.tile_cnt = w.tile_cnt.p; T.tile_off = w.tile_off.p;
+    T.look = reinterpret_cast<unsigned long long *>(w.counters.p + 8);
     T.tpos = w.tpos_valid ? w.tpos.p : nullptr;
-    T.tiles = w.tiles.p; T.step_cnt = w.step_cnt.p; T.step_off = w.step_off.p; T.steps = w.steps.p;
-    T.ntile = w.tile_off.p + nrowt; T.cap_steps = plan.cap_steps; T.flags = w.counters.p;
+    T.tiles = w.tiles.p; T.step_rng = w.step_rng.p; T.steps = w.steps.p;
+    T.cap_steps = plan.cap_steps; T.flags = w.counters.p;
     static_assert(kTileRowWords == kStepWords, "one window bound for both plan builders");
     T.max_words = w.knobs.window_words > 0 && w.knobs.window_words < kTileRowWords ? w.knobs.window_words
                                                                                     : kTileRowWords;
-    const int rgrid = (nrowt + kTileRowWarps - 1) / kTileRowWarps;
     const int sgrid = (int)std::min<int64_t>(max_tile, 152 * 16);
-    k_tile_rows<G><<<rgrid, 32 * kTileRowWarps, 0, st>>>(T, 0);
+    k_tile_rows<G><<<rgrid, 32 * kTileRowWarps, 0, st>>>(T);
     RDM_LAUNCH_CHECK();
-    scan_exclusive_i32(w.tile_cnt.p, w.tile_off.p, nrowt, w.scan32.p, st);
-    k_tile_rows<G><<<rgrid, 32 * kTileRowWarps, 0, st>>>(T, 1);
-    RDM_LAUNCH_CHECK();
-    k_tile_steps<G><<<sgrid, 32 * kStepWarps, 0, st>>>(T, 0);
-    RDM_LAUNCH_CHECK();
-    scan_exclusive_i64(w.step_cnt.p, w.step_off.p, (int)max_tile, w.scan64.p, st, T.ntile);
-    k_tile_steps<G><<<sgrid, 32 * kStepWarps, 0, st>>>(T, 1);
+    k_tile_steps<G><<<sgrid, 32 * kStepWarps, 0, st>>>(T);
     RDM_LAUNCH_CHECK();
     return plan;
 }
-
 
 }  // namespace
 }  // namespace rdm

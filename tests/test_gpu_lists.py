@@ -1,0 +1,67 @@
+"""Tile lists, K-step lists and the compaction's pattern of long, thin block
+matrices: their offsets are prefix sums across the CTAs of one launch (8 rows
+or super-rows each, 32 CTAs looked at in one go), and the K-step lists start in
+room guessed from the number of block pairs.  Entries are small integers, so
+every arithmetic gives the exact product."""
+
+import numpy as np
+import pytest
+import scipy.sparse as sp
+
+from synth import Bsr
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def rdm():
+    from paper_2009_03551_gb300 import build as b
+    b.build()
+    from paper_2009_03551_gb300 import rdm as mod
+    return mod
+
+
+def band(rng, nb, b, off):
+    """Symmetric matrix with the block diagonals 0 and +-off, integer entries."""
+    i = np.arange(nb)
+    d = rng.integers(-2, 3, (nb, b, b)).astype(float)
+    u = rng.integers(-2, 3, (max(nb - off, 0), b, b)).astype(float) if off else np.zeros((0, b, b))
+    k = i[:len(u)]
+    rows = np.concatenate([i, k, k + off])
+    cols = np.concatenate([i, k + off, k])
+    vals = np.concatenate([d + d.transpose(0, 2, 1), u, u.transpose(0, 2, 1)])
+    o = np.lexsort((cols, rows))
+    rp = np.concatenate([[0], np.cumsum(np.bincount(rows, minlength=nb))]).astype(np.int32)
+    return rp, cols[o].astype(np.int32), np.ascontiguousarray(vals[o])
+
+
+@pytest.mark.parametrize("nb,b,off,mode", [
+    (1, 2, 0, "fp64"), (8, 2, 1, "fp64"), (9, 4, 2, "fp64"),              # one CTA, two
+    (256, 2, 1, "fp64"), (257, 4, 3, "fp64"), (8400, 2, 7, "fp64"),       # 32, 33 and 1,050 CTAs of the compaction
+    (2047, 16, 3, "mixed_fp16"), (2112, 16, 1, "mixed_bf16"),             # 32 and 33 CTAs of the tile list
+    (521, 64, 2, "mixed_bf16"), (1100, 32, 1, "mixed_fp16"), (1100, 32, 5, "fp64"),
+    (95000, 16, 0, "mixed_fp16"),      # one pair per K-step: more steps than the first guess has room for
+])
+def test_lists_of_long_matrices(rdm, nb, b, off, mode):
+    rng = np.random.default_rng(nb + b)
+    rp, ci, va = band(rng, nb, b, off)
+    n = nb * b
+    A = Bsr(nb, b, n, rp, ci, va)
+    S = sp.bsr_matrix((va, ci, rp), shape=(n, n))
+    exact = sp.bsr_matrix(S @ S + 2.0 * S, blocksize=(b, b))
+    exact.sort_indices()
+    # a threshold inside the widest gap between the middle half of the block norms
+    nrm = np.sqrt((exact.data ** 2).sum((1, 2)))
+    mid = np.sort(nrm)[len(nrm) // 4:max(3 * len(nrm) // 4, 2)]
+    k = int(np.argmax(np.diff(mid))) if off else 0
+    tau = float(0.5 * (mid[k] + mid[k + 1])) if off else 0.0
+    keep = nrm >= tau
+    row = np.repeat(np.arange(nb), np.diff(exact.indptr))
+    h = rdm.rdm_create(0)
+    try:
+        got = rdm.rdm_block_product(h, A, None, A, 2.0, 1.0, 1, tau, rdm.MODES[mode])
+    finally:
+        rdm.rdm_destroy(h)
+    assert np.array_equal(got.row_ptr, np.concatenate([[0], np.cumsum(np.bincount(row[keep], minlength=nb))]))
+    assert np.array_equal(got.col_idx, exact.indices[keep])
+    assert np.array_equal(got.vals, exact.data[keep])
