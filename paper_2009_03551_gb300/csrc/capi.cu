@@ -535,6 +535,9 @@ struct StepStats {
     // times of the launches; the last group's are added by finish_step
     float t_simt[3] = {0, 0, 0}, t_tc = 0, t_cmp = 0, t_oz = 0;
     bool oz_is_fp64 = false;                // the slice launch held FP64 products only
+    bool simt64 = true;                     // FP64 products run on the CUDA cores
+    bool tc = false, oz = false, f32_t = false, pending = false;   // what check_step looks at
+    double tc_flops = 0, oz_flops = 0;      // per K-step
 };
 
 // Uploads the scalars of a step (per system) in one copy.  Every step waits
@@ -585,6 +588,47 @@ void finish_step(rdm_handle *h, StepStats &ss) {
     ss.ms[5] = ss.t_simt[1];     // double-FP32 products
     ss.ms[6] = ss.t_oz;          // tensor-core slice products
     ss.ms[0] = std::max(0.f, mall - rest);   // mask, lists, plans
+}
+
+// Once the counters of a group's launches are on the host: throws what the
+// kernels report; false: a K-step list outgrew its buffer (the next lists get
+// the room) and the launches have to be repeated.
+bool check_step(rdm_handle *h, StepStats &ss) {
+    const HostStep *hs = h->step_host.p;
+    if (hs->ctr[kCtrLook]) throw Error{RDM_ETIMEOUT, "compaction: a wait for other blocks of the kernel ran out"};
+    if (hs->ctr[kCtrErr])
+        throw Error{RDM_ECUDA,
+                    "internal error: pair lists inconsistent with the mask (code " + std::to_string(hs->ctr[kCtrErr]) + ")"};
+    const int64_t nst_tc = ss.tc ? *reinterpret_cast<const int64_t *>(hs->tc + 4) : 0;
+    const int64_t nst_oz = ss.oz ? *reinterpret_cast<const int64_t *>(hs->oz + 4) : 0;
+    if ((ss.tc && hs->tc[1]) || (ss.oz && hs->oz[1])) {
+        h->tcw.need_steps = nst_tc;
+        h->tcw_oz.need_steps = nst_oz;
+        return false;
+    }
+    h->tcw.need_steps = h->tcw_oz.need_steps = 0;
+    const int err = (ss.f32_t ? hs->pre_err & 8 : 0) | (ss.tc ? hs->tc[0] : 0) | (ss.oz ? hs->oz[0] : 0);
+    if (err & 8) throw Error{RDM_EBADBSR, "an operand's block pattern is not symmetric"};
+    if (err)
+        throw Error{err & 1 ? RDM_ETIMEOUT : RDM_ECUDA, "tensor-core product kernel failed (code " + std::to_string(err) + ")"};
+    ss.issued_tc += (double)nst_tc * ss.tc_flops;
+    ss.issued_oz += (double)nst_oz * ss.oz_flops;
+    return true;
+}
+
+// sizes of the result, pairs per kernel class
+void close_step(rdm_handle *h, StepStats &ss, MatSet &out) {
+    const HostStep *hs = h->step_host.p;
+    const unsigned long long *cls = reinterpret_cast<const unsigned long long *>(hs->ctr + kCtrClass);
+    ss.pairs_tc = (int64_t)cls[0];
+    ss.pairs_64 = (int64_t)cls[1];
+    ss.pairs_32 = (int64_t)cls[2];
+    ss.pairs_ff = (int64_t)cls[3];
+    ss.pairs_oz = (int64_t)cls[4];
+    ss.pairs_simt = (ss.simt64 ? ss.pairs_64 : 0) + ss.pairs_32 + ss.pairs_ff;
+    out.total = hs->kept;
+    out.nnzb.assign(out.nmat, 0);
+    for (int p = 0; p < out.nmat; ++p) out.nnzb[p] = hs->rp[p + 1] - hs->rp[p];
 }
 
 bool is_tc(Arith a) { return a == AR_BF16X3 || a == AR_FP16X3; }
@@ -656,11 +700,16 @@ Arith fp64_arith(int mode, int b, double tau) {
 // lin: an active system's c_lin is not 0; copies: some system is not active
 // (its blocks are copied); next_ar: split arithmetic (Arith) of a step that takes
 // `out` as its input, whose operands the compaction then writes (-1: none).
-// The host waits twice, for the size of the mask and
-// for that of the result (and once more per further group); the device may
+// The host waits for the size of the mask and then, once per group, for that of
+// the result.  With `defer` a small result is not waited for: its blocks are
+// copied into room for the whole mask (at most kDeferBytes, and a sixteenth of
+// the free memory where the room has to be made), and the caller, after its
+// own wait, calls check_step and close_step (StepStats::pending).  The device may
 // still be working on the compaction when the call returns (finish_step).
+constexpr size_t kDeferBytes = size_t(256) << 20;   // (a wait costs ~20 us, the room 256 MB of up to 280 GB)
 StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
-                   const Arith (*tab)[kMaxJobs], unsigned tiers_present, bool lin, bool copies, int next_ar = -1) {
+                   const Arith (*tab)[kMaxJobs], unsigned tiers_present, bool lin, bool copies, int next_ar = -1,
+                   bool defer = false) {
     cudaStream_t st = h->stream;
     const int NB = in.NB, b = in.b, njob = jt.njob;
     const size_t bb = (size_t)b * b;
@@ -894,6 +943,21 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
     for (int g = 0; g < ngroup; ++g) gslots = std::max(gslots, gslot(gunit[g + 1]) - gslot(gunit[g]));
     h->cpsrc.ensure(gslots);
     int kept = 0;
+    ss.tc = tc;
+    ss.oz = any_oz;
+    ss.f32_t = f32_t;
+    ss.tc_flops = tc ? tc_step_flops(b) : 0.0;
+    ss.oz_flops = any_oz ? oz_step_flops(h->ozw) : 0.0;
+    if (defer && ngroup == 1) {
+        const size_t need = (size_t)ns1 * bb;
+        ss.pending = need * sizeof(double) <= kDeferBytes;
+        if (ss.pending && out.val.cap < need) {
+            size_t fr = 0, tot = 0;
+            RDM_CUDA_TRY(cudaMemGetInfo(&fr, &tot));
+            ss.pending = need * sizeof(double) <= fr / 16;
+        }
+        if (ss.pending) out.val.ensure(need);
+    }
     const int ev_simt[kSimt] = {5, 6, 4};   // events after each CUDA-core class
     for (int g = 0; g < ngroup; ++g) {
         const int ua = gunit[g], ub = gunit[g + 1];
@@ -902,9 +966,8 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
         // room for the K-steps (a tile of 4 x 8 blocks has 5 to 12 pairs to a
         // step, one of 4 x 2 about 3); a plan that needs more is built again
         const int64_t gpairs = (int64_t)((double)npairs * (double)nup / (double)std::max<int64_t>(nupper, 1)) + 1;
-        int64_t steps_tc = std::min(gpairs, gpairs / 4 + 65536) + 1024, steps_oz = gpairs / 2 + 1024;
+        const int64_t steps_tc = std::min(gpairs, gpairs / 4 + 65536) + 1024, steps_oz = gpairs / 2 + 1024;
         CompactArgs ca{};
-        int kept_end = 0;
         for (int attempt = 0;; ++attempt) {
             RDM_CUDA_TRY(cudaMemsetAsync(h->counters.p + kCtrWork, 0, (kCtrInts - kCtrWork) * sizeof(int), st));
             // CUDA-core work per class: the selected jobs, and in the first class
@@ -915,8 +978,10 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
                                       h->sd.sys_of_row.p, h->sd.active.p, h->slot_job.p, h->sd.tier.p, cm[c],
                                       c == first_c ? 1 : 0);
             TcPlan plan{}, oplan{};
-            if (tc) plan = build_tc_plan(in, jt, h->sd, h->out_rp.p, mcol, h->tcw, tcm, ua, ub, nup, steps_tc, st);
-            if (any_oz) oplan = build_oz_plan(in, jt, h->sd, h->out_rp.p, mcol, h->tcw_oz, ozm, ua, ub, nup, steps_oz, st);
+            if (tc) plan = build_tc_plan(in, jt, h->sd, h->out_rp.p, mcol, h->tcw, tcm, ua, ub, nup,
+                                       std::max(steps_tc, h->tcw.need_steps), st);
+            if (any_oz) oplan = build_oz_plan(in, jt, h->sd, h->out_rp.p, mcol, h->tcw_oz, ozm, ua, ub, nup,
+                                            std::max(steps_oz, h->tcw_oz.need_steps), st);
 
             NumArgs a{};
             a.in_val = in.val.p; a.in_nrm = in.nrm.p;
@@ -971,30 +1036,17 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
             if (g == ngroup - 1 && NB)
                 RDM_CUDA_TRY(cudaMemcpy2DAsync(hs->rp, sizeof(int), out.row_ptr.p, (size_t)NB * sizeof(int), sizeof(int),
                                                njob + 1, cudaMemcpyDeviceToHost, st));
+            if (ss.pending) break;
             sync(h);
-            if (hs->ctr[kCtrLook]) throw Error{RDM_ETIMEOUT, "compaction: a wait for other blocks of the kernel ran out"};
-            if (hs->ctr[kCtrErr])
-                throw Error{RDM_ECUDA, "internal error: pair lists inconsistent with the mask (code " +
-                                           std::to_string(hs->ctr[kCtrErr]) + ")"};
-            const int64_t nst_tc = tc ? *reinterpret_cast<int64_t *>(hs->tc + 4) : 0;
-            const int64_t nst_oz = any_oz ? *reinterpret_cast<int64_t *>(hs->oz + 4) : 0;
-            const bool again = (tc && hs->tc[1]) || (any_oz && hs->oz[1]);
-            if (!again) {
-                ss.issued_tc += (double)nst_tc * tc_step_flops(b);
-                if (any_oz) ss.issued_oz += (double)nst_oz * oz_step_flops(h->ozw);
-                break;
-            }
+            if (check_step(h, ss)) break;
             if (attempt == 3) throw Error{RDM_ECAPACITY, "K-step lists outgrew their buffers repeatedly"};
-            steps_tc = std::max(steps_tc, nst_tc);
-            steps_oz = std::max(steps_oz, nst_oz);
         }
-        kept_end = hs->kept;
-        const int tc_err = (f32_t ? hs->pre_err & 8 : 0) | (tc ? hs->tc[0] : 0) | (any_oz ? hs->oz[0] : 0);
-        if (tc_err & 8) throw Error{RDM_EBADBSR, "an operand's block pattern is not symmetric"};
-        if (tc_err)
-            throw Error{tc_err & 1 ? RDM_ETIMEOUT : RDM_ECUDA,
-                        "tensor-core product kernel failed (code " + std::to_string(tc_err) + ")"};
-        if (g == 0) {
+        // blocks up to this group's end: not known yet if the result is not
+        // waited for, then at most the mask's
+        const int kept_end = ss.pending ? (int)nslot : hs->kept;
+        if (ss.pending) {
+            // room made above
+        } else if (g == 0) {
             // the output set's old contents are dead; reserve about the input's size
             const int64_t want = ngroup > 1 ? std::max<int64_t>(kept_end, in.total) : kept_end;
             out.val.ensure((size_t)std::max<int64_t>(want, 1) * bb);
@@ -1005,7 +1057,7 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
         ca.slot_job = h->slot_job.p;
         if (next_ar >= 0 && ngroup == 1 && tc_block_size_ok(b) && !h->tcw.knobs.block_copies)
             operands_from_compaction(ca, out, in.ophi, kept_end, njob, (Arith)next_ar, h->tcw);
-        launch_compact_copy(ca, kept_end, st);
+        launch_compact_copy(ca, kept_end - kept, st);
         kept = kept_end;
         RDM_CUDA_TRY(cudaEventRecord(h->ev[3], st));
         if (g + 1 < ngroup) {
@@ -1013,20 +1065,12 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
             add_times(h, ss);
         }
     }
-    const unsigned long long *cls = reinterpret_cast<unsigned long long *>(hs->ctr + kCtrClass);
-    ss.pairs_tc = (int64_t)cls[0];
-    ss.pairs_64 = (int64_t)cls[1];
-    ss.pairs_32 = (int64_t)cls[2];
-    ss.pairs_ff = (int64_t)cls[3];
-    ss.pairs_oz = (int64_t)cls[4];
-    ss.pairs_simt = (any_oz8 ? 0 : ss.pairs_64) + ss.pairs_32 + ss.pairs_ff;
     ss.oz_is_fp64 = any_oz8;
     for (int t = 0; t < kMaxTiers; ++t) ss.oz_is_fp64 = ss.oz_is_fp64 && !moz.m[t];
     ss.bytes = ((double)in.total * (tc ? 4.0 : 8.0) + (any_oz ? (double)in.nnzb[0] * 2.0 * h->ozw.nslice : 0.0) +
                 (double)nupper * 8.0) * (double)bb;
-    out.total = kept;
-    out.nnzb.assign(njob, 0);
-    for (int p = 0; p < njob; ++p) out.nnzb[p] = hs->rp[p + 1] - hs->rp[p];
+    ss.simt64 = !any_oz8;
+    if (!ss.pending) close_step(h, ss, out);
     return ss;
 }
 
@@ -1510,10 +1554,21 @@ int run_solve(rdm_handle *h, rdm_info *info_out) {
         upload_step(h, c_lin, c_sq, t0, t1, act, tier_of);
         RDM_CUDA_TRY(cudaEventRecord(ev0, st));
         MatSet &Xn = h->X[1 - h->cur];
-        StepStats sst = multiply(h, Xc, Xn, jt, tab, tiers_present, lin, copies,
-                                 P.mode == RDM_MODE_MIXED_BF16 ? AR_BF16X3 : mixed ? AR_FP16X3 : -1);
+        const int next_ar = P.mode == RDM_MODE_MIXED_BF16 ? AR_BF16X3 : mixed ? AR_FP16X3 : -1;
+        StepStats sst = multiply(h, Xc, Xn, jt, tab, tiers_present, lin, copies, next_ar, true);
         RDM_CUDA_TRY(cudaEventRecord(ev1, st));
         q = stats(h, Xn);                     // waits for the step
+        if (sst.pending) {
+            if (!check_step(h, sst)) {
+                // once more, waiting for the lists; the operands' buffer went to Xn
+                Xc.planes_ar = -1;
+                sst = multiply(h, Xc, Xn, jt, tab, tiers_present, lin, copies, next_ar);
+                RDM_CUDA_TRY(cudaEventRecord(ev1, st));
+                q = stats(h, Xn);
+            } else {
+                close_step(h, sst, Xn);
+            }
+        }
         finish_step(h, sst);
         float ms = 0;
         cudaEventElapsedTime(&ms, ev0, ev1);

@@ -109,8 +109,9 @@ __global__ void __launch_bounds__(32 * kRowWarps) k_compact_rows(CompactArgs c) 
 // CTA per block (grid-stride), upper blocks are copied, lower ones transposed
 // through shared memory (b x (b+1) doubles) from their upper partner, which is
 // in this group's buffer or already compacted.
-__global__ void __launch_bounds__(128) k_compact_vals(CompactArgs c, int d1) {
+__global__ void __launch_bounds__(128) k_compact_vals(CompactArgs c) {
     extern __shared__ double tile[];
+    const int d1 = c.new_rp[c.r0 + c.nrows];
     const int b = c.b, bb = b * b, ld = b + 1;
     for (int d = c.d0 + blockIdx.x; d < d1; d += gridDim.x) {
         const int p = c.src[d - c.d0];
@@ -142,7 +143,8 @@ __global__ void __launch_bounds__(128) k_compact_vals(CompactArgs c, int d1) {
 // 300,000 blocks of 32: 292 + 271 us per step in two passes, 537 in one;
 // 150 atoms, 5,500 blocks: 16.5 + 13.5 us, 21 in one, and four launches less).
 template <int B, int PL>
-__global__ void __launch_bounds__(128) k_compact_blocks(CompactArgs c, int d1) {
+__global__ void __launch_bounds__(128) k_compact_blocks(CompactArgs c) {
+    const int d1 = c.new_rp[c.r0 + c.nrows];
     constexpr int BB = B * B, C8 = B / 8;
     const int lane = threadIdx.x & 31;
     if (PL && blockIdx.x == 0 && (int)threadIdx.x < c.njob) c.scale[threadIdx.x] = matrix_scale(c.mx[threadIdx.x], PL == 1);
@@ -238,11 +240,11 @@ __global__ void __launch_bounds__(128) k_compact_blocks(CompactArgs c, int d1) {
 }
 
 template <int B>
-void launch_blocks(const CompactArgs &c, int d1, cudaStream_t st) {
-    const int grid = (int)std::min<int64_t>(((int64_t)d1 - c.d0 + 3) / 4, 152 * 16);
-    if (!c.planes) k_compact_blocks<B, 0><<<grid, 128, 0, st>>>(c, d1);
-    else if (c.bf16) k_compact_blocks<B, 2><<<grid, 128, 0, st>>>(c, d1);
-    else k_compact_blocks<B, 1><<<grid, 128, 0, st>>>(c, d1);
+void launch_blocks(const CompactArgs &c, int max_blocks, cudaStream_t st) {
+    const int grid = (int)std::min((max_blocks + 3) / 4, 152 * 16);
+    if (!c.planes) k_compact_blocks<B, 0><<<grid, 128, 0, st>>>(c);
+    else if (c.bf16) k_compact_blocks<B, 2><<<grid, 128, 0, st>>>(c);
+    else k_compact_blocks<B, 1><<<grid, 128, 0, st>>>(c);
     RDM_LAUNCH_CHECK();
 }
 
@@ -272,17 +274,17 @@ void launch_compact_rows(CompactArgs &c, unsigned long long *look, cudaStream_t 
     RDM_LAUNCH_CHECK();
 }
 
-void launch_compact_copy(const CompactArgs &c, int d1, cudaStream_t st) {
-    if (d1 <= c.d0) return;
+void launch_compact_copy(const CompactArgs &c, int max_blocks, cudaStream_t st) {
+    if (max_blocks <= 0 || c.nrows == 0) return;
     switch (c.b) {
-        case 16: return launch_blocks<16>(c, d1, st);
-        case 32: return launch_blocks<32>(c, d1, st);
-        case 64: return launch_blocks<64>(c, d1, st);
+        case 16: return launch_blocks<16>(c, max_blocks, st);
+        case 32: return launch_blocks<32>(c, max_blocks, st);
+        case 64: return launch_blocks<64>(c, max_blocks, st);
         default: break;
     }
     const size_t smem = (size_t)c.b * (c.b + 1) * sizeof(double);
-    const int grid = (int)std::min<int64_t>((int64_t)d1 - c.d0, 152 * 16);
-    k_compact_vals<<<grid, 128, smem, st>>>(c, d1);
+    const int grid = std::min(max_blocks, 152 * 16);
+    k_compact_vals<<<grid, 128, smem, st>>>(c);
     RDM_LAUNCH_CHECK();
 }
 

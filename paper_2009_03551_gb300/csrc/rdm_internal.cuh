@@ -380,11 +380,11 @@ struct CompactArgs {
     const int *slot_job;
 };
 // pattern of the kept blocks of rows [r0, r0 + nrows) (fills mx and look from
-// `look`, compact_look_words(nrows) words of scratch), then the values of the
-// output blocks [d0, d1)
+// `look`, compact_look_words(nrows) words of scratch), then the values of its
+// kept blocks (at most max_blocks; how many is read on the device)
 int64_t compact_look_words(int nrows);
 void launch_compact_rows(CompactArgs &c, unsigned long long *look, cudaStream_t st);
-void launch_compact_copy(const CompactArgs &c, int d1, cudaStream_t st);
+void launch_compact_copy(const CompactArgs &c, int max_blocks, cudaStream_t st);
 
 // k_lowdin.cu: out = fac[sys] * val for every block of the first NB block rows
 // (pad_one: the diagonal of padding rows set to 1), and identity blocks.

@@ -21,6 +21,7 @@ struct TcWork {
     DevBuf<uint16_t> zero;      // zero operand blocks: one per CTA and K-step slot
     DevBuf<int> tiles;          // per tile: job, I, -, nsteps, mask slot[TBM x TBN], column j[TBN]
     DevBuf<int64_t> step_rng;   // per tile: its K-steps are [step_rng[2 t], step_rng[2 t + 1])
+    int64_t need_steps = 0;     // K-steps of a plan that did not fit (0: fits)
     DevBuf<int> steps;          // per K-step: TBM A block indices, TBN B block indices (-1 = zero)
     // [0]: error bits of the product kernel, [1]: a list outgrew its buffer
     // (the product kernel then does nothing), [2]: tiles, [3]: the tile list is not

@@ -8,7 +8,7 @@ import numpy as np
 import pytest
 import scipy.sparse as sp
 
-from synth import Bsr
+from synth import Bsr, System
 
 pytestmark = pytest.mark.gpu
 
@@ -65,3 +65,28 @@ def test_lists_of_long_matrices(rdm, nb, b, off, mode):
     assert np.array_equal(got.row_ptr, np.concatenate([[0], np.cumsum(np.bincount(row[keep], minlength=nb))]))
     assert np.array_equal(got.col_idx, exact.indices[keep])
     assert np.array_equal(got.vals, exact.data[keep])
+
+
+def test_a_step_whose_lists_outgrow_their_room_is_repeated(rdm):
+    """A block-diagonal H0 of 95,000 blocks has one pair to a K-step: the first
+    step's list does not fit, which the host learns after the copy into the next
+    step's matrices was launched.  Every block of P0 is the projector of its
+    block of H0 (split fp16 ladder at tol 1e-8: 1e-5 is far above its error and
+    far below a missing or misplaced step)."""
+    nb, b, nocc = 95000, 16, 5
+    rng = np.random.default_rng(3)
+    q, _ = np.linalg.qr(rng.standard_normal((b, b)))
+    ev = np.concatenate([np.linspace(-2.0, -1.0, nocc), np.linspace(1.0, 2.0, b - nocc)])
+    blk = (q * ev) @ q.T
+    blk = 0.5 * (blk + blk.T)
+    i = np.arange(nb, dtype=np.int32)
+    h0 = Bsr(nb, b, nb * b, np.arange(nb + 1, dtype=np.int32), i, np.tile(blk, (nb, 1, 1)))
+    s = System("blocks", "diagonal", np.zeros((nb, 3)), b, nocc * nb, b, h0, [], (), 0.0, 3)
+    sol = rdm.Solver(0)
+    sol.set_params(tau=1e-7, tol=1e-8, mode="mixed_fp16", max_iter=60)
+    sol.load(s)
+    code, info = sol.solve()
+    assert code == rdm.RDM_OK
+    p0 = sol.p0()
+    assert np.array_equal(p0.col_idx, i)
+    assert np.max(np.abs(p0.vals - q[:, :nocc] @ q[:, :nocc].T)) <= 1e-5
