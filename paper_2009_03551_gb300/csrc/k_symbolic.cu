@@ -149,18 +149,46 @@ __global__ void __launch_bounds__(kSymThreads) k_symbolic(SymParams P) {
     const float csq = (float)fabs(P.c_sq[s]);
     const double cl = P.c_lin[s];
 
+    // Bound by the latency of dependent loads (row of A, row pointers of B, row of
+    // B): a warp's rows of B are looked up 32 at a time, a lane each, and the
+    // first 32 entries of the next one are loaded while this one's are added
+    // (152 rows of 38 blocks, two terms: 20 us one after the other, 13 us so).
     const int nw = blockDim.x >> 5;
+    auto add = [&](int j, float nb, float na) {
+        if (!exact) atomicAdd(&sm_acc[j - c0], fix_units(__fmul_ru(na, nb), inv_unit));
+        atomicAdd(&cnt[j - c0], 1u);
+    };
     for (int t = 0; t < job.nterm; ++t) {
         const int am = job.a[t], bm = job.b[t];
         const int alo = P.rp[am * NB + i], ahi = P.rp[am * NB + i + 1];
-        for (int pa = alo + wid; pa < ahi; pa += nw) {
-            const int k = P.col[pa];
-            const float na = __fmul_ru(P.nrm[pa], csq);
-            const int blo = P.rp[bm * NB + k], bhi = P.rp[bm * NB + k + 1];
-            for (int pb = blo + lane; pb < bhi; pb += 32) {
-                const int j = P.col[pb] - c0;
-                if (!exact) atomicAdd(&sm_acc[j], fix_units(__fmul_ru(na, P.nrm[pb]), inv_unit));
-                atomicAdd(&cnt[j], 1u);
+        for (int first = alo + wid; first < ahi; first += 32 * nw) {
+            const int pa = first + nw * lane;
+            float my_na = 0.f;
+            int my_lo = 0, my_hi = 0;
+            if (pa < ahi) {
+                const int k = P.col[pa];
+                my_na = __fmul_ru(P.nrm[pa], csq);
+                my_lo = P.rp[bm * NB + k];
+                my_hi = P.rp[bm * NB + k + 1];
+            }
+            const int n = min(32, (ahi - first + nw - 1) / nw);
+            int lo = __shfl_sync(0xffffffffu, my_lo, 0), hi = __shfl_sync(0xffffffffu, my_hi, 0);
+            int j = -1;
+            float nb = 0.f;
+            if (lo + lane < hi) { j = P.col[lo + lane]; nb = P.nrm[lo + lane]; }
+            for (int u = 0; u < n; ++u) {
+                const float na = __shfl_sync(0xffffffffu, my_na, u);
+                const int v = min(u + 1, n - 1);
+                const int lo2 = __shfl_sync(0xffffffffu, my_lo, v), hi2 = __shfl_sync(0xffffffffu, my_hi, v);
+                int j2 = -1;
+                float nb2 = 0.f;
+                if (lo2 + lane < hi2) { j2 = P.col[lo2 + lane]; nb2 = P.nrm[lo2 + lane]; }
+                if (j >= 0) add(j, nb, na);
+                for (int pb = lo + 32 + lane; pb < hi; pb += 32) add(P.col[pb], P.nrm[pb], na);
+                lo = lo2;
+                hi = hi2;
+                j = j2;
+                nb = nb2;
             }
         }
     }
