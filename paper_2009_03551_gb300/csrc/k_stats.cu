@@ -42,9 +42,17 @@ __device__ __forceinline__ int warp_find_col(const int *__restrict__ col, int lo
 // elements of its share.  Bound by the FP64 pipe (2 FMAs per clock and SM); the
 // chains of a row (8 warps, 2 + nmat sums) are spread over 2 (1 + nmat) CTAs, so
 // that a system of few block rows fills the chip (38 block rows, 1,300 blocks of
-// X0: 155 us in one CTA per row, 27 us spread).
+// X0: 155 us in one CTA per row, 27 us spread, 22 us with the next 256
+// elements of a warp's share loaded while these are added, and with the blocks
+// of X looked up by 32 lanes at once).
 constexpr int kStatWarps = 8;    // warps per block row
 constexpr int kStatCta = 4;      // of them in one CTA
+
+// 256 elements, a lane every 32nd
+__device__ __forceinline__ void load8(double (&v)[8], const double *__restrict__ x) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = x[32 * k];
+}
 
 __global__ void __launch_bounds__(kStatCta * 32) k_row_stats(
     const int *__restrict__ rp, const int *__restrict__ col, const double *__restrict__ val, int NB, int b,
@@ -53,26 +61,30 @@ __global__ void __launch_bounds__(kStatCta * 32) k_row_stats(
     const int lane = threadIdx.x & 31;
     const int slot = blockIdx.x * kStatCta + (threadIdx.x >> 5);     // row, warp of the row
     const int i = slot / kStatWarps, w = slot % kStatWarps;
-    const int bb = b * b;
+    const int bb = b * b, n8 = bb >> 8;          // 256 elements at a time (blocks of 16 and more)
     const size_t nslot = (size_t)NB * kStatWarps;
     if (blockIdx.y == 0) {
         // trace and squared norm of X0
         double tr = 0.0, ss = 0.0;
-        for (int p = rp[i] + w; p < rp[i + 1]; p += kStatWarps) {
+        int p = rp[i] + w;
+        const int end = rp[i + 1];
+        double v[8], nx[8];
+        if (n8 && p < end) load8(v, val + (size_t)p * bb + lane);
+        for (; p < end; p += kStatWarps) {
             const double *x = val + (size_t)p * bb;
-            int e = lane;
-            for (; e + 224 < bb; e += 256) {
-                double v[8];
-#pragma unroll
-                for (int k = 0; k < 8; ++k) v[k] = x[e + 32 * k];
+            for (int q = 0; q < n8; ++q) {
+                const int pn = q + 1 < n8 ? p : p + kStatWarps;
+                if (pn < end) load8(nx, val + (size_t)pn * bb + (q + 1 < n8 ? 256 * (q + 1) : 0) + lane);
 #pragma unroll
                 for (int k = 0; k < 8; ++k) ss = fma(v[k], v[k], ss);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) v[k] = nx[k];
             }
-            for (; e < bb; e += 32) ss = fma(x[e], x[e], ss);
+            for (int e = 256 * n8 + lane; e < bb; e += 32) ss = fma(x[e], x[e], ss);
             if (col[p] == i)
                 // the lane's elements in order, those on the diagonal
-                for (e = lane; e < bb; e += 32)
-                    if (e / b == e % b) tr += x[e];
+                for (int e = 0; e < bb; e += b + 1)
+                    if ((e & 31) == lane) tr += x[e];
         }
         tr = warp_sum(tr);
         ss = warp_sum(ss);
@@ -85,27 +97,58 @@ __global__ void __launch_bounds__(kStatCta * 32) k_row_stats(
     // band energy of matrix m over the pattern of H0
     const int m = blockIdx.y - 1;
     const int *rpm = rp + (size_t)m * NB;
-    const int lo = rpm[i], hi = rpm[i + 1];
+    const int lo = rpm[i], hi = rpm[i + 1], hend = hrp[i + 1];
     double q = 0.0;
-    for (int ph = hrp[i] + w; ph < hrp[i + 1]; ph += kStatWarps) {
-        const int p = warp_find_col(col, lo, hi, hcol[ph], lane);
-        if (p < 0) continue;
-        const double *h = hval + (size_t)ph * bb;
-        const double *x = val + (size_t)p * bb;
-        double eb = 0.0;
-        int e = lane;
-        for (; e + 224 < bb; e += 256) {
-            double v[8], u[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                v[k] = x[e + 32 * k];
-                u[k] = h[e + 32 * k];
+    for (int first = hrp[i] + w; first < hend; first += 32 * kStatWarps) {
+        const int ph = first + kStatWarps * lane;
+        int mine = -1;                           // the block of X at H0's block ph
+        if (ph < hend) {
+            const int j = hcol[ph];
+            int a = lo, z = hi;
+            while (a < z) {
+                const int mid = (a + z) >> 1;
+                if (col[mid] < j) a = mid + 1; else z = mid;
             }
-#pragma unroll
-            for (int k = 0; k < 8; ++k) eb = fma(v[k], u[k], eb);
+            if (a < hi && col[a] == j) mine = a;
         }
-        for (; e < bb; e += 32) eb = fma(x[e], h[e], eb);
-        q += eb;
+        unsigned todo = __ballot_sync(0xffffffffu, mine >= 0);
+        if (!todo) continue;
+        int u = __ffs(todo) - 1;
+        const double *x = val + (size_t)__shfl_sync(0xffffffffu, mine, u) * bb + lane;
+        const double *h = hval + (size_t)(first + kStatWarps * u) * bb + lane;
+        double v[8], g[8], nv[8], ng[8];
+        if (n8) {
+            load8(v, x);
+            load8(g, h);
+        }
+        for (;;) {
+            todo &= todo - 1;
+            u = todo ? __ffs(todo) - 1 : 0;
+            const double *xn = val + (size_t)__shfl_sync(0xffffffffu, mine, u) * bb + lane;
+            const double *hn = hval + (size_t)(first + kStatWarps * u) * bb + lane;
+            double eb = 0.0;
+            for (int k8 = 0; k8 < n8; ++k8) {
+                if (k8 + 1 < n8) {
+                    load8(nv, x + 256 * (k8 + 1));
+                    load8(ng, h + 256 * (k8 + 1));
+                } else if (todo) {
+                    load8(nv, xn);
+                    load8(ng, hn);
+                }
+#pragma unroll
+                for (int k = 0; k < 8; ++k) eb = fma(v[k], g[k], eb);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    v[k] = nv[k];
+                    g[k] = ng[k];
+                }
+            }
+            for (int e = 256 * n8; e + lane < bb; e += 32) eb = fma(x[e], h[e], eb);
+            q += eb;
+            if (!todo) break;
+            x = xn;
+            h = hn;
+        }
     }
     q = warp_sum(q);
     if (lane == 0) row_part[(2 + m) * nslot + slot] = q;
