@@ -97,7 +97,7 @@ struct PinBuf {
     T *ensure(size_t n) {
         if (n <= cap && p) return p;
         release();
-        RDM_CUDA_TRY(cudaHostAlloc((void **)&p, n * sizeof(T), cudaHostAllocDefault));
+        RDM_CUDA_TRY(cudaHostAlloc((void **)&p, n * sizeof(T), cudaHostAllocMapped));
         cap = n;
         return p;
     }
@@ -106,25 +106,6 @@ struct PinBuf {
         p = nullptr;
         cap = 0;
     }
-};
-
-// device counters of a multiplication step (rdm_handle::counters, ints)
-enum {
-    kCtrTop = 0,         // pool_top, overflow of the symbolic phase
-    kCtrErr = 2,         // error bits of the pair lists
-    kCtrPairs = 4,       // 64 bits: pairs of all upper slots
-    kCtrClass = 6,       // 5 x 64 bits: pairs per kernel class
-    kCtrWork = 16,       // work items of the three CUDA-core classes (zeroed for every group, with the next)
-    kCtrNext = 20,       // next item to hand out, per class
-    kCtrLook = 23,       // a wait of the compaction ran out
-    kCtrInts = 24
-};
-struct HostStep {
-    int ctr[kCtrInts];
-    int nupper, kept;
-    int tc[8], oz[8];                 // TcWork::counters of the two plans
-    int pre_err;                      // error bits of the transposed positions (FP32 products)
-    int rp[kMaxJobs + 1];             // first block of every output matrix
 };
 
 struct rdm_handle {
@@ -170,7 +151,6 @@ struct rdm_handle {
     DevBuf<int> out_rp, slot_row, slot_job, slot_npair, slot_x, slot_t, work, work2, work3;
     DevBuf<int64_t> pair_off, scan_tmp64;
     DevBuf<int> pair_a, pair_b;
-    DevBuf<unsigned long long> look;                  // prefix sums of the compaction
     DevBuf<int> uidx, urp, dest, cpsrc;               // upper-slot ranks, compaction maps
     DevBuf<double> out_val, row_part, sys_q;
     DevBuf<float> out_nrm;
@@ -535,6 +515,8 @@ struct StepStats {
     // times of the launches; the last group's are added by finish_step
     float t_simt[3] = {0, 0, 0}, t_tc = 0, t_cmp = 0, t_oz = 0;
     bool oz_is_fp64 = false;                // the slice launch held FP64 products only
+    unsigned ran = 0;                       // classes of launches of the last group (add_times)
+    float all_ms = 0;                       // the whole step
     bool simt64 = true;                     // FP64 products run on the CUDA cores
     bool tc = false, oz = false, f32_t = false, pending = false;   // what check_step looks at
     double tc_flops = 0, oz_flops = 0;      // per K-step
@@ -560,18 +542,18 @@ void upload_step(rdm_handle *h, const std::vector<double> &c_lin, const std::vec
 
 // adds the times of the events of the last group, which must have completed
 void add_times(rdm_handle *h, StepStats &ss) {
-    const int ev_simt[3] = {5, 6, 4};   // events after each CUDA-core class
-    float m[6] = {0, 0, 0, 0, 0, 0};
-    cudaEventElapsedTime(&m[0], h->ev[1], h->ev[ev_simt[0]]);             // FP64 class
-    cudaEventElapsedTime(&m[1], h->ev[ev_simt[0]], h->ev[ev_simt[1]]);    // double-FP32 class
-    cudaEventElapsedTime(&m[2], h->ev[ev_simt[1]], h->ev[ev_simt[2]]);    // FP32 class (and copies)
-    cudaEventElapsedTime(&m[3], h->ev[ev_simt[2]], h->ev[2]);             // tensor-core launch
-    cudaEventElapsedTime(&m[4], h->ev[2], h->ev[7]);                      // slice-product launch
-    cudaEventElapsedTime(&m[5], h->ev[7], h->ev[3]);                      // compaction
-    for (int c = 0; c < 3; ++c) ss.t_simt[c] += m[c];
-    ss.t_tc += m[3];
-    ss.t_oz += m[4];
-    ss.t_cmp += m[5];
+    // events after each class of launches, in their order; only those of the
+    // classes that ran were recorded (an event holds the stream up for ~2 us)
+    const int ev_of[6] = {5, 6, 4, 2, 7, 3};   // FP64, double-FP32, FP32 (and copies), tensor cores, slices, compaction
+    float *const to[6] = {&ss.t_simt[0], &ss.t_simt[1], &ss.t_simt[2], &ss.t_tc, &ss.t_oz, &ss.t_cmp};
+    int prev = 1;
+    for (int k = 0; k < 6; ++k) {
+        if (!((ss.ran >> k) & 1u)) continue;
+        float m = 0;
+        cudaEventElapsedTime(&m, h->ev[prev], h->ev[ev_of[k]]);
+        *to[k] += m;
+        prev = ev_of[k];
+    }
 }
 
 // the step's times per kernel class, once the device has finished it
@@ -579,6 +561,7 @@ void finish_step(rdm_handle *h, StepStats &ss) {
     add_times(h, ss);
     float mall = 0;
     cudaEventElapsedTime(&mall, h->ev[0], h->ev[3]);
+    ss.all_ms = mall;
     const float rest = ss.t_simt[0] + ss.t_simt[1] + ss.t_simt[2] + ss.t_tc + ss.t_cmp + ss.t_oz;
     if (ss.oz_is_fp64) std::swap(ss.t_simt[0], ss.t_oz);
     ss.ms[1] = ss.t_tc;          // tensor-core products
@@ -811,7 +794,15 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
     h->out_rp.ensure(nrows + 1);
     h->urp.ensure(nrows + 1);
     h->scan_tmp64.ensure(scan_tmp_elems(nrows + 1));
-    h->counters.ensure(kCtrInts);
+    // one buffer for everything a step starts with zeros in: the counters, those
+    // of the two plans and the state of the prefix sums
+    const int TR = tc_tile_rows(b), NBT = (NB + TR - 1) / TR, nunit = njob * NBT;
+    const int64_t plan_ints = plan_counter_ints(nunit);
+    const int64_t zero_ints = kCtrInts + 2 * plan_ints + 2 * compact_look_words(nrows);
+    h->counters.ensure(zero_ints);
+    h->tcw.counters = h->counters.p + kCtrInts;
+    h->tcw_oz.counters = h->tcw.counters + plan_ints;
+    unsigned long long *look = reinterpret_cast<unsigned long long *>(h->tcw_oz.counters + plan_ints);
     HostStep *hs = h->step_host.ensure(1);
     int64_t cap = std::max<int64_t>(h->pool_cap_hint, 4 * in.total + 1024);
     SymOut so{};
@@ -819,14 +810,14 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
         if (cap > INT32_MAX / 2) throw Error{RDM_ECAPACITY, "symbolic pool exceeds 2^30 blocks"};
         h->pool_col.ensure(cap);
         h->pool_npair.ensure(cap);
-        RDM_CUDA_TRY(cudaMemsetAsync(h->counters.p, 0, kCtrInts * sizeof(int), st));
+        RDM_CUDA_TRY(cudaMemsetAsync(h->counters.p, 0, zero_ints * sizeof(int), st));
         so = SymOut{h->row_cnt.p, h->row_off.p, h->pool_col.p, h->pool_npair.p, h->counters.p + kCtrTop,
                     (int)h->pool_col.cap, h->counters.p + kCtrTop + 1,
                     reinterpret_cast<unsigned long long *>(h->counters.p + kCtrPairs)};
         launch_symbolic(in, jt, h->sd, h->S, so, st, h->prm.symbolic_hash ? kSymMaxNs + 1 : max_ns);
         scan_exclusive_pair(h->row_cnt.p, h->out_rp.p, h->urp.p, nrows, h->scan_tmp64.p, st);
-        d2h(hs->ctr, h->counters.p, kCtrInts, st);
-        d2h(&hs->nupper, h->urp.p + nrows, 1, st);
+        launch_publish(PublishArgs{hs, h->counters.p, h->urp.p + nrows, nullptr, nullptr, nullptr, nullptr, nullptr, NB, njob},
+                       st);
         sync(h);
         const int top = hs->ctr[kCtrTop], over = hs->ctr[kCtrTop + 1];
         if (!over) break;
@@ -900,7 +891,6 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
         const size_t cap = std::min(avail, std::max(totm / 16, size_t(4) << 30));
         budget = std::max<int64_t>(1, (int64_t)(cap / slot_bytes));
     }
-    const int TR = tc_tile_rows(b), NBT = (NB + TR - 1) / TR, nunit = njob * NBT;
     auto unit_row = [&](int u) {   // first flat row of super-row unit u (u = nunit: nrows)
         if (u >= nunit) return nrows;
         return (u / NBT) * NB + TR * (u % NBT);
@@ -933,7 +923,6 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
     h->out_nrm.ensure(std::max<int64_t>(nslot, 1));
     h->keep.ensure(std::max<int64_t>(nslot, 1));
     h->dest.ensure(std::max<int64_t>(nslot, 1));
-    h->look.ensure(compact_look_words(nrows));
     // the pattern of the output is written before its size is known, into room
     // for the whole mask (12 bytes per block, against b x b values for a kept one)
     out.row_ptr.ensure(nrows + 1);
@@ -943,6 +932,8 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
     for (int g = 0; g < ngroup; ++g) gslots = std::max(gslots, gslot(gunit[g + 1]) - gslot(gunit[g]));
     h->cpsrc.ensure(gslots);
     int kept = 0;
+    for (int c = 0; c < kSimt; ++c) ss.ran |= run_c[c] ? 1u << c : 0u;
+    ss.ran |= (tc ? 8u : 0u) | (any_oz ? 16u : 0u) | 32u;
     ss.tc = tc;
     ss.oz = any_oz;
     ss.f32_t = f32_t;
@@ -969,7 +960,8 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
         const int64_t steps_tc = std::min(gpairs, gpairs / 4 + 65536) + 1024, steps_oz = gpairs / 2 + 1024;
         CompactArgs ca{};
         for (int attempt = 0;; ++attempt) {
-            RDM_CUDA_TRY(cudaMemsetAsync(h->counters.p + kCtrWork, 0, (kCtrInts - kCtrWork) * sizeof(int), st));
+            if (g > 0 || attempt > 0)
+                RDM_CUDA_TRY(cudaMemsetAsync(h->counters.p + kCtrWork, 0, (zero_ints - kCtrWork) * sizeof(int), st));
             // CUDA-core work per class: the selected jobs, and in the first class
             // the copies of converged systems
             for (int c = 0; c < kSimt; ++c)
@@ -1006,19 +998,21 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
                     ac.max_work = (int)nup;
                     ac.work_next = h->counters.p + kCtrNext + c;
                     launch_numeric_simt(ac, simt_ar[c], st);
+                    RDM_CUDA_TRY(cudaEventRecord(h->ev[ev_simt[c]], st));
                 }
-                RDM_CUDA_TRY(cudaEventRecord(h->ev[ev_simt[c]], st));
             }
             ss.simt_launches += (int)(g_kernel_launches - lg);
             const long long lt = g_kernel_launches;
-            if (tc) launch_numeric_tc(a, in, jt, tc_ar, h->tcw, NB, plan, st);
-            ss.tc_launches += (int)(g_kernel_launches - lt);
-            RDM_CUDA_TRY(cudaEventRecord(h->ev[2], st));
+            if (tc) {
+                launch_numeric_tc(a, in, jt, tc_ar, h->tcw, NB, plan, st);
+                ss.tc_launches += (int)(g_kernel_launches - lt);
+                RDM_CUDA_TRY(cudaEventRecord(h->ev[2], st));
+            }
             const long long lo = g_kernel_launches;
             if (any_oz) launch_numeric_oz(a, in, jt, mcol, h->ozw, h->tcw_oz, oplan, st);
             ss.oz_launches += (int)(g_kernel_launches - lo);
             if (any_oz8) launch_diag_fp64(a, in, jt, m64, h->out_rp.p, mcol, h->sd.tier.p, r0, nr, st);
-            RDM_CUDA_TRY(cudaEventRecord(h->ev[7], st));
+            if (any_oz) RDM_CUDA_TRY(cudaEventRecord(h->ev[7], st));
 
             // compaction of the group's rows, appended after the previous groups
             ca = CompactArgs{};
@@ -1027,15 +1021,11 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
             ca.u0 = u0; ca.dest = h->dest.p; ca.new_rp = out.row_ptr.p; ca.r0 = r0; ca.nrows = nr; ca.b = b;
             ca.new_col = out.col.p; ca.new_nrm = out.nrm.p; ca.src = h->cpsrc.p; ca.d0 = kept; ca.NB = NB;
             ca.look_err = h->counters.p + kCtrLook;
-            launch_compact_rows(ca, h->look.p, st);
-            d2h(&hs->kept, out.row_ptr.p + r0 + nr, 1, st);
-            d2h(hs->ctr, h->counters.p, kCtrInts, st);
-            if (tc) d2h(hs->tc, h->tcw.counters.p, 8, st);
-            if (any_oz) d2h(hs->oz, h->tcw_oz.counters.p, 8, st);
-            if (f32_t) d2h(&hs->pre_err, h->tcw.pre_err.p, 1, st);
-            if (g == ngroup - 1 && NB)
-                RDM_CUDA_TRY(cudaMemcpy2DAsync(hs->rp, sizeof(int), out.row_ptr.p, (size_t)NB * sizeof(int), sizeof(int),
-                                               njob + 1, cudaMemcpyDeviceToHost, st));
+            launch_compact_rows(ca, look, st);
+            launch_publish(PublishArgs{hs, h->counters.p, nullptr, out.row_ptr.p + r0 + nr, tc ? h->tcw.counters : nullptr,
+                                       any_oz ? h->tcw_oz.counters : nullptr, f32_t ? h->tcw.pre_err.p : nullptr,
+                                       g == ngroup - 1 && NB ? out.row_ptr.p : nullptr, NB, njob},
+                           st);
             if (ss.pending) break;
             sync(h);
             if (check_step(h, ss)) break;
@@ -1086,13 +1076,12 @@ JobTable solve_jobs(int nd) {
 std::vector<double> stats(rdm_handle *h, MatSet &X) {
     const int nq = 3 + h->nd, parts = row_stats_parts();
     h->row_part.ensure((size_t)nq * h->NB * parts);
-    h->sys_q.ensure((size_t)nq * h->S);
-    launch_row_stats(X.row_ptr.p, X.col.p, X.val.p, X.nmat, h->NB, h->bs, h->H0.row_ptr.p,
-                     h->H0.col.p, h->H0.val.p, h->row_part.p, h->stream);
-    launch_sys_sum(h->row_part.p, nq, h->NB, h->sd.row0.p, h->sd.nbs.p, h->S, h->sys_q.p, h->stream, parts);
+    // the sums go straight to page-locked memory
     const size_t n = (size_t)nq * h->S;
     double *q = h->scalars_host.ensure(std::max(n, SysDev::step_doubles(h->S)));
-    d2h(q, h->sys_q.p, n, h->stream);
+    launch_row_stats(X.row_ptr.p, X.col.p, X.val.p, X.nmat, h->NB, h->bs, h->H0.row_ptr.p,
+                     h->H0.col.p, h->H0.val.p, h->row_part.p, h->stream);
+    launch_sys_sum(h->row_part.p, nq, h->NB, h->sd.row0.p, h->sd.nbs.p, h->S, q, h->stream, parts);
     sync(h);
     return std::vector<double>(q, q + n);
 }
@@ -1404,9 +1393,6 @@ int run_solve(rdm_handle *h, rdm_info *info_out) {
     double kms[7] = {0, 0, 0, 0, 0, 0, 0};
     int tc_launches = 0, oz_launches = 0, simt_launches = 0, max_groups = 1;
     g_dev_bytes_peak = g_dev_bytes.load();
-    cudaEvent_t ev0, ev1;
-    RDM_CUDA_TRY(cudaEventCreate(&ev0));
-    RDM_CUDA_TRY(cudaEventCreate(&ev1));
     int it = 0;
     bool any_active = true;
     std::vector<double> q = stats(h, X);      // of the current X, from here on
@@ -1552,26 +1538,22 @@ int run_solve(rdm_handle *h, rdm_info *info_out) {
             copies = copies || !act[s];
         }
         upload_step(h, c_lin, c_sq, t0, t1, act, tier_of);
-        RDM_CUDA_TRY(cudaEventRecord(ev0, st));
         MatSet &Xn = h->X[1 - h->cur];
         const int next_ar = P.mode == RDM_MODE_MIXED_BF16 ? AR_BF16X3 : mixed ? AR_FP16X3 : -1;
         StepStats sst = multiply(h, Xc, Xn, jt, tab, tiers_present, lin, copies, next_ar, true);
-        RDM_CUDA_TRY(cudaEventRecord(ev1, st));
         q = stats(h, Xn);                     // waits for the step
         if (sst.pending) {
             if (!check_step(h, sst)) {
                 // once more, waiting for the lists; the operands' buffer went to Xn
                 Xc.planes_ar = -1;
                 sst = multiply(h, Xc, Xn, jt, tab, tiers_present, lin, copies, next_ar);
-                RDM_CUDA_TRY(cudaEventRecord(ev1, st));
-                q = stats(h, Xn);
+                        q = stats(h, Xn);
             } else {
                 close_step(h, sst, Xn);
             }
         }
         finish_step(h, sst);
-        float ms = 0;
-        cudaEventElapsedTime(&ms, ev0, ev1);
+        const float ms = sst.all_ms;
         const double fpb = 2.0 * b * b * b;
         useful += (double)sst.npairs * fpb;
         flops_tc += (double)sst.pairs_tc * fpb;
@@ -1607,8 +1589,6 @@ int run_solve(rdm_handle *h, rdm_info *info_out) {
                     (long long)Xn.nnzb[0], ms, sst.ms[0], sst.ms[1], sst.ms[2] + sst.ms[3], sst.ms[4]);
         }
     }
-    cudaEventDestroy(ev0);
-    cudaEventDestroy(ev1);
 
     // polarizability: alpha[g][d] = -spin * <P1_d, H1_g>
     MatSet &Xf = h->X[h->cur];

@@ -105,6 +105,22 @@ __global__ void __launch_bounds__(32 * kRowWarps) k_compact_rows(CompactArgs c) 
     if (row && lane == 0 && mx > 0.f) atomicMax(&c.mx[r / c.NB], __float_as_uint(mx));
 }
 
+// A step's counters and sizes to page-locked host memory, in one launch: a copy
+// each holds the stream up for ~2 us, and a step had seven of them.
+__global__ void __launch_bounds__(32) k_publish(PublishArgs a) {
+    static_assert(kCtrInts <= 32 && kMaxJobs < 32, "one warp");
+    const int t = threadIdx.x;
+    if (a.ctr && t < kCtrInts) a.dst->ctr[t] = a.ctr[t];
+    if (a.tc && t < 8) a.dst->tc[t] = a.tc[t];
+    if (a.oz && t < 8) a.dst->oz[t] = a.oz[t];
+    if (a.rp && t <= a.njob) a.dst->rp[t] = a.rp[(size_t)t * a.NB];
+    if (t == 0) {
+        if (a.nupper) a.dst->nupper = *a.nupper;
+        if (a.kept) a.dst->kept = *a.kept;
+        if (a.pre_err) a.dst->pre_err = *a.pre_err;
+    }
+}
+
 // Values of the kept blocks, block sizes that the tensor cores do not take: one
 // CTA per block (grid-stride), upper blocks are copied, lower ones transposed
 // through shared memory (b x (b+1) doubles) from their upper partner, which is
@@ -263,7 +279,6 @@ void launch_build_work(const int *slot_row, const int *out_col, int64_t s0, int6
 int64_t compact_look_words(int nrows) { return kMaxJobs + lookback_words((nrows + kRowWarps - 1) / kRowWarps); }
 
 void launch_compact_rows(CompactArgs &c, unsigned long long *look, cudaStream_t st) {
-    RDM_CUDA_TRY(cudaMemsetAsync(look, 0, compact_look_words(c.nrows) * sizeof(unsigned long long), st));
     c.mx = reinterpret_cast<unsigned *>(look);
     c.look = look + kMaxJobs;
     if (c.nrows == 0) {
@@ -271,6 +286,11 @@ void launch_compact_rows(CompactArgs &c, unsigned long long *look, cudaStream_t 
         return;
     }
     k_compact_rows<<<(c.nrows + kRowWarps - 1) / kRowWarps, kRowWarps * 32, 0, st>>>(c);
+    RDM_LAUNCH_CHECK();
+}
+
+void launch_publish(const PublishArgs &a, cudaStream_t st) {
+    k_publish<<<1, 32, 0, st>>>(a);
     RDM_LAUNCH_CHECK();
 }
 

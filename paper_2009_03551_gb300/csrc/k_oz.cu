@@ -704,7 +704,7 @@ void launch_numeric_oz(const NumArgs &a, const MatSet &in, const JobTable &jt, c
     A.slices_b = ow.slices_b.p;
     A.e = ow.e.p;
     A.NB = in.NB;
-    A.tiles = w.tiles.p; A.step_rng = w.step_rng.p; A.steps = w.steps.p; A.flags = w.counters.p;
+    A.tiles = w.tiles.p; A.step_rng = w.step_rng.p; A.steps = w.steps.p; A.flags = w.counters;
     A.in_val = a.in_val; A.slot_row = a.slot_row; A.slot_job = a.slot_job; A.slot_x = a.slot_x; A.mcol = mcol;
     A.sys_of_row = a.sys_of_row; A.c_lin = a.c_lin; A.c_sq = a.c_sq; A.tau0 = a.tau0; A.tau1 = a.tau1;
     for (int p = 0; p < kMaxJobs; ++p) A.job_tau_sel[p] = a.job_tau_sel[p];
@@ -716,7 +716,7 @@ void launch_numeric_oz(const NumArgs &a, const MatSet &in, const JobTable &jt, c
         }
     }
     A.out_val = a.out_val; A.out_nrm = a.out_nrm; A.keep = a.keep; A.uidx = a.uidx; A.u0 = a.u0;
-    A.err = w.counters.p;
+    A.err = w.counters;
     A.wait_cycles = w.knobs.wait_cycles > 0 ? w.knobs.wait_cycles : kWaitCycles;
     if (ow.nslice == 8) launch_oz<8>(A, plan, ow, st);
     else launch_oz<7>(A, plan, ow, st);

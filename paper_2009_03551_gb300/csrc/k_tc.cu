@@ -875,7 +875,7 @@ void launch_tc(const NumArgs &a, const MatSet &in, const JobTable &jt, Arith ar,
     }
     TcArgs A{};
     A.planes = in.ophi.p; A.zero = w.zero.p;
-    A.tiles = w.tiles.p; A.step_rng = w.step_rng.p; A.steps = w.steps.p; A.flags = w.counters.p;
+    A.tiles = w.tiles.p; A.step_rng = w.step_rng.p; A.steps = w.steps.p; A.flags = w.counters;
     // kind::f16: D = F32 (bit 4), A/B = BF16 (1) or F16 (0), K-major, N = kTileN, M = 128
     const uint32_t ab = ar == AR_BF16X3 ? 1u : 0u;
     A.idesc = (1u << 4) | (ab << 7) | (ab << 10) | (((uint32_t)kTileN >> 3) << 17) | ((128u >> 4) << 24);
@@ -889,7 +889,7 @@ void launch_tc(const NumArgs &a, const MatSet &in, const JobTable &jt, Arith ar,
     A.tau0 = a.tau0; A.tau1 = a.tau1;
     for (int p = 0; p < kMaxJobs; ++p) A.job_tau_sel[p] = a.job_tau_sel[p];
     A.out_val = a.out_val; A.out_nrm = a.out_nrm; A.keep = a.keep; A.uidx = a.uidx; A.u0 = a.u0;
-    A.err = w.counters.p;
+    A.err = w.counters;
     A.wait_cycles = w.knobs.wait_cycles > 0 ? w.knobs.wait_cycles : kWaitCycles;
     A.hold = w.knobs.hold;
     A.runs = w.tpos_valid ? 1 : 0;
@@ -903,6 +903,8 @@ void launch_tc(const NumArgs &a, const MatSet &in, const JobTable &jt, Arith ar,
 }  // namespace
 
 bool tc_block_size_ok(int b) { return b == 16 || b == 32 || b == 64; }
+
+int64_t plan_counter_ints(int units) { return 8 + 2 * lookback_words((units + kTileRowWarps - 1) / kTileRowWarps); }
 
 int tc_tile_rows(int b) { return tc_block_size_ok(b) ? 128 / b : 4; }
 

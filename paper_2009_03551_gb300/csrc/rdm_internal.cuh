@@ -379,11 +379,39 @@ struct CompactArgs {
     int bf16, njob;
     const int *slot_job;
 };
-// pattern of the kept blocks of rows [r0, r0 + nrows) (fills mx and look from
-// `look`, compact_look_words(nrows) words of scratch), then the values of its
+// pattern of the kept blocks of rows [r0, r0 + nrows) (`look`:
+// compact_look_words(nrows) zeroed words, for mx and look), then the values of its
 // kept blocks (at most max_blocks; how many is read on the device)
 int64_t compact_look_words(int nrows);
 void launch_compact_rows(CompactArgs &c, unsigned long long *look, cudaStream_t st);
+
+// device counters of a multiplication step (ints)
+enum {
+    kCtrTop = 0,         // pool_top, overflow of the symbolic phase
+    kCtrErr = 2,         // error bits of the pair lists
+    kCtrPairs = 4,       // 64 bits: pairs of all upper slots
+    kCtrClass = 6,       // 5 x 64 bits: pairs per kernel class
+    kCtrWork = 16,       // work items of the three CUDA-core classes (zeroed for every group, with the next)
+    kCtrNext = 20,       // next item to hand out, per class
+    kCtrLook = 23,       // a wait of the compaction ran out
+    kCtrInts = 24
+};
+// what the host reads of a step, in page-locked memory
+struct HostStep {
+    int ctr[kCtrInts];
+    int nupper, kept;
+    int tc[8], oz[8];                 // TcWork::counters of the two plans
+    int pre_err;                      // error bits of the transposed positions (FP32 products)
+    int rp[kMaxJobs + 1];             // first block of every output matrix
+};
+// one launch that writes the listed values (null: not this one) into *dst,
+// which the host reads after its next wait; rp: row_ptr, every NB-th entry
+struct PublishArgs {
+    HostStep *dst;
+    const int *ctr, *nupper, *kept, *tc, *oz, *pre_err, *rp;
+    int NB, njob;
+};
+void launch_publish(const PublishArgs &a, cudaStream_t st);
 void launch_compact_copy(const CompactArgs &c, int max_blocks, cudaStream_t st);
 
 // k_lowdin.cu: out = fac[sys] * val for every block of the first NB block rows

@@ -26,8 +26,9 @@ struct TcWork {
     // [0]: error bits of the product kernel, [1]: a list outgrew its buffer
     // (the product kernel then does nothing), [2]: tiles, [3]: the tile list is not
     // complete (a wait ran out; the lists are built again), [4..5]: K-steps (64
-    // bits), [8..]: state of the tile list's prefix sums
-    DevBuf<int> counters;
+    // bits), [8..]: state of the tile list's prefix sums.  plan_counter_ints(units)
+    // ints of the caller's memory, zeroed before a plan is built
+    int *counters = nullptr;
     DevBuf<float> scale;        // per matrix: power-of-two scale of its operand planes
     DevBuf<int> tpos;           // per block (i, k) of the input set: global index of block (k, i)
     // [0]: error bits of the operand preparation (8: a transposed block missing);
@@ -61,6 +62,7 @@ struct TcPlan {
 // super-row of the CUDA-core path).
 bool tc_block_size_ok(int b);
 int tc_tile_rows(int b);
+int64_t plan_counter_ints(int units);
 
 // Convert the FP64 master values of `in` into hi/lo operand planes of
 // arithmetic `ar` in the K-major core-matrix layout of the MMA.  For fp16

@@ -446,11 +446,7 @@ TcPlan build_plan(const MatSet &in, const JobTable &jt, const SysDev &sd, const 
     TcPlan plan{};
     const int NB = in.NB, NBT = (NB + G::TBM - 1) / G::TBM;
     const int nrowt = unit1 - unit0;
-    // the counters, and behind them the running sums of k_tile_rows' CTAs
     const int rgrid = std::max(0, (nrowt + kTileRowWarps - 1) / kTileRowWarps);
-    const size_t nctr = 8 + 2 * (size_t)lookback_words(rgrid);
-    w.counters.ensure(nctr);
-    RDM_CUDA_TRY(cudaMemsetAsync(w.counters.p, 0, nctr * sizeof(int), st));
     if (nrowt <= 0 || nupper <= 0) return plan;
     // every tile of a super-row but its last one has TBN columns, each with at
     // least one upper slot
@@ -466,10 +462,10 @@ TcPlan build_plan(const MatSet &in, const JobTable &jt, const SysDev &sd, const 
     T.job_mask = job_mask;
     T.u0 = unit0; T.u1 = unit1;
     T.sys_tier = sd.tier.p;
-    T.look = reinterpret_cast<unsigned long long *>(w.counters.p + 8);
+    T.look = reinterpret_cast<unsigned long long *>(w.counters + 8);
     T.tpos = w.tpos_valid ? w.tpos.p : nullptr;
     T.tiles = w.tiles.p; T.step_rng = w.step_rng.p; T.steps = w.steps.p;
-    T.cap_steps = plan.cap_steps; T.flags = w.counters.p;
+    T.cap_steps = plan.cap_steps; T.flags = w.counters;
     static_assert(kTileRowWords == kStepWords, "one window bound for both plan builders");
     T.max_words = w.knobs.window_words > 0 && w.knobs.window_words < kTileRowWords ? w.knobs.window_words
                                                                                     : kTileRowWords;
