@@ -34,16 +34,22 @@
 // (j_0..j_7, k) wherever row k holds them all, and a copy warp moves every
 // run of slots whose blocks are neighbours in memory with one copy.
 //
-// Warp roles (384 threads, one CTA per SM, persistent over a static tile
-// schedule, tiles round robin): warps 0 and 2 issue the bulk copies into a
+// Tiles are handed out by an atomic counter: a CTA claims its next one when the
+// copies of the one before it begin (warp 3, which passes the tiles and their
+// K-step ranges on to the other warps through a ring of four entries).  Round
+// robin left the SMs idle for 14% of the launch on the 1,000-atom cluster,
+// since tiles have from a few to a few hundred K-steps (28.8 -> 24.5 ms of
+// products; 2,000 atoms 57.3 -> 47.4, slab of 5,000 atoms 263 -> 209).
+//
+// Warp roles (384 threads, one CTA per SM, persistent): warps 0 and 2 issue the bulk copies into a
 // ring of stages, every second K-step each, warp 1 owns the tensor-memory
 // allocation and one thread issues the MMAs, warps 4-11 (two per TMEM lane
 // quarter, 128 accumulator columns each) run the epilogue.  Two copy warps,
 // because finding and issuing a K-step's ~3.5 copies keeps one busy for 930
 // clocks (index load, ballots, ~100 per copy), longer than the K-step's MMAs
 // (768): with one, a K-step of the 2,000-atom cluster took 1,158 clocks, with
-// two 1,026 (919 where the operands stay in L2), and the MMA thread's wait for
-// a stage fell from 495 to 313 clocks, what L2 misses leave.  Twelve warps put
+// two 1,026 (919 where the operands stay in L2; tiles round robin), and the MMA
+// thread's wait for a stage fell from 495 to 313 clocks, what L2 misses leave.  Twelve warps put
 // three on every SM sub-partition, which allows a thread 168 registers: the
 // epilogue keeps its 128 accumulators in registers and the tile metadata in
 // shared memory, gathered a tile ahead.  At b = 64 an output block spans two
@@ -265,11 +271,22 @@ struct TcArgs {
     long long wait_cycles;        // bound of every mbarrier wait
     int hold;                     // test setting: the MMA thread waits for g_never_set first
     int runs;                     // 1: slots whose blocks are neighbours in memory share a copy
+    int *next_tile;               // tiles handed out beyond every CTA's first
     const int *pre_err;           // error bits of the operand preparation, passed on to err
 };
 
-struct __align__(8) SmemCtl {
+// one entry of the CTA's sequence of tiles
+struct __align__(16) TileEntry {
+    int64_t s0, s1;               // K-steps
+    int t;                        // >= number of tiles: the end
+};
+constexpr int kSeq = 4;           // entries kept
+constexpr int kSeqReaders = 3 + kEpiWarps;
+
+struct __align__(16) SmemCtl {
     uint64_t full[8], empty[8];
+    uint64_t seq_full[kSeq], seq_empty[kSeq], seq_go;
+    TileEntry seq[kSeq];
     uint64_t seg_full[kSegBufs], seg_empty[kSegBufs];
     uint64_t drain;
     uint64_t pair[4];             // b = 64: handshake of the two epilogue warps of a column range
@@ -354,6 +371,23 @@ __device__ __forceinline__ bool pair_sync(SmemCtl *ctl, int pair, uint32_t &roun
     return ok != 0;
 }
 
+// Entry k of the tile sequence, by a warp (LANES = 32) or by one lane (1).  Every
+// reader takes every entry once, in order.
+template <int LANES>
+__device__ __forceinline__ bool take_tile(SmemCtl *ctl, uint32_t k, int lane, volatile int *abort_flag, long long limit,
+                                          TileEntry &e) {
+    const int slot = k % kSeq;
+    // every lane waits by itself, and the reads are plain shared loads of the
+    // same address, so that what follows is uniform control flow
+    if (!mbar_wait(&ctl->seq_full[slot], (k / kSeq) & 1, abort_flag, limit)) return false;
+    const uint32_t q = smem_u32(&ctl->seq[slot]);
+    asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(e.s0), "=l"(e.s1) : "r"(q) : "memory");
+    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(e.t) : "r"(q + 16) : "memory");
+    if (LANES > 1) __syncwarp();
+    if (LANES == 1 || lane == 0) mbar_arrive(&ctl->seq_empty[slot]);
+    return true;
+}
+
 template <int B>
 __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
     using G = Geo<B>;
@@ -372,6 +406,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
         if (blockIdx.x == 0 && *A.pre_err) atomicOr(A.err, *A.pre_err);
         for (int s = 0; s < G::kStages; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
         for (int b = 0; b < kSegBufs; ++b) { mbar_init(&ctl->seg_full[b], 1); mbar_init(&ctl->seg_empty[b], kEpiWarps); }
+        for (int b = 0; b < kSeq; ++b) { mbar_init(&ctl->seq_full[b], 1); mbar_init(&ctl->seq_empty[b], kSeqReaders); }
+        mbar_init(&ctl->seq_go, 1);
         mbar_init(&ctl->drain, 1);
         for (int q = 0; q < 4; ++q) mbar_init(&ctl->pair[q], 2);
         ctl->abort_flag = 0;
@@ -404,26 +440,26 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
         uint32_t zmask[G::kStages / 2];
 #pragma unroll
         for (int k = 0; k < G::kStages / 2; ++k) zmask[k] = 0u;
-        // lq < le: the next step of this warp, in tile lt; [nq, ne): the tile
-        // after it (its range is loaded a tile ahead)
-        int lt = blockIdx.x;
-        int64_t lq = 0, le = 0, nq = 0, ne = 0;
-        if (lt < ntile) { lq = A.step_rng[2 * lt]; le = A.step_rng[2 * lt + 1]; }
-        if (lt + (int)gridDim.x < ntile) { nq = A.step_rng[2 * (lt + gridDim.x)]; ne = A.step_rng[2 * (lt + gridDim.x) + 1]; }
-        lq += pr;
+        // lq < le: the next step of this warp, in the tile of entry k - 1
+        TileEntry e{};
+        uint32_t k = 0;
+        bool more = true;
+        int64_t lq = 0, le = 0;
         // block index of this lane's slot in the warp's next step, loaded
         // while the current step's copies are issued
         int nxt = -1;
         auto fetch = [&]() {
-            while (lq >= le && lt < ntile) {
-                lt += gridDim.x;
-                lq = nq + (lq - le);
-                le = ne;
-                if (lt + (int)gridDim.x < ntile) { nq = A.step_rng[2 * (lt + gridDim.x)]; ne = A.step_rng[2 * (lt + gridDim.x) + 1]; }
+            while (more && lq >= le) {
+                more = take_tile<32>(ctl, k++, lane, abort_flag, A.wait_cycles, e) && e.t < ntile;
+                if (!more) break;
+                if (pr == 0 && lane == 0) mbar_arrive(&ctl->seq_go);
+                lq = e.s0 + (lq - le);
+                le = e.s1;
             }
-            if (lt < ntile && lane < G::kSlots) nxt = A.steps[lq * G::kSlots + lane];
+            if (more && lane < G::kSlots) nxt = A.steps[lq * G::kSlots + lane];
         };
-        for (fetch(); lt < ntile; it += 2) {
+        lq = pr;
+        for (fetch(); more; it += 2) {
             const int cur = nxt;
             lq += 2;
             fetch();
@@ -481,11 +517,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
             if (A.hold) hold_until_timeout(abort_flag, A.wait_cycles);
             uint32_t it = 0, seg = 0;
             bool issued = false;
-            int64_t n0 = 0, n1 = 0;          // step range of the next tile, loaded a tile ahead
-            if (blockIdx.x < ntile) { n0 = A.step_rng[2 * blockIdx.x]; n1 = A.step_rng[2 * blockIdx.x + 1]; }
-            for (int t = blockIdx.x; t < ntile && !*abort_flag; t += gridDim.x) {
-                const int64_t s0 = n0, s1 = n1;
-                if (t + (int)gridDim.x < ntile) { n0 = A.step_rng[2 * (t + gridDim.x)]; n1 = A.step_rng[2 * (t + gridDim.x) + 1]; }
+            TileEntry e{};
+            for (uint32_t k = 0; take_tile<1>(ctl, k, 0, abort_flag, A.wait_cycles, e) && e.t < ntile; ++k) {
+                const int64_t s0 = e.s0, s1 = e.s1;
                 bool ok = true;
                 for (int64_t q = s0; q < s1 && ok; ++seg) {
                     // one segment: up to kSegSteps K-steps into a fresh accumulator
@@ -527,6 +561,30 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
                 }
             }
         }
+    } else if (warp == 3) {
+        // ---------------- tile sequence ----------------
+        // The first tile is the CTA's own, every further one the next that no
+        // CTA has taken, claimed when the copies of the one before it begin.
+        if (lane == 0) {
+            for (uint32_t k = 0;; ++k) {
+                int t = blockIdx.x;
+                if (k > 0) {
+                    if (!mbar_wait(&ctl->seq_go, (k - 1) & 1, abort_flag, A.wait_cycles)) break;
+                    t = gridDim.x + atomicAdd(A.next_tile, 1);
+                }
+                const int slot = k % kSeq;
+                if (!mbar_wait(&ctl->seq_empty[slot], ((k / kSeq) & 1) ^ 1, abort_flag, A.wait_cycles)) break;
+                volatile TileEntry *q = &ctl->seq[slot];
+                q->t = t;
+                if (t < ntile) {
+                    q->s0 = A.step_rng[2 * t];
+                    q->s1 = A.step_rng[2 * t + 1];
+                }
+                mbar_arrive(&ctl->seq_full[slot]);
+                if (t >= ntile) break;
+            }
+        }
+        __syncwarp();
     } else if (warp >= kEpiWarp0) {
         // ---------------- epilogue: warps 4..11 ----------------
         const int eq = warp & 3;                        // TMEM lanes 32*eq .. 32*eq+31
@@ -546,12 +604,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
         };
         uint32_t seg = 0, pround = 0;
         int par = 0;
-        if (blockIdx.x < ntile) gather(blockIdx.x, 0);
-        for (int t = blockIdx.x; t < ntile && !*abort_flag; t += gridDim.x, par ^= 1) {
+        uint32_t k = 0;
+        TileEntry e{};
+        bool more = take_tile<32>(ctl, k++, lane, abort_flag, A.wait_cycles, e) && e.t < ntile;
+        if (more) gather(e.t, 0);
+        while (more && !*abort_flag) {
             const float *meta = meta2 + par * blocks_per_warp<B>() * 8;
             __syncwarp();
             const int nst = nst_next;
-            const bool more = t + (int)gridDim.x < ntile;
             if (nst < 0 && lane == 0) atomicOr(A.err, 4);
             // the tile's accumulator: sum of its segments, added with
             // round-to-nearest in registers (row 32*eq + lane, this warp's 128 columns)
@@ -563,9 +623,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
             for (int g = 0; g < nseg; ++g, ++seg) {
                 const int buf = seg & (kSegBufs - 1);
                 const uint32_t use = seg / kSegBufs;
-                if (g == (nseg > 2 ? nseg - 2 : 0) && more) {
-                    prefetch_old_blocks<B, G>(A, t + gridDim.x, eq, colhalf, lane);
-                    gather(t + gridDim.x, par ^ 1);
+                if (g == (nseg > 2 ? nseg - 2 : 0)) {
+                    more = take_tile<32>(ctl, k++, lane, abort_flag, A.wait_cycles, e) && e.t < ntile;
+                    if (more) {
+                        prefetch_old_blocks<B, G>(A, e.t, eq, colhalf, lane);
+                        gather(e.t, par ^ 1);
+                    }
                 }
                 if (!mbar_wait(&ctl->seg_full[buf], use & 1, abort_flag, A.wait_cycles)) { ok = false; break; }
                 fence_after();
@@ -582,7 +645,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
                 if (lane == 0) mbar_arrive(&ctl->seg_empty[buf]);
             }
             if (!ok) break;
-            if (nseg == 0 && more) gather(t + gridDim.x, par ^ 1);
+            if (nseg == 0) {
+                more = take_tile<32>(ctl, k++, lane, abort_flag, A.wait_cycles, e) && e.t < ntile;
+                if (more) gather(e.t, par ^ 1);
+            }
+            par ^= 1;
 
             if constexpr (B == 32) {
                 // lane l holds row l of 4 blocks of 32 columns
@@ -843,6 +910,11 @@ constexpr size_t smem_bytes() {
 }
 static_assert(smem_bytes<16>() <= 227 * 1024 && smem_bytes<32>() <= 227 * 1024 && smem_bytes<64>() <= 227 * 1024,
               "shared memory of the tensor-core kernel exceeds 227 KB");
+template <int B>
+constexpr bool ctl_aligned() {
+    return (smem_bytes<B>() - sizeof(SmemCtl)) % alignof(SmemCtl) == 0;
+}
+static_assert(ctl_aligned<16>() && ctl_aligned<32>() && ctl_aligned<64>(), "SmemCtl's alignment");
 static_assert(Geo<16>::kStages <= 8 && Geo<32>::kStages <= 8 && Geo<64>::kStages <= 8, "mbarrier arrays");
 
 template <int B>
@@ -890,6 +962,7 @@ void launch_tc(const NumArgs &a, const MatSet &in, const JobTable &jt, Arith ar,
     for (int p = 0; p < kMaxJobs; ++p) A.job_tau_sel[p] = a.job_tau_sel[p];
     A.out_val = a.out_val; A.out_nrm = a.out_nrm; A.keep = a.keep; A.uidx = a.uidx; A.u0 = a.u0;
     A.err = w.counters;
+    A.next_tile = w.counters + 6;
     A.wait_cycles = w.knobs.wait_cycles > 0 ? w.knobs.wait_cycles : kWaitCycles;
     A.hold = w.knobs.hold;
     A.runs = w.tpos_valid ? 1 : 0;

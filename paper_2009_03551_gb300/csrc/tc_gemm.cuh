@@ -26,7 +26,7 @@ struct TcWork {
     // [0]: error bits of the product kernel, [1]: a list outgrew its buffer
     // (the product kernel then does nothing), [2]: tiles, [3]: the tile list is not
     // complete (a wait ran out; the lists are built again), [4..5]: K-steps (64
-    // bits), [8..]: state of the tile list's prefix sums.  plan_counter_ints(units)
+    // bits), [6]: tiles handed out, [8..]: state of the tile list's prefix sums.  plan_counter_ints(units)
     // ints of the caller's memory, zeroed before a plan is built
     int *counters = nullptr;
     DevBuf<float> scale;        // per matrix: power-of-two scale of its operand planes
