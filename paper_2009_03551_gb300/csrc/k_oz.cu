@@ -308,6 +308,7 @@ struct OzArgs {
     const int64_t *step_rng;
     const int *steps;
     const int *flags;             // TcWork::counters
+    int *next_tile;               // tiles handed out beyond every CTA's first
     int NB;
     // epilogue
     const double *in_val;
@@ -325,7 +326,8 @@ struct OzArgs {
     long long wait_cycles;
 };
 
-struct __align__(8) OzCtl {
+struct __align__(16) OzCtl {
+    TileSeq seq;
     uint64_t full[2], empty[2];
     uint64_t seg_full[2], seg_empty[2];      // per block column of the tile
     uint64_t drain;
@@ -352,6 +354,7 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_tc_oz(OzArgs A) {
     if (threadIdx.x == 0) {
         for (int s = 0; s < G::kStages; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
         for (int b = 0; b < 2; ++b) { mbar_init(&ctl->seg_full[b], 1); mbar_init(&ctl->seg_empty[b], kOzEpiWarps / 2); }
+        init_seq(&ctl->seq, 2 + kOzEpiWarps);
         mbar_init(&ctl->drain, 1);
         ctl->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -377,8 +380,18 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_tc_oz(OzArgs A) {
 #pragma unroll
         for (int k = 0; k < G::kStages; ++k) zmask[k] = 0u;
         const uint16_t *base = lane < G::TBM ? A.slices_a : A.slices_b;
-        for (int t = blockIdx.x; t < ntile && ok; t += gridDim.x) {
-            const int64_t s0 = A.step_rng[2 * t], s1 = A.step_rng[2 * t + 1];
+        // lane 0 claims the CTA's next tile once the first copies of this one are issued
+        TileEntry e{};
+        uint32_t k = 0;
+        auto claim = [&]() {
+            if (lane == 0) put_tile(&ctl->seq, k, ntile, A.step_rng, A.next_tile, abort_flag, A.wait_cycles);
+            __syncwarp();
+        };
+        claim();
+        while (ok && take_tile<32>(&ctl->seq, k, lane, abort_flag, A.wait_cycles, e) && e.t < ntile) {
+            const int64_t s0 = e.s0, s1 = e.s1;
+            ++k;
+            if (s0 == s1) claim();
             int nxt = (s0 < s1 && lane < G::kSlots) ? A.steps[s0 * G::kSlots + lane] : -1;
             for (int64_t q = s0; q < s1; ++q, ++it) {
                 const int cur = nxt;
@@ -407,9 +420,10 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_tc_oz(OzArgs A) {
                                                    : A.zero + ((size_t)blockIdx.x * G::kSlots + lane) * G::kBlockElems;
                     bulk_g2s(stages + st * G::kStageBytes + lane * G::kBlockBytes, src, G::kBlockBytes, &ctl->full[st]);
                 }
+                if (q == s0) claim();
             }
         }
-        if (!ok && lane == 0) {
+        if ((!ok || *abort_flag) && lane == 0) {
             // after an abort, wait (bounded) for the copies still in flight
             const uint32_t n = it < (uint32_t)G::kStages ? it : (uint32_t)G::kStages;
             for (uint32_t q = it - n; q < it; ++q)
@@ -423,8 +437,9 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_tc_oz(OzArgs A) {
             const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 4) << 24);
             uint32_t it = 0, seg = 0;
             bool issued = false;
-            for (int t = blockIdx.x; t < ntile && !*abort_flag; t += gridDim.x) {
-                const int *d = A.tiles + (size_t)t * G::kTileInts;
+            TileEntry e{};
+            for (uint32_t k = 0; take_tile<1>(&ctl->seq, k, 0, abort_flag, A.wait_cycles, e) && e.t < ntile; ++k) {
+                const int *d = A.tiles + (size_t)e.t * G::kTileInts;
                 const int nst = d[3], n1 = d[2];
                 bool ok = true;
                 for (int q = 0; q < nst && ok; ++seg) {
@@ -474,8 +489,9 @@ __global__ void __launch_bounds__(kOzThreads, 1) k_tc_oz(OzArgs A) {
         const int bc = (warp - kOzEpiWarp0) >> 2;       // block column of the tile
         const uint32_t ta = tmem + ((uint32_t)(32 * eq) << 16) + bc * G::kAccCols;
         uint32_t seg = 0;
-        for (int t = blockIdx.x; t < ntile && !*abort_flag; t += gridDim.x) {
-            const int *d = A.tiles + (size_t)t * G::kTileInts;
+        TileEntry e{};
+        for (uint32_t k = 0; take_tile<32>(&ctl->seq, k, lane, abort_flag, A.wait_cycles, e) && e.t < ntile; ++k) {
+            const int *d = A.tiles + (size_t)e.t * G::kTileInts;
             const int s = d[4 + eq * G::TBN + bc];
             const int nst = d[3], n1 = d[2];
             if ((nst < 0 || n1 < 0 || n1 > nst) && lane == 0) atomicOr(A.err, 4);
@@ -717,6 +733,7 @@ void launch_numeric_oz(const NumArgs &a, const MatSet &in, const JobTable &jt, c
     }
     A.out_val = a.out_val; A.out_nrm = a.out_nrm; A.keep = a.keep; A.uidx = a.uidx; A.u0 = a.u0;
     A.err = w.counters;
+    A.next_tile = w.counters + 6;
     A.wait_cycles = w.knobs.wait_cycles > 0 ? w.knobs.wait_cycles : kWaitCycles;
     if (ow.nslice == 8) launch_oz<8>(A, plan, ow, st);
     else launch_oz<7>(A, plan, ow, st);

@@ -275,18 +275,10 @@ struct TcArgs {
     const int *pre_err;           // error bits of the operand preparation, passed on to err
 };
 
-// one entry of the CTA's sequence of tiles
-struct __align__(16) TileEntry {
-    int64_t s0, s1;               // K-steps
-    int t;                        // >= number of tiles: the end
-};
-constexpr int kSeq = 4;           // entries kept
-constexpr int kSeqReaders = 3 + kEpiWarps;
-
 struct __align__(16) SmemCtl {
     uint64_t full[8], empty[8];
-    uint64_t seq_full[kSeq], seq_empty[kSeq], seq_go;
-    TileEntry seq[kSeq];
+    TileSeq seq;
+    uint64_t seq_go;              // the copies of a tile begin: the next one may be claimed
     uint64_t seg_full[kSegBufs], seg_empty[kSegBufs];
     uint64_t drain;
     uint64_t pair[4];             // b = 64: handshake of the two epilogue warps of a column range
@@ -371,23 +363,6 @@ __device__ __forceinline__ bool pair_sync(SmemCtl *ctl, int pair, uint32_t &roun
     return ok != 0;
 }
 
-// Entry k of the tile sequence, by a warp (LANES = 32) or by one lane (1).  Every
-// reader takes every entry once, in order.
-template <int LANES>
-__device__ __forceinline__ bool take_tile(SmemCtl *ctl, uint32_t k, int lane, volatile int *abort_flag, long long limit,
-                                          TileEntry &e) {
-    const int slot = k % kSeq;
-    // every lane waits by itself, and the reads are plain shared loads of the
-    // same address, so that what follows is uniform control flow
-    if (!mbar_wait(&ctl->seq_full[slot], (k / kSeq) & 1, abort_flag, limit)) return false;
-    const uint32_t q = smem_u32(&ctl->seq[slot]);
-    asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(e.s0), "=l"(e.s1) : "r"(q) : "memory");
-    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(e.t) : "r"(q + 16) : "memory");
-    if (LANES > 1) __syncwarp();
-    if (LANES == 1 || lane == 0) mbar_arrive(&ctl->seq_empty[slot]);
-    return true;
-}
-
 template <int B>
 __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
     using G = Geo<B>;
@@ -406,7 +381,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
         if (blockIdx.x == 0 && *A.pre_err) atomicOr(A.err, *A.pre_err);
         for (int s = 0; s < G::kStages; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
         for (int b = 0; b < kSegBufs; ++b) { mbar_init(&ctl->seg_full[b], 1); mbar_init(&ctl->seg_empty[b], kEpiWarps); }
-        for (int b = 0; b < kSeq; ++b) { mbar_init(&ctl->seq_full[b], 1); mbar_init(&ctl->seq_empty[b], kSeqReaders); }
+        init_seq(&ctl->seq, 3 + kEpiWarps);
         mbar_init(&ctl->seq_go, 1);
         mbar_init(&ctl->drain, 1);
         for (int q = 0; q < 4; ++q) mbar_init(&ctl->pair[q], 2);
@@ -450,7 +425,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
         int nxt = -1;
         auto fetch = [&]() {
             while (more && lq >= le) {
-                more = take_tile<32>(ctl, k++, lane, abort_flag, A.wait_cycles, e) && e.t < ntile;
+                more = take_tile<32>(&ctl->seq, k++, lane, abort_flag, A.wait_cycles, e) && e.t < ntile;
                 if (!more) break;
                 if (pr == 0 && lane == 0) mbar_arrive(&ctl->seq_go);
                 lq = e.s0 + (lq - le);
@@ -501,7 +476,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
                          &ctl->full[st]);
             }
         }
-        if (!ok && lane == 0) {
+        if ((!ok || *abort_flag) && lane == 0) {
             // after an abort, wait (bounded) until this warp's copies still in
             // flight have landed before the CTA leaves: those of its last
             // kStages / 2 issued steps, each at the phase of its last use
@@ -518,7 +493,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
             uint32_t it = 0, seg = 0;
             bool issued = false;
             TileEntry e{};
-            for (uint32_t k = 0; take_tile<1>(ctl, k, 0, abort_flag, A.wait_cycles, e) && e.t < ntile; ++k) {
+            for (uint32_t k = 0; take_tile<1>(&ctl->seq, k, 0, abort_flag, A.wait_cycles, e) && e.t < ntile; ++k) {
                 const int64_t s0 = e.s0, s1 = e.s1;
                 bool ok = true;
                 for (int64_t q = s0; q < s1 && ok; ++seg) {
@@ -567,20 +542,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
         // CTA has taken, claimed when the copies of the one before it begin.
         if (lane == 0) {
             for (uint32_t k = 0;; ++k) {
-                int t = blockIdx.x;
-                if (k > 0) {
-                    if (!mbar_wait(&ctl->seq_go, (k - 1) & 1, abort_flag, A.wait_cycles)) break;
-                    t = gridDim.x + atomicAdd(A.next_tile, 1);
-                }
-                const int slot = k % kSeq;
-                if (!mbar_wait(&ctl->seq_empty[slot], ((k / kSeq) & 1) ^ 1, abort_flag, A.wait_cycles)) break;
-                volatile TileEntry *q = &ctl->seq[slot];
-                q->t = t;
-                if (t < ntile) {
-                    q->s0 = A.step_rng[2 * t];
-                    q->s1 = A.step_rng[2 * t + 1];
-                }
-                mbar_arrive(&ctl->seq_full[slot]);
+                if (k > 0 && !mbar_wait(&ctl->seq_go, (k - 1) & 1, abort_flag, A.wait_cycles)) break;
+                const int t = put_tile(&ctl->seq, k, ntile, A.step_rng, A.next_tile, abort_flag, A.wait_cycles);
                 if (t >= ntile) break;
             }
         }
@@ -606,7 +569,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
         int par = 0;
         uint32_t k = 0;
         TileEntry e{};
-        bool more = take_tile<32>(ctl, k++, lane, abort_flag, A.wait_cycles, e) && e.t < ntile;
+        bool more = take_tile<32>(&ctl->seq, k++, lane, abort_flag, A.wait_cycles, e) && e.t < ntile;
         if (more) gather(e.t, 0);
         while (more && !*abort_flag) {
             const float *meta = meta2 + par * blocks_per_warp<B>() * 8;
@@ -624,7 +587,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
                 const int buf = seg & (kSegBufs - 1);
                 const uint32_t use = seg / kSegBufs;
                 if (g == (nseg > 2 ? nseg - 2 : 0)) {
-                    more = take_tile<32>(ctl, k++, lane, abort_flag, A.wait_cycles, e) && e.t < ntile;
+                    more = take_tile<32>(&ctl->seq, k++, lane, abort_flag, A.wait_cycles, e) && e.t < ntile;
                     if (more) {
                         prefetch_old_blocks<B, G>(A, e.t, eq, colhalf, lane);
                         gather(e.t, par ^ 1);
@@ -646,7 +609,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_tc_bf16x3(TcArgs A) {
             }
             if (!ok) break;
             if (nseg == 0) {
-                more = take_tile<32>(ctl, k++, lane, abort_flag, A.wait_cycles, e) && e.t < ntile;
+                more = take_tile<32>(&ctl->seq, k++, lane, abort_flag, A.wait_cycles, e) && e.t < ntile;
                 if (more) gather(e.t, par ^ 1);
             }
             par ^= 1;

@@ -113,5 +113,58 @@ __device__ __forceinline__ void tmem_wait_ld(float (&v)[4][8]) {
                    "+f"(v[3][0]), "+f"(v[3][1]), "+f"(v[3][2]), "+f"(v[3][3]), "+f"(v[3][4]), "+f"(v[3][5]), "+f"(v[3][6]), "+f"(v[3][7]));
 }
 
+// ---------------------------------------------------------------------------
+// The tiles of a persistent CTA, handed from the thread that claims them to the
+// warps that work on them through a ring in shared memory.  The first tile is
+// the CTA's own, every further one the next that no CTA has taken.
+// ---------------------------------------------------------------------------
+struct __align__(16) TileEntry {
+    int64_t s0, s1;               // K-steps
+    int t;                        // >= number of tiles: the end
+};
+constexpr int kSeq = 4;           // entries kept
+struct __align__(16) TileSeq {
+    TileEntry e[kSeq];
+    uint64_t full[kSeq], empty[kSeq];
+};
+__device__ __forceinline__ void init_seq(TileSeq *q, int readers) {
+    for (int k = 0; k < kSeq; ++k) {
+        mbar_init(&q->full[k], 1);
+        mbar_init(&q->empty[k], readers);
+    }
+}
+// entry k, by one thread; returns the tile (the end too when the wait is given up)
+__device__ __forceinline__ int put_tile(TileSeq *q, uint32_t k, int ntile, const int64_t *step_rng, int *next_tile,
+                                        volatile int *abort_flag, long long limit) {
+    const int t = k == 0 ? (int)blockIdx.x : (int)gridDim.x + atomicAdd(next_tile, 1);
+    const int slot = k % kSeq;
+    if (!mbar_wait(&q->empty[slot], ((k / kSeq) & 1) ^ 1, abort_flag, limit)) return ntile;
+    volatile TileEntry *e = &q->e[slot];
+    e->t = t;
+    if (t < ntile) {
+        e->s0 = step_rng[2 * t];
+        e->s1 = step_rng[2 * t + 1];
+    }
+    mbar_arrive(&q->full[slot]);
+    return t;
+}
+// Entry k, by a warp (LANES = 32) or by one lane (1).  Every reader takes every
+// entry once, in order.  Every lane waits by itself and reads by shared loads of
+// one address, which leaves the control flow that follows uniform for the
+// compiler: read through a generic pointer, the loops over a tile's K-steps
+// and segments were compiled as divergent and 1.7 times slower.
+template <int LANES>
+__device__ __forceinline__ bool take_tile(TileSeq *q, uint32_t k, int lane, volatile int *abort_flag, long long limit,
+                                          TileEntry &e) {
+    const int slot = k % kSeq;
+    if (!mbar_wait(&q->full[slot], (k / kSeq) & 1, abort_flag, limit)) return false;
+    const uint32_t at = smem_u32(&q->e[slot]);
+    asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(e.s0), "=l"(e.s1) : "r"(at) : "memory");
+    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(e.t) : "r"(at + 16) : "memory");
+    if (LANES > 1) __syncwarp();
+    if (LANES == 1 || lane == 0) mbar_arrive(&q->empty[slot]);
+    return true;
+}
+
 }  // namespace
 }  // namespace rdm
