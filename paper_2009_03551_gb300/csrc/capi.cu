@@ -690,9 +690,9 @@ Arith fp64_arith(int mode, int b, double tau) {
 // own wait, calls check_step and close_step (StepStats::pending).  The device may
 // still be working on the compaction when the call returns (finish_step).
 constexpr size_t kDeferBytes = size_t(256) << 20;   // (a wait costs ~20 us, the room 256 MB of up to 280 GB)
-StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
-                   const Arith (*tab)[kMaxJobs], unsigned tiers_present, bool lin, bool copies, int next_ar = -1,
-                   bool defer = false) {
+StepStats multiply_once(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
+                        const Arith (*tab)[kMaxJobs], unsigned tiers_present, bool lin, bool copies, int next_ar,
+                        bool defer) {
     cudaStream_t st = h->stream;
     const int NB = in.NB, b = in.b, njob = jt.njob;
     const size_t bb = (size_t)b * b;
@@ -733,7 +733,13 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
     }
     h->ensure_events();
     RDM_CUDA_TRY(cudaEventRecord(h->ev[0], st));
-    if (any_oz && !prepare_oz_operands(in, oz_nmat, any_oz8 ? 8 : 7, h->ozw, st)) {
+    // 8-slice products have FP64 FMAs to fall back on: their slices leave room for
+    // the result (about the input set's size) and the step's buffers
+    const size_t out_bytes = (size_t)in.total * bb * sizeof(double) * 9 / 8, out_held = out.val.cap * sizeof(double);
+    const size_t grow = out_bytes > out_held ? out_bytes - out_held : 0;
+    const size_t reserve = any_oz8 ? grow + (size_t(4) << 30) : h->tcw.lean ? grow : 0;
+    if (any_oz && ((any_oz8 && h->tcw.lean) ||
+                   !prepare_oz_operands(in, oz_nmat, any_oz8 ? 8 : 7, reserve, h->ozw, st))) {
         // no room for the slices: the FP64 pipe
         for (int t = 0; t < kMaxTiers; ++t) {
             cm[0].m[t] |= ozm.m[t];
@@ -939,7 +945,7 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
     ss.f32_t = f32_t;
     ss.tc_flops = tc ? tc_step_flops(b) : 0.0;
     ss.oz_flops = any_oz ? oz_step_flops(h->ozw) : 0.0;
-    if (defer && ngroup == 1) {
+    if (defer && ngroup == 1 && !h->tcw.lean) {
         const size_t need = (size_t)ns1 * bb;
         ss.pending = need * sizeof(double) <= kDeferBytes;
         if (ss.pending && out.val.cap < need) {
@@ -1045,7 +1051,7 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
         }
         ca.new_val = out.val.p;
         ca.slot_job = h->slot_job.p;
-        if (next_ar >= 0 && ngroup == 1 && tc_block_size_ok(b) && !h->tcw.knobs.block_copies)
+        if (next_ar >= 0 && ngroup == 1 && !h->tcw.lean && tc_block_size_ok(b) && !h->tcw.knobs.block_copies)
             operands_from_compaction(ca, out, in.ophi, kept_end, njob, (Arith)next_ar, h->tcw);
         launch_compact_copy(ca, kept_end - kept, st);
         kept = kept_end;
@@ -1062,6 +1068,25 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt,
     ss.simt64 = !any_oz8;
     if (!ss.pending) close_step(h, ss, out);
     return ss;
+}
+
+// A step that runs out of memory is repeated without what it can do without: the
+// FP32 copy of the linear terms, operands written by the compaction, room for the
+// whole mask, 8-slice products (then FP64 FMAs); the solve goes on that way.
+StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt, const Arith (*tab)[kMaxJobs],
+                   unsigned tiers_present, bool lin, bool copies, int next_ar = -1, bool defer = false) {
+    try {
+        return multiply_once(h, in, out, jt, tab, tiers_present, lin, copies, next_ar, defer);
+    } catch (const Error &e) {
+        if (e.code != RDM_ENOMEM || h->tcw.lean) throw;
+    }
+    sync(h);
+    h->tcw.lean = true;
+    h->tcw.xlin.release();
+    h->ozw.slices_a.release();
+    h->ozw.slices_b.release();
+    in.planes_ar = -1;
+    return multiply_once(h, in, out, jt, tab, tiers_present, lin, copies, -1, false);
 }
 
 JobTable solve_jobs(int nd) {
@@ -1342,6 +1367,14 @@ int run_solve(rdm_handle *h, rdm_info *info_out) {
         return fail(h, RDM_EINVAL, "the mixed modes run their products on the tensor cores, which take 16 x 16, 32 x 32 or 64 x 64 blocks");
     auto t_start = std::chrono::steady_clock::now();
     const long long launches0 = g_kernel_launches;
+    // large optional buffers of the solve before: made again where there is room
+    const size_t big = (size_t(4) << 30);
+    h->tcw.lean = false;
+    if (h->tcw.xlin.cap * sizeof(float) > big) h->tcw.xlin.release();
+    if ((h->ozw.slices_a.cap + h->ozw.slices_b.cap) * sizeof(uint16_t) > big) {
+        h->ozw.slices_a.release();
+        h->ozw.slices_b.release();
+    }
     if (h->keep_assembled) init_x(h);
     else assemble(h);
     if (h->has_s && !h->keep_assembled) {
@@ -2014,6 +2047,8 @@ void release_work(rdm_handle *h) {
     h->tcw.step_rng.release();
     h->tcw.zero.release();
     h->tcw.xlin.release();
+    h->ozw.slices_a.release();
+    h->ozw.slices_b.release();
     h->pool_cap_hint = 0;
     h->solved = false;
 }

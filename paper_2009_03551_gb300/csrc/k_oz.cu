@@ -672,7 +672,7 @@ void launch_oz(OzArgs &A, const TcPlan &plan, OzWork &ow, cudaStream_t st) {
 
 }  // namespace
 
-bool prepare_oz_operands(const MatSet &in, int nmat, int slices, OzWork &w, cudaStream_t st) {
+bool prepare_oz_operands(const MatSet &in, int nmat, int slices, size_t reserve, OzWork &w, cudaStream_t st) {
     if (in.b != 32) throw Error{-1, "the slice-product (FP64-class tensor-core) path handles 32 x 32 blocks"};
     const int nrows = nmat * in.NB;
     int64_t nblk = 0;
@@ -682,7 +682,7 @@ bool prepare_oz_operands(const MatSet &in, int nmat, int slices, OzWork &w, cuda
         // room for both layouts (and their headroom), or the caller's other path
         size_t fr = 0, tot = 0;
         RDM_CUDA_TRY(cudaMemGetInfo(&fr, &tot));
-        const size_t need = 5 * elems + (size_t(1) << 30);       // 2 layouts x 2 bytes x 5/4
+        const size_t need = 5 * elems + reserve;       // 2 layouts x 2 bytes x 5/4
         if (need > fr + (w.slices_a.cap + w.slices_b.cap) * sizeof(uint16_t)) return false;
     }
     w.nslice = slices;

@@ -947,6 +947,7 @@ int tc_tile_rows(int b) { return tc_block_size_ok(b) ? 128 / b : 4; }
 namespace {
 // room for an FP32 copy of n elements, if that is at most a quarter of the free memory
 bool xlin_room(size_t n, TcWork &w) {
+    if (w.lean) return false;
     if (w.xlin.cap >= n) return true;
     size_t fr = 0, tot = 0;
     RDM_CUDA_TRY(cudaMemGetInfo(&fr, &tot));

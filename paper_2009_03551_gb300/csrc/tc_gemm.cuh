@@ -37,6 +37,7 @@ struct TcWork {
     DevBuf<float> xlin;         // FP32 values of the input set's upper blocks (layout f32_index)
     bool lin = false;           // xlin is filled for this step
     uint64_t gen = 0;           // counts the rewrites of tpos, scale and xlin
+    bool lean = false;          // memory is short: no FP32 copy
     bool xlin_valid = false;    // xlin was written with the planes
     bool tpos_valid = false;    // the planes sit at tpos and the K-step lists point there
 };
@@ -105,8 +106,9 @@ void launch_numeric_tc(const NumArgs &a, const MatSet &in, const JobTable &jt, A
 // first nmat matrices of `in` (false, with nothing done, when the device has
 // no room for them), the tile lists (128 x 64 tiles) of the jobs in job_mask,
 // and the launch (same output contract as the other numeric launches).
-// tc_step_flops / oz_step_flops: the MMA flops issued per K-step.
-bool prepare_oz_operands(const MatSet &in, int nmat, int slices, OzWork &w, cudaStream_t st);
+// tc_step_flops / oz_step_flops: the MMA flops issued per K-step; reserve:
+// bytes the slices leave free.
+bool prepare_oz_operands(const MatSet &in, int nmat, int slices, size_t reserve, OzWork &w, cudaStream_t st);
 TcPlan build_oz_plan(const MatSet &in, const JobTable &jt, const SysDev &sd, const int *out_rp, const int *mcol,
                      TcWork &w, JobMask job_mask, int unit0, int unit1, int64_t nupper, int64_t min_steps,
                      cudaStream_t st);

@@ -90,3 +90,41 @@ def test_a_step_whose_lists_outgrow_their_room_is_repeated(rdm):
     p0 = sol.p0()
     assert np.array_equal(p0.col_idx, i)
     assert np.max(np.abs(p0.vals - q[:, :nocc] @ q[:, :nocc].T)) <= 1e-5
+
+
+@pytest.mark.parametrize("mode", ["fp64", "mixed_fp16"])
+def test_solve_with_little_memory(rdm, mode):
+    """With three quarters of the memory that a solve takes when it has all it
+    wants, it goes on without its optional buffers: the split ladder to the same
+    bits (the copies it does without hold the same numbers), the FP64 mode to the
+    rounding of its products (1e-16 each, amplified by at most 2^20)."""
+    import torch
+    from synth import make_cluster
+    s = make_cluster(600, opa=8, b=32, cutoff=10.0, seed=4, dirs=("x",))
+
+    def solve():
+        sol = rdm.Solver(0)
+        sol.set_params(tau=1e-6, tol=1e-9, mode=mode, max_iter=60)
+        sol.load(s)
+        code, info = sol.solve()
+        assert code == rdm.RDM_OK
+        p1 = sol.p1(0, 0)
+        peak = info.device_bytes_peak
+        sol.close()
+        return p1, peak
+
+    ref, peak = solve()
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    hold = [torch.empty(int(free - 0.75 * peak) >> 20, 1 << 20, dtype=torch.uint8, device="cuda")]
+    try:
+        got, less = solve()
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    assert less < peak
+    if mode == "fp64":
+        assert np.array_equal(got.row_ptr, ref.row_ptr)
+        assert np.max(np.abs(got.vals - ref.vals)) <= 1e-9 * np.max(np.abs(ref.vals))
+    else:
+        assert np.array_equal(got.col_idx, ref.col_idx) and np.array_equal(got.vals, ref.vals)
