@@ -44,7 +44,8 @@ FP64_PEAK_NOTE = ("GB300 FP64: 152 SMs x 2 FP64 FMA/clk/SM x 2 flop x 2.07 GHz =
 FP32_PEAK_NOTE = "GB300 FP32: 152 SMs x 128 FMA/clk/SM x 2 flop x 2.07 GHz = 80.5 TFLOP/s"
 DENSE_MAX_N = 16000       # largest system the dense CPU oracle may be given (N x N FP64: 2 GB)
 SAMPLE_ATOMS = 250        # atoms of the carve-out the CPU oracle solves (N = 2,000)
-SLICE_PAIRS = 28          # bf16 slice pairs one FP64-class slice product issues per useful product
+SLICE_PAIRS = 28          # bf16 slice pairs one FP64-class slice product issues per useful product (7 slices)
+FP64_SLICE_PAIRS = 36     # the same with 8 slices (FP64 mode)
 # MMA work of one K-step of the tensor-core kernel at block size b: 3 products of 128 x 256 x b
 def tc_flops_per_kstep(b):
     return 3 * 2 * 128 * 256 * b
@@ -530,14 +531,20 @@ def run_ours(args, systems, wname, rank, world, torch, dist):
     issued_tc = max(0.0, issued - (kfl[1] + kfl[2] + kfl[3]) - kfl[4] * SLICE_PAIRS)
     bsz = int(last.block_size) or sys_.b
     ksteps_per_launch = issued_tc / tc_flops_per_kstep(bsz) / tc_launches if tc_launches else 0.0
+    # FP64 products of 32 x 32 blocks with a truncation threshold run as 8-slice products
+    fp64_slices = mode == "fp64" and kfl[1] > 0 and int(last.simt_launches) == 0
     classes = {
         "tc": ("k_tc_bf16x3 (tcgen05 split-precision block SpGEMM + fused truncation)", tc_ms, kfl[0],
                peaks["bf16_tflops"] * 1e12 / 3.0, "tensor",
                f"measured bf16 dense burst / 3 (a split product issues 3 MMAs per useful product; {peak_kind}, "
                "MEASURED_PEAKS.json bf16_tflops; fp16 has the same nominal rate)"),
-        "fp64": ("k_numeric_simt<32,double> (FP64 block SpGEMM + fused truncation)", f64_ms, kfl[1], 1.26e12,
+        "fp64": ("k_tc_oz<8> (tcgen05 exact bf16 slice products in place of FP64 FMAs, + fused truncation)", f64_ms,
+                 kfl[1], peaks["bf16_tflops"] * 1e12 / FP64_SLICE_PAIRS, "tensor",
+                 f"measured bf16 dense burst / {FP64_SLICE_PAIRS} (36 slice-pair MMAs per useful product; {peak_kind}, "
+                 "MEASURED_PEAKS.json bf16_tflops)") if fp64_slices else
+                ("k_numeric_simt<32,double> (FP64 block SpGEMM + fused truncation)", f64_ms, kfl[1], 1.26e12,
                  "alu", FP64_PEAK_NOTE + " (derived from unit counts and clock)"),
-        "fp32": ("k_numeric_f32_t84 (FP32 block SpGEMM + fused truncation)", f32_ms, kfl[2], 80.5e12, "alu",
+        "fp32": ("k_numeric_f32_x2 (FP32 block SpGEMM + fused truncation)", f32_ms, kfl[2], 80.5e12, "alu",
                  FP32_PEAK_NOTE + " (derived from unit counts and clock)"),
         "ff": ("k_numeric_ff_b32 (double-FP32 block SpGEMM, error-free transformations, + fused truncation)", ff_ms, kfl[3],
                80.5e12 / 12.0, "alu", FP32_PEAK_NOTE + "; 12 FP32-pipe operations per multiply-add "

@@ -663,7 +663,7 @@ void tier_arith(int mode, int tier, int njob, Arith *ar, int refine_x1 = 0, int 
 }
 
 // FP64 products of an FP64-mode step with threshold tau: 8-slice products on
-// the tensor cores for 32 x 32 blocks (12 times the FP64 pipe's rate on the
+// the tensor cores for 32 x 32 blocks (20 times the FP64 pipe's rate on the
 // 300-atom cluster, and closer to the exact product, k_oz.cu).  Their error is
 // absolute, ~2^-60 of the largest elements of a row and a column; an element
 // far below that, which an FP64 FMA chain might still resolve, lies in a block

@@ -45,6 +45,11 @@
 // segment finishes block column 0 half a step before block column 1, and the
 // next segment's first K-step starts with block column 0, so that each of the
 // two is drained by its four epilogue warps while the MMAs of the other run.
+// (Running both last steps' block column 0 before their block column 1, to hide
+// more of the draining, holds both stages longer and exposes their refill:
+// 19.1 -> 23.0 ms per solve of the 2,000-atom cluster.)  Tiles are handed out by
+// an atomic counter (round robin: 22.2 ms): the copy warp claims the next one
+// after the first copies of this one.
 //
 // Epilogue, S = 8.  The group sums are integers and are added up as integers,
 // four groups at a time in 64-bit words (units 2^-36 and 2^-68), converted
@@ -66,8 +71,8 @@
 // for S = 8) for 128 x 64 x 32 FP64-class multiply-adds.  A block needs its 8-row
 // groups equally spaced over the 4 stacked blocks (groups outermost, slices
 // inside) and B its slices (slices outermost), so both layouts are stored.
-// FP64 solve of a 300-atom cluster: products 652 ms on the FP64 pipe, 37 ms here
-// (21 TFLOP/s useful, the 2 ms of k_diag_fp64 included: the diagonal elements
+// FP64 solve of a 300-atom cluster: products 652 ms on the FP64 pipe, 33 ms here
+// (24 TFLOP/s useful, the 2 ms of k_diag_fp64 included: the diagonal elements
 // of X0^2 keep the FMA chains' rounding, because the trace decides branches).  Bounded waits and the abort drain are those of the
 // split kernel (k_tc.cu).
 #include <cuda_bf16.h>
