@@ -860,7 +860,7 @@ StepStats multiply_once(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &
     }
     const ClassMasks masks{{tcm, m64, cm[2], cm[1], moz}};
     launch_gather(so, njob, NB, h->out_rp.p, h->urp.p, mcol, h->slot_row.p, h->slot_job.p,
-                  lists ? h->slot_npair.p : nullptr, h->uidx.p, h->sd, masks,
+                  lists ? h->slot_npair.p : nullptr, h->uidx.p, h->slot_t.p, h->sd, masks,
                   reinterpret_cast<unsigned long long *>(h->counters.p + kCtrClass), st);
     if (lists) scan_exclusive_i64(h->slot_npair.p, h->pair_off.p, (int)nslot, h->scan_tmp64.p, st);
     launch_pairs(in, jt, h->sd, h->out_rp.p, mcol, h->slot_row.p, h->slot_job.p, lists ? h->pair_off.p : nullptr,
@@ -1170,6 +1170,7 @@ void concat(rdm_handle *h, std::initializer_list<SetRange> parts, MatSet &out) {
         off += a1 - a0;
     }
     launch_block_norms(out.val.p, out.nrm.p, total, b, h->stream);
+    launch_symmetric_norms(out.row_ptr.p, out.col.p, out.nrm.p, nmat, NB, h->stream);
 }
 
 // every job of jt, C = c_lin X + c_sq (A B [+ B A]) with per-system
@@ -1269,6 +1270,7 @@ void lowdin_forward(rdm_handle *h) {
     launch_scale_sys(Y.row_ptr.p, Y.col.p, Y.val.p, NB, b, h->sd.sys_of_row.p, h->sd.row0.p, h->sd.n_orb.p, fac.p, 1,
                      Y.val.p, st);
     launch_block_norms(Y.val.p, Y.nrm.p, Y.total, b, st);
+    launch_symmetric_norms(Y.row_ptr.p, Y.col.p, Y.nrm.p, 1, NB, st);
     make_identity(h, I);
     concat(h, {{&I, 0, 1}}, Z);
     JobTable jt{};
@@ -1312,6 +1314,7 @@ void lowdin_forward(rdm_handle *h) {
     launch_scale_sys(h->Zm.row_ptr.p, h->Zm.col.p, h->Zm.val.p, NB, b, h->sd.sys_of_row.p, h->sd.row0.p,
                      h->sd.n_orb.p, fac.p, 0, h->Zm.val.p, st);
     launch_block_norms(h->Zm.val.p, h->Zm.nrm.p, h->Zm.total, b, st);
+    launch_symmetric_norms(h->Zm.row_ptr.p, h->Zm.col.p, h->Zm.nrm.p, 1, NB, st);
     Y.release(); Z.release(); T.release(); YZ.release(); I.release();
     concat(h, {{&h->Zm, 0, 1}}, in);
     jt.njob = 1;
@@ -1405,6 +1408,7 @@ int run_solve(rdm_handle *h, rdm_info *info_out) {
                           X.nrm.p + h->H0.total, nd * NB, NB, b, h->sd.sys_of_row.p,
                           h->sd.row0.p, h->sd.n_orb.p, h->sd.emin.p, h->sd.emax.p, 0, st);
     }
+    launch_symmetric_norms(X.row_ptr.p, X.col.p, X.nrm.p, 1 + nd, NB, st);
     std::vector<double> emin(S), emax(S);
     d2h(emin.data(), h->sd.emin.p, S, st);
     d2h(emax.data(), h->sd.emax.p, S, st);
@@ -2609,6 +2613,7 @@ int rdm_block_product(rdm_handle *h, const rdm_bsr *A, const rdm_bsr *B, const r
             off += n;
         }
         launch_block_norms(in.val.p, in.nrm.p, top, b, t.stream);
+        launch_symmetric_norms(in.row_ptr.p, in.col.p, in.nrm.p, nm, NB, t.stream);
         t.NB = NB;
         t.b = b;
         t.nbs = {NB};

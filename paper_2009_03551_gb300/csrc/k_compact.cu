@@ -56,8 +56,8 @@ __global__ void __launch_bounds__(32 * kRowWarps) k_compact_rows(CompactArgs c) 
     const int rbeg = row ? c.out_rp[r] : 0, rend = row ? c.out_rp[r + 1] : 0;
     int n = 0;
     for (int p = rbeg + lane; p < rend; p += 32) {
-        const bool up = c.out_col[p] >= c.slot_row[p];
-        n += c.keep[up ? p : c.slot_t[p]] & kKeepBlock;
+        const int partner = c.slot_t[p];     // -1: the mask lacks it
+        n += partner >= 0 ? c.keep[c.out_col[p] >= c.slot_row[p] ? p : partner] & kKeepBlock : 0;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
@@ -85,8 +85,9 @@ __global__ void __launch_bounds__(32 * kRowWarps) k_compact_rows(CompactArgs c) 
         bool k = false;
         int src = p;
         if (p < rend) {
-            src = c.out_col[p] >= c.slot_row[p] ? p : c.slot_t[p];
-            k = (c.keep[src] & kKeepBlock) != 0;
+            const int partner = c.slot_t[p];
+            src = c.out_col[p] >= c.slot_row[p] ? p : partner;
+            k = partner >= 0 && (c.keep[src] & kKeepBlock);
         }
         const unsigned m = __ballot_sync(0xffffffffu, k);
         if (k) {

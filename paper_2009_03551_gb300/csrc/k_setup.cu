@@ -150,6 +150,23 @@ __global__ void k_block_norms(const double *__restrict__ val, float *__restrict_
     if (lane == 0) nrm[p] = __double2float_ru(sqrt(ss));
 }
 
+// The norm bounds of block (i, j) and its mirror (j, i) both become the larger of
+// the two, one warp per flat block row.  Values are symmetric to the tolerance of
+// the uploads only, and sums over a block and over its transpose round
+// differently: a mask made from unequal bounds can hold (i, j) without (j, i).
+__global__ void k_symmetric_norms(const int *__restrict__ rp, const int *__restrict__ col, int nrows, int NB,
+                                  float *__restrict__ nrm) {
+    const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (r >= nrows) return;
+    const int i = r % NB, m0 = r - i;
+    for (int p = rp[r] + (threadIdx.x & 31); p < rp[r + 1]; p += 32) {
+        const int j = col[p];
+        if (j <= i) continue;
+        const int q = find_col(col, rp[m0 + j], rp[m0 + j + 1], i);
+        if (q >= 0) nrm[p] = nrm[q] = fmaxf(nrm[p], nrm[q]);
+    }
+}
+
 __global__ void k_max_abs(const double *__restrict__ val, int64_t n, unsigned long long *out) {
     double m = 0.0;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n;
@@ -229,6 +246,13 @@ void launch_block_norms(const double *val, float *nrm, int64_t nblk, int b, cuda
     if (nblk == 0) return;
     int64_t grid = (nblk + 7) / 8;
     k_block_norms<<<(unsigned)grid, 256, 0, st>>>(val, nrm, nblk, b);
+    RDM_LAUNCH_CHECK();
+}
+
+void launch_symmetric_norms(const int *row_ptr, const int *col, float *nrm, int nmat, int NB, cudaStream_t st) {
+    const int nrows = nmat * NB;
+    if (nrows == 0) return;
+    k_symmetric_norms<<<(nrows + 7) / 8, 256, 0, st>>>(row_ptr, col, nrows, NB, nrm);
     RDM_LAUNCH_CHECK();
 }
 

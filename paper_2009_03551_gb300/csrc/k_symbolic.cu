@@ -4,7 +4,7 @@
 // Mask.  For output row i of job p (C = c_lin X + c_sq sum_t A_t B_t) every
 // column j reached by the Gustavson row expansion (Algorithm 1: for k in row
 // i of A, for j in row k of B) accumulates the bound
-//     beta_ij = |c_sq| sum_k ||A_ik|| ||B_kj||  +  |c_lin| ||X_ij||,
+//     beta_ij = sum_k ||A_ik|| ||B_kj|| |c_sq|  +  |c_lin| ||X_ij||,
 // which by the triangle inequality and Frobenius submultiplicativity is >=
 // ||C_ij||.  Column j is kept iff beta_ij >= tau (any contribution when
 // tau = 0), so every block that survives the truncation of Sec. 2.3 is in the
@@ -14,8 +14,10 @@
 //
 // Determinism and symmetry.  beta is accumulated in 64-bit fixed point (each
 // term rounded UP to a unit of tau * 2^-24 and capped), so the sum does not
-// depend on the order of the shared-memory atomics and beta_ij == beta_ji
-// exactly: the mask of a symmetric product is exactly symmetric.
+// depend on the order of the shared-memory atomics, the two norms are multiplied
+// before |c_sq|, and the norm bounds of a block and its mirror are equal
+// (k_symmetric_norms, or the compaction's copy): beta_ij == beta_ji exactly, and
+// the mask of a symmetric product is exactly symmetric.
 //
 // Pairs.  For an upper-triangle output block (j >= i) the pairs are the k in
 // row i of A_t whose block (j,k) exists in B_t (B symmetric: B_kj = B_jk^T),
@@ -155,7 +157,7 @@ __global__ void __launch_bounds__(kSymThreads) k_symbolic(SymParams P) {
     // (152 rows of 38 blocks, two terms: 20 us one after the other, 13 us so).
     const int nw = blockDim.x >> 5;
     auto add = [&](int j, float nb, float na) {
-        if (!exact) atomicAdd(&sm_acc[j - c0], fix_units(__fmul_ru(na, nb), inv_unit));
+        if (!exact) atomicAdd(&sm_acc[j - c0], fix_units(__fmul_ru(__fmul_ru(na, nb), csq), inv_unit));
         atomicAdd(&cnt[j - c0], 1u);
     };
     for (int t = 0; t < job.nterm; ++t) {
@@ -167,7 +169,7 @@ __global__ void __launch_bounds__(kSymThreads) k_symbolic(SymParams P) {
             int my_lo = 0, my_hi = 0;
             if (pa < ahi) {
                 const int k = P.col[pa];
-                my_na = __fmul_ru(P.nrm[pa], csq);
+                my_na = P.nrm[pa];
                 my_lo = P.rp[bm * NB + k];
                 my_hi = P.rp[bm * NB + k + 1];
             }
@@ -323,12 +325,12 @@ __global__ void __launch_bounds__(kSymThreads) k_symbolic_hash(SymParams P) {
         const int alo = P.rp[am * NB + i], ahi = P.rp[am * NB + i + 1];
         for (int pa = alo + wid; pa < ahi; pa += nw) {
             const int k = P.col[pa];
-            const float na = __fmul_ru(P.nrm[pa], csq);
+            const float na = P.nrm[pa];
             const int blo = P.rp[bm * NB + k], bhi = P.rp[bm * NB + k + 1];
             for (int pb = blo + lane; pb < bhi; pb += 32) {
                 const int h = hash_find(keys, P.col[pb], &sh_fill);
                 if (h < 0) { sh_bad = 1; continue; }
-                if (!exact) atomicAdd(&sm_acc[h], fix_units(__fmul_ru(na, P.nrm[pb]), inv_unit));
+                if (!exact) atomicAdd(&sm_acc[h], fix_units(__fmul_ru(__fmul_ru(na, P.nrm[pb]), csq), inv_unit));
                 atomicAdd(&cnt[h], 1u);
             }
         }
@@ -409,7 +411,7 @@ struct GatherParams {
     SymOut so;
     int nrows, NB;
     const int *out_rp, *out_urp;
-    int *out_col, *slot_row, *slot_job, *slot_npair, *uidx;
+    int *out_col, *slot_row, *slot_job, *slot_npair, *uidx, *slot_t;
     const int *sys_of_row, *active, *sys_tier;
     ClassMasks cm;
     unsigned long long *cls;
@@ -434,6 +436,7 @@ __global__ void k_gather(GatherParams P) {
         P.slot_row[dst + t] = i;
         P.slot_job[dst + t] = p;
         if (t >= nlow) P.uidx[dst + t] = u0 + (t - nlow);
+        else P.slot_t[dst + t] = -1;
         np += (unsigned long long)c;       // 0 for lower slots
     }
     const int sys = P.sys_of_row[i];
@@ -526,6 +529,9 @@ __global__ void k_pairs(PairParams P) {
             blo = lower_bound(P.col, blo, bhi, last);
         }
     }
+    // fewer than counted: the rest points at a block that exists, since the
+    // products run before the host reads the error
+    for (int64_t q = w + lane; q < wend; q += 32) P.pair_a[q] = P.pair_b[q] = 0;
     if (lane == 0 && w != wend) atomicOr(P.err, 2);
 }
 
@@ -552,11 +558,11 @@ void launch_symbolic(const MatSet &in, const JobTable &jt, const SysDev &sd, int
 }
 
 void launch_gather(const SymOut &so, int njob, int NB, const int *out_row_ptr, const int *out_urp, int *out_col,
-                   int *slot_row, int *slot_job, int *slot_npair, int *uidx, const SysDev &sd,
+                   int *slot_row, int *slot_job, int *slot_npair, int *uidx, int *slot_t, const SysDev &sd,
                    const ClassMasks &cm, unsigned long long *cls, cudaStream_t st) {
     const int nrows = njob * NB;
     if (nrows == 0) return;
-    GatherParams P{so, nrows, NB, out_row_ptr, out_urp, out_col, slot_row, slot_job, slot_npair, uidx,
+    GatherParams P{so, nrows, NB, out_row_ptr, out_urp, out_col, slot_row, slot_job, slot_npair, uidx, slot_t,
                    sd.sys_of_row.p, sd.active.p, sd.tier.p, cm, cls};
     const int wpb = 8;
     k_gather<<<(nrows + wpb - 1) / wpb, wpb * 32, 0, st>>>(P);

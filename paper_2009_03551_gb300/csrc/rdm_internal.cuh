@@ -234,6 +234,8 @@ void launch_init_scale(const int *row_ptr, const int *col, const double *hval, d
                        const int *row0, const int *n_orb, const double *emin,
                        const double *emax, int is_x0, cudaStream_t st);
 void launch_block_norms(const double *val, float *nrm, int64_t nblk, int b, cudaStream_t st);
+// norm bounds equal for every block and its mirror (the larger of the two)
+void launch_symmetric_norms(const int *row_ptr, const int *col, float *nrm, int nmat, int NB, cudaStream_t st);
 void launch_check_values(const int *row_ptr, const int *col, const double *val, int64_t nval,
                          int NB, int b, const int *sys_of_row, const int *row0, const int *n_orb,
                          double rel_tol, int *err, cudaStream_t st);
@@ -276,12 +278,13 @@ void launch_symbolic(const MatSet &in, const JobTable &jt, const SysDev &sd, int
 // Gathers the pool into the output pattern: columns, row and job of every
 // slot, its pair count (slot_npair may be null), and uidx, the rank of an
 // upper slot (col >= row) among the upper slots (out_urp: their count before
-// each row).  cls accumulates the pairs of active systems per kernel class.
+// each row); slot_t of a lower slot is -1 until launch_pairs finds its partner.
+// cls accumulates the pairs of active systems per kernel class.
 struct ClassMasks {
     JobMask m[5];        // tensor cores, FP64, FP32, double-FP32, tensor-core slices
 };
 void launch_gather(const SymOut &so, int njob, int NB, const int *out_row_ptr, const int *out_urp, int *out_col,
-                   int *slot_row, int *slot_job, int *slot_npair, int *uidx, const SysDev &sd,
+                   int *slot_row, int *slot_job, int *slot_npair, int *uidx, int *slot_t, const SysDev &sd,
                    const ClassMasks &cm, unsigned long long *cls, cudaStream_t st);
 // pair lists of the jobs in `fill` (pair_off: offsets of every slot's list;
 // null when no job is) and slot_x / slot_t of every slot
@@ -349,6 +352,8 @@ void launch_build_work(const int *slot_row, const int *out_col, int64_t s0, int6
                        int with_inactive);
 // Compaction of the rows [r0, r0 + nrows) of the mask.  An upper slot is kept
 // on its own flag; a lower slot t on that of its upper partner slot_t[t],
+// (a slot without a partner is dropped, whatever its flag: no index is taken
+// from it, and the host reads the error bit of the pair lists afterwards)
 // and receives that block's transpose, read from out_val when the partner
 // belongs to the current group (uidx >= u0) and otherwise from the already
 // compacted output (dest[partner]).  dest[s] receives the output position of
