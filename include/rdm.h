@@ -415,12 +415,14 @@ typedef struct {
                                 positions and every block is one bulk copy (0: at the positions of the
                                 transposed blocks, so that neighbouring slots of a K-step share a copy).
                                 Results do not depend on it. */
-    int32_t pad0;            /* zero */
+    int32_t inject;          /* failures of the next step, which is then repeated with the same results:
+                                1: a wait of the tile lists' prefix sums runs out, 2: one of the
+                                compaction's, 4: the K-step lists find no room; sums of these */
 } rdm_test_knobs;
 
 /* Set the test settings of h (NULL restores all zeros).  RDM_EINVAL for a
- * negative value, a window that is not a multiple of 32 up to 16,384, or a
- * flag other than 0 or 1. */
+ * negative value, a window that is not a multiple of 32 up to 16,384, a flag
+ * other than 0 or 1, or an `inject` above 7. */
 int rdm_set_test_knobs(rdm_handle *h, const rdm_test_knobs *k);
 
 /* Library version string. */

@@ -24,6 +24,7 @@
 #include <vector>
 
 #include "../../include/rdm.h"
+#include "lookback.cuh"
 #include "rdm_internal.cuh"
 #include "tc_gemm.cuh"
 
@@ -575,10 +576,10 @@ void finish_step(rdm_handle *h, StepStats &ss) {
 
 // Once the counters of a group's launches are on the host: throws what the
 // kernels report; false: a K-step list outgrew its buffer (the next lists get
-// the room) and the launches have to be repeated.
+// the room) or a wait between the CTAs of a prefix sum ran out, and the launches
+// have to be repeated.
 bool check_step(rdm_handle *h, StepStats &ss) {
     const HostStep *hs = h->step_host.p;
-    if (hs->ctr[kCtrLook]) throw Error{RDM_ETIMEOUT, "compaction: a wait for other blocks of the kernel ran out"};
     if (hs->ctr[kCtrErr])
         throw Error{RDM_ECUDA,
                     "internal error: pair lists inconsistent with the mask (code " + std::to_string(hs->ctr[kCtrErr]) + ")"};
@@ -589,6 +590,7 @@ bool check_step(rdm_handle *h, StepStats &ss) {
         h->tcw_oz.need_steps = nst_oz;
         return false;
     }
+    if (hs->ctr[kCtrLook]) return false;
     h->tcw.need_steps = h->tcw_oz.need_steps = 0;
     const int err = (ss.f32_t ? hs->pre_err & 8 : 0) | (ss.tc ? hs->tc[0] : 0) | (ss.oz ? hs->oz[0] : 0);
     if (err & 8) throw Error{RDM_EBADBSR, "an operand's block pattern is not symmetric"};
@@ -1027,6 +1029,8 @@ StepStats multiply_once(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &
             ca.u0 = u0; ca.dest = h->dest.p; ca.new_rp = out.row_ptr.p; ca.r0 = r0; ca.nrows = nr; ca.b = b;
             ca.new_col = out.col.p; ca.new_nrm = out.nrm.p; ca.src = h->cpsrc.p; ca.d0 = kept; ca.NB = NB;
             ca.look_err = h->counters.p + kCtrLook;
+            ca.look_polls = h->tcw.knobs.inject & kInjectRowWait ? 0 : kLookPolls;
+            h->tcw.knobs.inject &= ~kInjectRowWait;
             launch_compact_rows(ca, look, st);
             launch_publish(PublishArgs{hs, h->counters.p, nullptr, out.row_ptr.p + r0 + nr, tc ? h->tcw.counters : nullptr,
                                        any_oz ? h->tcw_oz.counters : nullptr, f32_t ? h->tcw.pre_err.p : nullptr,
@@ -1035,7 +1039,10 @@ StepStats multiply_once(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &
             if (ss.pending) break;
             sync(h);
             if (check_step(h, ss)) break;
-            if (attempt == 3) throw Error{RDM_ECAPACITY, "K-step lists outgrew their buffers repeatedly"};
+            if (attempt < 3) continue;
+            if (hs->ctr[kCtrLook] || (tc && hs->tc[3]) || (any_oz && hs->oz[3]))
+                throw Error{RDM_ETIMEOUT, "a wait for other blocks of a kernel ran out repeatedly"};
+            throw Error{RDM_ECAPACITY, "K-step lists outgrew their buffers repeatedly"};
         }
         // blocks up to this group's end: not known yet if the result is not
         // waited for, then at most the mask's
@@ -1584,7 +1591,7 @@ int run_solve(rdm_handle *h, rdm_info *info_out) {
                 // once more, waiting for the lists; the operands' buffer went to Xn
                 Xc.planes_ar = -1;
                 sst = multiply(h, Xc, Xn, jt, tab, tiers_present, lin, copies, next_ar);
-                        q = stats(h, Xn);
+                q = stats(h, Xn);
             } else {
                 close_step(h, sst, Xn);
             }
@@ -2468,12 +2475,13 @@ int rdm_set_test_knobs(rdm_handle *h, const rdm_test_knobs *k) {
     if (!k) k = &z;
     if (k->tc_wait_cycles < 0 || k->tc_hold < 0 || k->tc_hold > 1 || k->tc_window_cols < 0 ||
         k->tc_window_cols > 16384 || (k->tc_window_cols & 31) || k->tc_block_copies < 0 ||
-        k->tc_block_copies > 1 || k->pad0 != 0)
+        k->tc_block_copies > 1 || k->inject < 0 || k->inject > 7)
         return fail(h, RDM_EINVAL, "invalid test settings");
     h->tcw.knobs.wait_cycles = k->tc_wait_cycles;
     h->tcw.knobs.hold = k->tc_hold;
     h->tcw.knobs.window_words = k->tc_window_cols / 32;
     h->tcw.knobs.block_copies = k->tc_block_copies;
+    h->tcw.knobs.inject = h->tcw_oz.knobs.inject = k->inject;
     return RDM_OK;
 }
 

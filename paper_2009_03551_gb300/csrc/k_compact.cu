@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(32 * kRowWarps) k_compact_rows(CompactArgs c) 
         total += cnt_s[k];
     }
     if (wq == 0) {
-        const int first = lookback_sum(c.look, bid, total, c.look_err) + c.d0;
+        const int first = lookback_sum(c.look, bid, total, c.look_err, c.look_polls) + c.d0;
         if (lane == 0) {
             sh_base = first;
             if (bid == (int)gridDim.x - 1) c.new_rp[c.r0 + c.nrows] = first + total;
@@ -128,6 +128,7 @@ __global__ void __launch_bounds__(32) k_publish(PublishArgs a) {
 // in this group's buffer or already compacted.
 __global__ void __launch_bounds__(128) k_compact_vals(CompactArgs c) {
     extern __shared__ double tile[];
+    if (*c.look_err) return;                 // src is not complete: the host repeats the step
     const int d1 = c.new_rp[c.r0 + c.nrows];
     const int b = c.b, bb = b * b, ld = b + 1;
     for (int d = c.d0 + blockIdx.x; d < d1; d += gridDim.x) {
@@ -161,6 +162,7 @@ __global__ void __launch_bounds__(128) k_compact_vals(CompactArgs c) {
 // 150 atoms, 5,500 blocks: 16.5 + 13.5 us, 21 in one, and four launches less).
 template <int B, int PL>
 __global__ void __launch_bounds__(128) k_compact_blocks(CompactArgs c) {
+    if (*c.look_err) return;
     const int d1 = c.new_rp[c.r0 + c.nrows];
     constexpr int BB = B * B, C8 = B / 8;
     const int lane = threadIdx.x & 31;

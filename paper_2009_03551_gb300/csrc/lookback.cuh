@@ -11,7 +11,9 @@
 namespace rdm {
 namespace {
 
-constexpr long long kLookCycles = 200000000ll;   // ~0.1 s
+// A wait is bounded by the number of looks (~1 us each), not by the clock, which
+// runs on while the whole context is descheduled.
+constexpr int kLookPolls = 1 << 21;
 
 // 64-bit words of state for `grid` CTAs, zeroed before the launch: the number of
 // CTAs that have started, then per CTA 1 << 32 | sum or 2 << 32 | prefix + sum
@@ -25,8 +27,10 @@ __device__ __forceinline__ int lookback_id(unsigned long long *look, int *sh) {
 }
 
 // sum over the CTAs numbered below `bid`, all lanes of one warp; `total`: this
-// CTA's sum.  On timeout *err is set and the missing sums count as 0.
-__device__ __forceinline__ int lookback_sum(unsigned long long *look, int bid, int total, int *err) {
+// CTA's sum.  A wait that runs out sets *err and the missing sums count as 0, so
+// that a place computed from them is too small but never outside the list
+// (polls = 0, a test setting: every wait runs out).
+__device__ __forceinline__ int lookback_sum(unsigned long long *look, int bid, int total, int *err, int polls) {
     const int lane = threadIdx.x & 31;
     volatile unsigned long long *st = look + 1;
     if (lane == 0) st[bid] = ((bid == 0 ? 2ull : 1ull) << 32) | (unsigned)total;
@@ -35,9 +39,8 @@ __device__ __forceinline__ int lookback_sum(unsigned long long *look, int bid, i
     for (int j = bid - 1;; j -= 32) {
         unsigned long long v = 2ull << 32;
         if (j - lane >= 0) {
-            v = st[j - lane];
-            const long long t0 = clock64();
-            while (v == 0ull && clock64() - t0 < kLookCycles) v = st[j - lane];
+            v = 0ull;
+            for (int n = 0; v == 0ull && n < polls; ++n) v = st[j - lane];
             if (v == 0ull) {
                 atomicOr(err, 1);
                 v = 2ull << 32;

@@ -374,7 +374,8 @@ struct CompactArgs {
     int NB;
     unsigned *mx;           // per matrix: largest block norm of the group (bit pattern)
     unsigned long long *look;
-    int *look_err;          // set when a wait for other CTAs ran out
+    int look_polls;         // bound of the waits for other CTAs (lookback.cuh)
+    int *look_err;          // set when one ran out: the pattern is not complete and no values are copied
     // the next step's operands (null: not made): planes at the transposed
     // positions, those positions, operand scales, FP32 copy for the linear
     // terms (may be null)
@@ -386,7 +387,8 @@ struct CompactArgs {
 };
 // pattern of the kept blocks of rows [r0, r0 + nrows) (`look`:
 // compact_look_words(nrows) zeroed words, for mx and look), then the values of its
-// kept blocks (at most max_blocks; how many is read on the device)
+// kept blocks (at most max_blocks; how many is read on the device).  In a pattern
+// that a wait cut short, row pointers and columns lie inside the mask's room.
 int64_t compact_look_words(int nrows);
 void launch_compact_rows(CompactArgs &c, unsigned long long *look, cudaStream_t st);
 

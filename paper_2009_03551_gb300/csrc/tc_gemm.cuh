@@ -7,7 +7,9 @@ namespace rdm {
 
 // Test settings of the tensor-core path (rdm_set_test_knobs); zeros keep the
 // production behaviour.
+constexpr int kInjectTileWait = 1, kInjectRowWait = 2, kInjectStepRoom = 4;
 struct TcKnobs {
+    int inject = 0;             // kInject*: failures of one plan or compaction to come
     long long wait_cycles = 0;  // bound of every mbarrier wait in SM clock cycles (0: ~2 s)
     int hold = 0;               // 1: the MMA thread first waits for a flag that nothing sets
     int window_words = 0;       // bitmap window of the tile-plan builders in 32-column words

@@ -36,6 +36,7 @@ struct TileBuild {
     JobMask job_mask;    // jobs computed on the tensor cores, per tier
     int u0, u1;          // super-row units (job * NBT + I) of this plan
     unsigned long long *look;   // running sums of k_tile_rows' CTAs (lookback.cuh), zeroed
+    int look_polls;             // bound of its waits
     int *tiles;          // [ntile * kTileInts]
     int64_t *step_rng;   // [2 ntile]: a tile's K-steps are [step_rng[2 t], step_rng[2 t + 1])
     int *steps;          // [nsteps * kSlots]
@@ -148,7 +149,7 @@ __global__ void __launch_bounds__(32 * kTileRowWarps) k_tile_rows(TileBuild T) {
 #pragma unroll
     for (int k = 0; k < kTileRowWarps; ++k) total += cnt_s[k];
     if (wq == 0) {
-        const int first = lookback_sum(T.look, bid, total, T.flags + 3);
+        const int first = lookback_sum(T.look, bid, total, T.flags + 3, T.look_polls);
         if (lane == 0) {
             sh_base = first;
             if (bid == (int)gridDim.x - 1) T.flags[2] = first + total;
@@ -467,6 +468,10 @@ TcPlan build_plan(const MatSet &in, const JobTable &jt, const SysDev &sd, const 
     w.step_rng.ensure(2 * (size_t)max_tile);
     w.steps.ensure((size_t)std::max<int64_t>(min_steps, 1) * G::kSlots);
     plan.cap_steps = (int64_t)(w.steps.cap / G::kSlots);
+    // test settings, each for one plan
+    const int inject = w.knobs.inject & (kInjectTileWait | kInjectStepRoom);
+    w.knobs.inject &= ~inject;
+    if (inject & kInjectStepRoom) plan.cap_steps = 1;
     TileBuild T{};
     T.rp = in.row_ptr.p; T.col = in.col.p; T.NB = NB; T.NBT = NBT; T.jt = jt;
     T.out_rp = out_rp; T.mcol = mcol; T.sys_of_row = sd.sys_of_row.p; T.active = sd.active.p;
@@ -474,6 +479,7 @@ TcPlan build_plan(const MatSet &in, const JobTable &jt, const SysDev &sd, const 
     T.u0 = unit0; T.u1 = unit1;
     T.sys_tier = sd.tier.p;
     T.look = reinterpret_cast<unsigned long long *>(w.counters + 8);
+    T.look_polls = inject & kInjectTileWait ? 0 : kLookPolls;
     T.tpos = w.tpos_valid ? w.tpos.p : nullptr;
     T.tiles = w.tiles.p; T.step_rng = w.step_rng.p; T.steps = w.steps.p;
     T.cap_steps = plan.cap_steps; T.flags = w.counters;

@@ -85,7 +85,7 @@ class rdm_info(C.Structure):
 
 class rdm_test_knobs(C.Structure):
     _fields_ = [("tc_wait_cycles", C.c_int64), ("tc_hold", C.c_int32), ("tc_window_cols", C.c_int32),
-                ("tc_block_copies", C.c_int32), ("pad0", C.c_int32)]
+                ("tc_block_copies", C.c_int32), ("inject", C.c_int32)]
 
 
 class rdm_iter_log(C.Structure):
@@ -387,10 +387,10 @@ def rdm_bsr_dot_noalloc(A, B, out_ptr: int, stream=None) -> None:
 
 
 def rdm_set_test_knobs(h, tc_wait_cycles: int = 0, tc_hold: int = 0, tc_window_cols: int = 0,
-                       tc_block_copies: int = 0) -> None:
+                       tc_block_copies: int = 0, inject: int = 0) -> None:
     """Test settings of the tensor-core path (see include/rdm.h); all zeros
     restore production behaviour."""
-    k = rdm_test_knobs(tc_wait_cycles, tc_hold, tc_window_cols, tc_block_copies, 0)
+    k = rdm_test_knobs(tc_wait_cycles, tc_hold, tc_window_cols, tc_block_copies, inject)
     _check(h, _lib.rdm_set_test_knobs(h, C.byref(k)))
 
 
