@@ -506,8 +506,8 @@ void init_sys_scalars(rdm_handle *h) {
 struct StepStats {
     int64_t npairs = 0;
     int64_t nslot = 0;
-    int64_t pairs_tc = 0, pairs_64 = 0, pairs_32 = 0, pairs_ff = 0, pairs_oz = 0;   // block triples per class
-    int64_t pairs_simt = 0;                 // block triples computed on the CUDA cores
+    // block triples per class (64: FP64 FMAs, oz: 7 slices, oz8: FP64 products as 8 slices)
+    int64_t pairs_tc = 0, pairs_64 = 0, pairs_32 = 0, pairs_ff = 0, pairs_oz = 0, pairs_oz8 = 0;
     double issued_tc = 0, issued_oz = 0;
     double bytes = 0;
     double ms[7] = {0, 0, 0, 0, 0, 0, 0};   // symbolic, tc, fp64, fp32, compaction, double-fp32, slice products
@@ -515,10 +515,9 @@ struct StepStats {
     int groups = 1;                         // job groups of the numeric phase
     // times of the launches; the last group's are added by finish_step
     float t_simt[3] = {0, 0, 0}, t_tc = 0, t_cmp = 0, t_oz = 0;
-    bool oz_is_fp64 = false;                // the slice launch held FP64 products only
+    bool oz8 = false;                       // the slice launch holds FP64 products
     unsigned ran = 0;                       // classes of launches of the last group (add_times)
     float all_ms = 0;                       // the whole step
-    bool simt64 = true;                     // FP64 products run on the CUDA cores
     bool tc = false, oz = false, f32_t = false, pending = false;   // what check_step looks at
     double tc_flops = 0, oz_flops = 0;      // per K-step
 };
@@ -564,13 +563,13 @@ void finish_step(rdm_handle *h, StepStats &ss) {
     cudaEventElapsedTime(&mall, h->ev[0], h->ev[3]);
     ss.all_ms = mall;
     const float rest = ss.t_simt[0] + ss.t_simt[1] + ss.t_simt[2] + ss.t_tc + ss.t_cmp + ss.t_oz;
-    if (ss.oz_is_fp64) std::swap(ss.t_simt[0], ss.t_oz);
     ss.ms[1] = ss.t_tc;          // tensor-core products
-    ss.ms[2] = ss.t_simt[0];     // FP64 products: on the CUDA cores, or slices
+    // FP64 products: on the CUDA cores and as slices, a job's threshold decides
+    ss.ms[2] = ss.t_simt[0] + (ss.oz8 ? ss.t_oz : 0.f);
     ss.ms[3] = ss.t_simt[2];     // FP32 products (and copies of converged systems)
     ss.ms[4] = ss.t_cmp;
     ss.ms[5] = ss.t_simt[1];     // double-FP32 products
-    ss.ms[6] = ss.t_oz;          // tensor-core slice products
+    ss.ms[6] = ss.oz8 ? 0.f : ss.t_oz;   // tensor-core slice products
     ss.ms[0] = std::max(0.f, mall - rest);   // mask, lists, plans
 }
 
@@ -610,7 +609,7 @@ void close_step(rdm_handle *h, StepStats &ss, MatSet &out) {
     ss.pairs_32 = (int64_t)cls[2];
     ss.pairs_ff = (int64_t)cls[3];
     ss.pairs_oz = (int64_t)cls[4];
-    ss.pairs_simt = (ss.simt64 ? ss.pairs_64 : 0) + ss.pairs_32 + ss.pairs_ff;
+    ss.pairs_oz8 = (int64_t)cls[5];
     out.total = hs->kept;
     out.nnzb.assign(out.nmat, 0);
     for (int p = 0; p < out.nmat; ++p) out.nnzb[p] = hs->rp[p + 1] - hs->rp[p];
@@ -704,7 +703,7 @@ StepStats multiply_once(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &
     // CUDA-core classes, launched in this order: FP64, double-FP32, FP32
     constexpr int kSimt = 3;
     const Arith simt_ar[kSimt] = {AR_FP64, AR_FF, AR_FP32};
-    JobMask tcm{}, cm[kSimt]{}, simt{}, ozm{}, m64{}, moz{};   // m64, moz: accounting (FP64, slices)
+    JobMask tcm{}, cm[kSimt]{}, simt{}, ozm{}, moz{}, moz8{};   // ozm = moz or moz8
     Arith tc_ar = AR_FP16X3;
     bool any_tc = false, any_oz = false, any_oz8 = false, any_c[kSimt] = {false, false, false};
     int oz_nmat = 0;
@@ -714,7 +713,7 @@ StepStats multiply_once(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &
             const Arith a = tab[t][p];
             if (a == AR_OZ || a == AR_OZ8) {
                 ozm.m[t] |= 1u << p;
-                (a == AR_OZ ? moz : m64).m[t] |= 1u << p;
+                (a == AR_OZ ? moz : moz8).m[t] |= 1u << p;
                 any_oz = true;
                 any_oz8 = any_oz8 || a == AR_OZ8;
                 for (int k = 0; k < jt.job[p].nterm; ++k)
@@ -731,7 +730,6 @@ StepStats multiply_once(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &
             cm[c].m[t] |= 1u << p;
             any_c[c] = true;
         }
-        m64.m[t] |= cm[0].m[t];
     }
     h->ensure_events();
     RDM_CUDA_TRY(cudaEventRecord(h->ev[0], st));
@@ -745,7 +743,7 @@ StepStats multiply_once(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &
         // no room for the slices: the FP64 pipe
         for (int t = 0; t < kMaxTiers; ++t) {
             cm[0].m[t] |= ozm.m[t];
-            ozm.m[t] = 0;
+            ozm.m[t] = moz.m[t] = moz8.m[t] = 0;
         }
         any_oz = any_oz8 = false;
         any_c[0] = true;
@@ -860,7 +858,7 @@ StepStats multiply_once(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &
         h->pair_a.ensure(std::max<int64_t>(npairs, 1));
         h->pair_b.ensure(std::max<int64_t>(npairs, 1));
     }
-    const ClassMasks masks{{tcm, m64, cm[2], cm[1], moz}};
+    const ClassMasks masks{{tcm, cm[0], cm[2], cm[1], moz, moz8}};
     launch_gather(so, njob, NB, h->out_rp.p, h->urp.p, mcol, h->slot_row.p, h->slot_job.p,
                   lists ? h->slot_npair.p : nullptr, h->uidx.p, h->slot_t.p, h->sd, masks,
                   reinterpret_cast<unsigned long long *>(h->counters.p + kCtrClass), st);
@@ -944,6 +942,7 @@ StepStats multiply_once(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &
     ss.ran |= (tc ? 8u : 0u) | (any_oz ? 16u : 0u) | 32u;
     ss.tc = tc;
     ss.oz = any_oz;
+    ss.oz8 = any_oz8;
     ss.f32_t = f32_t;
     ss.tc_flops = tc ? tc_step_flops(b) : 0.0;
     ss.oz_flops = any_oz ? oz_step_flops(h->ozw) : 0.0;
@@ -1019,7 +1018,7 @@ StepStats multiply_once(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &
             const long long lo = g_kernel_launches;
             if (any_oz) launch_numeric_oz(a, in, jt, mcol, h->ozw, h->tcw_oz, oplan, st);
             ss.oz_launches += (int)(g_kernel_launches - lo);
-            if (any_oz8) launch_diag_fp64(a, in, jt, m64, h->out_rp.p, mcol, h->sd.tier.p, r0, nr, st);
+            if (any_oz8) launch_diag_fp64(a, in, jt, moz8, h->out_rp.p, mcol, h->sd.tier.p, r0, nr, st);
             if (any_oz) RDM_CUDA_TRY(cudaEventRecord(h->ev[7], st));
 
             // compaction of the group's rows, appended after the previous groups
@@ -1068,11 +1067,8 @@ StepStats multiply_once(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &
             add_times(h, ss);
         }
     }
-    ss.oz_is_fp64 = any_oz8;
-    for (int t = 0; t < kMaxTiers; ++t) ss.oz_is_fp64 = ss.oz_is_fp64 && !moz.m[t];
     ss.bytes = ((double)in.total * (tc ? 4.0 : 8.0) + (any_oz ? (double)in.nnzb[0] * 2.0 * h->ozw.nslice : 0.0) +
                 (double)nupper * 8.0) * (double)bb;
-    ss.simt64 = !any_oz8;
     if (!ss.pending) close_step(h, ss, out);
     return ss;
 }
@@ -1601,11 +1597,11 @@ int run_solve(rdm_handle *h, rdm_info *info_out) {
         const double fpb = 2.0 * b * b * b;
         useful += (double)sst.npairs * fpb;
         flops_tc += (double)sst.pairs_tc * fpb;
-        flops_64 += (double)sst.pairs_64 * fpb;
+        flops_64 += (double)(sst.pairs_64 + sst.pairs_oz8) * fpb;
         flops_32 += (double)sst.pairs_32 * fpb;
         flops_ff += (double)sst.pairs_ff * fpb;
         flops_oz += (double)sst.pairs_oz * fpb;
-        issued += sst.issued_tc + sst.issued_oz + (double)sst.pairs_simt * fpb;
+        issued += sst.issued_tc + sst.issued_oz + (double)(sst.pairs_64 + sst.pairs_32 + sst.pairs_ff) * fpb;
         nbytes += sst.bytes;
         tc_launches += sst.tc_launches;
         oz_launches += sst.oz_launches;

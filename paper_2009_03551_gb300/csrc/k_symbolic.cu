@@ -443,7 +443,7 @@ __global__ void k_gather(GatherParams P) {
     if (!P.active[sys]) return;
     const int tier = P.sys_tier[sys] & (kMaxTiers - 1);
 #pragma unroll
-    for (int k = 0; k < 5; ++k)
+    for (int k = 0; k < kClasses; ++k)
         if ((P.cm.m[k].m[tier] >> p) & 1u) {
             add_pairs(np, &P.cls[k]);
             return;

@@ -280,8 +280,9 @@ void launch_symbolic(const MatSet &in, const JobTable &jt, const SysDev &sd, int
 // upper slot (col >= row) among the upper slots (out_urp: their count before
 // each row); slot_t of a lower slot is -1 until launch_pairs finds its partner.
 // cls accumulates the pairs of active systems per kernel class.
+constexpr int kClasses = 6;
 struct ClassMasks {
-    JobMask m[5];        // tensor cores, FP64, FP32, double-FP32, tensor-core slices
+    JobMask m[kClasses]; // tensor cores, FP64 FMAs, FP32, double-FP32, 7 slices, 8 slices (FP64 products)
 };
 void launch_gather(const SymOut &so, int njob, int NB, const int *out_row_ptr, const int *out_urp, int *out_col,
                    int *slot_row, int *slot_job, int *slot_npair, int *uidx, int *slot_t, const SysDev &sd,
@@ -397,12 +398,13 @@ enum {
     kCtrTop = 0,         // pool_top, overflow of the symbolic phase
     kCtrErr = 2,         // error bits of the pair lists
     kCtrPairs = 4,       // 64 bits: pairs of all upper slots
-    kCtrClass = 6,       // 5 x 64 bits: pairs per kernel class
-    kCtrWork = 16,       // work items of the three CUDA-core classes (zeroed for every group, with the next)
-    kCtrNext = 20,       // next item to hand out, per class
-    kCtrLook = 23,       // a wait of the compaction ran out
-    kCtrInts = 24
+    kCtrClass = 6,       // kClasses x 64 bits: pairs per kernel class
+    kCtrWork = 18,       // work items of the three CUDA-core classes (zeroed for every group, with the next)
+    kCtrNext = 22,       // next item to hand out, per class
+    kCtrLook = 25,       // a wait of the compaction ran out
+    kCtrInts = 26        // even: 64-bit words follow
 };
+static_assert(kCtrClass + 2 * kClasses <= kCtrWork && kCtrInts % 2 == 0, "counters");
 // what the host reads of a step, in page-locked memory
 struct HostStep {
     int ctr[kCtrInts];

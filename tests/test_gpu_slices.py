@@ -64,3 +64,29 @@ def test_slices_need_a_threshold(rdm):
     assert out[0.0][1] > 0 and out[1e-11][1] > 0 and out[2e-10][1] == 0
     for tau in (1e-11, 2e-10):
         assert rel_frobenius(out[tau][0], out[0.0][0]) <= 1e-9
+
+
+@pytest.mark.parametrize("tau,tau_x1", [(1e-6, 0.0), (0.0, 1e-6)])
+def test_accounting_of_thresholds_on_either_side_of_the_bound(rdm, tau, tau_x1):
+    """X0^2 as slices and X1's products as FP64 FMAs, and the other way round:
+    both count as FP64 products, in flops and in time, and the FMA chains
+    appear among the issued ones."""
+    s = make_cluster(17, opa=8, b=32, cutoff=10.0, seed=2, dirs=("x", "y"))
+    info = {}
+    for dirs in (0, 2):
+        y = type(s)(**{**s.__dict__, "h1": s.h1[:dirs], "dirs": s.dirs[:dirs]})
+        sol = rdm.Solver(0)
+        sol.set_params(tau=tau, tau_x1=tau_x1, tol=0.0, mode="fp64", max_iter=12)
+        sol.load(y)
+        code, info[dirs] = sol.solve()
+        assert code == rdm.RDM_NOT_CONVERGED and info[dirs].iterations == 12
+        sol.close()
+    i0, i2 = info[0], info[2]
+    assert i2.oz_launches > 0 and i2.simt_launches > 0
+    assert i2.kernel_flops[1] == i2.useful_flops and i2.kernel_flops[4] == 0
+    assert i2.kernel_ms[2] > 0 and i2.kernel_ms[7] == 0
+    # X0's recursion does not depend on X1: the FMA part is issued as it is useful
+    if tau > 0:
+        assert i2.issued_flops - i0.issued_flops == i2.useful_flops - i0.useful_flops
+    else:
+        assert i0.issued_flops == i0.useful_flops < i2.issued_flops - (i2.useful_flops - i0.useful_flops)
