@@ -60,9 +60,17 @@ extern "C" {
 
 /* ---- precision modes (rdm_params.mode) ------------------------------- */
 #define RDM_MODE_FP64        0   /* every product to FP64 accuracy: FP64 FMAs on the CUDA cores, or
-                                    (32 x 32 blocks, truncation threshold >= 1e-10) exact sums of
+                                    (32 x 32 blocks, truncation threshold >= 1e-10) sums of
                                     products of 8 bf16 slices per element on the tensor cores,
-                                    rounded to FP64 once */
+                                    added exactly and rounded to FP64 once.  Slices hold an element
+                                    to 2^-62 of the largest of its row: errors are below those of
+                                    FMA chains against the largest elements of a product, not
+                                    against an element 2^-9 or less of its row's largest.
+                                    refine_x0 = RDM_REFINE_FP64 keeps the FMAs.  Which of the two
+                                    runs depends on sizes alone, unless the device has no room
+                                    for the slices: the solve then starts again with FMAs.
+                                    rdm_info: oz_launches > 0 with slices, simt_launches > 0 with
+                                    FMAs (or copies of converged systems) */
 #define RDM_MODE_FP32        1   /* every product in FP32 (CUDA cores), FP64 scalars */
 #define RDM_MODE_MIXED_BF16  2   /* bf16 hi+lo split products on the tensor cores
                                     (tcgen05, FP32 accumulate) until the idempotency
@@ -144,7 +152,8 @@ typedef struct {
                                (RDM_REFINE_SLICES with 32 x 32 blocks, otherwise
                                RDM_REFINE_FP64), RDM_REFINE_FP64, RDM_REFINE_FP32X2
                                (32 x 32 blocks only), or RDM_REFINE_FP32 (the final tier then ends
-                               on the FP32 idempotency stall) */
+                               on the FP32 idempotency stall).  FP64 mode: RDM_REFINE_FP64 computes
+                               every product with FMA chains; other values make no difference */
     int32_t stall_window;   /* mixed modes: the idempotency error e "stalls" when |e_n| >= |e_{n-w}| / 2
                                with w = stall_window iterations (0: 2); a stall moves a system to the
                                final tier, and in the final tier ends its iteration */
@@ -417,12 +426,13 @@ typedef struct {
                                 Results do not depend on it. */
     int32_t inject;          /* failures of the next step, which is then repeated with the same results:
                                 1: a wait of the tile lists' prefix sums runs out, 2: one of the
-                                compaction's, 4: the K-step lists find no room; sums of these */
+                                compaction's, 4: the K-step lists find no room, sums of these; plus
+                                8 k: the k-th device allocation of the next steps fails */
 } rdm_test_knobs;
 
 /* Set the test settings of h (NULL restores all zeros).  RDM_EINVAL for a
- * negative value, a window that is not a multiple of 32 up to 16,384, a flag
- * other than 0 or 1, or an `inject` above 7. */
+ * negative value, a window that is not a multiple of 32 up to 16,384, or a flag
+ * other than 0 or 1. */
 int rdm_set_test_knobs(rdm_handle *h, const rdm_test_knobs *k);
 
 /* Library version string. */

@@ -131,6 +131,8 @@ struct rdm_handle {
     int nd = 0;
     int dirs[3] = {0, 0, 0};
     int dir_only = -1;          // >= 0: assemble only this field direction (split_directions)
+    bool fp64_fma = false;      // FP64-mode products of this solve as FMA chains (fp64_arith)
+    size_t dev_total = 0;       // the device's memory, once asked for
     bool keep_assembled = false;  // run_solve starts from the current H0, H1 (the correction's response solves)
     std::vector<int> stop_at;     // non-empty: system s stops after stop_at[s] updates (the same)
     std::vector<int> row0, nbs, norb;
@@ -673,9 +675,27 @@ void tier_arith(int mode, int tier, int njob, Arith *ar, int refine_x1 = 0, int 
 // FP64 pipe.  So do the FP64 products of the mixed modes: their results go
 // through the rounding of the split operands, where a last-bit difference
 // comes out as one of 2^-22.
+// A caller who wants the chains asks for them with refine_x0.
+// Which of the two a step takes must not depend on what else holds memory on the
+// device: last bits decide branches at convergence.  It follows from the sizes
+// (slices_fit); when the device has no room for slices that fit by that rule, the
+// whole solve starts again with FMA chains throughout (NoRoomForSlices).
 constexpr double kSliceTau = 1e-10;
-Arith fp64_arith(int mode, int b, double tau) {
-    return mode == RDM_MODE_FP64 && b == 32 && tau >= kSliceTau ? AR_OZ8 : AR_FP64;
+Arith fp64_arith(const rdm_handle *h, double tau) {
+    return h->prm.mode == RDM_MODE_FP64 && h->bs == 32 && tau >= kSliceTau && !h->fp64_fma ? AR_OZ8 : AR_FP64;
+}
+struct NoRoomForSlices {};
+
+// Slices of nblk blocks in a step whose input set has `total`: both layouts with
+// their headroom (40 KB per block), the input and the result (8 and 9 KB) take at
+// most three quarters of the device's memory (3.7 million blocks on 277 GB; the
+// step's lists, untruncated blocks and uploaded matrices share the rest).
+bool slices_fit(rdm_handle *h, int64_t nblk, int64_t total) {
+    if (!h->dev_total) {
+        size_t fr = 0;
+        RDM_CUDA_TRY(cudaMemGetInfo(&fr, &h->dev_total));
+    }
+    return ((size_t)nblk * 40 + (size_t)total * 17) * 1024 <= h->dev_total / 4 * 3;
 }
 
 // tab[t][p]: arithmetic of job p for the systems in tier t; tiers_present:
@@ -733,19 +753,31 @@ StepStats multiply_once(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &
     }
     h->ensure_events();
     RDM_CUDA_TRY(cudaEventRecord(h->ev[0], st));
-    // 8-slice products have FP64 FMAs to fall back on: their slices leave room for
-    // the result (about the input set's size) and the step's buffers
+    if (any_oz8) {
+        int64_t nblk = 0;
+        for (int m = 0; m < oz_nmat; ++m) nblk += in.nnzb[m];
+        if (!slices_fit(h, nblk, in.total)) {
+            for (int t = 0; t < kMaxTiers; ++t) {
+                cm[0].m[t] |= moz8.m[t];
+                ozm.m[t] = moz8.m[t] = 0;
+            }
+            any_oz = any_oz8 = false;
+            any_c[0] = true;
+        }
+    }
+    // 8-slice products leave room for the result (about the input set's size) and
+    // for the step's untruncated blocks and lists
     const size_t out_bytes = (size_t)in.total * bb * sizeof(double) * 9 / 8, out_held = out.val.cap * sizeof(double);
     const size_t grow = out_bytes > out_held ? out_bytes - out_held : 0;
-    const size_t reserve = any_oz8 ? grow + (size_t(4) << 30) : h->tcw.lean ? grow : 0;
-    if (any_oz && ((any_oz8 && h->tcw.lean) ||
-                   !prepare_oz_operands(in, oz_nmat, any_oz8 ? 8 : 7, reserve, h->ozw, st))) {
-        // no room for the slices: the FP64 pipe
+    const size_t reserve = any_oz8 ? grow + out_bytes : h->tcw.lean ? grow : 0;
+    if (any_oz && !prepare_oz_operands(in, oz_nmat, any_oz8 ? 8 : 7, reserve, h->ozw, st)) {
+        if (any_oz8) throw NoRoomForSlices{};
+        // no room for the 7 slices: the FP64 pipe
         for (int t = 0; t < kMaxTiers; ++t) {
             cm[0].m[t] |= ozm.m[t];
-            ozm.m[t] = moz.m[t] = moz8.m[t] = 0;
+            ozm.m[t] = moz.m[t] = 0;
         }
-        any_oz = any_oz8 = false;
+        any_oz = false;
         any_c[0] = true;
     }
     for (int t = 0; t < kMaxTiers; ++t) simt.m[t] = cm[0].m[t] | cm[1].m[t] | cm[2].m[t];
@@ -1075,15 +1107,25 @@ StepStats multiply_once(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &
 
 // A step that runs out of memory is repeated without what it can do without: the
 // FP32 copy of the linear terms, operands written by the compaction, room for the
-// whole mask, 8-slice products (then FP64 FMAs); the solve goes on that way.
+// whole mask; the solve goes on that way.  With 8-slice products the solve starts
+// again (NoRoomForSlices).
 StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt, const Arith (*tab)[kMaxJobs],
                    unsigned tiers_present, bool lin, bool copies, int next_ar = -1, bool defer = false) {
+    // test setting: an allocation of a step fails
+    struct FailAlloc {
+        int &k;
+        explicit FailAlloc(int &knob) : k(knob) { g_fail_alloc = k; }
+        ~FailAlloc() { k = g_fail_alloc; g_fail_alloc = 0; }
+    } fail_alloc{h->tcw.knobs.fail_alloc};
     try {
         return multiply_once(h, in, out, jt, tab, tiers_present, lin, copies, next_ar, defer);
     } catch (const Error &e) {
         if (e.code != RDM_ENOMEM || h->tcw.lean) throw;
     }
     sync(h);
+    for (int t = 0; t < kMaxTiers; ++t)
+        for (int p = 0; p < jt.njob; ++p)
+            if (((tiers_present >> t) & 1u) && tab[t][p] == AR_OZ8) throw NoRoomForSlices{};
     h->tcw.lean = true;
     h->tcw.xlin.release();
     h->ozw.slices_a.release();
@@ -1183,7 +1225,7 @@ void set_products(rdm_handle *h, MatSet &in, const JobTable &jt, const std::vect
     const int S = h->S;
     const std::vector<double> t(S, tau);
     upload_step(h, cl, cq, t, t, std::vector<int>(S, 1), std::vector<int>(S, 0));
-    if (ar == AR_FP64) ar = fp64_arith(h->prm.mode, h->bs, tau);
+    if (ar == AR_FP64) ar = fp64_arith(h, tau);
     Arith tab[kMaxTiers][kMaxJobs];
     for (int p = 0; p < kMaxJobs; ++p) tab[0][p] = ar;
     multiply(h, in, out, jt, tab, 1u, std::any_of(cl.begin(), cl.end(), [](double c) { return c != 0.0; }), false);
@@ -1199,7 +1241,7 @@ void fp64_products(rdm_handle *h, MatSet &in, const JobTable &jt, double c_lin, 
 // would run on the FP64 pipe, FP64 ones otherwise
 void fp64_class_products(rdm_handle *h, MatSet &in, const JobTable &jt, const std::vector<double> &cl,
                          const std::vector<double> &cq, double tau, MatSet &out) {
-    set_products(h, in, jt, cl, cq, tau, h->bs == 32 && fp64_arith(h->prm.mode, 32, tau) == AR_FP64 ? AR_FF : AR_FP64, out);
+    set_products(h, in, jt, cl, cq, tau, h->bs == 32 && fp64_arith(h, tau) == AR_FP64 ? AR_FF : AR_FP64, out);
 }
 
 // Job: out p = c_lin X_x + c_sq (A B + B A), or A A (a == b, one term)
@@ -1559,7 +1601,7 @@ int run_solve(rdm_handle *h, rdm_info *info_out) {
             const bool ref = mixed && t == final_tier;
             for (int p = 0; p < jt.njob; ++p)
                 if (tab[t][p] == AR_FP64)
-                    tab[t][p] = fp64_arith(P.mode, b, jt.job[p].tau_sel ? (ref ? tau1_ref : tau1) : (ref ? tau_ref : tau0));
+                    tab[t][p] = fp64_arith(h, jt.job[p].tau_sel ? (ref ? tau1_ref : tau1) : (ref ? tau_ref : tau0));
         }
         for (int s = 0; s < S; ++s) {
             tier_of[s] = ss[s].tier;
@@ -2067,6 +2109,18 @@ void release_work(rdm_handle *h) {
 int solve_entry(rdm_handle *h, rdm_info *info_out) {
     DeviceGuard dg(h->device);
     const rdm_params &P = h->prm;
+    auto run = [&] {
+        h->fp64_fma = P.refine_x0 == RDM_REFINE_FP64;
+        try {
+            return run_solve_dirs(h, nullptr);
+        } catch (const NoRoomForSlices &) {
+        }
+        sync(h);
+        h->ozw.slices_a.release();
+        h->ozw.slices_b.release();
+        h->fp64_fma = true;
+        return run_solve_dirs(h, nullptr);
+    };
     if (h->hs.empty() || !h->b) return fail(h, RDM_ESTATE, "no system uploaded");
     bool have_result = false;
     int status = RDM_OK;
@@ -2091,7 +2145,7 @@ int solve_entry(rdm_handle *h, rdm_info *info_out) {
             try {
                 for (int sy = 0; sy < h->S; ++sy)
                     if (h->hs[sy].has_h0) ensure_reblocked(h, sy, cand[k]);   // outside the timed solve
-                st = run_solve_dirs(h, nullptr);
+                st = run();
             } catch (const Error &e) {
                 st = e.code;
                 h->err = e.msg;
@@ -2120,7 +2174,7 @@ int solve_entry(rdm_handle *h, rdm_info *info_out) {
         const int want = P.autotune ? h->tuned_b : P.block_size > 0 ? P.block_size : h->b;
         if (P.autotune && h->bs != want) release_work(h);
         h->bs = want;
-        status = run_solve_dirs(h, nullptr);
+        status = run();
         if (status < 0) return status;
     }
     for (auto &I : h->info) {
@@ -2471,13 +2525,14 @@ int rdm_set_test_knobs(rdm_handle *h, const rdm_test_knobs *k) {
     if (!k) k = &z;
     if (k->tc_wait_cycles < 0 || k->tc_hold < 0 || k->tc_hold > 1 || k->tc_window_cols < 0 ||
         k->tc_window_cols > 16384 || (k->tc_window_cols & 31) || k->tc_block_copies < 0 ||
-        k->tc_block_copies > 1 || k->inject < 0 || k->inject > 7)
+        k->tc_block_copies > 1 || k->inject < 0)
         return fail(h, RDM_EINVAL, "invalid test settings");
     h->tcw.knobs.wait_cycles = k->tc_wait_cycles;
     h->tcw.knobs.hold = k->tc_hold;
     h->tcw.knobs.window_words = k->tc_window_cols / 32;
     h->tcw.knobs.block_copies = k->tc_block_copies;
-    h->tcw.knobs.inject = h->tcw_oz.knobs.inject = k->inject;
+    h->tcw.knobs.inject = h->tcw_oz.knobs.inject = k->inject & 7;
+    h->tcw.knobs.fail_alloc = k->inject >> 3;
     return RDM_OK;
 }
 

@@ -60,9 +60,12 @@ void func_smem_once(const void *func, int bytes);
 inline std::atomic<size_t> g_dev_bytes{0};
 inline std::atomic<size_t> g_dev_bytes_peak{0};
 
+// test setting: > 0: the g_fail_alloc-th allocation of this thread from now on fails
+inline thread_local int g_fail_alloc = 0;
+
 inline void *dev_alloc(size_t bytes) {
     void *p = nullptr;
-    cudaError_t e = cudaMalloc(&p, bytes);
+    cudaError_t e = g_fail_alloc > 0 && --g_fail_alloc == 0 ? cudaErrorMemoryAllocation : cudaMalloc(&p, bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
         throw Error{-3, "cudaMalloc of " + std::to_string(bytes) + " bytes failed (" +

@@ -10,6 +10,7 @@ namespace rdm {
 constexpr int kInjectTileWait = 1, kInjectRowWait = 2, kInjectStepRoom = 4;
 struct TcKnobs {
     int inject = 0;             // kInject*: failures of one plan or compaction to come
+    int fail_alloc = 0;         // > 0: that many device allocations of the steps on, one fails
     long long wait_cycles = 0;  // bound of every mbarrier wait in SM clock cycles (0: ~2 s)
     int hold = 0;               // 1: the MMA thread first waits for a flag that nothing sets
     int window_words = 0;       // bitmap window of the tile-plan builders in 32-column words
@@ -106,7 +107,7 @@ void launch_numeric_tc(const NumArgs &a, const MatSet &in, const JobTable &jt, A
 // FP64-class products on the tensor cores from exact bf16 slices (32 x 32
 // blocks; k_oz.cu): the slices (7 or 8 per element) and row scales of the
 // first nmat matrices of `in` (false, with nothing done, when the device has
-// no room for them), the tile lists (128 x 64 tiles) of the jobs in job_mask,
+// no room for them; then the caller has another way), the tile lists (128 x 64 tiles) of the jobs in job_mask,
 // and the launch (same output contract as the other numeric launches).
 // tc_step_flops / oz_step_flops: the MMA flops issued per K-step; reserve:
 // bytes the slices leave free.

@@ -54,3 +54,49 @@ def test_a_repeated_step_gives_the_same_bits(rdm, system, prm, inject):
     for r, g in zip(ref, got):
         assert np.array_equal(r.row_ptr, g.row_ptr) and np.array_equal(r.col_idx, g.col_idx)
         assert np.array_equal(r.vals, g.vals)
+
+
+@pytest.mark.parametrize("mode,b", [("mixed_fp16", 32), ("mixed_bf16", 16), ("fp32", 32)])
+def test_a_step_without_memory_is_repeated_without_its_optional_buffers(rdm, system, mode, b):
+    """Whichever allocation of a step fails, the results keep their bits."""
+    ref, i0 = solve(rdm, system, mode=mode, block_size=b)
+    for k in range(1, 60, 2):
+        got, i1 = solve(rdm, system, inject=8 * k, mode=mode, block_size=b)
+        assert i1.iterations == i0.iterations
+        for r, g in zip(ref, got):
+            assert np.array_equal(r.col_idx, g.col_idx) and np.array_equal(r.vals, g.vals), k
+
+
+def test_an_fp64_solve_has_one_arithmetic(rdm, system):
+    """FP64 mode at 32 x 32 blocks: slices, or FMA chains where the caller asks
+    for them or where a step with slices finds no memory, in every step of the
+    solve; the info tells which."""
+    slices, i0 = solve(rdm, system, mode="fp64", block_size=32)
+    fma, i1 = solve(rdm, system, mode="fp64", block_size=32, refine_x0=1)
+    assert i0.oz_launches > 0 and i0.simt_launches == 0
+    assert i1.oz_launches == 0 and i1.simt_launches > 0
+    failed = 0
+    for k in range(1, 60, 2):
+        got, i = solve(rdm, system, inject=8 * k, mode="fp64", block_size=32)
+        assert (i.oz_launches > 0) != (i.simt_launches > 0)
+        failed += i.oz_launches == 0
+        for r, g in zip(slices if i.oz_launches else fma, got):
+            assert np.array_equal(r.col_idx, g.col_idx) and np.array_equal(r.vals, g.vals), k
+    assert failed > 10
+    # rounding of either (1e-16 a product, doubled by each of ~20 steps)
+    for r, g in zip(slices, fma):
+        assert np.max(np.abs(r.to_dense() - g.to_dense())) <= 1e-9 * np.max(np.abs(g.vals))
+
+
+@pytest.mark.parametrize("prm", [dict(correct=1), dict(split_directions=1)], ids=["correct", "directions"])
+def test_solves_of_several_passes_start_again_as_a_whole(rdm, system, prm):
+    """A pass after the first one that finds no room for its slices."""
+    prm = dict(prm, mode="fp64", block_size=32)
+    ref = {True: solve(rdm, system, **prm)[0], False: solve(rdm, system, refine_x0=1, **prm)[0]}
+    seen = set()
+    for k in range(3, 260, 16):
+        got, i = solve(rdm, system, inject=8 * k, **prm)
+        seen.add(i.oz_launches > 0)
+        for r, g in zip(ref[i.oz_launches > 0], got):
+            assert np.array_equal(r.col_idx, g.col_idx) and np.array_equal(r.vals, g.vals), k
+    assert seen == {True, False}
