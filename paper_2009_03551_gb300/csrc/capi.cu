@@ -854,7 +854,7 @@ StepStats multiply_once(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &
                     reinterpret_cast<unsigned long long *>(h->counters.p + kCtrPairs)};
         launch_symbolic(in, jt, h->sd, h->S, so, st, h->prm.symbolic_hash ? kSymMaxNs + 1 : max_ns);
         scan_exclusive_pair(h->row_cnt.p, h->out_rp.p, h->urp.p, nrows, h->scan_tmp64.p, st);
-        launch_publish(PublishArgs{hs, h->counters.p, h->urp.p + nrows, nullptr, nullptr, nullptr, nullptr, nullptr, NB, njob},
+        launch_publish(PublishArgs{hs, h->counters.p, h->urp.p, nullptr, nullptr, nullptr, nullptr, nullptr, NB, njob},
                        st);
         sync(h);
         const int top = hs->ctr[kCtrTop], over = hs->ctr[kCtrTop + 1];
@@ -864,8 +864,13 @@ StepStats multiply_once(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &
         if (attempt == 3) throw Error{RDM_ECAPACITY, "symbolic pool overflow after retries"};
         cap = (int64_t)top + top / 4 + 1024;
     }
-    const int64_t nslot = hs->ctr[kCtrTop], nupper = hs->nupper;
-    const int64_t npairs = *reinterpret_cast<int64_t *>(hs->ctr + kCtrPairs);
+    const int64_t nslot = hs->ctr[kCtrTop], nupper = hs->upper[njob];
+    int64_t npairs = 0, job_pairs[kMaxJobs], job_upper[kMaxJobs];
+    for (int p = 0; p < njob; ++p) {
+        job_pairs[p] = reinterpret_cast<int64_t *>(hs->ctr + kCtrPairs)[p];
+        job_upper[p] = hs->upper[p + 1] - hs->upper[p];
+        npairs += job_pairs[p];
+    }
     h->pool_cap_hint = std::max<int64_t>(h->pool_cap_hint, nslot);
     ss.nslot = nslot;
     ss.npairs = npairs;
@@ -988,15 +993,34 @@ StepStats multiply_once(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &
         }
         if (ss.pending) out.val.ensure(need);
     }
+    // upper slots and (estimated, where a group cuts a job) pairs of the super-row
+    // units [ua, ub) of the jobs in a mask
+    struct PlanSize { int64_t upper = 0, pairs = 0; };
+    auto plan_size = [&](const JobMask &m, int ua, int ub) {
+        PlanSize z;
+        for (int p = 0; p < njob; ++p) {
+            const int lo = std::max(unit_row(ua), p * NB), hi = std::min(unit_row(ub), (p + 1) * NB);
+            bool mine = false;
+            for (int t = 0; t < kMaxTiers; ++t) mine = mine || ((m.m[t] >> p) & 1u);
+            if (!mine || lo >= hi || job_upper[p] == 0) continue;
+            const int64_t u = ngroup == 1 ? job_upper[p] : hurp[hi] - hurp[lo];
+            z.upper += u;
+            z.pairs += (int64_t)((double)job_pairs[p] * (double)u / (double)job_upper[p]) + 1;
+        }
+        return z;
+    };
     const int ev_simt[kSimt] = {5, 6, 4};   // events after each CUDA-core class
     for (int g = 0; g < ngroup; ++g) {
         const int ua = gunit[g], ub = gunit[g + 1];
         const int64_t s0 = gslot(ua), s1 = gslot(ub), u0 = gupper(ua), nup = gupper(ub) - u0;
         const int r0 = unit_row(ua), nr = unit_row(ub) - r0;
         // room for the K-steps (a tile of 4 x 8 blocks has 5 to 12 pairs to a
-        // step, one of 4 x 2 about 3); a plan that needs more is built again
-        const int64_t gpairs = (int64_t)((double)npairs * (double)nup / (double)std::max<int64_t>(nupper, 1)) + 1;
-        const int64_t steps_tc = std::min(gpairs, gpairs / 4 + 65536) + 1024, steps_oz = gpairs / 2 + 1024;
+        // step, one of 4 x 2 about 3; a quarter of it when memory is short); a plan
+        // that needs more is built again
+        const PlanSize zt = plan_size(tcm, ua, ub), zo = plan_size(ozm, ua, ub);
+        const int less = h->tcw.lean ? 4 : 1;
+        const int64_t steps_tc = std::min(zt.pairs, zt.pairs / 4 / less + 65536) + 1024,
+                      steps_oz = zo.pairs / 2 / less + 1024;
         CompactArgs ca{};
         for (int attempt = 0;; ++attempt) {
             if (g > 0 || attempt > 0)
@@ -1009,9 +1033,9 @@ StepStats multiply_once(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &
                                       h->sd.sys_of_row.p, h->sd.active.p, h->slot_job.p, h->sd.tier.p, cm[c],
                                       c == first_c ? 1 : 0);
             TcPlan plan{}, oplan{};
-            if (tc) plan = build_tc_plan(in, jt, h->sd, h->out_rp.p, mcol, h->tcw, tcm, ua, ub, nup,
+            if (tc) plan = build_tc_plan(in, jt, h->sd, h->out_rp.p, mcol, h->tcw, tcm, ua, ub, zt.upper,
                                        std::max(steps_tc, h->tcw.need_steps), st);
-            if (any_oz) oplan = build_oz_plan(in, jt, h->sd, h->out_rp.p, mcol, h->tcw_oz, ozm, ua, ub, nup,
+            if (any_oz) oplan = build_oz_plan(in, jt, h->sd, h->out_rp.p, mcol, h->tcw_oz, ozm, ua, ub, zo.upper,
                                             std::max(steps_oz, h->tcw_oz.need_steps), st);
 
             NumArgs a{};
@@ -1107,7 +1131,7 @@ StepStats multiply_once(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &
 
 // A step that runs out of memory is repeated without what it can do without: the
 // FP32 copy of the linear terms, operands written by the compaction, room for the
-// whole mask; the solve goes on that way.  With 8-slice products the solve starts
+// whole mask, K-step lists sized for few pairs to a step; the solve goes on that way.  With 8-slice products the solve starts
 // again (NoRoomForSlices).
 StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt, const Arith (*tab)[kMaxJobs],
                    unsigned tiers_present, bool lin, bool copies, int next_ar = -1, bool defer = false) {
@@ -1130,6 +1154,12 @@ StepStats multiply(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &jt, c
     h->tcw.xlin.release();
     h->ozw.slices_a.release();
     h->ozw.slices_b.release();
+    for (TcWork *w : {&h->tcw, &h->tcw_oz}) {
+        w->steps.release();
+        w->tiles.release();
+        w->step_rng.release();
+        w->need_steps = 0;
+    }
     in.planes_ar = -1;
     return multiply_once(h, in, out, jt, tab, tiers_present, lin, copies, -1, false);
 }

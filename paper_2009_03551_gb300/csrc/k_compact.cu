@@ -109,14 +109,15 @@ __global__ void __launch_bounds__(32 * kRowWarps) k_compact_rows(CompactArgs c) 
 // A step's counters and sizes to page-locked host memory, in one launch: a copy
 // each holds the stream up for ~2 us, and a step had seven of them.
 __global__ void __launch_bounds__(32) k_publish(PublishArgs a) {
-    static_assert(kCtrInts <= 32 && kMaxJobs < 32, "one warp");
+    static_assert(kMaxJobs < 32, "one warp");
     const int t = threadIdx.x;
-    if (a.ctr && t < kCtrInts) a.dst->ctr[t] = a.ctr[t];
+    if (a.ctr)
+        for (int k = t; k < kCtrInts; k += 32) a.dst->ctr[k] = a.ctr[k];
     if (a.tc && t < 8) a.dst->tc[t] = a.tc[t];
     if (a.oz && t < 8) a.dst->oz[t] = a.oz[t];
     if (a.rp && t <= a.njob) a.dst->rp[t] = a.rp[(size_t)t * a.NB];
+    if (a.upper && t <= a.njob) a.dst->upper[t] = a.upper[(size_t)t * a.NB];
     if (t == 0) {
-        if (a.nupper) a.dst->nupper = *a.nupper;
         if (a.kept) a.dst->kept = *a.kept;
         if (a.pre_err) a.dst->pre_err = *a.pre_err;
     }

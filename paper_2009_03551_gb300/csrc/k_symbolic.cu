@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(kSymThreads) k_symbolic(SymParams P) {
     int total, upper;
     block_excl_scan<int>(my, sh_scan, &total);
     block_excl_scan<int>(up, sh_scan, &upper);
-    add_pairs(np, P.so.npairs);
+    add_pairs(np, P.so.npairs + p);
     if (tid == 0) {
         int off = atomicAdd(P.so.pool_top, total);
         if (off + total > P.so.pool_cap) { atomicExch(P.so.overflow, 1); off = -1; }
@@ -376,7 +376,7 @@ __global__ void __launch_bounds__(kSymThreads) k_symbolic_hash(SymParams P) {
     int total, upper;
     block_excl_scan<int>(my, sh_scan, &total);
     block_excl_scan<int>(up, sh_scan, &upper);
-    add_pairs(npt, P.so.npairs);
+    add_pairs(npt, P.so.npairs + p);
     // bitonic sort of the packed keys (ascending)
     for (int k = 2; k <= kHashSlots; k <<= 1) {
         for (int jj = k >> 1; jj > 0; jj >>= 1) {

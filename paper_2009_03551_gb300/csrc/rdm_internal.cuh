@@ -272,7 +272,7 @@ struct SymOut {
     int *pool_top;       // [1] pool allocation counter
     int pool_cap;
     int *overflow;       // [1] set when the pool is too small
-    unsigned long long *npairs;   // [1] pairs of the kept upper-triangle blocks
+    unsigned long long *npairs;   // [njob] pairs of the kept upper-triangle blocks
 };
 // largest system (in block rows) the shared-memory row accumulator handles
 constexpr int kSymMaxNs = 8192;
@@ -400,27 +400,29 @@ void launch_compact_rows(CompactArgs &c, unsigned long long *look, cudaStream_t 
 enum {
     kCtrTop = 0,         // pool_top, overflow of the symbolic phase
     kCtrErr = 2,         // error bits of the pair lists
-    kCtrPairs = 4,       // 64 bits: pairs of all upper slots
-    kCtrClass = 6,       // kClasses x 64 bits: pairs per kernel class
-    kCtrWork = 18,       // work items of the three CUDA-core classes (zeroed for every group, with the next)
-    kCtrNext = 22,       // next item to hand out, per class
-    kCtrLook = 25,       // a wait of the compaction ran out
-    kCtrInts = 26        // even: 64-bit words follow
+    kCtrPairs = 4,       // 64 bits per job: pairs of its upper slots
+    kCtrClass = kCtrPairs + 2 * kMaxJobs,   // kClasses x 64 bits: pairs per kernel class
+    kCtrWork = 32,       // work items of the three CUDA-core classes (zeroed for every group, with the next)
+    kCtrNext = 36,       // next item to hand out, per class
+    kCtrLook = 39,       // a wait of the compaction ran out
+    kCtrInts = 40        // even: 64-bit words follow
 };
 static_assert(kCtrClass + 2 * kClasses <= kCtrWork && kCtrInts % 2 == 0, "counters");
 // what the host reads of a step, in page-locked memory
 struct HostStep {
     int ctr[kCtrInts];
-    int nupper, kept;
+    int kept;
+    int upper[kMaxJobs + 1];          // upper slots before every job, and their number
     int tc[8], oz[8];                 // TcWork::counters of the two plans
     int pre_err;                      // error bits of the transposed positions (FP32 products)
     int rp[kMaxJobs + 1];             // first block of every output matrix
 };
 // one launch that writes the listed values (null: not this one) into *dst,
-// which the host reads after its next wait; rp: row_ptr, every NB-th entry
+// which the host reads after its next wait; upper, rp: every NB-th entry of the
+// upper slots' and of the result's row pointers
 struct PublishArgs {
     HostStep *dst;
-    const int *ctr, *nupper, *kept, *tc, *oz, *pre_err, *rp;
+    const int *ctr, *upper, *kept, *tc, *oz, *pre_err, *rp;
     int NB, njob;
 };
 void launch_publish(const PublishArgs &a, cudaStream_t st);

@@ -91,8 +91,8 @@ void find_transposes(const MatSet &in, TcWork &w, cudaStream_t st);
 // Tile and K-step lists of one multiplication step from the output mask, for
 // the jobs selected by job_mask (per system tier) and the super-row units
 // [unit0, unit1) (unit = job * ceil(NB/TR) + I covers block rows
-// TR I .. TR I + TR - 1 of the job, TR = tc_tile_rows(b)), which have nupper
-// upper slots.  Nothing is waited for: min_steps is the least room made for
+// TR I .. TR I + TR - 1 of the job, TR = tc_tile_rows(b)); those of the selected
+// jobs have nupper upper slots.  Nothing is waited for: min_steps is the least room made for
 // K-steps, and a list that needs more (counters[1], with the number in
 // counters[4..5]) has to be built again.
 TcPlan build_tc_plan(const MatSet &in, const JobTable &jt, const SysDev &sd, const int *out_rp,

@@ -100,3 +100,12 @@ def test_solves_of_several_passes_start_again_as_a_whole(rdm, system, prm):
         for r, g in zip(ref[i.oz_launches > 0], got):
             assert np.array_equal(r.col_idx, g.col_idx) and np.array_equal(r.vals, g.vals), k
     assert seen == {True, False}
+
+
+def test_slice_plans_make_room_for_their_own_jobs(rdm):
+    """The final tier's slice plan holds X0^2 alone, a small part of a step's
+    pairs with three field directions: its lists, made for every pair at 24 bytes
+    per two, held 38 of the 2,146 MB of this solve beyond what they need."""
+    s = make_cluster(600, opa=8, b=32, cutoff=10.0, seed=4)
+    _, info = solve(rdm, s, mode="mixed_fp16")
+    assert 1.5e9 < info.device_bytes_peak <= 2.125e9
