@@ -69,7 +69,30 @@ struct HostSys {
     std::vector<int> rps, cols;
     DevBuf<double> vals;
     SysMats rb;                        // the same matrices at the solve's block size (when it differs)
+    size_t bytes() const {
+        size_t n = val.cap + vals.cap + rb.val.cap + rb.vals.cap;
+        for (int d = 0; d < 3; ++d) n += val1[d].cap + rb.val1[d].cap;
+        return n * sizeof(double);
+    }
+    // buffers that an earlier upload left and this one does not use
+    void release_unused() {
+        if (rb.b == 0) rb = SysMats{};
+        for (int d = 0; d < 3; ++d)
+            if (!has_h1[d]) {
+                val1[d].release();
+                rb.val1[d].release();
+            }
+        if (!has_s) {
+            vals.release();
+            rb.vals.release();
+        }
+    }
 };
+// Device buffers that uploaded systems may leave for the next uploads, per
+// handle: allocations cost a tenth of a millisecond and more each (uploads of a
+// batch of five 2,000-atom clusters 5.4 -> 2.3 ms), beside milliseconds of
+// solve; above this bound the solve's time dwarfs them.
+constexpr size_t kKeepUploadBytes = size_t(2) << 30;
 
 struct SysState {
     int iters = 0;
@@ -358,6 +381,7 @@ void assemble(rdm_handle *h) {
     for (int s = 0; s < S; ++s) {
         if (!h->hs[s].has_h0) throw Error{RDM_ESTATE, "H0 of system " + std::to_string(s) + " not uploaded"};
         if (rb) ensure_reblocked(h, s, h->bs);
+        h->hs[s].release_unused();
         h->row0[s] = NB;
         h->nbs[s] = rb ? h->hs[s].rb.nb : h->hs[s].nb;
         h->norb[s] = h->hs[s].n;
@@ -2419,8 +2443,14 @@ int rdm_batch_create(rdm_handle *h, int n_systems) {
     return guarded(h, [&] {
         DeviceGuard dg(h->device);
         // the systems' device buffers stay for the next uploads (those of
-        // systems beyond n_systems are freed)
+        // systems beyond n_systems and what exceeds the bound are freed)
         h->hs.resize(n_systems);
+        size_t kept = 0;
+        for (HostSys &y : h->hs)
+            if ((kept += y.bytes()) > kKeepUploadBytes) {
+                kept -= y.bytes();
+                y = HostSys{};
+            }
         for (HostSys &y : h->hs) {
             y.has_h0 = y.has_s = false;
             for (bool &f : y.has_h1) f = false;

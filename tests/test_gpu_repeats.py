@@ -109,3 +109,23 @@ def test_slice_plans_make_room_for_their_own_jobs(rdm):
     s = make_cluster(600, opa=8, b=32, cutoff=10.0, seed=4)
     _, info = solve(rdm, s, mode="mixed_fp16")
     assert 1.5e9 < info.device_bytes_peak <= 2.125e9
+
+
+def test_uploads_give_back_what_the_next_problem_does_not_use(rdm):
+    """A handle that held H1 matrices solves a system without them in the memory that
+    a new handle takes."""
+    s = make_cluster(400, opa=8, b=32, cutoff=10.0, seed=4)
+    bare = type(s)(**{**s.__dict__, "h1": [], "dirs": ()})
+
+    def peak(first):        # (of every handle of the process)
+        sol = rdm.Solver(0)
+        sol.set_params(tau=1e-6, tol=1e-9, mode="fp64", max_iter=60)
+        if first is not None:
+            sol.load(first)
+        sol.load(bare)
+        code, info = sol.solve()
+        assert code == rdm.RDM_OK
+        sol.close()
+        return info.device_bytes_peak
+
+    assert peak(s) == peak(None)
