@@ -130,6 +130,7 @@ struct PinBuf {
         p = nullptr;
         cap = 0;
     }
+    void swap(PinBuf &o) noexcept { std::swap(p, o.p); std::swap(cap, o.cap); }
 };
 
 struct rdm_handle {
@@ -2686,6 +2687,17 @@ int rdm_block_product(rdm_handle *h, const rdm_bsr *A, const rdm_bsr *B, const r
         t.stream = h->stream;
         t.S = 1;
         t.hs.resize(1);
+        // with the page-locked memory of h (two buffers made and freed in every call:
+        // 1.02 ms for a product of 4 x 4 blocks, 0.70 so)
+        struct Lend {
+            rdm_handle &a, &b;
+            Lend(rdm_handle &x, rdm_handle &y) : a(x), b(y) { swap(); }
+            ~Lend() { swap(); }
+            void swap() {
+                a.step_host.swap(b.step_host);
+                a.scalars_host.swap(b.scalars_host);
+            }
+        } lend(*h, t);
         const rdm_bsr *mats[3] = {A, terms == 2 ? B : nullptr, X};
         std::vector<int> rps[3], cols[3];
         DevBuf<double> vals[3];

@@ -129,3 +129,25 @@ def test_uploads_give_back_what_the_next_problem_does_not_use(rdm):
         return info.device_bytes_peak
 
     assert peak(s) == peak(None)
+
+
+def test_products_between_solves(rdm, system):
+    """A block product borrows the handle's page-locked memory: solves before and
+    after it, and the product itself, are what they are on handles of their own."""
+    ref, _ = solve(rdm, system, mode="mixed_fp16")
+    h = rdm.rdm_create(0)
+    want = rdm.rdm_block_product(h, system.h0, None, None, 0.0, 1.0, 1, 1e-6)
+    rdm.rdm_destroy(h)
+    sol = rdm.Solver(0)
+    sol.set_params(tau=1e-6, tol=1e-9, max_iter=60, mode="mixed_fp16")
+    sol.load(system)
+    for _ in range(2):
+        prod = rdm.rdm_block_product(sol.h, system.h0, None, None, 0.0, 1.0, 1, 1e-6)
+        with pytest.raises(rdm.RdmError):       # a product that fails gives it back too
+            rdm.rdm_block_product(sol.h, system.h0, system.h1[0], system.h0, 0.0, 1.0, 2, -1.0)
+        code, _ = sol.solve()
+        assert code == rdm.RDM_OK
+        assert np.array_equal(prod.vals, want.vals)
+        for r, g in zip(ref, [sol.p0()] + [sol.p1(0, d) for d in range(3)]):
+            assert np.array_equal(r.vals, g.vals)
+    sol.close()
