@@ -322,8 +322,8 @@ void upload_matrix(rdm_handle *h, const rdm_bsr *A, std::vector<int> &rp, std::v
     int herr[4];
     d2h(herr, derr.p, 4, h->stream);
     sync(h);
-    if (herr[0] & 1) throw Error{RDM_EBADBSR, "matrix has non-finite values"};
     if (herr[0] & 8) throw Error{RDM_EBADBSR, "block pattern is not symmetric"};
+    if (herr[0] & 1) throw Error{RDM_EBADBSR, "matrix has non-finite values"};
     if (herr[0] & 2) throw Error{RDM_EBADBSR, "matrix values are not symmetric (tolerance 1e-12 max|H|)"};
     if (herr[0] & 4) throw Error{RDM_EBADBSR, "padding rows/columns (index >= n) must be zero"};
     h->b = A->b;
