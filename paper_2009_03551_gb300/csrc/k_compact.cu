@@ -108,11 +108,11 @@ __global__ void __launch_bounds__(32 * kRowWarps) k_compact_rows(CompactArgs c) 
 
 // A step's counters and sizes to page-locked host memory, in one launch: a copy
 // each holds the stream up for ~2 us, and a step had seven of them.
-__global__ void __launch_bounds__(32) k_publish(PublishArgs a) {
-    static_assert(kMaxJobs < 32, "one warp");
+constexpr int kPublishThreads = 64;    // a thread per counter: one load's latency
+__global__ void __launch_bounds__(kPublishThreads) k_publish(PublishArgs a) {
+    static_assert(kCtrInts <= kPublishThreads && kMaxJobs < kPublishThreads, "one thread per value");
     const int t = threadIdx.x;
-    if (a.ctr)
-        for (int k = t; k < kCtrInts; k += 32) a.dst->ctr[k] = a.ctr[k];
+    if (a.ctr && t < kCtrInts) a.dst->ctr[t] = a.ctr[t];
     if (a.tc && t < 8) a.dst->tc[t] = a.tc[t];
     if (a.oz && t < 8) a.dst->oz[t] = a.oz[t];
     if (a.rp && t <= a.njob) a.dst->rp[t] = a.rp[(size_t)t * a.NB];
@@ -129,8 +129,8 @@ __global__ void __launch_bounds__(32) k_publish(PublishArgs a) {
 // in this group's buffer or already compacted.
 __global__ void __launch_bounds__(128) k_compact_vals(CompactArgs c) {
     extern __shared__ double tile[];
-    if (*c.look_err) return;                 // src is not complete: the host repeats the step
-    const int d1 = c.new_rp[c.r0 + c.nrows];
+    // nothing where src is not complete: the host repeats the step
+    const int bad = *c.look_err, end = c.new_rp[c.r0 + c.nrows], d1 = bad ? c.d0 : end;
     const int b = c.b, bb = b * b, ld = b + 1;
     for (int d = c.d0 + blockIdx.x; d < d1; d += gridDim.x) {
         const int p = c.src[d - c.d0];
@@ -163,8 +163,7 @@ __global__ void __launch_bounds__(128) k_compact_vals(CompactArgs c) {
 // 150 atoms, 5,500 blocks: 16.5 + 13.5 us, 21 in one, and four launches less).
 template <int B, int PL>
 __global__ void __launch_bounds__(128) k_compact_blocks(CompactArgs c) {
-    if (*c.look_err) return;
-    const int d1 = c.new_rp[c.r0 + c.nrows];
+    const int bad = *c.look_err, end = c.new_rp[c.r0 + c.nrows], d1 = bad ? c.d0 : end;
     constexpr int BB = B * B, C8 = B / 8;
     const int lane = threadIdx.x & 31;
     if (PL && blockIdx.x == 0 && (int)threadIdx.x < c.njob) c.scale[threadIdx.x] = matrix_scale(c.mx[threadIdx.x], PL == 1);
@@ -294,7 +293,7 @@ void launch_compact_rows(CompactArgs &c, unsigned long long *look, cudaStream_t 
 }
 
 void launch_publish(const PublishArgs &a, cudaStream_t st) {
-    k_publish<<<1, 32, 0, st>>>(a);
+    k_publish<<<1, kPublishThreads, 0, st>>>(a);
     RDM_LAUNCH_CHECK();
 }
 
