@@ -51,10 +51,9 @@ def tc_flops_per_kstep(b):
     return 3 * 2 * 128 * 256 * b
 
 
-# DRAM traffic of the product kernels, from one ncu capture each (profiles/):
+# DRAM traffic of the tensor-core product kernel, from an ncu capture (profiles/):
 # dram__bytes_read.sum + dram__bytes_write.sum per launch, divided by the work
-# units of that launch (K-steps for the tensor-core kernel, block triples for
-# the CUDA-core kernels), so that a capture on a small case scales to the
+# units of that launch (K-steps), so that a capture on a small case scales to the
 # launches of the bench workload by the units they process.  A figure is
 # reported only while the code of the kernel's source file is unchanged since
 # the capture (SHA-256 of the file with comments and whitespace removed).
@@ -64,9 +63,6 @@ PROFILED_TRAFFIC = {
            "sha256": "8144a972ed0c44d892c544a9ba616a6284ee8c6341aa764fb7532f003327a28b",
            "bytes_per_unit": 10598.0, "unit": "K-step", "b": 32,
            "capture": "profiles/k_tc_bf16x3_dram_cluster1000.md"},
-    "ff": {"file": "paper_2009_03551_gb300/csrc/k_numeric.cu",
-           "sha256": "1c9d3e76e36659e5d06b0d237474522761ebecc2732c37eb20f037dc4adcb12e",
-           "bytes_per_unit": None, "unit": "block triple"},
 }
 
 
@@ -113,7 +109,7 @@ def profiled_traffic(cls, units_per_launch, b=32):
     capture by the units the launch processes; None if there is no capture of
     the current code at this block size."""
     rec = PROFILED_TRAFFIC.get(cls)
-    if rec is None or rec["bytes_per_unit"] is None or not units_per_launch or rec.get("b", 32) != b:
+    if rec is None or not units_per_launch or rec.get("b", 32) != b:
         return None
     root = os.path.dirname(os.path.abspath(__file__))
     files = rec["file"] if isinstance(rec["file"], list) else [rec["file"]]

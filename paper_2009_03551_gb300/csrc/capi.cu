@@ -1064,7 +1064,7 @@ StepStats multiply_once(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &
                                             std::max(steps_oz, h->tcw_oz.need_steps), st);
 
             NumArgs a{};
-            a.in_val = in.val.p; a.in_nrm = in.nrm.p;
+            a.in_val = in.val.p;
             a.in_f32 = f32_planes ? in.opf32.p : nullptr;
             a.tpos = f32_t ? h->tcw.tpos.p : nullptr;
             a.in_f32lo = any_c[1] ? in.opf32lo.p : nullptr;
@@ -1092,7 +1092,7 @@ StepStats multiply_once(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &
             ss.simt_launches += (int)(g_kernel_launches - lg);
             const long long lt = g_kernel_launches;
             if (tc) {
-                launch_numeric_tc(a, in, jt, tc_ar, h->tcw, NB, plan, st);
+                launch_numeric_tc(a, in, jt, tc_ar, h->tcw, plan, st);
                 ss.tc_launches += (int)(g_kernel_launches - lt);
                 RDM_CUDA_TRY(cudaEventRecord(h->ev[2], st));
             }

@@ -24,7 +24,7 @@ namespace {
 
 template <int B>
 struct Cfg {
-    static constexpr int NT = (B * B >= 256) ? 256 : ((B * B < 32) ? 32 : B * B);
+    static constexpr int NT = B * B >= 256 ? 256 : B * B;      // B = 8 and up
     static constexpr int PER = (B * B + NT - 1) / NT;
     static constexpr int LD = B + 1;
 };

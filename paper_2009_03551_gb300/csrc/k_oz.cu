@@ -101,7 +101,6 @@ struct GeoOz : PlanGeo<4, 2> {
     static constexpr uint32_t kSBOA = S * 512;                      // bytes between 8-row groups of an A slice
     static constexpr uint32_t kSBOB = 512;                          // ... of a B slice, and on to the next slice
     static constexpr int kAccCols = 32 * S;                         // accumulator columns of a block column
-    static constexpr int kPairs = S * (S + 1) / 2;
     static_assert(2 * kAccCols <= 512, "group accumulators exceed tensor memory");
 };
 constexpr int kOzEpiWarp0 = 2, kOzEpiWarps = 8;

@@ -105,7 +105,7 @@ struct Geo : PlanGeo<128 / B, 256 / B> {
 
 constexpr int kTileN = 256;                  // MMA N = accumulator columns in tensor memory
 constexpr int kEpiWarps = 8;                 // epilogue warps: 2 per TMEM lane quarter
-constexpr int kEpiWarp0 = 4;                 // warps 0 and 2 copy, warp 1 issues the MMAs, warp 3 idles
+constexpr int kEpiWarp0 = 4;                 // warps 0 and 2 copy, 1 issues the MMAs, 3 claims the tiles
 constexpr int kThreads = 32 * (kEpiWarp0 + kEpiWarps);
 constexpr int kSegBufs = 512 / kTileN;       // segment accumulators: the 512 TMEM columns
 // output blocks whose metadata an epilogue warp holds (one lane each)
@@ -1033,8 +1033,7 @@ void prepare_operands(MatSet &in, Arith ar, bool lin, TcWork &w, cudaStream_t st
 double tc_step_flops(int b) { return 3.0 * 2.0 * 128.0 * kTileN * b; }
 
 void launch_numeric_tc(const NumArgs &a, const MatSet &in, const JobTable &jt, Arith ar, TcWork &w,
-                       int NB, const TcPlan &plan, cudaStream_t st) {
-    (void)NB;
+                       const TcPlan &plan, cudaStream_t st) {
     if (!tc_block_size_ok(in.b)) throw Error{-1, "the tensor-core path handles 16 x 16, 32 x 32 and 64 x 64 blocks"};
     if (plan.max_tile == 0) return;
     switch (in.b) {

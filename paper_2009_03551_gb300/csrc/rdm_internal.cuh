@@ -313,7 +313,6 @@ struct NumArgs {
     const float *in_f32;       // FP32 copy of in_val (FP32 products), may be null
     const int *tpos;           // position of every block's transpose (with in_f32 and b = 32)
     const float *in_f32lo;     // in_val - in_f32 rounded to FP32 (double-FP32 products), may be null
-    const float *in_nrm;
     const int *pair_a, *pair_b;
     const int64_t *pair_off;   // null: no slot has pairs (copies of converged systems only)
     const int *slot_row, *slot_job, *slot_x, *slot_t;

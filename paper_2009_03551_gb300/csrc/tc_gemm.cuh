@@ -102,7 +102,7 @@ TcPlan build_tc_plan(const MatSet &in, const JobTable &jt, const SysDev &sd, con
 // Numeric phase on the tensor cores; same output contract as
 // launch_numeric_simt for the slots of active systems.
 void launch_numeric_tc(const NumArgs &a, const MatSet &in, const JobTable &jt, Arith ar, TcWork &w,
-                         int NB, const TcPlan &plan, cudaStream_t st);
+                       const TcPlan &plan, cudaStream_t st);
 
 // FP64-class products on the tensor cores from exact bf16 slices (32 x 32
 // blocks; k_oz.cu): the slices (7 or 8 per element) and row scales of the
