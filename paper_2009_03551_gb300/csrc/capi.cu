@@ -712,15 +712,16 @@ Arith fp64_arith(const rdm_handle *h, double tau) {
 struct NoRoomForSlices {};
 
 // Slices of nblk blocks in a step whose input set has `total`: both layouts with
-// their headroom (40 KB per block), the input and the result (8 and 9 KB) take at
-// most three quarters of the device's memory (3.7 million blocks on 277 GB; the
-// step's lists, untruncated blocks and uploaded matrices share the rest).
+// their headroom (34 KB per block), the input and the result (8 and 9 KB) take at
+// most three quarters of the device's memory (4.1 million blocks on 277 GB; the
+// step's lists, untruncated blocks and uploaded matrices share the rest).  FP64
+// solve of 20,000 atoms at tau = 1e-7: 596 s with 40 KB counted, 572 s so.
 bool slices_fit(rdm_handle *h, int64_t nblk, int64_t total) {
     if (!h->dev_total) {
         size_t fr = 0;
         RDM_CUDA_TRY(cudaMemGetInfo(&fr, &h->dev_total));
     }
-    return ((size_t)nblk * 40 + (size_t)total * 17) * 1024 <= h->dev_total / 4 * 3;
+    return ((size_t)nblk * 34 + (size_t)total * 17) * 1024 <= h->dev_total / 4 * 3;
 }
 
 // tab[t][p]: arithmetic of job p for the systems in tier t; tiers_present:
@@ -791,10 +792,11 @@ StepStats multiply_once(rdm_handle *h, MatSet &in, MatSet &out, const JobTable &
         }
     }
     // 8-slice products leave room for the result (about the input set's size) and
-    // for the step's untruncated blocks and lists
+    // for the step's untruncated blocks (where the buffers do not have it yet)
     const size_t out_bytes = (size_t)in.total * bb * sizeof(double) * 9 / 8, out_held = out.val.cap * sizeof(double);
     const size_t grow = out_bytes > out_held ? out_bytes - out_held : 0;
-    const size_t reserve = any_oz8 ? grow + out_bytes : h->tcw.lean ? grow : 0;
+    const size_t held = h->out_val.cap * sizeof(double), slots = std::min(out_bytes, size_t(4) << 30);
+    const size_t reserve = any_oz8 ? grow + (slots > held ? slots - held : 0) : h->tcw.lean ? grow : 0;
     if (any_oz && !prepare_oz_operands(in, oz_nmat, any_oz8 ? 8 : 7, reserve, h->ozw, st)) {
         if (any_oz8) throw NoRoomForSlices{};
         // no room for the 7 slices: the FP64 pipe

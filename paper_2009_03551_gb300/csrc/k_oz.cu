@@ -28,7 +28,11 @@
 // element over the largest result (uniform, normal and decaying entries, one
 // and two terms, 3 to 96 blocks deep): 5e-17 to 1.6e-16, that of the FP64 FMA
 // chains on the same operands 4e-16 to 9e-15; in the Frobenius norm 4e-17 to
-// 1e-16 against 3e-16 to 3e-15.  (7 slices: up to 2e-13 by the test's bound.)
+// 1e-16 against 3e-16 to 3e-15.  That error is absolute: an element below 2^-9 of
+// its row's largest keeps fewer than 53 bits.  X0^2 of a 100-atom cluster, largest
+// error of a block over the block's own norm: 9e-16 for norms above 0.1, 2.3e-14
+// above 1e-3, 2.5e-11 above 1e-7, where FMA chains have 9e-16 throughout; the
+// filter (tau >= 1e-10) drops blocks of such norms.  (7 slices: up to 2e-13 by the test's bound.)
 //
 // MMAs.  The accumulators of a block column lie side by side, 32 columns per
 // group, and the slices of a B block one after another in shared memory, so
@@ -74,7 +78,8 @@
 // FP64 solve of a 300-atom cluster: products 652 ms on the FP64 pipe, 33 ms here
 // (24 TFLOP/s useful, the 2 ms of k_diag_fp64 included: the diagonal elements
 // of X0^2 keep the FMA chains' rounding, because the trace decides branches).  Bounded waits and the abort drain are those of the
-// split kernel (k_tc.cu).
+// split kernel (k_tc.cu).  ptxas: 162 registers for S = 7; 168, the bound of its
+// launch, and 196 bytes of spills for S = 8.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -686,7 +691,7 @@ bool prepare_oz_operands(const MatSet &in, int nmat, int slices, size_t reserve,
         // room for both layouts (and their headroom), or the caller's other path
         size_t fr = 0, tot = 0;
         RDM_CUDA_TRY(cudaMemGetInfo(&fr, &tot));
-        const size_t need = 5 * elems + reserve;       // 2 layouts x 2 bytes x 5/4
+        const size_t need = 4 * DevBuf<uint16_t>::with_headroom(elems) + reserve;   // 2 layouts x 2 bytes
         if (need > fr + (w.slices_a.cap + w.slices_b.cap) * sizeof(uint16_t)) return false;
     }
     w.nslice = slices;
