@@ -60,8 +60,8 @@ def tc_flops_per_kstep(b):
 PROFILED_TRAFFIC = {
     "tc": {"file": ["paper_2009_03551_gb300/csrc/k_tc.cu", "paper_2009_03551_gb300/csrc/tc_ptx.cuh",
                     "paper_2009_03551_gb300/csrc/tc_plan.cuh"],
-           "sha256": "8144a972ed0c44d892c544a9ba616a6284ee8c6341aa764fb7532f003327a28b",
-           "bytes_per_unit": 10598.0, "unit": "K-step", "b": 32,
+           "sha256": "53e9c3aca925d9d92417b223367ea841224d45593784f8b4b4926472314d1b8f",
+           "bytes_per_unit": 10605.0, "unit": "K-step", "b": 32,
            "capture": "profiles/k_tc_bf16x3_dram_cluster1000.md"},
 }
 
